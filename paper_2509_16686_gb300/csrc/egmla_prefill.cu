@@ -239,12 +239,28 @@ __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfG
 }
 
 // ============================================================================ 2. key/value up-projection
-// Each CTA owns RT tiles of 128 token rows and walks the output blocks
-// (head h, key rows or value rows) in order; every 16 KB chunk of W (128
-// output rows x 64 of d_c) that it pulls in feeds the MMAs of all RT row
-// tiles, so the weights cross into the SM once per RT x 128 tokens (the
-// weight stream, not the tensor pipe, bounds a CTA of one row tile).
+// A unit is (RT tiles of 128 token rows, output block of 128 columns: the key
+// or the value rows of a head).  The units, row tiles outermost, are cut into
+// equal contiguous ranges, one per CTA, so a short prompt's few row tiles
+// still spread over every SM and a long batch does not end in a part-filled
+// wave of whole tiles.  A CTA keeps its row tile's K chunks in shared memory
+// across the blocks of the range; where the range enters the next tile, each
+// chunk is refilled as soon as its last MMA is done.  Every 16 KB chunk of W
+// (128 output rows x 64 of d_c) feeds the MMAs of all RT row tiles.
+// Measured at d_c 256, 16 heads (kernel alone, cold caches): one whole tile per
+// CTA 52 us at 777 tokens (7 CTAs) and 109 us at 32768 (256 CTAs, two waves);
+// equal ranges and the single issuing thread below 9 us and 70 us.  Whole tiles
+// with that thread: 89 us at 32768, so the cut itself is worth 19 us there.  A
+// unit then takes about 1.3 us per SM: its 64 KB of weights and 32 KB of
+// output cross the SM's port, and its 16 MMAs take 0.83 us.
+//
+// Output: the kv buffer is kept in planes of 64 columns (plane 4 h + c:
+// k^C columns 0-63, 64-127, v^C columns 0-63, 64-127 of head h), each
+// [T, 64], so that both the boxes stored here (32 rows) and the tiles the
+// attention copies (128 rows) are contiguous runs of memory (measured no
+// faster and no slower than rows of all heads).
 constexpr int kKvFeat = kPfDn + kPfDv;                      // 256 output features per head
+constexpr int kKvPlanes = kKvFeat / kPfChunk;               // 64-column planes of a head
 constexpr int kKvBlock = 128;                               // output columns per block (key or value rows)
 constexpr uint32_t kKvBBytes = kKvBlock * kPfChunk * 2;     // 16 KB: one K chunk of a block's W rows
 constexpr int kKvMaxStages = 4;
@@ -255,8 +271,10 @@ constexpr uint32_t kKvStageOut = 32 * kPfChunk * 2;         // 4 KB
 constexpr uint32_t kKvOutBytes = kKvEpiWarps * 2 * kKvStageOut;   // 64 KB
 constexpr int kKvThreads = 32 * (2 + kKvEpiWarps);          // warp 0 TMA, warp 1 MMA
 
+constexpr int kKvMaxA = 8;   // row-tile K chunks: RT x d_c / 64
+
 struct KvBars {
-  uint64_t afull;
+  uint64_t afull[kKvMaxA], aempty[kKvMaxA];
   uint64_t bfull[kKvMaxStages], bempty[kKvMaxStages];
   uint64_t dfull[2], dfree[2];
   uint64_t drain;
@@ -265,8 +283,8 @@ struct KvBars {
 };
 
 struct KvParams {
-  __nv_bfloat16* kv;   // [T, H, 256]
-  int total, H, nkc, stages;
+  int nkc, stages;
+  long long units;     // row tiles x nblocks, shared equally by the CTAs
   // kv_mode 1: block b is the key (b even) or value (b odd) rows of head b / 2
   // from the two weight maps; kv_mode 0: block b is rows 128 b .. 128 b + 127
   // of the first map (a plain x W^T, e.g. the gate table E W^UE^T)
@@ -304,12 +322,17 @@ __global__ void __launch_bounds__(kKvThreads, 1)
   KvBars& bars = *reinterpret_cast<KvBars*>(smem + b_off + kKvStages * kKvBBytes);
   volatile int* abort_flag = &bars.abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.x * RT * kPfRows;
   const int nblocks = p.nblocks;
-  const int nsteps = nblocks * p.nkc;
+  // this CTA's units
+  const long long u0 = p.units * blockIdx.x / gridDim.x;
+  const int nunits = static_cast<int>(p.units * (blockIdx.x + 1) / gridDim.x - u0);
+  const int tile0 = static_cast<int>(u0 / nblocks), blk0 = static_cast<int>(u0 % nblocks);
 
   if (tid == 0) {
-    mbar_init(smem_u32(&bars.afull), 1);
+    for (int a = 0; a < RT * p.nkc; ++a) {
+      mbar_init(smem_u32(&bars.afull[a]), 1);
+      mbar_init(smem_u32(&bars.aempty[a]), 1);
+    }
     for (int s = 0; s < kKvStages; ++s) {
       mbar_init(smem_u32(&bars.bfull[s]), 1);
       mbar_init(smem_u32(&bars.bempty[s]), 1);
@@ -338,26 +361,52 @@ __global__ void __launch_bounds__(kKvThreads, 1)
   if (warp == 0) {
     if (elect_one()) {
       const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
-      mbar_arrive_expect_tx(smem_u32(&bars.afull), static_cast<uint32_t>(RT * p.nkc) * kPfAtom);
-      for (int t = 0; t < RT; ++t)
-        for (int kc = 0; kc < p.nkc; ++kc)
-          tma_load_2d(sbase + (t * p.nkc + kc) * kPfAtom, &cmap, kc * kPfChunk, row0 + t * kPfRows,
-                      smem_u32(&bars.afull), pol_stream);
-      int issued = 0;
-      for (int i = 0; i < nsteps; ++i) {
-        const int s = i % kKvStages;
-        if (i >= kKvStages &&
-            !mbar_wait(smem_u32(&bars.bempty[s]), ((i / kKvStages) & 1) ^ 1, abort_flag, p.wait_ns))
-          break;
-        const int blk = i / p.nkc, kc = i % p.nkc;
-        mbar_arrive_expect_tx(smem_u32(&bars.bfull[s]), kKvBBytes);
-        tma_load_2d(sbase + b_off + s * kKvBBytes, (p.kv_mode && (blk & 1)) ? &wvmap : &wkmap, kc * kPfChunk,
-                    (p.kv_mode ? blk >> 1 : blk) * kKvBlock, smem_u32(&bars.bfull[s]), pol_keep);
-        issued = i + 1;
+      int issued = 0, tiles = 0;   // W chunks and whole row tiles issued
+      uint32_t part = 0;           // chunks of the row tile being entered that are issued
+      int s = 0;
+      uint32_t ph = 0;             // phase of the weight ring's slot s
+      bool ok = true;
+      for (int u = 0, blk = blk0, tile = tile0; ok && u < nunits; ++u) {
+        const bool enter = u == 0 || blk == 0;   // the row tile's first unit here
+        for (int kc = 0; kc < p.nkc; ++kc) {
+          if (enter) {
+            // the tile's chunk kc, once the previous tile's last MMA on it is done
+            for (int t = 0; ok && t < RT; ++t) {
+              const int a = t * p.nkc + kc;
+              ok = tiles == 0 || mbar_wait(smem_u32(&bars.aempty[a]), (tiles - 1) & 1, abort_flag, p.wait_ns);
+              if (!ok) break;
+              mbar_arrive_expect_tx(smem_u32(&bars.afull[a]), kPfAtom);
+              tma_load_2d(sbase + a * kPfAtom, &cmap, kc * kPfChunk, (tile * RT + t) * kPfRows,
+                          smem_u32(&bars.afull[a]), pol_stream);
+              part |= 1u << a;
+            }
+          }
+          ok = ok && (issued < kKvStages || mbar_wait(smem_u32(&bars.bempty[s]), ph ^ 1, abort_flag, p.wait_ns));
+          if (!ok) break;
+          mbar_arrive_expect_tx(smem_u32(&bars.bfull[s]), kKvBBytes);
+          tma_load_2d(sbase + b_off + s * kKvBBytes, (p.kv_mode && (blk & 1)) ? &wvmap : &wkmap, kc * kPfChunk,
+                      (p.kv_mode ? blk >> 1 : blk) * kKvBlock, smem_u32(&bars.bfull[s]), pol_keep);
+          ++issued;
+          if (++s == kKvStages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+        if (ok && enter) {
+          ++tiles;
+          part = 0;
+        }
+        if (++blk == nblocks) {
+          blk = 0;
+          ++tile;
+        }
       }
       // every copy issued lands before the CTA can leave
       volatile int own = 0;
-      if (!mbar_wait(smem_u32(&bars.afull), 0, &own, p.wait_ns)) *abort_flag = 1;
+      for (int a = 0; a < RT * p.nkc; ++a) {
+        const int n = tiles + ((part >> a) & 1);
+        if (n > 0 && !mbar_wait(smem_u32(&bars.afull[a]), (n - 1) & 1, &own, p.wait_ns)) *abort_flag = 1;
+      }
       for (int i = issued > kKvStages ? issued - kKvStages : 0; i < issued; ++i)
         if (!mbar_wait(smem_u32(&bars.bfull[i % kKvStages]), (i / kKvStages) & 1, &own, p.wait_ns))
           *abort_flag = 1;
@@ -365,38 +414,54 @@ __global__ void __launch_bounds__(kKvThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     constexpr uint32_t idesc = idesc_bf16(kPfRows, kKvBlock, 0, 0);
-    bool ok = pf_warp_wait(smem_u32(&bars.afull), 0, abort_flag, p.wait_ns);
-    bool issued = false;
-    for (int blk = 0; ok && blk < nblocks; ++blk) {
-      const int db = blk & 1;
-      if (blk >= 2) ok = pf_warp_wait(smem_u32(&bars.dfree[db]), ((blk - 2) >> 1) & 1, abort_flag, p.wait_ns);
-      for (int kc = 0; ok && kc < p.nkc; ++kc) {
-        const int i = blk * p.nkc + kc, s = i % kKvStages;
-        ok = pf_warp_wait(smem_u32(&bars.bfull[s]), (i / kKvStages) & 1, abort_flag, p.wait_ns);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
+    // One thread waits and issues, and the ring's slot and phase are stepped,
+    // not divided out: what lies between two chunks' MMAs adds to the kernel's
+    // period (a whole warp that waits, votes and elects per chunk, with the
+    // divisions, took 135 us where this takes 89: whole tiles, 32768 tokens).
+    if (elect_one()) {
+      bool ok = true, issued = false;
+      int s = 0;
+      uint32_t ph = 0, aph = 0;   // phases of the weight ring's slot s and of the row tile's chunks
+      for (int u = 0, blk = blk0; ok && u < nunits; ++u) {
+        const int db = u & 1;
+        const bool enter = u == 0 || blk == 0;
+        const bool leave = blk == nblocks - 1;   // the tile's last unit: its chunks may be refilled
+        const uint32_t d = tmem + db * (RT * kKvBlock);
+        if (u >= 2) ok = mbar_wait(smem_u32(&bars.dfree[db]), ((u - 2) >> 1) & 1, abort_flag, p.wait_ns);
+        for (int kc = 0; ok && kc < p.nkc; ++kc) {
+          if (enter)
+            for (int t = 0; ok && t < RT; ++t)
+              ok = mbar_wait(smem_u32(&bars.afull[t * p.nkc + kc]), aph, abort_flag, p.wait_ns);
+          ok = ok && mbar_wait(smem_u32(&bars.bfull[s]), ph, abort_flag, p.wait_ns);
+          if (!ok) break;
+          tc_fence_after();
           const uint64_t bd = smem_desc(sbase + b_off + s * kKvBBytes, 16, 1024, kSwizzle128B);
 #pragma unroll
           for (int t = 0; t < RT; ++t) {
             const uint64_t ad = smem_desc(sbase + (t * p.nkc + kc) * kPfAtom, 16, 1024, kSwizzle128B);
 #pragma unroll
             for (int kk = 0; kk < kPfChunk / 16; ++kk)
-              mma_bf16_ss(tmem + db * (RT * kKvBlock) + t * kKvBlock, ad + ((kk * 32) >> 4), bd + ((kk * 32) >> 4),
-                          idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+              mma_bf16_ss(d + t * kKvBlock, ad + ((kk * 32) >> 4), bd + ((kk * 32) >> 4), idesc,
+                          (kc > 0 || kk > 0) ? 1u : 0u);
           }
           mma_commit(smem_u32(&bars.bempty[s]));
-          if (kc == p.nkc - 1) mma_commit(smem_u32(&bars.dfull[db]));
+          if (leave)
+            for (int t = 0; t < RT; ++t) mma_commit(smem_u32(&bars.aempty[t * p.nkc + kc]));
+          issued = true;
+          if (++s == kKvStages) {
+            s = 0;
+            ph ^= 1;
+          }
         }
-        __syncwarp();
-        issued = true;
+        if (ok) mma_commit(smem_u32(&bars.dfull[db]));
+        if (leave) aph ^= 1;
+        if (++blk == nblocks) blk = 0;
       }
-    }
-    if (issued) {
-      if (elect_one()) mma_commit(smem_u32(&bars.drain));
-      __syncwarp();
-      volatile int own = 0;
-      if (!mbar_wait(smem_u32(&bars.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
+      if (issued) {
+        mma_commit(smem_u32(&bars.drain));
+        volatile int own = 0;
+        if (!mbar_wait(smem_u32(&bars.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
+      }
     }
     __syncwarp();
   } else {
@@ -409,14 +474,14 @@ __global__ void __launch_bounds__(kKvThreads, 1)
     const int t = RT == 2 ? g : 0;
     constexpr int kCols = RT == 2 ? kKvBlock : kKvBlock / 2;
     const int cbase = RT == 2 ? 0 : g * kCols;
-    const int y0 = row0 + t * kPfRows + 32 * quad;           // the warp's first token row
     const uint32_t stg = sbase + o_off + (warp - 2) * 2 * kKvStageOut;
     const uint32_t rowoff = (lane >> 3) * 1024 + (lane & 7) * 128;
     bool ok = true;
     int nst = 0;   // boxes stored so far (buffer nst % 2)
-    for (int blk = 0; blk < nblocks; ++blk) {
-      const int db = blk & 1;
-      ok = ok && pf_warp_wait(smem_u32(&bars.dfull[db]), (blk >> 1) & 1, abort_flag, p.wait_ns);
+    for (int u = 0, blk = blk0, tile = tile0; u < nunits; ++u) {
+      const int db = u & 1;
+      const int y0 = (tile * RT + t) * kPfRows + 32 * quad;   // the warp's first token row
+      ok = ok && pf_warp_wait(smem_u32(&bars.dfull[db]), (u >> 1) & 1, abort_flag, p.wait_ns);
       if (!ok) break;
       tc_fence_after();
 #pragma unroll
@@ -442,14 +507,18 @@ __global__ void __launch_bounds__(kKvThreads, 1)
         if (lane == 0) {
           // every chunk commits a group (possibly empty), so the buffer
           // rotation above stays in step
-          if (blk * kKvBlock + cbase + c0 < p.out_cols)
-            tma_store_2d(&omap, blk * kKvBlock + cbase + c0, y0, stg + (nst & 1) * kKvStageOut);
+          const int col = blk * kKvBlock + cbase + c0;
+          if (col < p.out_cols) tma_store_3d(&omap, 0, y0, col / kPfChunk, stg + (nst & 1) * kKvStageOut);
           bulk_commit_group();
         }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars.dfree[db]));
+      if (++blk == nblocks) {
+        blk = 0;
+        ++tile;
+      }
     }
     if (lane == 0) bulk_wait_group_all();
     __syncwarp();
@@ -652,8 +721,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             }
             mbar_arrive_expect_tx(smem_u32(&bars.kfull[s]), kPfAtom);
             if (c < 2)
-              tma_load_2d(sbase + kOffK + s * kPfAtom, &kvmap, it.h * kKvFeat + c * kPfChunk, y,
-                          smem_u32(&bars.kfull[s]), pol_k);
+              tma_load_3d(sbase + kOffK + s * kPfAtom, &kvmap, 0, y, it.h * kKvPlanes + c, smem_u32(&bars.kfull[s]),
+                          pol_k);
             else
               tma_load_2d(sbase + kOffK + s * kPfAtom, &krmap, 0, y, smem_u32(&bars.kfull[s]), pol_k);
           }
@@ -692,9 +761,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           const int y = it.start + j * kAttnKeys;
           const uint32_t dst = sbase + kOffV + s * kAttnVBytes;
           mbar_arrive_expect_tx(smem_u32(&bars.vfull[s]), kAttnVBytes);
-          tma_load_2d(dst, &kvmap, it.h * kKvFeat + kPfDn, y, smem_u32(&bars.vfull[s]), pol_v);
-          tma_load_2d(dst + kPfAtom, &kvmap, it.h * kKvFeat + kPfDn + kPfChunk, y, smem_u32(&bars.vfull[s]),
-                      pol_v);
+          tma_load_3d(dst, &kvmap, 0, y, it.h * kKvPlanes + 2, smem_u32(&bars.vfull[s]), pol_v);
+          tma_load_3d(dst + kPfAtom, &kvmap, 0, y, it.h * kKvPlanes + 3, smem_u32(&bars.vfull[s]), pol_v);
         }
       }
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
@@ -938,16 +1006,32 @@ EncodeFn pf_encode_fn() {
   return fn;
 }
 
+// bf16 planes of [rows, 64] with row stride `ld` and plane stride `plane`
+// elements; boxes of 64 columns x box_rows rows of one plane, 128-byte swizzle,
+// rows past the end read as zero and are not written
+bool pf_encode_planes(CUtensorMap* map, const void* base, uint64_t rows, uint64_t ld, uint64_t planes, uint64_t plane,
+                      uint32_t box_rows) {
+  EncodeFn enc = pf_encode_fn();
+  if (enc == nullptr) return false;
+  std::memset(map, 0, sizeof(*map));
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(kPfChunk), rows, planes};
+  const cuuint64_t strides[2] = {ld * 2, plane * 2};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(kPfChunk), box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // row-major bf16 [rows, cols] with row stride `ld` elements; boxes of 64
-// columns x box_rows rows, 128-byte swizzle, rows past the end read as zero
-bool pf_encode(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
-               uint32_t box_rows = kPfRows) {
+// columns x 128 rows, 128-byte swizzle, rows past the end read as zero
+bool pf_encode(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld) {
   EncodeFn enc = pf_encode_fn();
   if (enc == nullptr) return false;
   std::memset(map, 0, sizeof(*map));
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {ld * 2};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(kPfChunk), box_rows};
+  const cuuint32_t box[2] = {static_cast<cuuint32_t>(kPfChunk), static_cast<cuuint32_t>(kPfRows)};
   const cuuint32_t estr[2] = {1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1022,22 +1106,22 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
-  // 2. keys and values of every head: one 128-row tile per CTA.  Its output
-  // stores and its weight copies bound it about equally per SM, so spreading
-  // the stores over more CTAs beats reading the weights fewer times (measured:
-  // two tiles per CTA took 114 us against 109 at 8 x 4096)
+  // 2. keys and values of every head: the units shared equally by one CTA per SM
   CUtensorMap cmap, wkmap, wvmap;
   if (!pf_encode(&cmap, ctil, a.total, a.d_c, a.d_c)) return cudaErrorInvalidValue;
   if (!pf_encode(&wkmap, a.w_uk, static_cast<uint64_t>(a.H) * kPfDn, a.d_c, a.d_c)) return cudaErrorInvalidValue;
   if (!pf_encode(&wvmap, a.w_uv, static_cast<uint64_t>(a.H) * kPfDv, a.d_c, a.d_c)) return cudaErrorInvalidValue;
   const int nkc = a.d_c / kPfChunk;
-  CUtensorMap omap;   // the kv buffer, stored in boxes of 64 columns x 32 rows
-  if (!pf_encode(&omap, kv, a.total, static_cast<uint64_t>(a.H) * kKvFeat, static_cast<uint64_t>(a.H) * kKvFeat, 32))
-    return cudaErrorInvalidValue;
+  // the kv buffer's planes: stored 32 rows, read 128 rows at a time
+  const uint64_t planes = static_cast<uint64_t>(a.H) * kKvPlanes, plane = static_cast<uint64_t>(a.total) * kPfChunk;
+  CUtensorMap omap, kvmap;
+  if (!pf_encode_planes(&omap, kv, a.total, kPfChunk, planes, plane, 32)) return cudaErrorInvalidValue;
+  if (!pf_encode_planes(&kvmap, kv, a.total, kPfChunk, planes, plane, kPfRows)) return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   KvParams kp;
-  kp.kv = kv;
-  kp.total = a.total;
-  kp.H = a.H;
   kp.nkc = nkc;
   kp.wait_ns = kWaitLimitNs;
   kp.status = a.status;
@@ -1049,17 +1133,16 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
     const int kv_smem = static_cast<int>(kv_smem_bytes<1>(nkc));
     e = cudaFuncSetAttribute(prefill_kv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kv_smem);
     if (e != cudaSuccess) return e;
-    prefill_kv_kernel<1><<<(a.total + kPfRows - 1) / kPfRows, kKvThreads, kv_smem, st>>>(cmap, wkmap, wvmap, omap,
-                                                                                         kp);
+    kp.units = static_cast<long long>((a.total + kPfRows - 1) / kPfRows) * kp.nblocks;
+    const int grid = static_cast<int>(kp.units < sms ? kp.units : sms);
+    prefill_kv_kernel<1><<<grid, kKvThreads, kv_smem, st>>>(cmap, wkmap, wvmap, omap, kp);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
   // 3. causal attention
-  CUtensorMap qmap, kvmap, krmap;
+  CUtensorMap qmap, krmap;
   if (!pf_encode(&qmap, a.q, a.total, static_cast<uint64_t>(a.H) * kPfDqk, static_cast<uint64_t>(a.H) * kPfDqk))
-    return cudaErrorInvalidValue;
-  if (!pf_encode(&kvmap, kv, a.total, static_cast<uint64_t>(a.H) * kKvFeat, static_cast<uint64_t>(a.H) * kKvFeat))
     return cudaErrorInvalidValue;
   if (!pf_encode(&krmap, a.kr, a.total, kPfDr, kPfDr)) return cudaErrorInvalidValue;
   e = cudaFuncSetAttribute(prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1081,10 +1164,6 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   const long long items = static_cast<long long>(a.batch) * a.H * ap.qblocks;
   if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
   ap.items = static_cast<int>(items);
-  int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
   const int grid = static_cast<int>(items < sms ? items : sms);
   if (mark) mark(st, true);
   prefill_attn_kernel<<<grid, kAttnThreads, kAttnSmem, st>>>(qmap, kvmap, krmap, ap);
@@ -1099,12 +1178,9 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
   CUtensorMap amap, wmap, omap;
   if (!pf_encode(&amap, emb, vocab, d_e, d_e)) return cudaErrorInvalidValue;
   if (!pf_encode(&wmap, w_ue, d_c, d_e, d_e)) return cudaErrorInvalidValue;
-  if (!pf_encode(&omap, table, vocab, d_c, d_c, 32)) return cudaErrorInvalidValue;
+  if (!pf_encode_planes(&omap, table, vocab, d_c, d_c / kPfChunk, kPfChunk, 32)) return cudaErrorInvalidValue;
   const int nkc = d_e / kPfChunk;
   KvParams kp;
-  kp.kv = static_cast<__nv_bfloat16*>(table);
-  kp.total = vocab;
-  kp.H = 0;
   kp.nkc = nkc;
   kp.wait_ns = kWaitLimitNs;
   kp.status = status;
@@ -1117,14 +1193,17 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
     const int smem = static_cast<int>(kv_smem_bytes<2>(nkc));
     e = cudaFuncSetAttribute(prefill_kv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    prefill_kv_kernel<2><<<(vocab + 2 * kPfRows - 1) / (2 * kPfRows), kKvThreads, smem, st>>>(amap, wmap, wmap, omap,
-                                                                                              kp);
+    const int tiles = (vocab + 2 * kPfRows - 1) / (2 * kPfRows);
+    kp.units = static_cast<long long>(tiles) * kp.nblocks;   // whole tiles: a table row's few blocks share its copy
+    prefill_kv_kernel<2><<<tiles, kKvThreads, smem, st>>>(amap, wmap, wmap, omap, kp);
   } else {
     kp.stages = kv_stages<1>(nkc);
     const int smem = static_cast<int>(kv_smem_bytes<1>(nkc));
     e = cudaFuncSetAttribute(prefill_kv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    prefill_kv_kernel<1><<<(vocab + kPfRows - 1) / kPfRows, kKvThreads, smem, st>>>(amap, wmap, wmap, omap, kp);
+    const int tiles = (vocab + kPfRows - 1) / kPfRows;
+    kp.units = static_cast<long long>(tiles) * kp.nblocks;
+    prefill_kv_kernel<1><<<tiles, kKvThreads, smem, st>>>(amap, wmap, wmap, omap, kp);
   }
   return cudaGetLastError();
 }

@@ -78,6 +78,31 @@ def test_prefill_matches_oracle(gpu_lib, name):
     check_close(got, orc.prefill(pc), positions_of(pc))
 
 
+@pytest.mark.parametrize("heads,d_c,prompts,length", [(1, 128, 310, 71), (3, 192, 41, 150), (2, 512, 61, 130)])
+def test_prefill_packed_prompts_equal_each_prompt_alone(gpu_lib, heads, d_c, prompts, length):
+    """Row tiles x output blocks of the up-projection that are no multiple of
+    the SMs: a CTA's range of them starts and ends inside a tile and enters one
+    or two more.  No row's arithmetic depends on where the ranges are cut, so
+    every prompt's rows are bit for bit those of a call with that prompt alone
+    (which the tests above hold to the oracle)."""
+    dims = synth.Dims(num_heads=heads, d_nope=128, d_rope=64, d_v=128, d_c=d_c, page_size=64, vocab=500,
+                      dtype="bf16")
+    pc = synth.make_prefill_case("packed", dims, [length] * prompts, seed=69, affine_ln=True)
+    dp, _ = run(pc)
+    assert dp.read_status() == 0
+    one = device.upload_prefill(synth.make_prefill_case("one", dims, [length], seed=69))
+    for name in ("gate_table", "ln_gamma", "ln_beta", "w_uk", "w_uv"):
+        setattr(one, name, getattr(dp, name))
+    for b in range(0, prompts, 3):
+        rows = slice(b * length, (b + 1) * length)
+        for name in ("q", "c", "kr", "ids"):
+            getattr(one, name).copy_(getattr(dp, name)[rows])
+        one.out.fill_(float("nan"))
+        one.run(write_cache=False)
+        assert torch.equal(one.out, dp.out[rows]), b
+    assert one.read_status() == 0
+
+
 def test_prefill_cache_write_is_bit_exact(gpu_lib):
     pc = synth.make_prefill_case("pool", synth.dims_bf16(d_c=192, vocab=3000), [70, 0, 129, 1], seed=62,
                                  extra_pages=4)
