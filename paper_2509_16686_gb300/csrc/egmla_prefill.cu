@@ -579,7 +579,8 @@ struct AttnBars {
   uint64_t qfull, qempty;
   uint64_t kfull[kAttnKSlots], kempty[kAttnKSlots];
   uint64_t vfull[kAttnVStages], vempty[kAttnVStages];
-  uint64_t sfull[2], pfull[2], odone[2], ofree[2];   // per query tile
+  uint64_t sfull[2], odone[2], ofree[2];   // per query tile
+  uint64_t pfull[2][2];                    // per query tile, halves of 64 keys
   uint64_t ifull[2], iempty[2];                      // the work-item ring
   uint64_t drain;
   AttnItem item[2];
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(smem_u32(&bars.sfull[x]), 1);
-      mbar_init(smem_u32(&bars.pfull[x]), 4);
+      for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&bars.pfull[x][h]), 4);
       mbar_init(smem_u32(&bars.odone[x]), 1);
       mbar_init(smem_u32(&bars.ofree[x]), 4);
       mbar_init(smem_u32(&bars.ifull[x]), 1);
@@ -784,91 +785,92 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // V [keys x features] is the B operand MN-major: 64-feature atoms 16 KB
     // apart, 8-key groups 1 KB apart
     const uint64_t vdesc = smem_desc(sbase + kOffV, kPfAtom, 1024, kSwizzle128B);
-    bool ok = true, issued = false;
-    int g0 = 0, v0 = 0;              // first key chunk and value tile of the item
-    int tx[2] = {0, 0};              // tiles of query tile X before this item
-    int kx[2] = {0, 0};              // items in which query tile X had rows
-    int kseen = -1;                  // the last key chunk whose arrival was waited for
-    for (int n = 0; ok; ++n) {
-      AttnItem it;
-      if (!read_item(n, it, true) || it.b < 0) break;
-      int ntile[2];
-      tiles_of(it, ntile);
-      const int nkt = ntile[1] > 0 ? ntile[1] : ntile[0];
-      ok = pf_warp_wait(smem_u32(&bars.qfull), n & 1, abort_flag, p.wait_ns);
-      auto wait_k = [&](int g) {
-        if (kseen < g) {
-          ok = ok && pf_warp_wait(smem_u32(&bars.kfull[g % kAttnKSlots]), (g / kAttnKSlots) & 1, abort_flag,
-                                  p.wait_ns);
-          kseen = g;
-        }
-      };
-      // O_X += P_X(i) V(i); the last reader of V(i) frees it, the last PV of X signals its epilogue
-      auto issue_pv = [&](int x, int i) {
-        const int vi = v0 + i, vs = vi % kAttnVStages;
-        if (x == 0 || ntile[0] <= i)   // first reader of V(i)
-          ok = ok && pf_warp_wait(smem_u32(&bars.vfull[vs]), (vi / kAttnVStages) & 1, abort_flag, p.wait_ns);
-        // the first PV MMA of X in this item overwrites O_X: its last item's epilogue has read it
-        if (i == 0 && kx[x] >= 1)
-          ok = ok && pf_warp_wait(smem_u32(&bars.ofree[x]), (kx[x] - 1) & 1, abort_flag, p.wait_ns);
-        ok = ok && pf_warp_wait(smem_u32(&bars.pfull[x]), (tx[x] + i) & 1, abort_flag, p.wait_ns);
-        if (!ok) return;
-        tc_fence_after();
-        if (elect_one()) {
+    // one thread waits and issues (no warp-wide wait, vote or election between MMAs)
+    if (elect_one()) {
+      bool ok = true, issued = false;
+      int g0 = 0, v0 = 0;              // first key chunk and value tile of the item
+      int tx[2] = {0, 0};              // tiles of query tile X before this item
+      int kx[2] = {0, 0};              // items in which query tile X had rows
+      int kseen = -1;                  // the last key chunk whose arrival was waited for
+      for (int n = 0; ok; ++n) {
+        if (!mbar_wait(smem_u32(&bars.ifull[n & 1]), (n >> 1) & 1, abort_flag, p.wait_ns)) break;
+        const AttnItem it = bars.item[n & 1];
+        mbar_arrive(smem_u32(&bars.iempty[n & 1]));
+        if (it.b < 0) break;
+        int ntile[2];
+        tiles_of(it, ntile);
+        const int nkt = ntile[1] > 0 ? ntile[1] : ntile[0];
+        ok = mbar_wait(smem_u32(&bars.qfull), n & 1, abort_flag, p.wait_ns);
+        // O_X += P_X(i) V(i); the last reader of V(i) frees it, the last PV of X signals its epilogue
+        auto issue_pv = [&](int x, int i) {
+          const int vi = v0 + i, vs = vi % kAttnVStages;
+          if (x == 0 || ntile[0] <= i)   // first reader of V(i)
+            ok = mbar_wait(smem_u32(&bars.vfull[vs]), (vi / kAttnVStages) & 1, abort_flag, p.wait_ns);
+          // the first PV MMA of X in this item overwrites O_X: its last item's epilogue has read it
+          if (i == 0 && kx[x] >= 1)
+            ok = ok && mbar_wait(smem_u32(&bars.ofree[x]), (kx[x] - 1) & 1, abort_flag, p.wait_ns);
           const uint64_t vd = vdesc + ((vs * kAttnVBytes) >> 4);
-          // A = P_X from tensor memory: 16 keys per MMA are 8 columns of bf16 pairs
+          // A = P_X from tensor memory: 16 keys per MMA are 8 columns of bf16
+          // pairs; the first 64 keys' MMAs run while the softmax does the others
 #pragma unroll
-          for (int ks = 0; ks < kAttnKeys / 16; ++ks)
-            mma_bf16_ts(tmem + col_o(x), tmem + col_s(x) + ks * 8, vd + ((ks * 2048) >> 4), idesc_o,
-                        (i > 0 || ks > 0) ? 1u : 0u);
+          for (int h = 0; h < 2; ++h) {
+            ok = ok && mbar_wait(smem_u32(&bars.pfull[x][h]), (tx[x] + i) & 1, abort_flag, p.wait_ns);
+            if (!ok) return;
+            tc_fence_after();
+#pragma unroll
+            for (int ks = 4 * h; ks < 4 * h + 4; ++ks)
+              mma_bf16_ts(tmem + col_o(x), tmem + col_s(x) + ks * 8, vd + ((ks * 2048) >> 4), idesc_o,
+                          (i > 0 || ks > 0) ? 1u : 0u);
+            issued = true;
+          }
           if (x == 1 || ntile[1] <= i) mma_commit(smem_u32(&bars.vempty[vs]));
           if (i == ntile[x] - 1) mma_commit(smem_u32(&bars.odone[x]));
-        }
-        __syncwarp();
-        issued = true;
-      };
-      auto issue_s = [&](int x, int j) {
-        const uint64_t qd = qdesc + ((x * kAttnQBytes) >> 4);
-        // the last reader of a key chunk (B, or A when B has no tile j) frees its slot
-        const bool last_reader = x == 1 || ntile[1] <= j;
-        for (int c = 0; c < 3; ++c) {
-          const int g = g0 + 3 * j + c, s = g % kAttnKSlots;
-          wait_k(g);
-          if (!ok) return;
-          tc_fence_after();
-          if (elect_one()) {
+        };
+        auto issue_s = [&](int x, int j) {
+          const uint64_t qd = qdesc + ((x * kAttnQBytes) >> 4);
+          // the last reader of a key chunk (B, or A when B has no tile j) frees its slot
+          const bool last_reader = x == 1 || ntile[1] <= j;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const int g = g0 + 3 * j + c, s = g % kAttnKSlots;
+            if (kseen < g) {
+              ok = mbar_wait(smem_u32(&bars.kfull[s]), (g / kAttnKSlots) & 1, abort_flag, p.wait_ns);
+              kseen = g;
+            }
+            if (!ok) return;
+            tc_fence_after();
             const uint64_t kd = kdesc + ((s * kPfAtom) >> 4);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
               mma_bf16_ss(tmem + col_s(x), qd + ((c * kPfAtom + kk * 32) >> 4), kd + ((kk * 32) >> 4), idesc_s,
                           (c > 0 || kk > 0) ? 1u : 0u);
+            issued = true;
             if (c == 2) mma_commit(smem_u32(&bars.sfull[x]));
             if (last_reader) mma_commit(smem_u32(&bars.kempty[s]));
             // the item's last score MMAs done: the query tiles may be refilled
             if (c == 2 && last_reader && j == nkt - 1) mma_commit(smem_u32(&bars.qempty));
           }
-          __syncwarp();
+        };
+        for (int j = 0; ok && j <= nkt; ++j) {
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            if (ok && j >= 1 && j - 1 < ntile[x]) issue_pv(x, j - 1);
+            if (ok && j < ntile[x]) issue_s(x, j);
+          }
         }
-        issued = true;
-      };
-      for (int j = 0; ok && j <= nkt; ++j) {
-        for (int x = 0; ok && x < 2; ++x) {
-          if (j >= 1 && j - 1 < ntile[x]) issue_pv(x, j - 1);
-          if (ok && j < ntile[x]) issue_s(x, j);
+        g0 += 3 * nkt;
+        v0 += nkt;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          tx[x] += ntile[x];
+          if (ntile[x] > 0) ++kx[x];
         }
       }
-      g0 += 3 * nkt;
-      v0 += nkt;
-      for (int x = 0; x < 2; ++x) {
-        tx[x] += ntile[x];
-        if (ntile[x] > 0) ++kx[x];
+      if (issued) {
+        mma_commit(smem_u32(&bars.drain));
+        volatile int own = 0;
+        if (!mbar_wait(smem_u32(&bars.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
       }
-    }
-    if (issued) {
-      if (elect_one()) mma_commit(smem_u32(&bars.drain));
-      __syncwarp();
-      volatile int own = 0;
-      if (!mbar_wait(smem_u32(&bars.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
     }
     __syncwarp();
   } else {
@@ -906,15 +908,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           for (int c = 0; c < kAttnKeys; ++c)
             if (k0 + c > qrow) sv[c] = -INFINITY;
         }
-        // row maximum and sum as eight interleaved chains (short dependencies)
+        // row maximum and sum as interleaved chains (short dependencies)
         float m8[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) m8[e] = sv[e];
 #pragma unroll
-        for (int c = 8; c < kAttnKeys; ++c) m8[c & 7] = fmaxf(m8[c & 7], sv[c]);
-        float mx =
-            fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])), fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
-        mx *= sl2;
+        for (int c = 8; c < kAttnKeys; c += 16)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            m8[e] = c + 8 < kAttnKeys ? fmaxf(fmaxf(m8[e], sv[c + e]), sv[(c + 8 + e) % kAttnKeys])
+                                      : fmaxf(m8[e], sv[c + e]);
+        float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), m8[2]), fmaxf(fmaxf(m8[3], m8[4]), m8[5]));
+        mx = fmaxf(fmaxf(mx, m8[6]), m8[7]) * sl2;
         float alpha = 1.f;
         if (j == 0) {
           m_ref = mx;
@@ -922,17 +927,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
           alpha = pf_ex2(m_ref - mx);
           m_ref = mx;
         }
-        float pk[kAttnKeys / 2];   // bf16 pairs, kept as 32-bit words for the TMEM store
-        float r8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int c = 0; c < kAttnKeys; c += 2) {
-          const float p0 = pf_ex2(fmaf(sv[c], sl2, -m_ref));
-          const float p1 = pf_ex2(fmaf(sv[c + 1], sl2, -m_ref));
-          r8[(c >> 1) & 7] += p0 + p1;
-          pk[c / 2] = __uint_as_float(pack_bf16x2(p0, p1));
-        }
-        const float rs = ((r8[0] + r8[1]) + (r8[2] + r8[3])) + ((r8[4] + r8[5]) + (r8[6] + r8[7]));
-        l = fmaf(l, alpha, rs);
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
 #pragma unroll
           for (int c = 0; c < kPfDv; c += 16) {
@@ -944,14 +938,31 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             tmem_st16(lane_base + col_o(x) + c, o);
           }
         }
-        // P_X over the first 64 columns of S_X
+        // P_X over the first 64 columns of S_X, each half of 64 keys handed to
+        // the PV MMAs as soon as it is written
+        const float2 sl2v = make_float2(sl2, sl2), mrv = make_float2(-m_ref, -m_ref);
+        float2 r4[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
-        for (int c = 0; c < kAttnKeys / 2; c += 16)
-          tmem_st16(lane_base + col_s(x) + c, *reinterpret_cast<const float(*)[16]>(&pk[c]));
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars.pfull[x]));
+        for (int h = 0; h < 2; ++h) {
+          float pk[kAttnKeys / 4];   // bf16 pairs, kept as 32-bit words for the TMEM store
+#pragma unroll
+          for (int i = 0; i < kAttnKeys / 4; ++i) {
+            const int c = h * (kAttnKeys / 2) + 2 * i;
+            const float2 e = __ffma2_rn(make_float2(sv[c], sv[c + 1]), sl2v, mrv);
+            const float2 pr = make_float2(pf_ex2(e.x), pf_ex2(e.y));
+            r4[i & 3] = __fadd2_rn(r4[i & 3], pr);
+            pk[i] = __uint_as_float(pack_bf16x2(pr.x, pr.y));
+          }
+#pragma unroll
+          for (int c = 0; c < kAttnKeys / 4; c += 16)
+            tmem_st16(lane_base + col_s(x) + h * (kAttnKeys / 4) + c, *reinterpret_cast<const float(*)[16]>(&pk[c]));
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bars.pfull[x][h]));
+        }
+        const float2 rs2 = __fadd2_rn(__fadd2_rn(r4[0], r4[1]), __fadd2_rn(r4[2], r4[3]));
+        l = fmaf(l, alpha, rs2.x + rs2.y);
       }
       // ---- epilogue: O_X / l of the live rows, then O_X is free for the next item
       if (ok) ok = pf_warp_wait(smem_u32(&bars.odone[x]), kx & 1, abort_flag, p.wait_ns);
