@@ -201,8 +201,8 @@ int eg_mla_decode(const eg_mla_dims* dims, const void* q, const void* c_pool,
  * checked before anything is launched; host errors return the same codes as
  * the two calls, device errors go to *dev_status.
  *
- * On the bf16 path the append runs inside the grid of the query-absorption
- * kernel (which reads no pool), one launch fewer per step; the split-KV
+ * The append runs inside the grid of the query-absorption kernel (which
+ * reads no pool), one launch fewer per step; on the bf16 path the split-KV
  * kernel starts its setup while that kernel finishes and waits for its
  * completion before it reads the cache.
  */

@@ -348,8 +348,7 @@ int fill_append_args(egmla::AppendArgs& a, const eg_mla_dims* dims, void* c_pool
 }
 
 // eg_mla_decode, preceded by the append of `app` when it is non-null (in the
-// query-absorption kernel's grid on the tensor-core path; as its own launch
-// otherwise).  Every argument is checked before anything is launched.
+// query-absorption kernel's grid).  Every argument is checked before anything is launched.
 int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, const void* krope_pool,
                 const int32_t* id_pool, const int32_t* block_table, int32_t max_pages_per_seq,
                 const int32_t* seq_lens, int32_t max_seq_len, int32_t batch, int32_t num_pages,
@@ -386,8 +385,7 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
     if (e == cudaSuccess && !fused) e = egmla::launch_combine(a, true, st);
     return to_status(e);
   }
-  cudaError_t e = app != nullptr ? egmla::launch_append(*app, st) : cudaSuccess;
-  if (e == cudaSuccess) e = egmla::launch_decode_f32(a, st);
+  cudaError_t e = egmla::launch_decode_f32(a, app, st);
   if (e == cudaSuccess) e = egmla::launch_combine(a, false, st);
   return to_status(e);
 }

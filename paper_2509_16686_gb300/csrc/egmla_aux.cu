@@ -351,29 +351,80 @@ __global__ void prologue_tc_kernel(const __nv_bfloat16* __restrict__ q, const __
   }
 }
 
-// fp32 path: q^ [H, d_c] and q^R [H, d_rope] in fp32, row-major.
-__global__ void prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
-                                    const int32_t* __restrict__ seq_lens, int batch, int H, int d_nope,
-                                    int d_rope, int d_c, int page_size, uint8_t* __restrict__ qprep,
-                                    size_t qstride, int32_t* __restrict__ cu) {
-  __shared__ float qn[256];
-  if (blockIdx.x == static_cast<unsigned>(batch * H)) {
+// fp32 path: q^ [H, d_c] and q^R [H, d_rope] in fp32, row-major.  Block 0: the
+// page prefix sums; then one block per (head, 64 features, group of up to
+// kPfBatch sequences); then the append blocks of a step.  A thread takes four
+// features of W_UK,h and every 16th of its d_nope rows, each row loaded once
+// for all the group's sequences with no load depending on another; the 16
+// parts of a sum are added in shared memory.  Bound by the latency of one
+// round of loads: 17.5 us for 8 sequences when a thread walked all of d_nope
+// for one sequence, 9 us now (ncu, cold caches).
+constexpr int kPfBatch = 8, kPfFeat = 64, kPfParts = 16;
+
+__global__ void __launch_bounds__(256)
+prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk, const int32_t* __restrict__ seq_lens,
+                    int batch, int H, int d_nope, int d_rope, int d_c, int page_size, uint8_t* __restrict__ qprep,
+                    size_t qstride, int32_t* __restrict__ cu, const AppendArgs app) {
+  __shared__ float qn[kPfBatch][256];
+  __shared__ __align__(16) float red[kPfParts][kPfBatch][kPfFeat];
+  const int nfc = (d_c + kPfFeat - 1) / kPfFeat, nbg = (batch + kPfBatch - 1) / kPfBatch;
+  const int nabs = H * nfc * nbg;
+  if (blockIdx.x == 0) {
     page_prefix_sums(seq_lens, batch, page_size, cu);
     return;
   }
-  const int b = blockIdx.x / H, h = blockIdx.x % H;
-  const float* qv = q + (static_cast<size_t>(b) * H + h) * (d_nope + d_rope);
-  for (int n = threadIdx.x; n < d_nope; n += blockDim.x) qn[n] = qv[n];
-  __syncthreads();
-  float* qh = reinterpret_cast<float*>(qprep + static_cast<size_t>(b) * qstride);
-  const float* w = w_uk + static_cast<size_t>(h) * d_nope * d_c;
-  for (int f = threadIdx.x; f < d_c; f += blockDim.x) {
-    float acc = 0.f;
-    for (int n = 0; n < d_nope; ++n) acc = fmaf(w[static_cast<size_t>(n) * d_c + f], qn[n], acc);
-    qh[static_cast<size_t>(h) * d_c + f] = acc;
+  if (blockIdx.x > static_cast<unsigned>(nabs)) {   // no block of this kernel reads the pools
+    append_row(app, blockIdx.x - (nabs + 1));
+    return;
   }
-  float* qr = qh + static_cast<size_t>(H) * d_c;
-  for (int r = threadIdx.x; r < d_rope; r += blockDim.x) qr[static_cast<size_t>(h) * d_rope + r] = qv[d_nope + r];
+  const int item = static_cast<int>(blockIdx.x) - 1;
+  const int h = item % H, fc = (item / H) % nfc, b0 = (item / (H * nfc)) * kPfBatch;
+  const int nb = min(kPfBatch, batch - b0), tid = threadIdx.x;
+  const int qrow = d_nope + d_rope;
+  for (int i = tid; i < kPfBatch * d_nope; i += 256) {
+    const int j = i / d_nope, n = i % d_nope;
+    qn[j][n] = j < nb ? q[(static_cast<size_t>(b0 + j) * H + h) * qrow + n] : 0.f;
+  }
+  __syncthreads();
+  const int f4 = 4 * (tid % (kPfFeat / 4)), part = tid / (kPfFeat / 4), f = fc * kPfFeat + f4;
+  float4 acc[kPfBatch];
+#pragma unroll
+  for (int j = 0; j < kPfBatch; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (f < d_c) {
+    const float* w = w_uk + static_cast<size_t>(h) * d_nope * d_c + f;
+#pragma unroll 8
+    for (int n = part; n < d_nope; n += kPfParts) {
+      const float4 wv = __ldg(reinterpret_cast<const float4*>(w + static_cast<size_t>(n) * d_c));
+#pragma unroll
+      for (int j = 0; j < kPfBatch; ++j) {
+        const float x = qn[j][n];
+        acc[j].x = fmaf(wv.x, x, acc[j].x);
+        acc[j].y = fmaf(wv.y, x, acc[j].y);
+        acc[j].z = fmaf(wv.z, x, acc[j].z);
+        acc[j].w = fmaf(wv.w, x, acc[j].w);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kPfBatch; ++j) *reinterpret_cast<float4*>(&red[part][j][f4]) = acc[j];
+  __syncthreads();
+  for (int i = tid; i < nb * kPfFeat; i += 256) {
+    const int j = i / kPfFeat, e = i % kPfFeat;
+    float sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < kPfParts; ++k) sum += red[k][j][e];
+    if (fc * kPfFeat + e < d_c)
+      reinterpret_cast<float*>(qprep + static_cast<size_t>(b0 + j) * qstride)[static_cast<size_t>(h) * d_c +
+                                                                              fc * kPfFeat + e] = sum;
+  }
+  if (fc == 0) {
+    for (int i = tid; i < nb * d_rope; i += 256) {
+      const int j = i / d_rope, r = i % d_rope;
+      reinterpret_cast<float*>(qprep + static_cast<size_t>(b0 + j) * qstride)[static_cast<size_t>(H) * d_c +
+                                                                              static_cast<size_t>(h) * d_rope + r] =
+          q[(static_cast<size_t>(b0 + j) * H + h) * qrow + d_nope + r];
+    }
+  }
 }
 
 // ------------------------------------------------------------------ combine
@@ -390,25 +441,33 @@ __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <>
 __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
-// Block per (head h, group of kCombineGroup sequences), 256 threads: the
+// Block per (head h, group of kCombineGroup sequences; blockIdx.y: a part of the
+// d_v output rows, each part repeating the merge), 256 threads: the
 // sequences of a group share one pass over W_UV,h.  The splits that covered
 // sequence b are the CTAs c0..c1 of the page schedule; their partials sit in
 // slots c + b.  M = max_s m_s; o = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M)
 // l_s (m in log2 units); then u = W_UV,h o.  A sequence of length 0 gets
 // u = 0.
-//  - merge: warp j takes sequence b0 + j: lane k holds slot k's (m, l) of
-//    each group of 32 slots, and every lane the O values of its features
-//    (f = lane + 32 i) for one slot at a time, the slot's weight broadcast
-//    from the lane that holds it;
+//  - weights: warp j takes sequence b0 + j, its lanes the slots: M, then
+//    2^(m_s - M) into shared memory, kCombineSlots at a time, and the
+//    denominator;
+//  - merge: thread t takes (sequence, 4 features) pairs t, t + 256, ..: up to
+//    four pairs and four slots of each in flight, so that the time is a few
+//    round trips whatever the number of slots (a warp per sequence, one slot
+//    after another, took 60 us of an fp32 step of 8 sequences of 100 to 3000
+//    tokens, up to 47 slots each; 15 us now, and 20 us against
+//    26.3 us at 128 sequences with d_c 512: ncu, cold caches);
 //  - u: warp w takes groups of four W_UV,h rows; a lane loads its 16-byte
 //    pieces of the four rows once and multiplies them into all the group's
 //    merged vectors (shared memory), then the 32 sums (sequence, row) are
 //    reduced across the lanes by a transposing butterfly (31 shuffles), after
 //    which lane t holds sequence t / 4, row t % 4.
 constexpr int kCombineThreads = 256;
-constexpr int kCombineGroup = 8;        // sequences per block (one warp each in the merge)
+constexpr int kCombineGroup = 8;        // sequences per block (one warp each for the weights)
 constexpr int kCombineMaxDc = 512;
-constexpr int kCombineFeat = kCombineMaxDc / 32;   // features per lane in the merge, at most
+constexpr int kCombineBlocks = 304;     // two blocks per SM
+constexpr int kCombineSlots = 128;      // slots whose weights are in shared memory at a time
+constexpr int kCombinePairs = kCombineGroup * kCombineMaxDc / 4 / kCombineThreads;   // pairs per thread, at most
 
 // v[i] (i < 32) summed over the warp; lane t returns the sum of v[t]
 __device__ __forceinline__ float reduce32_transpose(float (&v)[32], int lane) {
@@ -433,59 +492,100 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
                const T* __restrict__ w_uv, T* __restrict__ out, int batch, int H, int d_c, int d_v,
                int num_splits) {
   __shared__ __align__(16) float olat[kCombineGroup][kCombineMaxDc];
+  __shared__ float wts[kCombineGroup][kCombineSlots];
+  __shared__ float inv_l[kCombineGroup];
+  __shared__ int slots_s[kCombineGroup], slot0_s[kCombineGroup];
   const int h = blockIdx.x % H, b0 = (blockIdx.x / H) * kCombineGroup;
   const int nb = min(kCombineGroup, batch - b0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kCombineThreads / 32;
   const int total = cu[batch];
   const int chunk = split_chunk(total, num_splits);
+  const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
+  // the slots of sequence b0 + warp and their maximum
+  int n = 0, c0 = 0;
+  float M = -INFINITY, lsum = 0.f;
+  const float* pml = part_ml;
   if (warp < nb) {
     const int b = b0 + warp;
     const int p0 = cu[b] + kSegCost, p1 = cu[b + 1];   // units of the sequence's pages
-    const int c0 = p0 / chunk;
-    const int n = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
-    float* ol = olat[warp];
-    if (n == 0) {
-      for (int f = lane; f < d_c; f += 32) ol[f] = 0.f;
-    } else {
-      const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
-      const float* pml = part_ml + (static_cast<size_t>(c0 + b) * H + h) * 2;
-      const float* po = part_o + (static_cast<size_t>(c0 + b) * H + h) * d_c;
-      float M = -INFINITY;
-      for (int k = lane; k < n; k += 32) M = fmaxf(M, pml[k * mlstride]);
+    c0 = p0 / chunk;
+    n = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
+    pml += (static_cast<size_t>(c0 + b) * H + h) * 2;
+    for (int k = lane; k < n; k += 32) M = fmaxf(M, pml[k * mlstride]);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      float acc[kCombineFeat];
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  }
+  if (warp < kCombineGroup && lane == 0) {
+    slots_s[warp] = n;
+    slot0_s[warp] = c0 + b0 + warp;
+  }
+  // this thread's (sequence, 4 features) pairs
+  const int ncol = d_c / 4;
+  int pj[kCombinePairs];
+  const float* po[kCombinePairs];
+  float4 acc4[kCombinePairs];
+  int nmax = 0;   // slots of the group's longest sequence
+  __syncthreads();
 #pragma unroll
-      for (int i = 0; i < kCombineFeat; ++i) acc[i] = 0.f;
-      float lsum = 0.f;
-      for (int k0 = 0; k0 < n; k0 += 32) {
-        const int kn = min(32, n - k0);
+  for (int j = 0; j < kCombineGroup; ++j) nmax = max(nmax, slots_s[j]);
+#pragma unroll
+  for (int u = 0; u < kCombinePairs; ++u) {
+    const int i = tid + u * kCombineThreads, j = i / ncol, f = 4 * (i - j * ncol);
+    pj[u] = j < nb ? j : -1;
+    acc4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    po[u] = part_o + (static_cast<size_t>(j < nb ? slot0_s[j] : 0) * H + h) * d_c + f;
+  }
+  for (int k0 = 0; k0 < nmax; k0 += kCombineSlots) {
+    if (warp < nb) {
+      for (int k = lane; k < kCombineSlots; k += 32) {
         float wk = 0.f;
-        if (lane < kn) {
-          const float2 ml = *reinterpret_cast<const float2*>(pml + (k0 + lane) * mlstride);
+        if (k0 + k < n) {
+          const float2 ml = *reinterpret_cast<const float2*>(pml + (k0 + k) * mlstride);
           wk = exp2f(ml.x - M);
           lsum = fmaf(wk, ml.y, lsum);
         }
-#pragma unroll 2
-        for (int kk = 0; kk < kn; ++kk) {
-          const float w = __shfl_sync(0xffffffffu, wk, kk);
-          const float* ps = po + (k0 + kk) * sstride;
+        wts[warp][k] = wk;
+      }
+    }
+    __syncthreads();
+    const int kn = min(kCombineSlots, nmax - k0);
+    for (int k = 0; k < kn; k += 4) {
+      float4 v[kCombinePairs][4];
 #pragma unroll
-          for (int i = 0; i < kCombineFeat; ++i) {
-            const int f = lane + 32 * i;
-            if (f < d_c) acc[i] = fmaf(w, ps[f], acc[i]);
-          }
+      for (int u = 0; u < kCombinePairs; ++u)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          v[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (pj[u] >= 0 && k0 + k + e < slots_s[pj[u]])
+            v[u][e] = *reinterpret_cast<const float4*>(po[u] + (k0 + k + e) * sstride);
         }
-      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-      const float invL = 1.f / lsum;
+      for (int u = 0; u < kCombinePairs; ++u)
 #pragma unroll
-      for (int i = 0; i < kCombineFeat; ++i) {
-        const int f = lane + 32 * i;
-        if (f < d_c) ol[f] = acc[i] * invL;
-      }
+        for (int e = 0; e < 4; ++e) {
+          const float w = pj[u] >= 0 ? wts[pj[u]][k + e] : 0.f;   // 0 past the sequence's slots
+          acc4[u].x = fmaf(w, v[u][e].x, acc4[u].x);
+          acc4[u].y = fmaf(w, v[u][e].y, acc4[u].y);
+          acc4[u].z = fmaf(w, v[u][e].z, acc4[u].z);
+          acc4[u].w = fmaf(w, v[u][e].w, acc4[u].w);
+        }
+    }
+    __syncthreads();   // the weights are read: the next slots' may overwrite them
+  }
+  if (warp < nb) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if (lane == 0) inv_l[warp] = n > 0 ? 1.f / lsum : 0.f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kCombinePairs; ++u) {
+    const int i = tid + u * kCombineThreads;
+    if (pj[u] >= 0) {
+      const float il = inv_l[pj[u]];
+      *reinterpret_cast<float4*>(&olat[pj[u]][4 * (i - pj[u] * ncol)]) =
+          make_float4(acc4[u].x * il, acc4[u].y * il, acc4[u].z * il, acc4[u].w * il);
     }
   }
   __syncthreads();
@@ -493,7 +593,7 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
   constexpr int VEC = 16 / sizeof(T);
   const int npieces = d_c / VEC;   // d_c is a multiple of VEC for both element types
   const T* wh = w_uv + static_cast<size_t>(h) * d_v * d_c;
-  for (int v0 = 4 * warp; v0 < d_v; v0 += 4 * kWarps) {
+  for (int v0 = 4 * (warp + kWarps * blockIdx.y); v0 < d_v; v0 += 4 * kWarps * gridDim.y) {
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
@@ -533,23 +633,37 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
 }
 
 // ------------------------------------------------------------------ fp32 decode
-// One block per split, 128 threads.  Each cached token of the block's page
-// range is processed in order: c~ = LN(c (*) G[id]) with a two-pass mean and
-// variance, per-head scores against q^ and q^R, online softmax, and the
-// running latent output sum_j p_j c~_j.  Writes the same partials as the
-// tensor-core kernel.
-constexpr int kF32Threads = 128;
+// One block of 16 warps per split, one 64-token page per tile:
+//   gate    warp w takes tokens w, w + 16, ..: c~ = LN(c (*) G[id]) (two-pass mean
+//           and variance) into shared memory with the RoPE key behind it, the
+//           loads of several tokens issued together;
+//   scores  warp = (8 heads, one of 8 parts of d_c + d_rope), lane = tokens
+//           lane and lane + 32: each shared-memory value read meets 8 heads or
+//           2 tokens;
+//   softmax warp = head: the parts added, the tile's maximum, P and the
+//           running max and denominator;
+//   output  thread = (4 features, 4 heads), accumulated in registers.
+// All sums are fp32 on CUDA cores.  A tile's four phases cost five block
+// barriers for 64 tokens; processing one token at a time cost 36 barriers per
+// token, 651 us for 8 sequences of 100 to 3000 tokens (d_c 256, 16 heads)
+// against 20 us now (ncu, cold caches).  At that size a split holds one
+// page, so the time is the latency of one tile's phases.
+constexpr int kF32Threads = 512, kF32Warps = kF32Threads / 32;
+constexpr int kF32Parts = 8;      // parts of a dot product
+constexpr int kF32Heads = 16;     // heads, at most
 
-__device__ __forceinline__ float block_sum_128(float v, float* red, int slot) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[slot * 4 + (threadIdx.x >> 5)] = v;
-  __syncthreads();
-  const float s = red[slot * 4] + red[slot * 4 + 1] + red[slot * 4 + 2] + red[slot * 4 + 3];
-  __syncthreads();
-  return s;
+// row stride of the tile in floats: a multiple of 4 and an odd number of 16-byte
+// units, so that the lanes' rows start in different bank groups
+__host__ __device__ constexpr int f32_row(int d) { return (d / 4) % 2 ? d : d + 4; }
+__host__ __device__ constexpr size_t f32_smem_floats(int d_c, int d_rope) {
+  const int d = d_c + d_rope;
+  return static_cast<size_t>(kF32Heads) * d + static_cast<size_t>(kPage) * f32_row(d) +
+         kF32Parts * kF32Heads * kPage + kPage * kF32Heads + kF32Heads;
 }
 
-__global__ void __launch_bounds__(kF32Threads)
+// NV: 16-byte units of a latent row per lane (d_c <= 128 NV)
+template <int NV>
+__global__ void __launch_bounds__(kF32Threads, 1)
 decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr_pool,
                   const int32_t* __restrict__ id_pool, const int32_t* __restrict__ block_table,
                   int max_pages, const int32_t* __restrict__ seq_lens, int batch, int num_pages,
@@ -559,15 +673,17 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
                   int H, int d_c, int d_rope, int vocab, int gate, int gate_add, int gate_ln, float scale_log2,
                   float eps,
                   int32_t* status) {
-  extern __shared__ float sm[];
-  float* qh = sm;                               // [H][d_c]
-  float* qr = qh + H * d_c;                     // [H][d_rope]
-  float* acc = qr + H * d_rope;                 // [H][d_c]
-  float* ct = acc + H * d_c;                    // [d_c]
-  float* krs = ct + d_c;                        // [d_rope]
-  float* red = krs + 64;                        // [20][4]
-  __shared__ float mrun[16], lrun[16], pcur[16], alph[16];
+  constexpr int kTok = kPage / kF32Warps;            // tokens of a page per warp
+  constexpr int kBatch = NV <= 2 ? kTok : kTok / 2;  // .. whose rows are in flight together
+  const int d = d_c + d_rope, row_f = f32_row(d), ncol = d_c / 4;
+  extern __shared__ __align__(16) float sm[];
+  float* qs = sm;                                    // [16][d]: q^_h, then q^R_h (0 past H)
+  float* ct = qs + kF32Heads * d;                    // [64][row_f]: c~, then k^R
+  float* sp = ct + kPage * row_f;                    // [8 parts][16 heads][64 tokens]
+  float* pw = sp + kF32Parts * kF32Heads * kPage;    // [64 tokens][16 heads]
+  float* al = pw + kPage * kF32Heads;                // [16]
 
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int total = cu[batch];
   const int chunk = split_chunk(total, gridDim.x);
   const int g0 = blockIdx.x * chunk;
@@ -575,86 +691,213 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
   if (g0 >= g1) return;
   int b = find_sequence(cu, batch, g0);
   int g = g0;
+  // output: features 4 ocol .., heads 4 ohg ..
+  const int ocol = tid % ncol, ohg = tid / ncol;
+  const bool oact = ohg < kF32Heads / 4 && 4 * ohg < H;
   while (g < g1) {
     const int pend = min(g1, cu[b + 1]);
     const int L = seq_lens[b];
-    const int s = cu[b] + kSegCost;   // unit of the sequence's first page
-    const int tok0 = max(g - s, 0) * kPage;
-    const int tok1 = min((pend - s) * kPage, L);
-    if (tok1 <= tok0) break;   // the range ends inside the sequence's start cost
+    const int s0 = cu[b] + kSegCost;   // unit of the sequence's first page
+    const int lp0 = max(g - s0, 0), lp1 = pend - s0;
+    if (min(lp1 * kPage, L) <= lp0 * kPage) break;   // the range ends inside the sequence's start cost
     const float* qsrc = reinterpret_cast<const float*>(qprep + static_cast<size_t>(b) * qstride);
-    for (int i = threadIdx.x; i < H * (d_c + d_rope); i += blockDim.x) qh[i] = qsrc[i];
-    for (int i = threadIdx.x; i < H * d_c; i += blockDim.x) acc[i] = 0.f;
-    if (threadIdx.x < 16) { mrun[threadIdx.x] = -INFINITY; lrun[threadIdx.x] = 0.f; }
-    __syncthreads();
-    for (int j = tok0; j < tok1; ++j) {
-      const int page = block_table[static_cast<size_t>(b) * max_pages + j / kPage];
+    for (int i = tid; i < kF32Heads * d; i += kF32Threads) {
+      const int h = i / d, f = i - h * d;
+      qs[i] = h >= H ? 0.f : f < d_c ? qsrc[h * d_c + f] : qsrc[H * d_c + h * d_rope + f - d_c];
+    }
+    float4 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float mrun = -INFINITY, lrun = 0.f;   // head `warp`, the same in every lane
+    for (int lp = lp0; lp < lp1; ++lp) {
+      const int ntok = min(kPage, L - lp * kPage);
+      const int page = block_table[static_cast<size_t>(b) * max_pages + lp];
       const bool page_ok = page >= 0 && page < num_pages;
-      const size_t row = static_cast<size_t>(page_ok ? page : 0) * kPage + j % kPage;
-      if (!page_ok && threadIdx.x == 0) report_status(status, kStatusOutOfRange);
-      int id = 0;
-      if (gate) {
-        id = id_pool[row];
-        if (id < 0 || id >= vocab) {
-          if (threadIdx.x == 0) report_status(status, kStatusOutOfRange);
-          id = 0;
+      if (!page_ok && tid == 0) report_status(status, kStatusOutOfRange);
+      const size_t row0 = static_cast<size_t>(page_ok ? page : 0) * kPage;
+      // ---- gate and LayerNorm
+#pragma unroll
+      for (int k0 = 0; k0 < kTok; k0 += kBatch) {
+        float4 z[kBatch][NV], gv[kBatch][NV], kr[kBatch];
+        int id[kBatch];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+          const int t = warp + kF32Warps * (k0 + k);
+          id[k] = gate && t < ntok ? id_pool[row0 + t] : 0;
         }
-      }
-      // gate and LayerNorm (two-pass statistics)
-      float s1 = 0.f;
-      for (int f = threadIdx.x; f < d_c; f += blockDim.x) {
-        float z = c_pool[row * d_c + f];
-        if (gate) {
-          const float g = gate_table[static_cast<size_t>(id) * d_c + f];
-          z = gate_add ? z + g : z * g;
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+          const int t = warp + kF32Warps * (k0 + k);
+          if (id[k] < 0 || id[k] >= vocab) {
+            if (lane == 0) report_status(status, kStatusOutOfRange);
+            id[k] = 0;
+          }
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            const int u = lane + 32 * i;
+            z[k][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            gv[k][i] = z[k][i];
+            if (t < ntok && u < ncol) {
+              z[k][i] = __ldg(reinterpret_cast<const float4*>(c_pool + (row0 + t) * d_c) + u);
+              if (gate) gv[k][i] = __ldg(reinterpret_cast<const float4*>(gate_table + static_cast<size_t>(id[k]) * d_c) + u);
+            }
+          }
+          kr[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (t < ntok && lane < d_rope / 4)
+            kr[k] = __ldg(reinterpret_cast<const float4*>(kr_pool + (row0 + t) * d_rope) + lane);
         }
-        ct[f] = z;
-        s1 += z;
-      }
-      for (int r = threadIdx.x; r < d_rope; r += blockDim.x) krs[r] = kr_pool[row * d_rope + r];
-      if (gate && gate_ln) {
-        const float mean = block_sum_128(s1, red, 0) / d_c;
-        float s2 = 0.f;
-        for (int f = threadIdx.x; f < d_c; f += blockDim.x) {
-          const float dz = ct[f] - mean;
-          s2 = fmaf(dz, dz, s2);
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+          const int t = warp + kF32Warps * (k0 + k);
+          float* row = ct + t * row_f;
+          if (gate) {
+            float s1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+              float4& v = z[k][i];
+              const float4 w = gv[k][i];
+              v = gate_add ? make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w)
+                           : make_float4(v.x * w.x, v.y * w.y, v.z * w.z, v.w * w.w);
+              s1 += (v.x + v.y) + (v.z + v.w);
+            }
+            if (gate_ln) {
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+              const float mean = s1 / d_c;
+              float s2 = 0.f;
+#pragma unroll
+              for (int i = 0; i < NV; ++i) {
+                float4& v = z[k][i];
+                if (lane + 32 * i < ncol) {
+                  v = make_float4(v.x - mean, v.y - mean, v.z - mean, v.w - mean);
+                  s2 = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s2))));
+                }
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+              const float rstd = rsqrtf(s2 / d_c + eps);
+#pragma unroll
+              for (int i = 0; i < NV; ++i) {
+                const int f = 4 * (lane + 32 * i);
+                if (f < d_c) {
+                  float4& v = z[k][i];
+                  v.x = v.x * rstd * (gamma ? gamma[f] : 1.f) + (beta ? beta[f] : 0.f);
+                  v.y = v.y * rstd * (gamma ? gamma[f + 1] : 1.f) + (beta ? beta[f + 1] : 0.f);
+                  v.z = v.z * rstd * (gamma ? gamma[f + 2] : 1.f) + (beta ? beta[f + 2] : 0.f);
+                  v.w = v.w * rstd * (gamma ? gamma[f + 3] : 1.f) + (beta ? beta[f + 3] : 0.f);
+                }
+              }
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            const int u = lane + 32 * i;
+            if (u < ncol) *reinterpret_cast<float4*>(row + 4 * u) = z[k][i];
+          }
+          if (lane < d_rope / 4) *reinterpret_cast<float4*>(row + d_c + 4 * lane) = kr[k];
         }
-        const float var = block_sum_128(s2, red, 1) / d_c;
-        const float rstd = rsqrtf(var + eps);
-        for (int f = threadIdx.x; f < d_c; f += blockDim.x)
-          ct[f] = (ct[f] - mean) * rstd * (gamma ? gamma[f] : 1.f) + (beta ? beta[f] : 0.f);
       }
       __syncthreads();
-      // scores of every head
-      for (int h = 0; h < H; ++h) {
-        float part = 0.f;
-        for (int f = threadIdx.x; f < d_c; f += blockDim.x) part = fmaf(qh[h * d_c + f], ct[f], part);
-        for (int r = threadIdx.x; r < d_rope; r += blockDim.x) part = fmaf(qr[h * d_rope + r], krs[r], part);
-        const float s = block_sum_128(part, red, 2 + h) * scale_log2;
-        if (threadIdx.x == 0) {
-          const float mn = fmaxf(mrun[h], s);
-          const float a = exp2f(mrun[h] - mn);
-          const float p = exp2f(s - mn);
-          lrun[h] = lrun[h] * a + p;
-          mrun[h] = mn;
-          alph[h] = a;
-          pcur[h] = p;
+      // ---- scores
+      {
+        const int h0 = 8 * (warp / kF32Parts), part = warp % kF32Parts;
+        const int u0 = d / 4 * part / kF32Parts, u1 = d / 4 * (part + 1) / kF32Parts;
+        float sa[2][8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sa[0][j] = sa[1][j] = 0.f;
+        if (h0 < H) {
+          const float *r0 = ct + lane * row_f, *r1 = ct + (lane + 32) * row_f, *qh = qs + h0 * d;
+          for (int u = u0; u < u1; ++u) {
+            const float4 x0 = *reinterpret_cast<const float4*>(r0 + 4 * u);
+            const float4 x1 = *reinterpret_cast<const float4*>(r1 + 4 * u);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float4 y = *reinterpret_cast<const float4*>(qh + j * d + 4 * u);
+              sa[0][j] = fmaf(y.x, x0.x, fmaf(y.y, x0.y, fmaf(y.z, x0.z, fmaf(y.w, x0.w, sa[0][j]))));
+              sa[1][j] = fmaf(y.x, x1.x, fmaf(y.y, x1.y, fmaf(y.z, x1.z, fmaf(y.w, x1.w, sa[1][j]))));
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            sp[(part * kF32Heads + h0 + j) * kPage + lane] = sa[0][j];
+            sp[(part * kF32Heads + h0 + j) * kPage + lane + 32] = sa[1][j];
+          }
         }
       }
       __syncthreads();
-      for (int i = threadIdx.x; i < H * d_c; i += blockDim.x) {
-        const int h = i / d_c;
-        acc[i] = fmaf(acc[i], alph[h], pcur[h] * ct[i - h * d_c]);
+      // ---- softmax of head `warp`
+      if (warp < H) {
+        float s[2], mx = mrun;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int t = lane + 32 * e;
+          float v = 0.f;
+#pragma unroll
+          for (int k = 0; k < kF32Parts; ++k) v += sp[(k * kF32Heads + warp) * kPage + t];
+          s[e] = t < ntok ? v * scale_log2 : -INFINITY;
+          mx = fmaxf(mx, s[e]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float ps = 0.f;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float pv = lane + 32 * e < ntok ? exp2f(s[e] - mx) : 0.f;
+          pw[(lane + 32 * e) * kF32Heads + warp] = pv;
+          ps += pv;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+        const float a = exp2f(mrun - mx);
+        lrun = lrun * a + ps;
+        mrun = mx;
+        if (lane == 0) al[warp] = a;
+      } else {
+        pw[lane * kF32Heads + warp] = 0.f;
+        pw[(lane + 32) * kF32Heads + warp] = 0.f;
+        if (lane == 0) al[warp] = 1.f;
       }
       __syncthreads();
+      // ---- output
+      if (oact) {
+        const float4 a4 = *reinterpret_cast<const float4*>(al + 4 * ohg);
+        const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          acc[k].x *= a[k];
+          acc[k].y *= a[k];
+          acc[k].z *= a[k];
+          acc[k].w *= a[k];
+        }
+        const float* zc = ct + 4 * ocol;
+        const float* pc = pw + 4 * ohg;
+#pragma unroll 4
+        for (int t = 0; t < ntok; ++t) {
+          const float4 x = *reinterpret_cast<const float4*>(zc + t * row_f);
+          const float4 p4 = *reinterpret_cast<const float4*>(pc + t * kF32Heads);
+          const float pk[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            acc[k].x = fmaf(pk[k], x.x, acc[k].x);
+            acc[k].y = fmaf(pk[k], x.y, acc[k].y);
+            acc[k].z = fmaf(pk[k], x.z, acc[k].z);
+            acc[k].w = fmaf(pk[k], x.w, acc[k].w);
+          }
+        }
+      }
+      __syncthreads();   // the tile is read: the next one may overwrite it
     }
-    const int slot = blockIdx.x + b;
-    for (int i = threadIdx.x; i < H * d_c; i += blockDim.x) part_o[static_cast<size_t>(slot) * H * d_c + i] = acc[i];
-    if (threadIdx.x < H) {
-      part_ml[(static_cast<size_t>(slot) * H + threadIdx.x) * 2] = mrun[threadIdx.x];
-      part_ml[(static_cast<size_t>(slot) * H + threadIdx.x) * 2 + 1] = lrun[threadIdx.x];
+    const size_t slot = blockIdx.x + b;
+    if (oact) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (4 * ohg + k < H)
+          *reinterpret_cast<float4*>(part_o + (slot * H + 4 * ohg + k) * d_c + 4 * ocol) = acc[k];
     }
-    __syncthreads();
+    if (warp < H && lane == 0) {
+      part_ml[(slot * H + warp) * 2] = mrun;
+      part_ml[(slot * H + warp) * 2 + 1] = lrun;
+    }
     g = pend;
     ++b;
     while (b < batch && cu[b + 1] <= g) ++b;
@@ -686,21 +929,15 @@ cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t launch_decode_f32(const DecodeArgs& a, cudaStream_t st) {
-  const WorkspaceLayout wl = workspace_layout(a.batch, a.num_splits, a.H, a.d_c, a.d_rope, false);
+namespace {
+template <int NV>
+cudaError_t launch_decode_f32_t(const DecodeArgs& a, const WorkspaceLayout& wl, cudaStream_t st) {
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
-  prologue_f32_kernel<<<a.batch * a.H + 1, 256, 0, st>>>(
-      static_cast<const float*>(a.q), static_cast<const float*>(a.w_uk), a.seq_lens, a.batch, a.H, a.d_nope,
-      a.d_rope, a.d_c, a.page_size, ws + wl.off_qprep, wl.qprep_stride,
-      reinterpret_cast<int32_t*>(ws + wl.off_cu));
-  cudaError_t e = cudaGetLastError();
+  const size_t smem = f32_smem_floats(a.d_c, a.d_rope) * sizeof(float);
+  const cudaError_t e =
+      cudaFuncSetAttribute(decode_f32_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const size_t smem = (static_cast<size_t>(a.H) * (2 * a.d_c + a.d_rope) + a.d_c + 64 + 80) * sizeof(float);
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(decode_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  decode_f32_kernel<<<a.num_splits, kF32Threads, smem, st>>>(
+  decode_f32_kernel<NV><<<a.num_splits, kF32Threads, smem, st>>>(
       static_cast<const float*>(a.c_pool), static_cast<const float*>(a.kr_pool), a.id_pool, a.block_table,
       a.max_pages, a.seq_lens, a.batch, a.num_pages, static_cast<const float*>(a.gate_table), a.ln_gamma,
       a.ln_beta, ws + wl.off_qprep, wl.qprep_stride, reinterpret_cast<const int32_t*>(ws + wl.off_cu),
@@ -708,12 +945,36 @@ cudaError_t launch_decode_f32(const DecodeArgs& a, cudaStream_t st) {
       a.vocab, a.gate, a.gate_add, a.gate_ln, a.scale_log2, a.eps, a.status);
   return cudaGetLastError();
 }
+}  // namespace
+
+cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaStream_t st) {
+  const WorkspaceLayout wl = workspace_layout(a.batch, a.num_splits, a.H, a.d_c, a.d_rope, false);
+  uint8_t* ws = static_cast<uint8_t*>(a.workspace);
+  AppendArgs none;
+  std::memset(&none, 0, sizeof(none));
+  const AppendArgs& ap = app != nullptr ? *app : none;
+  const int absorb =
+      a.H * ((a.d_c + kPfFeat - 1) / kPfFeat) * ((a.batch + kPfBatch - 1) / kPfBatch);
+  prologue_f32_kernel<<<absorb + 1 + ap.batch, 256, 0, st>>>(
+      static_cast<const float*>(a.q), static_cast<const float*>(a.w_uk), a.seq_lens, a.batch, a.H, a.d_nope,
+      a.d_rope, a.d_c, a.page_size, ws + wl.off_qprep, wl.qprep_stride,
+      reinterpret_cast<int32_t*>(ws + wl.off_cu), ap);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (a.d_c <= 128) return launch_decode_f32_t<1>(a, wl, st);
+  if (a.d_c <= 256) return launch_decode_f32_t<2>(a, wl, st);
+  return launch_decode_f32_t<4>(a, wl, st);
+}
 
 namespace {
 template <typename T>
 void launch_combine_t(const DecodeArgs& a, const int32_t* cu, const float* ml, const float* po, cudaStream_t st) {
-  const int grid = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup);
-  combine_kernel<T><<<grid, kCombineThreads, 0, st>>>(cu, ml, po, static_cast<const T*>(a.w_uv),
+  // small batches: the output rows spread over more blocks (a pass of the block's
+  // warps covers 32 rows), so that most SMs read a part of W_UV
+  const int groups = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup), passes = (a.d_v + 31) / 32;
+  int parts = kCombineBlocks / groups;
+  parts = parts < 1 ? 1 : parts > passes ? passes : parts;
+  combine_kernel<T><<<dim3(groups, parts), kCombineThreads, 0, st>>>(cu, ml, po, static_cast<const T*>(a.w_uv),
                                                       static_cast<T*>(a.out), a.batch, a.H, a.d_c, a.d_v,
                                                       a.num_splits);
 }

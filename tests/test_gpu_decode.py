@@ -99,6 +99,32 @@ def test_bf16_ablation_gates_match_oracle(gpu_lib, op, d_c):
         check_bf16(got, ref, f"{op} d_c={d_c} splits={splits}", scaled_abs=True)
 
 
+@pytest.mark.parametrize("heads,d_nope,d_rope,d_v,d_c,gate", [
+    (16, 256, 64, 256, 512, True),    # the largest shape: four units per lane, all shared memory
+    (3, 7, 12, 9, 100, True),         # d_c + d_rope an even number of units (padded rows), odd sizes
+    (5, 33, 4, 6, 132, True),         # an odd number of units, a part-filled second unit per lane
+    (1, 8, 4, 4, 4, True),            # the smallest latent: dot-product parts without a unit
+    (12, 64, 16, 40, 260, False),
+])
+def test_fp32_shapes_match_oracle(gpu_lib, heads, d_nope, d_rope, d_v, d_c, gate):
+    """The fp32 kernels at the edges of their tiles: heads, features, parts and
+    page remainders, more than eight sequences, and one split over all of them."""
+    dims = synth.Dims(num_heads=heads, d_nope=d_nope, d_rope=d_rope, d_v=d_v, d_c=d_c, page_size=64, vocab=300,
+                      dtype="fp32", gate=gate)
+    case = synth.make_case("f32-shape", dims, [1, 0, 63, 64, 65, 130, 2, 200, 31, 97], seed=33, affine_ln=True,
+                           layout="permuted", extra_pages=2)
+    for splits in (1, 0):
+        dc = device.upload(case, num_splits=splits)
+        dc.out.fill_(float("nan"))
+        dc.step()
+        torch.cuda.synchronize()
+        assert dc.read_status() == 0
+        got, ref = device.output_f64(dc.out), orc.decode_unabsorbed(case)
+        assert np.isfinite(got).all()
+        rel = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+        assert rel <= 1e-5, (splits, rel)
+
+
 @pytest.mark.parametrize("op", ["mul", "add_ln"])
 def test_fp32_ablation_gates_match_oracle(gpu_lib, op):
     dims = dataclasses.replace(synth.dims_tiny(), gate_op=op)
