@@ -354,7 +354,7 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
                 const int32_t* seq_lens, int32_t max_seq_len, int32_t batch, int32_t num_pages,
                 const void* gate_table, const float* ln_gamma, const float* ln_beta, const void* w_uk,
                 const void* w_uv, void* out, int32_t num_splits, void* workspace, size_t workspace_bytes,
-                int32_t* dev_status, const egmla::AppendArgs* app, cudaStream_t st) {
+                int32_t* dev_status, const egmla::AppendArgs* app, cudaStream_t st, bool early = false) {
   DecodeArgs a;
   int rc = fill_decode_args(a, dims, c_pool, krope_pool, id_pool, block_table, max_pages_per_seq, seq_lens,
                             max_seq_len, batch, num_pages, gate_table, num_splits, workspace, workspace_bytes,
@@ -370,6 +370,7 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
   a.w_uk = w_uk;
   a.w_uv = w_uv;
   a.out = out;
+  a.early = early ? 1 : 0;
   if (is_tc_path(dims)) {
     CUtensorMap maps[2];
     if (!encode_decode_maps(maps, dims, c_pool, krope_pool, num_pages)) return EG_MLA_ERR_CUDA;
@@ -391,6 +392,23 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
 }
 
 }  // namespace
+
+int egmla_layer_step(const eg_mla_dims* dims, bool append, void* c_pool, void* krope_pool, int32_t* id_pool,
+                     const void* c_new, const void* krope_new, const int32_t* ids_new, const int32_t* positions,
+                     const void* q, const int32_t* block_table, int32_t max_pages_per_seq, const int32_t* seq_lens,
+                     int32_t max_seq_len, int32_t batch, int32_t num_pages, const void* gate_table,
+                     const float* ln_gamma, const float* ln_beta, const void* w_uk, const void* w_uv, void* out,
+                     int32_t num_splits, void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
+  egmla::AppendArgs app;
+  if (append) {
+    const int rc = fill_append_args(app, dims, c_pool, krope_pool, id_pool, c_new, krope_new, ids_new, block_table,
+                                    max_pages_per_seq, positions, batch, num_pages, dev_status);
+    if (rc != EG_MLA_OK) return rc;
+  }
+  return decode_impl(dims, q, c_pool, krope_pool, id_pool, block_table, max_pages_per_seq, seq_lens, max_seq_len,
+                     batch, num_pages, gate_table, ln_gamma, ln_beta, w_uk, w_uv, out, num_splits, workspace,
+                     workspace_bytes, dev_status, append ? &app : nullptr, static_cast<cudaStream_t>(stream), true);
+}
 
 namespace {
 // shapes the prefill kernels cover; EG_MLA_OK or the error code

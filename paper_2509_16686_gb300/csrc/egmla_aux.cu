@@ -212,6 +212,7 @@ __global__ void prologue_tc_kernel(const __nv_bfloat16* __restrict__ q, const __
   // the decode kernel after this one may begin its setup (it waits for this
   // kernel's completion before it reads anything written here)
   grid_launch_dependents();
+  grid_dependency_wait();
   // block 0: the schedule (dispatched first, so that it never waits for a
   // second wave of the grid); blocks 1 .. A: the absorption items; then the
   // append blocks
@@ -369,6 +370,8 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
   __shared__ __align__(16) float red[kPfParts][kPfBatch][kPfFeat];
   const int nfc = (d_c + kPfFeat - 1) / kPfFeat, nbg = (batch + kPfBatch - 1) / kPfBatch;
   const int nabs = H * nfc * nbg;
+  grid_launch_dependents();
+  grid_dependency_wait();
   if (blockIdx.x == 0) {
     page_prefix_sums(seq_lens, batch, page_size, cu);
     return;
@@ -499,6 +502,7 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
   const int nb = min(kCombineGroup, batch - b0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kCombineThreads / 32;
+  grid_dependency_wait();
   const int total = cu[batch];
   const int chunk = split_chunk(total, num_splits);
   const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
@@ -684,6 +688,8 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
   float* al = pw + kPage * kF32Heads;                // [16]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int total = cu[batch];
   const int chunk = split_chunk(total, gridDim.x);
   const int g0 = blockIdx.x * chunk;
@@ -921,12 +927,12 @@ cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, cudaS
   AppendArgs none;
   std::memset(&none, 0, sizeof(none));
   const AppendArgs& ap = app != nullptr ? *app : none;
-  prologue_tc_kernel<<<16 * (a.d_c / kSumFeatures) * ngroups + 1 + ap.batch, 256, 0, st>>>(
+  return launch_chained(
+      prologue_tc_kernel, dim3(16 * (a.d_c / kSumFeatures) * ngroups + 1 + ap.batch), dim3(256), 0, st,
       static_cast<const __nv_bfloat16*>(a.q), static_cast<const __nv_bfloat16*>(a.w_uk), gamma, beta,
       a.seq_lens, a.batch, a.d_nope, a.d_rope, a.d_c, a.page_size, ws + wl.off_qprep, wl.qprep_stride,
       reinterpret_cast<int32_t*>(ws + wl.off_cu), reinterpret_cast<uint32_t*>(ws + wl.off_done), a.num_splits,
       a.block_table, a.max_pages, reinterpret_cast<SplitStart*>(ws + wl.off_start), ap);
-  return cudaGetLastError();
 }
 
 namespace {
@@ -937,13 +943,13 @@ cudaError_t launch_decode_f32_t(const DecodeArgs& a, const WorkspaceLayout& wl, 
   const cudaError_t e =
       cudaFuncSetAttribute(decode_f32_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  decode_f32_kernel<NV><<<a.num_splits, kF32Threads, smem, st>>>(
+  return launch_chained(
+      decode_f32_kernel<NV>, dim3(a.num_splits), dim3(kF32Threads), smem, st,
       static_cast<const float*>(a.c_pool), static_cast<const float*>(a.kr_pool), a.id_pool, a.block_table,
       a.max_pages, a.seq_lens, a.batch, a.num_pages, static_cast<const float*>(a.gate_table), a.ln_gamma,
       a.ln_beta, ws + wl.off_qprep, wl.qprep_stride, reinterpret_cast<const int32_t*>(ws + wl.off_cu),
       reinterpret_cast<float*>(ws + wl.off_ml), reinterpret_cast<float*>(ws + wl.off_o), a.H, a.d_c, a.d_rope,
       a.vocab, a.gate, a.gate_add, a.gate_ln, a.scale_log2, a.eps, a.status);
-  return cudaGetLastError();
 }
 }  // namespace
 
@@ -955,11 +961,11 @@ cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaSt
   const AppendArgs& ap = app != nullptr ? *app : none;
   const int absorb =
       a.H * ((a.d_c + kPfFeat - 1) / kPfFeat) * ((a.batch + kPfBatch - 1) / kPfBatch);
-  prologue_f32_kernel<<<absorb + 1 + ap.batch, 256, 0, st>>>(
+  const cudaError_t e = launch_chained(
+      prologue_f32_kernel, dim3(absorb + 1 + ap.batch), dim3(256), 0, st,
       static_cast<const float*>(a.q), static_cast<const float*>(a.w_uk), a.seq_lens, a.batch, a.H, a.d_nope,
       a.d_rope, a.d_c, a.page_size, ws + wl.off_qprep, wl.qprep_stride,
       reinterpret_cast<int32_t*>(ws + wl.off_cu), ap);
-  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.d_c <= 128) return launch_decode_f32_t<1>(a, wl, st);
   if (a.d_c <= 256) return launch_decode_f32_t<2>(a, wl, st);
@@ -968,15 +974,15 @@ cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaSt
 
 namespace {
 template <typename T>
-void launch_combine_t(const DecodeArgs& a, const int32_t* cu, const float* ml, const float* po, cudaStream_t st) {
+cudaError_t launch_combine_t(const DecodeArgs& a, const int32_t* cu, const float* ml, const float* po, cudaStream_t st) {
   // small batches: the output rows spread over more blocks (a pass of the block's
   // warps covers 32 rows), so that most SMs read a part of W_UV
   const int groups = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup), passes = (a.d_v + 31) / 32;
   int parts = kCombineBlocks / groups;
   parts = parts < 1 ? 1 : parts > passes ? passes : parts;
-  combine_kernel<T><<<dim3(groups, parts), kCombineThreads, 0, st>>>(cu, ml, po, static_cast<const T*>(a.w_uv),
-                                                      static_cast<T*>(a.out), a.batch, a.H, a.d_c, a.d_v,
-                                                      a.num_splits);
+  return launch_chained(combine_kernel<T>, dim3(groups, parts), dim3(kCombineThreads), 0, st, cu, ml, po,
+                        static_cast<const T*>(a.w_uv), static_cast<T*>(a.out), a.batch, a.H, a.d_c, a.d_v,
+                        a.num_splits);
 }
 }  // namespace
 
@@ -986,11 +992,7 @@ cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, cudaStream_t st) {
   const int32_t* cu = reinterpret_cast<const int32_t*>(ws + wl.off_cu);
   const float* ml = reinterpret_cast<const float*>(ws + wl.off_ml);
   const float* po = reinterpret_cast<const float*>(ws + wl.off_o);
-  if (a.dtype == 0)
-    launch_combine_t<__nv_bfloat16>(a, cu, ml, po, st);
-  else
-    launch_combine_t<float>(a, cu, ml, po, st);
-  return cudaGetLastError();
+  return a.dtype == 0 ? launch_combine_t<__nv_bfloat16>(a, cu, ml, po, st) : launch_combine_t<float>(a, cu, ml, po, st);
 }
 
 }  // namespace egmla

@@ -186,7 +186,7 @@ struct TcParams {
   __nv_bfloat16* out;
   uint32_t* seq_done;   // [0] CTAs done, [1 + b] split partials of sequence b stored
   int d_v, cmb_groups, cmb_g;
-  int fuse;
+  int fuse, early;
   // limit of every wait (ns); a test entry lowers it, together with a
   // withheld page copy (stall_cta, stall_tile; stall_cta < 0: none)
   uint64_t wait_ns;
@@ -662,9 +662,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   phase_mark<DBG == 2>(p, 0);
-  // a kernel launched after this one with programmatic stream serialisation
-  // (the layer's output projection) may take each SM this kernel leaves
-  grid_launch_dependents();
+  // the layer's output projection after this kernel may take each SM it
+  // leaves and stream its weights; any other kernel would crowd its blocks
+  // onto the first SMs to free up
+  if (p.early) grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) {
@@ -1587,6 +1588,7 @@ cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_
   const int g = std::min(static_cast<int>(kFusedMaxG), (a.batch + groups - 1) / groups);
   p.cmb_g = g;
   p.cmb_groups = (a.batch + g - 1) / g;
+  p.early = a.early;
   p.wait_ns = a.wait_ns;
   p.stall_cta = a.stall_cta;
   p.stall_tile = a.stall_tile;

@@ -14,6 +14,7 @@
 
 #include "../../include/egmla.h"
 #include "egmla_kernels.h"
+#include "egmla_ptx.cuh"
 
 namespace {
 
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(kQkvThreads) layer_qkv_kernel(
   const float* q = qkv32 + static_cast<size_t>(b) * (H * dq + dc + dr);   // [q (H dq) | c (dc) | k^R (dr)]
   const float* kv = q + H * dq;
   __nv_bfloat16* qo = q_out + static_cast<size_t>(b) * H * dq;
+  egmla::grid_dependency_wait();
 
   if (tid < np) {
     constexpr double kTwoPi = 6.283185307179586, kInvTwoPi = 0.15915494309189535;
@@ -174,20 +176,16 @@ int eg_mla_layer_decode(const eg_mla_dims* dims, const eg_mla_layer_dims* layer,
   if (egmla::launch_linear_tc(wt->w_qkv_a, do_kv ? nq + nkv : nq, E, x, batch, qkv32, nq + nkv, true, dev_status,
                               st) != cudaSuccess)
     return EG_MLA_ERR_CUDA;
-  layer_qkv_kernel<<<batch, kQkvThreads, 0, st>>>(
-      static_cast<const float*>(qkv32), positions,
+  if (egmla::launch_chained(
+      layer_qkv_kernel, dim3(batch), dim3(kQkvThreads), 0, st, static_cast<const float*>(qkv32), positions,
       static_cast<const __nv_bfloat16*>(wt->kv_norm_w), H, dims->d_nope, dims->d_rope, dims->d_c, freqs, eps,
-      do_kv ? 1 : 0, qb, cb, krb);
-  if (cudaGetLastError() != cudaSuccess) return EG_MLA_ERR_CUDA;
+      do_kv ? 1 : 0, qb, cb, krb) != cudaSuccess)
+    return EG_MLA_ERR_CUDA;
   // the append (first layer of a group) and the decode as one step
-  const int rc = do_kv ? eg_mla_step(dims, c_pool, krope_pool, id_pool, cb, krb, ids_new, positions, qb, block_table,
-                                     max_pages_per_seq, seq_lens, max_seq_len, batch, num_pages, wt->gate_table,
-                                     wt->ln_gamma, wt->ln_beta, wt->w_uk, wt->w_uv, ub, num_splits, base + ws.off_dec,
-                                     ws.dec_bytes, dev_status, stream)
-                       : eg_mla_decode(dims, qb, c_pool, krope_pool, id_pool, block_table, max_pages_per_seq,
-                                       seq_lens, max_seq_len, batch, num_pages, wt->gate_table, wt->ln_gamma,
-                                       wt->ln_beta, wt->w_uk, wt->w_uv, ub, num_splits, base + ws.off_dec,
-                                       ws.dec_bytes, dev_status, stream);
+  const int rc = egmla_layer_step(dims, do_kv, c_pool, krope_pool, id_pool, cb, krb, ids_new, positions, qb,
+                                  block_table, max_pages_per_seq, seq_lens, max_seq_len, batch, num_pages,
+                                  wt->gate_table, wt->ln_gamma, wt->ln_beta, wt->w_uk, wt->w_uv, ub, num_splits,
+                                  base + ws.off_dec, ws.dec_bytes, dev_status, stream);
   if (rc != EG_MLA_OK) return rc;
   // Eq. 14: the output projection of the heads' concatenated outputs
   if (egmla::launch_linear_tc(wt->w_o, E, nu, ub, batch, y, E, false, dev_status, st) != cudaSuccess)

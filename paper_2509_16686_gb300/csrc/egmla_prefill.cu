@@ -195,6 +195,8 @@ constexpr int kSortMaxBatch = 2048;   // larger batches keep the given order
 // One warp per token row.
 __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfGateParams p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  grid_launch_dependents();
+  grid_dependency_wait();
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) *p.next_item = 0;
     // the attention's launch order: longest prompts first (rank of each prompt
@@ -357,6 +359,8 @@ __global__ void __launch_bounds__(kKvThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
+  if (p.kv_mode) grid_launch_dependents();   // the attention kernel of the same call
+  grid_dependency_wait();
 
   if (warp == 0) {
     if (elect_one()) {
@@ -649,6 +653,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars.tmem_base;
+  grid_dependency_wait();
 
   // item n of this CTA sits in ring slot n % 2; a reader copies it out, then frees the slot
   auto read_item = [&](int n, AttnItem& it, bool arrive) -> bool {
@@ -1113,8 +1118,8 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   gp.gate_ln = a.gate_ln;
   gp.eps = a.eps;
   gp.status = a.status;
-  prefill_gate_kernel<<<(a.total + kGateWarps - 1) / kGateWarps, 32 * kGateWarps, 0, st>>>(gp);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e =
+      launch_chained(prefill_gate_kernel, dim3((a.total + kGateWarps - 1) / kGateWarps), dim3(32 * kGateWarps), 0, st, gp);
   if (e != cudaSuccess) return e;
 
   // 2. keys and values of every head: the units shared equally by one CTA per SM
@@ -1146,9 +1151,8 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
     if (e != cudaSuccess) return e;
     kp.units = static_cast<long long>((a.total + kPfRows - 1) / kPfRows) * kp.nblocks;
     const int grid = static_cast<int>(kp.units < sms ? kp.units : sms);
-    prefill_kv_kernel<1><<<grid, kKvThreads, kv_smem, st>>>(cmap, wkmap, wvmap, omap, kp);
+    e = launch_chained(prefill_kv_kernel<1>, dim3(grid), dim3(kKvThreads), kv_smem, st, cmap, wkmap, wvmap, omap, kp);
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
 
   // 3. causal attention
@@ -1177,8 +1181,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   ap.items = static_cast<int>(items);
   const int grid = static_cast<int>(items < sms ? items : sms);
   if (mark) mark(st, true);
-  prefill_attn_kernel<<<grid, kAttnThreads, kAttnSmem, st>>>(qmap, kvmap, krmap, ap);
-  e = cudaGetLastError();
+  e = launch_chained(prefill_attn_kernel, dim3(grid), dim3(kAttnThreads), kAttnSmem, st, qmap, kvmap, krmap, ap);
   if (mark) mark(st, false);
   return e;
 }
@@ -1206,7 +1209,7 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
     if (e != cudaSuccess) return e;
     const int tiles = (vocab + 2 * kPfRows - 1) / (2 * kPfRows);
     kp.units = static_cast<long long>(tiles) * kp.nblocks;   // whole tiles: a table row's few blocks share its copy
-    prefill_kv_kernel<2><<<tiles, kKvThreads, smem, st>>>(amap, wmap, wmap, omap, kp);
+    return launch_chained(prefill_kv_kernel<2>, dim3(tiles), dim3(kKvThreads), smem, st, amap, wmap, wmap, omap, kp);
   } else {
     kp.stages = kv_stages<1>(nkc);
     const int smem = static_cast<int>(kv_smem_bytes<1>(nkc));
@@ -1214,9 +1217,8 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
     if (e != cudaSuccess) return e;
     const int tiles = (vocab + kPfRows - 1) / kPfRows;
     kp.units = static_cast<long long>(tiles) * kp.nblocks;
-    prefill_kv_kernel<1><<<tiles, kKvThreads, smem, st>>>(amap, wmap, wmap, omap, kp);
+    return launch_chained(prefill_kv_kernel<1>, dim3(tiles), dim3(kKvThreads), smem, st, amap, wmap, wmap, omap, kp);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace egmla

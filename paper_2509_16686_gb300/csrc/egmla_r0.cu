@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(kR0Threads, 1)
     prefetch_tensormap(&cmap);
     prefetch_tensormap(&wmap);
   }
+  grid_dependency_wait();
   if (warp == 0) find_tile(p, sm, lane);
   __syncthreads();
   if (sm.tile_n[0] == 0 && sm.tile_n[1] == 0) return;   // past the last page (uniform)
@@ -507,6 +508,7 @@ __global__ void __launch_bounds__(kR0AttnThreads) r0_attend_kernel(const R0AttnP
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int hw = lane >> 4, c8 = 8 * (lane & 15);   // half-warp, first feature of the lane
   const int max_len = p.max_pages * kPage;
+  grid_dependency_wait();
   const int L = min(p.seq_lens[b], max_len);
   if (threadIdx.x == 0 && h == 0 && p.seq_lens[b] > max_len) report_status(p.status, kStatusOutOfRange);
   const float* lgb = p.logit + static_cast<size_t>(b) * max_len * kR0Heads + h;
@@ -675,8 +677,7 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   pp.status = a.status;
   // one CTA per two pages of the walk: the block table bounds the pages in use
   const int tiles = static_cast<int>((static_cast<int64_t>(a.batch) * a.max_pages + 1) / 2);
-  r0_project_kernel<<<tiles, kR0Threads, smem, st>>>(cmap, wmap, pp);
-  e = cudaGetLastError();
+  e = launch_chained(r0_project_kernel, dim3(tiles), dim3(kR0Threads), smem, st, cmap, wmap, pp);
   if (e != cudaSuccess) return e;
   R0AttnParams ap;
   ap.block_table = a.block_table;
@@ -691,8 +692,7 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   ap.num_pages = a.num_pages;
   ap.pool_rows = static_cast<int>(rows);
   ap.status = a.status;
-  r0_attend_kernel<<<a.batch * kR0Heads, kR0AttnThreads, 0, st>>>(ap);
-  return cudaGetLastError();
+  return launch_chained(r0_attend_kernel, dim3(a.batch * kR0Heads), dim3(kR0AttnThreads), 0, st, ap);
 }
 
 }  // namespace egmla
