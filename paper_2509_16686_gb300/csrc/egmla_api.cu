@@ -120,6 +120,29 @@ bool encode_decode_maps(CUtensorMap (&maps)[2], const eg_mla_dims* d, const void
   return encode_pool_map(&maps[1], krope_pool, rows, d->d_rope);
 }
 
+// bf16 tensor {d0, d1, d2} with strides s1, s2 (elements) in boxes {64, b1, b2},
+// 128-byte swizzle, elements past an end read as zero
+bool encode_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1, uint64_t s2,
+               uint32_t b1, uint32_t b2) {
+  EncodeFn enc = get_encode();
+  if (enc == nullptr) return false;
+  const cuuint64_t dims[3] = {d0, d1, d2};
+  const cuuint64_t strides[2] = {s1 * 2, s2 * 2};
+  const cuuint32_t box[3] = {64, b1, b2};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// maps of the tensor-core query absorption: {W_UK, q}
+bool encode_absorb_maps(CUtensorMap (&maps)[2], const DecodeArgs& a, int tile) {
+  std::memset(maps, 0, sizeof(maps));
+  const uint64_t dc = a.d_c, dn = a.d_nope, H = a.H, qrow = a.d_nope + a.d_rope;
+  return encode_3d(&maps[0], a.w_uk, dc, dn, H, dc, dn * dc, 64, 1) &&
+         encode_3d(&maps[1], a.q, dn, H, a.batch, qrow, H * qrow, 1, tile);   // q^C: the RoPE part is past the end
+}
+
 float resolve_scale(const eg_mla_dims* d) {
   return d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / std::sqrt(static_cast<float>(d->d_nope + d->d_rope));
 }
@@ -376,7 +399,9 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
     if (!encode_decode_maps(maps, dims, c_pool, krope_pool, num_pages)) return EG_MLA_ERR_CUDA;
     apply_trace(a);
     apply_fault(a);
-    cudaError_t e = egmla::launch_prologue_tc(a, app, st);
+    CUtensorMap amaps[2];
+    if (!encode_absorb_maps(amaps, a, egmla::absorb_tile(a.d_c, a.batch))) return EG_MLA_ERR_CUDA;
+    cudaError_t e = egmla::launch_prologue_tc(a, app, amaps, st);
     bool fused = false;
     if (e == cudaSuccess) {
       prof_mark(st, true);
@@ -762,7 +787,9 @@ int eg_mla_debug_gather(const eg_mla_dims* dims, const void* c_pool, const void*
   CUtensorMap maps[2];
   if (!encode_decode_maps(maps, dims, c_pool, krope_pool, num_pages)) return EG_MLA_ERR_CUDA;
   a.q = nullptr;  // prologue computes the page prefix sums only
-  cudaError_t e = egmla::launch_prologue_tc(a, nullptr, st);
+  CUtensorMap amaps[2];   // no query: not read
+  std::memset(amaps, 0, sizeof(amaps));
+  cudaError_t e = egmla::launch_prologue_tc(a, nullptr, amaps, st);
   if (e == cudaSuccess) e = egmla::launch_decode_tc(a, maps, true, st, nullptr);
   return to_status(e);
 }

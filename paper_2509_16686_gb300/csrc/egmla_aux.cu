@@ -23,53 +23,53 @@
 namespace egmla {
 
 // ------------------------------------------------------------------ append
-// The new token's rows of sequence b, copied by the calling block; the row
-// copies are 16-byte vectors (the row byte counts allow it for every
-// supported shape).
-__device__ void append_row(const AppendArgs& a, int b) {
+// The new token's rows of sequence b, copied by `nthr` threads (this one is
+// `thr`); the row copies are 16-byte vectors (the row byte counts allow it for
+// every supported shape).
+__device__ void append_row(const AppendArgs& a, int b, int thr, int nthr) {
   const int pos = a.positions[b];
   if (pos < 0) return;
   const int lp = pos / a.page_size;
   if (lp >= a.max_pages) {
-    if (threadIdx.x == 0) report_status(a.status, kStatusOutOfRange);
+    if (thr == 0) report_status(a.status, kStatusOutOfRange);
     return;
   }
   const int page = a.block_table[static_cast<size_t>(b) * a.max_pages + lp];
   if (page < 0 || page >= a.num_pages) {
-    if (threadIdx.x == 0) report_status(a.status, kStatusOutOfRange);
+    if (thr == 0) report_status(a.status, kStatusOutOfRange);
     return;
   }
   const size_t row = static_cast<size_t>(page) * a.page_size + pos % a.page_size;
   uint4* cd = reinterpret_cast<uint4*>(static_cast<uint8_t*>(a.c_pool) + row * a.c_row_bytes);
   const uint4* cs = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(a.c_new) +
                                                    static_cast<size_t>(b) * a.c_row_bytes);
-  for (int i = threadIdx.x; i < a.c_row_bytes / 16; i += blockDim.x) cd[i] = cs[i];
+  for (int i = thr; i < a.c_row_bytes / 16; i += nthr) cd[i] = cs[i];
   uint4* kd = reinterpret_cast<uint4*>(static_cast<uint8_t*>(a.kr_pool) + row * a.kr_row_bytes);
   const uint4* ks = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(a.kr_new) +
                                                    static_cast<size_t>(b) * a.kr_row_bytes);
-  for (int i = threadIdx.x; i < a.kr_row_bytes / 16; i += blockDim.x) kd[i] = ks[i];
-  if (a.id_pool != nullptr && a.ids_new != nullptr && threadIdx.x == 0) a.id_pool[row] = a.ids_new[b];
+  for (int i = thr; i < a.kr_row_bytes / 16; i += nthr) kd[i] = ks[i];
+  if (a.id_pool != nullptr && a.ids_new != nullptr && thr == 0) a.id_pool[row] = a.ids_new[b];
 }
 
 // one block per sequence
-__global__ void append_latent_kernel(const AppendArgs a) { append_row(a, blockIdx.x); }
+__global__ void append_latent_kernel(const AppendArgs a) { append_row(a, blockIdx.x, threadIdx.x, blockDim.x); }
 
 // ------------------------------------------------------------------ helpers
-// eight bf16 (or four fp32) of a 16-byte piece as floats
-__device__ __forceinline__ void unpack16(const uint4& raw, float (&w)[8]) {
-  const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&raw);
+// v[i] (i < 32) summed over the warp; lane t returns the sum of v[t]
+__device__ __forceinline__ float reduce32_transpose(float (&v)[32], int lane) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __bfloat1622float2(e[i]);
-    w[2 * i] = f.x;
-    w[2 * i + 1] = f.y;
+  for (int o = 16, len = 32; o > 0; o >>= 1, len >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < len / 2) {
+        const float keep = up ? v[i + len / 2] : v[i];
+        const float send = up ? v[i] : v[i + len / 2];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
   }
-}
-__device__ __forceinline__ void unpack16(const uint4& raw, float (&w)[4]) {
-  w[0] = __uint_as_float(raw.x);
-  w[1] = __uint_as_float(raw.y);
-  w[2] = __uint_as_float(raw.z);
-  w[3] = __uint_as_float(raw.w);
+  return v[0];
 }
 
 // ------------------------------------------------------------------ prologue
@@ -175,181 +175,194 @@ __device__ void split_starts(const int32_t* cu, const int32_t* seq_lens, int bat
   }
 }
 
-// Tensor-core path: block (head h, chunk of kSumFeatures = 32 latent features,
-// group of up to kPBatch sequences) computes q^_{b,h}[f] = sum_n W_UK,h[n][f] q^C_{b,h}[n]
-// in fp32 and stores (q^ (*) gamma) rounded to bf16 in the prepared query
-// block (qop_offset layout).  Its per-chunk partials of w_h = sum_f bf16(q^ gamma)_f
-// and b_h = q^_h . beta go to the block's slots of the sums area.  Chunk-0
-// blocks also copy q^R.  Block 0 computes the page prefix sums and the
-// splits' start records.
-//  - All 16-byte global loads of a thread are issued before any is stored
-//    (W_UK with an L2 evict-last hint: it stays in L2 across steps).
-//  - W_UK (bf16) and q^C (converted to fp32 once, as it is staged) are held
-//    row-major; a warp takes a quad of sequences and a part of the n range,
-//    reading per 8 n the lane's feature of 8 W rows and 8 n of each q^C row
-//    (two 16-byte broadcasts per sequence) for 32 FMAs.  With few sequences
-//    the spare warps split n further; the parts are added in shared memory.
-constexpr int kPBatch = 32;
-constexpr int kPMaxNope = 256;
-constexpr int kPThreads = 256;
-constexpr int kPLoads = kPMaxNope * kSumFeatures * 2 / 16 / kPThreads;   // 16-byte pieces per thread and array
+// The schedule, by one block of 256 threads: the combine's counters zeroed, the
+// page prefix sums and the splits' start records.  `smem` (`words` ints): the
+// prefix sums in shared memory too where they fit, so that the splits'
+// searches read them there; `wsum`: eight more ints.
+__device__ void schedule_block(const int32_t* seq_lens, int batch, int page_size, int32_t* cu, uint32_t* seq_done,
+                               int num_splits, const int32_t* block_table, int max_pages, SplitStart* starts,
+                               int32_t* smem, int words, int32_t* wsum) {
+  if (seq_done != nullptr)
+    for (int i = threadIdx.x; i <= batch; i += blockDim.x) seq_done[i] = 0u;
+  if (batch + 1 <= words) {
+    page_prefix_sums_block(seq_lens, batch, page_size, cu, smem, wsum);
+    __syncthreads();   // the prefix sums are visible to the whole block
+    split_starts(smem, seq_lens, batch, num_splits, block_table, max_pages, starts);
+  } else {
+    page_prefix_sums(seq_lens, batch, page_size, cu);
+    __syncthreads();
+    split_starts(cu, seq_lens, batch, num_splits, block_table, max_pages, starts);
+  }
+}
 
-// (no launch bound: with one, ptxas trims the kernel to 48 registers and spills)
-__global__ void prologue_tc_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ w_uk,
-                       const float* __restrict__ gamma, const float* __restrict__ beta,
-                       const int32_t* __restrict__ seq_lens, int batch, int d_nope, int d_rope, int d_c,
-                       int page_size, uint8_t* __restrict__ qprep, size_t qstride, int32_t* __restrict__ cu,
-                       uint32_t* __restrict__ seq_done, int num_splits, const int32_t* __restrict__ block_table,
-                       int max_pages, SplitStart* __restrict__ starts, const AppendArgs app) {
-  __shared__ __align__(16) __nv_bfloat16 ws[kPMaxNope][kSumFeatures];  // W_UK,h[n][f0 + f]
-  __shared__ __align__(16) float qs[kPBatch][kPMaxNope];              // q^C_{b0 + j, h}[n]
-  // partial sums [n part * 4 quads + j][f], written once every warp is done with ws
-  float (*red)[kSumFeatures] = reinterpret_cast<float (*)[kSumFeatures]>(&ws[0][0]);
-  static_assert(sizeof(ws) >= 32 * kSumFeatures * sizeof(float), "reduction buffer aliases ws");
+// Tensor-core path: the query absorption as a tcgen05 GEMM per head,
+//   D[f, b] = q^_{b,h}[f] = sum_n W_UK,h[n][f] q^C_{b,h}[n].
+// A block takes (head, 128 features, `nt` sequences): W_UK,h is the M = 128
+// operand read MN-major (features contiguous), q^C the K-major N operand, both
+// copied by TMA in 64-row / 64-column boxes (rows past d_nope and past the
+// batch read as zero; W_UK with an L2 evict-last hint: it stays in L2 across
+// steps).  The fp32 accumulator's lanes are features: a lane stores (q^ (*)
+// gamma) rounded to bf16 in the prepared query blocks (qop_offset layout), and
+// since a warp's quadrant is one chunk of kSumFeatures, the chunk's partials of
+// w_h = sum_f bf16(q^ gamma)_f and b_h = q^_h . beta for 16 sequences take one
+// transposing reduction of 32 values.  The blocks of the first features also
+// copy q^R.  Block 0: the schedule; the blocks after the tiles: the appends, a
+// warp per sequence (no block of this kernel reads the pools).
+// A block's time is one round of copies, its MMAs and its stores.  On CUDA
+// cores the absorption was bound by its shared-memory reads and grew with the
+// batch: 13.1 us at 128 sequences with d_c 192 and 18.9 with d_c 512, 8.3 at 64
+// with d_c 256; now 4.7, 6.2 and 4.6 (kernel alone, warm); equal at 8.
+constexpr int kPmThreads = 256;
+constexpr int kPmTile = 128;                    // features per block (the MMA's M)
+constexpr uint32_t kPmAtomRow = 128;            // bytes of a swizzled 64-element row
+constexpr int kPmMaxSeq = 128;                  // sequences per block, at most (the MMA's N)
+constexpr int kPmBlocks = 152;                  // one per SM
+constexpr int kPmMaxNope = 256;
+
+struct PmBars {
+  uint64_t full[kPmMaxNope / 64];
+  uint64_t done;
+  uint32_t tmem_base;
+  int abort;
+};
+
+__host__ __device__ constexpr uint32_t pm_smem(int nk, int nt) {
+  return static_cast<uint32_t>(nk) * 64 * kPmAtomRow * 2 + static_cast<uint32_t>(nk) * nt * kPmAtomRow + 1024 +
+         sizeof(PmBars);
+}
+
+__global__ void __launch_bounds__(kPmThreads)
+prologue_tc_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap qmap,
+                    const __nv_bfloat16* __restrict__ q, const float* __restrict__ gamma,
+                    const float* __restrict__ beta, const int32_t* __restrict__ seq_lens, int batch, int d_nope,
+                    int d_rope, int d_c, int page_size, uint8_t* __restrict__ qprep, size_t qstride,
+                    int32_t* __restrict__ cu, uint32_t* __restrict__ seq_done, int num_splits,
+                    const int32_t* __restrict__ block_table, int max_pages, SplitStart* __restrict__ starts, int nt,
+                    uint64_t wait_ns, int32_t* status, const AppendArgs app) {
+  extern __shared__ uint8_t pm_raw[];
+  uint8_t* smem = pm_raw + ((1024u - (smem_u32(pm_raw) & 1023u)) & 1023u);
   constexpr int H = 16;
-  const int nchunk = d_c / kSumFeatures;
-  const int ngroups = (batch + kPBatch - 1) / kPBatch;
-  // the decode kernel after this one may begin its setup (it waits for this
-  // kernel's completion before it reads anything written here)
+  const int mt = (d_c + kPmTile - 1) / kPmTile, nbg = (batch + nt - 1) / nt;
+  const int ntiles = q != nullptr ? H * mt * nbg : 0;   // (the cache-read test entry: the schedule only)
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (blockIdx.x == 0 || blockIdx.x > static_cast<unsigned>(ntiles)) {
+    grid_launch_dependents();
+    grid_dependency_wait();
+    if (blockIdx.x == 0) {
+      int32_t* words = reinterpret_cast<int32_t*>(smem);
+      constexpr int kWords = 4096;
+      static_assert(pm_smem(1, 16) >= 1024 + (kWords + 8) * 4, "schedule area");
+      schedule_block(seq_lens, batch, page_size, cu, seq_done, num_splits, block_table, max_pages, starts, words + 8,
+                     kWords, words);
+    } else {
+      const int b = (static_cast<int>(blockIdx.x) - (ntiles + 1)) * (kPmThreads / 32) + warp;
+      if (b < app.batch) append_row(app, b, lane, 32);
+    }
+    return;
+  }
+  const int item = static_cast<int>(blockIdx.x) - 1;
+  const int h = item % H, fm = (item / H) % mt, b0 = (item / (H * mt)) * nt;
+  // the last tile of a latent that is no multiple of 128 starts early and
+  // skips the features of the tile before it
+  const int f_first = fm * kPmTile, f0 = min(f_first, d_c - kPmTile);
+  const int nk = (d_nope + 63) / 64, nb = min(nt, batch - b0);
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t atom = static_cast<uint32_t>(nk) * 64 * kPmAtomRow;   // one 64-feature column of W, all rows
+  const uint32_t q_off = 2 * atom, q_chunk = static_cast<uint32_t>(nt) * kPmAtomRow;
+  PmBars& bars = *reinterpret_cast<PmBars*>(smem + q_off + nk * q_chunk);
+  volatile int* abort_flag = &bars.abort;
+  uint32_t tmem_cols = 32;
+  while (tmem_cols < static_cast<uint32_t>(nt)) tmem_cols <<= 1;
+  if (tid == 0) {
+    for (int k = 0; k < nk; ++k) mbar_init(smem_u32(&bars.full[k]), 1);
+    mbar_init(smem_u32(&bars.done), 1);
+    bars.abort = 0;
+    fence_mbar_init();
+    prefetch_tensormap(&wmap);
+    prefetch_tensormap(&qmap);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&bars.tmem_base), tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = bars.tmem_base;
   grid_launch_dependents();
   grid_dependency_wait();
-  // block 0: the schedule (dispatched first, so that it never waits for a
-  // second wave of the grid); blocks 1 .. A: the absorption items; then the
-  // append blocks
-  const int nabs = H * nchunk * ngroups;
-  if (blockIdx.x > static_cast<unsigned>(nabs)) {
-    // blocks after the schedule block: the new token of one sequence (a step
-    // that appends before it attends); no block of this kernel reads the pools
-    append_row(app, blockIdx.x - (nabs + 1));
-    return;
-  }
-  if (blockIdx.x == 0) {
-    if (seq_done != nullptr)
-      for (int i = threadIdx.x; i <= batch; i += blockDim.x) seq_done[i] = 0u;
-    // the prefix sums in shared memory too (the W_UK staging area is idle in
-    // this block), so that the splits' searches read them there
-    int32_t* cu_s = reinterpret_cast<int32_t*>(&ws[0][0]);
-    int32_t* wsum = reinterpret_cast<int32_t*>(&qs[0][0]);
-    constexpr int kCuSmem = static_cast<int>(sizeof(ws) / sizeof(int32_t));
-    if (batch + 1 <= kCuSmem) {
-      page_prefix_sums_block(seq_lens, batch, page_size, cu, cu_s, wsum);
-      __syncthreads();   // the prefix sums are visible to the whole block
-      split_starts(cu_s, seq_lens, batch, num_splits, block_table, max_pages, starts);
-    } else {
-      page_prefix_sums(seq_lens, batch, page_size, cu);
-      __syncthreads();
-      split_starts(cu, seq_lens, batch, num_splits, block_table, max_pages, starts);
+  if (warp == 0) {
+    if (elect_one()) {
+      const uint64_t keep = policy_evict_last(), once = policy_evict_first();
+      for (int k = 0; k < nk; ++k) {
+        const uint32_t fb = smem_u32(&bars.full[k]);
+        mbar_arrive_expect_tx(fb, 2 * 64 * kPmAtomRow + q_chunk);
+        for (int c = 0; c < 2; ++c)
+          tma_load_3d(sbase + c * atom + k * 64 * kPmAtomRow, &wmap, f0 + 64 * c, 64 * k, h, fb, keep);
+        tma_load_3d(sbase + q_off + k * q_chunk, &qmap, 64 * k, h, b0, fb, once);
+      }
+      const uint32_t idesc = idesc_bf16(kPmTile, nt, 1, 0);
+      const uint64_t wd = smem_desc(sbase, atom, 1024, kSwizzle128B);
+      for (int k = 0; k < nk; ++k) {
+        // every copy lands before the block can leave (own flag: bounded, not cut short)
+        volatile int own = 0;
+        if (!mbar_wait(smem_u32(&bars.full[k]), 0, &own, wait_ns)) *abort_flag = 1;
+        if (*abort_flag) continue;
+        tc_fence_after();
+        const uint64_t qd = smem_desc(sbase + q_off + k * q_chunk, 16, 1024, kSwizzle128B);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16_ss(tmem, wd + ((k * 64 * kPmAtomRow + kk * 2048) >> 4), qd + ((kk * 32) >> 4), idesc,
+                      (k > 0 || kk > 0) ? 1u : 0u);
+      }
+      mma_commit(smem_u32(&bars.done));
     }
-    return;
-  }
-  if (q == nullptr) return;  // cache-read test entry: prefix sums only
-  const int item = static_cast<int>(blockIdx.x) - 1;
-  const int h = item % H, fc = (item / H) % nchunk, bg = item / (H * nchunk);
-  const int b0 = bg * kPBatch, nb = min(kPBatch, batch - b0);
-  const int f0 = fc * kSumFeatures;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int qrow = d_nope + d_rope;
-  // W piece i: row n = i / 4, features 8 (i % 4) ..; q piece i: sequence j = i / (d_nope / 8), columns 8 (i % ..)
-  const int wpieces = d_nope * (kSumFeatures / 8), qpr = d_nope / 8, qpieces = kPBatch * qpr;
-  const uint64_t keep = policy_evict_last();
-  uint4 wv[kPLoads], qv[kPLoads];
-#pragma unroll
-  for (int k = 0; k < kPLoads; ++k) {
-    const int i = tid + k * kPThreads;
-    wv[k] = make_uint4(0, 0, 0, 0);
-    qv[k] = make_uint4(0, 0, 0, 0);
-    if (i < wpieces)
-      wv[k] = ldg_16_na_hint(w_uk + (static_cast<size_t>(h) * d_nope + i / 4) * d_c + f0 + 8 * (i % 4), keep);
-    if (i < qpieces && i / qpr < nb)
-      qv[k] = *reinterpret_cast<const uint4*>(q + (static_cast<size_t>(b0 + i / qpr) * H + h) * qrow + 8 * (i % qpr));
-  }
-#pragma unroll
-  for (int k = 0; k < kPLoads; ++k) {
-    const int i = tid + k * kPThreads;
-    if (i < wpieces) *reinterpret_cast<uint4*>(&ws[i / 4][8 * (i % 4)]) = wv[k];
-    if (i < qpieces) {
-      float x[8];
-      unpack16(qv[k], x);
-      float4* d = reinterpret_cast<float4*>(&qs[i / qpr][8 * (i % qpr)]);
-      d[0] = make_float4(x[0], x[1], x[2], x[3]);
-      d[1] = make_float4(x[4], x[5], x[6], x[7]);
+    __syncwarp();
+  } else if (fm == 0) {
+    // meanwhile: q^R of the block's sequences, 16 bytes at a time
+    const int qrow = d_nope + d_rope, pr = d_rope / 8;
+    for (int i = tid - 32; i < nb * pr; i += kPmThreads - 32) {
+      const int j = i / pr, r = 8 * (i % pr);
+      *reinterpret_cast<uint4*>(qprep + static_cast<size_t>(b0 + j) * qstride + qprep_lat_bytes(d_c) + qop_offset(h, r)) =
+          *reinterpret_cast<const uint4*>(q + (static_cast<size_t>(b0 + j) * H + h) * qrow + d_nope + r);
     }
   }
-  __syncthreads();
-  // warp -> (sequence quad sq, n part kp); nq quads, ks parts of the n range
-  const int nq = (nb + 3) / 4, nblk = d_nope / 8;
-  int ks = 8 / nq;
-  ks = ks >= 8 ? 8 : ks >= 4 ? 4 : ks >= 2 ? 2 : 1;
-  while (nblk % ks) ks >>= 1;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  const int sq = warp % nq, kp = warp / nq, bpk = nblk / ks;
-  if (warp < nq * ks) {
-    for (int blk = kp * bpk; blk < (kp + 1) * bpk; ++blk) {
-      float w[8];
+  // ---- epilogue: warp = (lane quadrant, every other group of 16 sequences)
+  const int quad = warp & 3, f = f0 + 32 * quad + lane;
+  const float gm = gamma ? gamma[f] : 1.f;
+  const float bt = beta ? beta[f] : 0.f;
+  __syncwarp();
+  bool ok = mbar_wait(smem_u32(&bars.done), 0, abort_flag, wait_ns);
+  ok = __all_sync(0xffffffffu, ok) && *abort_flag == 0;
+  tc_fence_after();
+  if (ok && f0 + 32 * quad >= f_first) {   // uniform in the warp
+    const int fc = (f0 + 32 * quad) / kSumFeatures;
+    for (int c0 = 16 * (warp >> 2); c0 < nb; c0 += 32) {
+      float v[16];
+      tmem_ld16(tmem + (static_cast<uint32_t>(32 * quad) << 16) + c0, v);
+      tmem_wait_ld();
+      float part[32];
+      uint8_t* qb = qprep + static_cast<size_t>(b0 + c0) * qstride + qop_offset(h, f);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = __bfloat162float(ws[blk * 8 + e][lane]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 x0 = *reinterpret_cast<const float4*>(&qs[4 * sq + i][blk * 8]);
-        const float4 x1 = *reinterpret_cast<const float4*>(&qs[4 * sq + i][blk * 8 + 4]);
-        acc[i] = fmaf(w[0], x0.x, acc[i]);
-        acc[i] = fmaf(w[1], x0.y, acc[i]);
-        acc[i] = fmaf(w[2], x0.z, acc[i]);
-        acc[i] = fmaf(w[3], x0.w, acc[i]);
-        acc[i] = fmaf(w[4], x1.x, acc[i]);
-        acc[i] = fmaf(w[5], x1.y, acc[i]);
-        acc[i] = fmaf(w[6], x1.z, acc[i]);
-        acc[i] = fmaf(w[7], x1.w, acc[i]);
+      for (int j = 0; j < 16; ++j) {
+        const __nv_bfloat16 bq = __float2bfloat16_rn(v[j] * gm);
+        part[j] = __bfloat162float(bq);
+        part[16 + j] = v[j] * bt;
+        if (c0 + j < nb) *reinterpret_cast<__nv_bfloat16*>(qb + j * qstride) = bq;
+      }
+      const float sum = reduce32_transpose(part, lane);   // lane t: value t
+      if (c0 + (lane & 15) < nb) {
+        float* sums = reinterpret_cast<float*>(qprep + static_cast<size_t>(b0 + c0 + (lane & 15)) * qstride +
+                                               qprep_lat_bytes(d_c) + qprep_rope_bytes(d_rope));
+        sums[(fc * 2 + (lane >> 4)) * 16 + h] = sum;
       }
     }
   }
-  const int f = f0 + lane;
-  const float gm = gamma ? gamma[f] : 1.f;
-  const float bt = beta ? beta[f] : 0.f;
-  // q^ of sequence j (its 32 features over the warp's lanes) -> prepared query block
-  auto emit = [&](int j, float a) {
-    const __nv_bfloat16 bq = __float2bfloat16_rn(a * gm);
-    float wpart = __bfloat162float(bq), bpart = a * bt;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      wpart += __shfl_xor_sync(0xffffffffu, wpart, o);
-      bpart += __shfl_xor_sync(0xffffffffu, bpart, o);
-    }
-    uint8_t* qb = qprep + static_cast<size_t>(b0 + j) * qstride;
-    *reinterpret_cast<__nv_bfloat16*>(qb + qop_offset(h, f)) = bq;
-    if (lane == 0) {
-      float* sums = reinterpret_cast<float*>(qb + qprep_lat_bytes(d_c) + qprep_rope_bytes(d_rope));
-      sums[(fc * 2) * 16 + h] = wpart;
-      sums[(fc * 2 + 1) * 16 + h] = bpart;
-    }
-  };
-  if (ks == 1) {
-    // each warp holds whole sums: emit from registers
-    if (warp < nq) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (4 * sq + i < nb) emit(4 * sq + i, acc[i]);
-    }
-  } else {
-    __syncthreads();   // every warp is done with ws, which red aliases
-    if (warp < nq * ks) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) red[kp * 4 * nq + 4 * sq + i][lane] = acc[i];
-    }
-    __syncthreads();
-    for (int j = warp; j < nb; j += kPThreads / 32) {
-      float a = 0.f;
-      for (int k = 0; k < ks; ++k) a += red[k * 4 * nq + j][lane];
-      emit(j, a);
-    }
-  }
-  if (fc == 0) {
-    for (int i = tid; i < nb * d_rope; i += kPThreads) {
-      const int j = i / d_rope, r = i % d_rope;
-      *reinterpret_cast<__nv_bfloat16*>(qprep + static_cast<size_t>(b0 + j) * qstride + qprep_lat_bytes(d_c) +
-                                        qop_offset(h, r)) = q[(static_cast<size_t>(b0 + j) * H + h) * qrow + d_nope + r];
-    }
-  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc(tmem, tmem_cols);
+  if (tid == 0 && *abort_flag) report_status(status, kStatusTimeout);
 }
 
 // fp32 path: q^ [H, d_c] and q^R [H, d_rope] in fp32, row-major.  Block 0: the
@@ -377,7 +390,7 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
     return;
   }
   if (blockIdx.x > static_cast<unsigned>(nabs)) {   // no block of this kernel reads the pools
-    append_row(app, blockIdx.x - (nabs + 1));
+    append_row(app, blockIdx.x - (nabs + 1), threadIdx.x, blockDim.x);
     return;
   }
   const int item = static_cast<int>(blockIdx.x) - 1;
@@ -471,23 +484,6 @@ constexpr int kCombineMaxDc = 512;
 constexpr int kCombineBlocks = 304;     // two blocks per SM
 constexpr int kCombineSlots = 128;      // slots whose weights are in shared memory at a time
 constexpr int kCombinePairs = kCombineGroup * kCombineMaxDc / 4 / kCombineThreads;   // pairs per thread, at most
-
-// v[i] (i < 32) summed over the warp; lane t returns the sum of v[t]
-__device__ __forceinline__ float reduce32_transpose(float (&v)[32], int lane) {
-#pragma unroll
-  for (int o = 16, len = 32; o > 0; o >>= 1, len >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      if (i < len / 2) {
-        const float keep = up ? v[i + len / 2] : v[i];
-        const float send = up ? v[i] : v[i + len / 2];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
-  }
-  return v[0];
-}
 
 template <typename T>
 __global__ void __launch_bounds__(kCombineThreads)
@@ -917,22 +913,37 @@ cudaError_t launch_append(const AppendArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, cudaStream_t st) {
+// The fewest sequences per block (a multiple of the MMA's 16) that leave at
+// most one block per SM, so that the blocks' epilogues are short.
+int absorb_tile(int d_c, int batch) {
+  const int mt = (d_c + kPmTile - 1) / kPmTile;
+  int nt = 16;
+  while (nt < kPmMaxSeq && 16 * mt * ((batch + nt - 1) / nt) > kPmBlocks) nt *= 2;
+  return nt;
+}
+
+cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, const CUtensorMap* maps, cudaStream_t st) {
   const WorkspaceLayout wl = workspace_layout(a.batch, a.num_splits, 16, a.d_c, a.d_rope, true);
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
   // with the gate off the latent is used as cached: no LayerNorm affine to fold into q^
   const float* gamma = a.gate && a.gate_ln ? a.ln_gamma : nullptr;
   const float* beta = a.gate && a.gate_ln ? a.ln_beta : nullptr;
-  const int ngroups = (a.batch + kPBatch - 1) / kPBatch;
   AppendArgs none;
   std::memset(&none, 0, sizeof(none));
   const AppendArgs& ap = app != nullptr ? *app : none;
+  const int nt = absorb_tile(a.d_c, a.batch), mt = (a.d_c + kPmTile - 1) / kPmTile, nk = (a.d_nope + 63) / 64;
+  const int tiles = a.q != nullptr ? 16 * mt * ((a.batch + nt - 1) / nt) : 0;
+  const int blocks = tiles + 1 + (ap.batch + kPmThreads / 32 - 1) / (kPmThreads / 32);
+  const size_t smem = pm_smem(nk, nt);
+  const cudaError_t e =
+      cudaFuncSetAttribute(prologue_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
   return launch_chained(
-      prologue_tc_kernel, dim3(16 * (a.d_c / kSumFeatures) * ngroups + 1 + ap.batch), dim3(256), 0, st,
-      static_cast<const __nv_bfloat16*>(a.q), static_cast<const __nv_bfloat16*>(a.w_uk), gamma, beta,
-      a.seq_lens, a.batch, a.d_nope, a.d_rope, a.d_c, a.page_size, ws + wl.off_qprep, wl.qprep_stride,
-      reinterpret_cast<int32_t*>(ws + wl.off_cu), reinterpret_cast<uint32_t*>(ws + wl.off_done), a.num_splits,
-      a.block_table, a.max_pages, reinterpret_cast<SplitStart*>(ws + wl.off_start), ap);
+      prologue_tc_kernel, dim3(blocks), dim3(kPmThreads), smem, st, maps[0], maps[1],
+      static_cast<const __nv_bfloat16*>(a.q), gamma, beta, a.seq_lens, a.batch, a.d_nope, a.d_rope, a.d_c,
+      a.page_size, ws + wl.off_qprep, wl.qprep_stride, reinterpret_cast<int32_t*>(ws + wl.off_cu),
+      reinterpret_cast<uint32_t*>(ws + wl.off_done), a.num_splits, a.block_table, a.max_pages,
+      reinterpret_cast<SplitStart*>(ws + wl.off_start), nt, kWaitLimitNs, a.status, ap);
 }
 
 namespace {

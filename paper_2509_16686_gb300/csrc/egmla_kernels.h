@@ -103,7 +103,11 @@ struct DecodeArgs {
 cudaError_t launch_append(const AppendArgs& a, cudaStream_t st);
 // query absorption and split schedule; with `app` non-null its blocks also
 // append the new token of every sequence (the pools are read by no block of it)
-cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, cudaStream_t st);
+// `maps`: W_UK as {d_c, d_nope, H} in boxes of {64, 64, 1} and q^C as {d_nope, H,
+// batch} in boxes of {64, 1, absorb_tile}
+cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, const CUtensorMap* maps, cudaStream_t st);
+// sequences per block of the absorption
+int absorb_tile(int d_c, int batch);
 // fp32: absorption (with the append blocks of `app` when it is non-null) and the split-KV kernel
 cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaStream_t st);
 cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, cudaStream_t st);

@@ -86,6 +86,28 @@ def test_bf16_small_matches_oracle(gpu_lib, d_c, lens):
         check_bf16(got, ref, f"d_c={d_c} lens={lens} splits={splits}", scaled_abs=min(lens) < 128)
 
 
+@pytest.mark.parametrize("d_c,gate", [(192, True), (256, True), (512, False)])
+@pytest.mark.parametrize("batch,d_nope", [(15, 128), (16, 40), (17, 128), (33, 256), (70, 72), (140, 128), (300, 64)])
+def test_bf16_query_absorption_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_nope):
+    """The query absorption at the edges of its tiles: sequences per block (16 to
+    128, part-filled last blocks, both sides of the batch from which it runs on
+    the tensor cores), d_nope below, on and off a multiple of 64, the
+    overlapping feature tile of d_c 192; short contexts."""
+    dims = synth.Dims(num_heads=16, d_nope=d_nope, d_rope=64, d_v=64, d_c=d_c, page_size=64, vocab=500, dtype="bf16",
+                      gate=gate)
+    lens = [1 + (37 * b) % 90 for b in range(batch)]
+    case = synth.make_case("absorb", dims, lens, seed=34, latent_scale=0.5, layout="permuted", affine_ln=True)
+    ref = orc.decode_unabsorbed(case)
+    _, got = run(case, 0)
+    assert np.isfinite(got).all()
+    # thousands of short sequences' rows: rel-L2 over each sequence instead of
+    # the largest of all elements' errors (the bf16 bound of one row, 2^-8 per
+    # rounding of q^, z, P and u, four independent roundings)
+    diff = np.linalg.norm((got - ref).reshape(batch, -1), axis=1)
+    rel = diff / np.linalg.norm(ref.reshape(batch, -1), axis=1)
+    assert rel.max() <= 4 * 2.0 ** -8 and rel_l2(got, ref) <= 5e-3, (float(rel.max()), rel_l2(got, ref))
+
+
 # --------------------------------------------------------------------------- gating ablations (Section 4.4)
 @pytest.mark.parametrize("op", ["mul", "add_ln"])
 @pytest.mark.parametrize("d_c", [256, 192])
