@@ -15,6 +15,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "egmla_common.cuh"
 #include "egmla_kernels.h"
@@ -443,20 +444,7 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
   }
 }
 
-// ------------------------------------------------------------------ combine
-template <typename T>
-__device__ __forceinline__ float to_f(T v);
-template <>
-__device__ __forceinline__ float to_f<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename T>
-__device__ __forceinline__ T from_f(float v);
-template <>
-__device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-
+// ------------------------------------------------------------------ combine, fp32
 // Block per (head h, group of kCombineGroup sequences; blockIdx.y: a part of the
 // d_v output rows, each part repeating the merge), 256 threads: the
 // sequences of a group share one pass over W_UV,h.  The splits that covered
@@ -471,8 +459,7 @@ __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return
 //    four pairs and four slots of each in flight, so that the time is a few
 //    round trips whatever the number of slots (a warp per sequence, one slot
 //    after another, took 60 us of an fp32 step of 8 sequences of 100 to 3000
-//    tokens, up to 47 slots each; 15 us now, and 20 us against
-//    26.3 us at 128 sequences with d_c 512: ncu, cold caches);
+//    tokens, up to 47 slots each; 15 us now: ncu, cold caches);
 //  - u: warp w takes groups of four W_UV,h rows; a lane loads its 16-byte
 //    pieces of the four rows once and multiplies them into all the group's
 //    merged vectors (shared memory), then the 32 sums (sequence, row) are
@@ -485,10 +472,9 @@ constexpr int kCombineBlocks = 304;     // two blocks per SM
 constexpr int kCombineSlots = 128;      // slots whose weights are in shared memory at a time
 constexpr int kCombinePairs = kCombineGroup * kCombineMaxDc / 4 / kCombineThreads;   // pairs per thread, at most
 
-template <typename T>
 __global__ void __launch_bounds__(kCombineThreads)
 combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml, const float* __restrict__ part_o,
-               const T* __restrict__ w_uv, T* __restrict__ out, int batch, int H, int d_c, int d_v,
+               const float* __restrict__ w_uv, float* __restrict__ out, int batch, int H, int d_c, int d_v,
                int num_splits) {
   __shared__ __align__(16) float olat[kCombineGroup][kCombineMaxDc];
   __shared__ float wts[kCombineGroup][kCombineSlots];
@@ -590,9 +576,9 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
   }
   __syncthreads();
   // u[j][v] = sum_f W_UV[h][v][f] olat[j][f]
-  constexpr int VEC = 16 / sizeof(T);
-  const int npieces = d_c / VEC;   // d_c is a multiple of VEC for both element types
-  const T* wh = w_uv + static_cast<size_t>(h) * d_v * d_c;
+  constexpr int VEC = 4;
+  const int npieces = d_c / VEC;   // d_c is a multiple of 4
+  const float* wh = w_uv + static_cast<size_t>(h) * d_v * d_c;
   for (int v0 = 4 * (warp + kWarps * blockIdx.y); v0 < d_v; v0 += 4 * kWarps * gridDim.y) {
     float acc[32];
 #pragma unroll
@@ -601,11 +587,12 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
       float wf[4][VEC];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        uint4 raw = make_uint4(0, 0, 0, 0);
-        if (v0 + r < d_v) raw = *reinterpret_cast<const uint4*>(wh + static_cast<size_t>(v0 + r) * d_c + pc * VEC);
-        const T* e = reinterpret_cast<const T*>(&raw);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) wf[r][i] = to_f<T>(e[i]);
+        float4 raw = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (v0 + r < d_v) raw = *reinterpret_cast<const float4*>(wh + static_cast<size_t>(v0 + r) * d_c + pc * VEC);
+        wf[r][0] = raw.x;
+        wf[r][1] = raw.y;
+        wf[r][2] = raw.z;
+        wf[r][3] = raw.w;
       }
 #pragma unroll
       for (int j = 0; j < kCombineGroup; ++j) {
@@ -628,8 +615,263 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
     }
     const float sum = reduce32_transpose(acc, lane);
     const int j = lane >> 2, v = v0 + (lane & 3);
-    if (j < nb && v < d_v) out[(static_cast<size_t>(b0 + j) * H + h) * d_v + v] = from_f<T>(sum);
+    if (j < nb && v < d_v) out[(static_cast<size_t>(b0 + j) * H + h) * d_v + v] = sum;
   }
+}
+
+// ------------------------------------------------------------------ combine, bf16
+// The merge and W_UV of the tensor-core path, for the launches whose decode
+// kernel does not fuse them.  A block takes (head h, `nt` sequences, 128 output
+// rows):
+//  - W_UV,h's rows (the MMA's M = 128 operand, K = d_c) are copied by TMA before
+//    the block waits for the decode kernel, which does not write them;
+//  - merge as in combine_kernel: weights per (sequence, slot) in shared memory,
+//    then thread t takes (sequence, 4 features) pairs; where the block has fewer
+//    pairs than threads, the slots are dealt to groups of threads whose sums
+//    are added in group order;
+//  - the merged fp32 vector is split into three bf16 pieces (o = o1 + o2 + o3 to
+//    2^-24 |o|), which become three columns of the N operand, so that
+//    u = W_UV,h o1 + W_UV,h o2 + W_UV,h o3 keeps the fp32 value of o (the weights
+//    are bf16 as stored), accumulated in fp32;
+//  - u: lanes are output rows; a sequence's three columns are added, rounded to
+//    bf16 and stored.
+// Bound by the merge's reads of the partials from L2 and the latency of its
+// phases: 9 us at 128 sequences with d_c 192 (the merge at the end of the
+// decode kernel, on CUDA cores after a grid-wide wait, and the cooperative
+// launch it needs cost that step 8 us more), and 13 us against 18 on CUDA cores
+// with d_c 512 (kernel alone, warm).
+constexpr int kCtThreads = 256;
+constexpr int kCtMaxSeq = 16;            // sequences per block, at most
+constexpr int kCtBlocks = 152;           // one per SM
+constexpr uint32_t kCtAtom = 128 * 128;  // 128 rows x 64 bf16
+
+// the N operand's rows: three per sequence, a multiple of the MMA's 16
+__host__ __device__ constexpr int ct_cols(int nt) { return (3 * nt + 15) / 16 * 16; }
+
+struct CtShared {
+  float wts[kCtMaxSeq][kCombineSlots];
+  float inv_l[kCtMaxSeq];
+  int slots[kCtMaxSeq], slot0[kCtMaxSeq];
+  float4 red[kCtThreads];
+  uint64_t afull, done;
+  uint32_t tmem_base;
+  int abort;
+};
+__host__ __device__ constexpr uint32_t ct_smem(int d_c, int nt) {
+  return static_cast<uint32_t>(d_c / 64) * (kCtAtom + ct_cols(nt) * 128) + sizeof(CtShared) + 1024;
+}
+
+// PPT: (sequence, 4 features) pairs per thread, at most
+template <int PPT>
+__global__ void __launch_bounds__(kCtThreads)
+combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __restrict__ cu,
+                  const float* __restrict__ part_ml, const float* __restrict__ part_o, __nv_bfloat16* __restrict__ out,
+                  int batch, int d_c, int d_v, int num_splits, int nt, int early, uint64_t wait_ns, int32_t* status) {
+  constexpr int H = 16;
+  constexpr int kFlight = PPT >= 8 ? 2 : PPT >= 4 ? 4 : 8;   // slots of a pair in flight
+  extern __shared__ uint8_t ct_raw[];
+  uint8_t* smem = ct_raw + ((1024u - (smem_u32(ct_raw) & 1023u)) & 1023u);
+  const uint32_t sbase = smem_u32(smem);
+  const int nkc = d_c / 64, cols = ct_cols(nt), ncol = d_c / 4, pairs = nt * ncol;
+  const uint32_t o_off = static_cast<uint32_t>(nkc) * kCtAtom, o_chunk = static_cast<uint32_t>(cols) * 128;
+  CtShared& sh = *reinterpret_cast<CtShared*>(smem + o_off + nkc * o_chunk);
+  volatile int* abort_flag = &sh.abort;
+  const int h = blockIdx.x % H, b0 = (blockIdx.x / H) * nt, v0 = blockIdx.y * 128;
+  const int nb = min(nt, batch - b0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kCtThreads / 32;
+  if (tid == 0) {
+    mbar_init(smem_u32(&sh.afull), 1);
+    mbar_init(smem_u32(&sh.done), 1);
+    sh.abort = 0;
+    fence_mbar_init();
+    prefetch_tensormap(&wmap);
+    const uint64_t keep = policy_evict_last();
+    mbar_arrive_expect_tx(smem_u32(&sh.afull), static_cast<uint32_t>(nkc) * kCtAtom);
+    for (int kc = 0; kc < nkc; ++kc) tma_load_3d(sbase + kc * kCtAtom, &wmap, 64 * kc, v0, h, smem_u32(&sh.afull), keep);
+  }
+  if (early) grid_launch_dependents();   // the layer's output projection, which streams weights of its own
+  const uint32_t tmem_cols = cols <= 32 ? 32u : 64u;
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&sh.tmem_base), tmem_cols);
+    tmem_relinquish();
+  }
+  grid_dependency_wait();
+  const int chunk = split_chunk(cu[batch], num_splits);
+  const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
+  // the slots of this warp's sequences (warp, warp + 8) and their maxima
+  int n[2] = {0, 0};
+  float M[2] = {-INFINITY, -INFINITY}, lsum[2] = {0.f, 0.f};
+  const float* pml[2] = {part_ml, part_ml};
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int j = warp + kWarps * e;
+    if (j >= nb) continue;
+    const int b = b0 + j, p0 = cu[b] + kSegCost, p1 = cu[b + 1], c0 = p0 / chunk;   // units of the sequence's pages
+    n[e] = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
+    pml[e] += (static_cast<size_t>(c0 + b) * H + h) * 2;
+    if (lane == 0) {
+      sh.slots[j] = n[e];
+      sh.slot0[j] = c0 + b;
+    }
+    for (int k = lane; k < n[e]; k += 32) M[e] = fmaxf(M[e], pml[e][k * mlstride]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M[e] = fmaxf(M[e], __shfl_xor_sync(0xffffffffu, M[e], o));
+  }
+  // this thread's pairs, and its group where the slots are dealt out
+  const int groups = pairs < kCtThreads ? kCtThreads / pairs : 1;
+  const int grp = groups > 1 ? tid / pairs : 0;
+  int pj[PPT], pf[PPT];
+  const float* po[PPT];
+  float4 acc[PPT];
+  __syncthreads();
+  int nmax = 0;
+  for (int j = 0; j < nb; ++j) nmax = max(nmax, sh.slots[j]);
+#pragma unroll
+  for (int u = 0; u < PPT; ++u) {
+    const int i = groups > 1 ? tid - grp * pairs : tid + u * kCtThreads;
+    const int j = i / ncol;
+    const bool live = grp < groups && j < nb && (groups == 1 || u == 0);
+    pj[u] = live ? j : -1;
+    pf[u] = 4 * (i - j * ncol);
+    acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    po[u] = part_o + (static_cast<size_t>(live ? sh.slot0[j] : 0) * H + h) * d_c + pf[u];
+  }
+  for (int k0 = 0; k0 < nmax; k0 += kCombineSlots) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = warp + kWarps * e;
+      if (j >= nb) continue;
+      for (int k = lane; k < kCombineSlots; k += 32) {
+        float wk = 0.f;
+        if (k0 + k < n[e]) {
+          const float2 ml = *reinterpret_cast<const float2*>(pml[e] + (k0 + k) * mlstride);
+          wk = exp2f(ml.x - M[e]);
+          lsum[e] = fmaf(wk, ml.y, lsum[e]);
+        }
+        sh.wts[j][k] = wk;
+      }
+    }
+    __syncthreads();
+    const int kn = min(kCombineSlots, nmax - k0);
+    for (int k = grp; k < kn; k += groups * kFlight) {
+      float4 v[PPT][kFlight];
+#pragma unroll
+      for (int u = 0; u < PPT; ++u)
+#pragma unroll
+        for (int e = 0; e < kFlight; ++e) {
+          const int kk = k + e * groups;
+          v[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (pj[u] >= 0 && kk < kn && k0 + kk < sh.slots[pj[u]])
+            v[u][e] = *reinterpret_cast<const float4*>(po[u] + (k0 + kk) * sstride);
+        }
+#pragma unroll
+      for (int u = 0; u < PPT; ++u)
+#pragma unroll
+        for (int e = 0; e < kFlight; ++e) {
+          const int kk = k + e * groups;
+          const float w = pj[u] >= 0 && kk < kn ? sh.wts[pj[u]][kk] : 0.f;   // 0 past the sequence's slots
+          acc[u].x = fmaf(w, v[u][e].x, acc[u].x);
+          acc[u].y = fmaf(w, v[u][e].y, acc[u].y);
+          acc[u].z = fmaf(w, v[u][e].z, acc[u].z);
+          acc[u].w = fmaf(w, v[u][e].w, acc[u].w);
+        }
+    }
+    __syncthreads();   // the weights are read: the next slots' may overwrite them
+  }
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int j = warp + kWarps * e;
+    if (j >= nb) continue;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lsum[e] += __shfl_xor_sync(0xffffffffu, lsum[e], o);
+    if (lane == 0) sh.inv_l[j] = n[e] > 0 ? 1.f / lsum[e] : 0.f;
+  }
+  if (groups > 1) sh.red[tid] = acc[0];
+  __syncthreads();
+  // the merged vectors as three bf16 pieces, rows j, nt + j and 2 nt + j of the N
+  // operand (K-major, 128-byte swizzle)
+#pragma unroll
+  for (int u = 0; u < PPT; ++u) {
+    if (pj[u] < 0 || grp > 0) continue;
+    float4 a = acc[u];
+    for (int g = 1; g < groups; ++g) {
+      const float4 r = sh.red[tid + g * pairs];
+      a = make_float4(a.x + r.x, a.y + r.y, a.z + r.z, a.w + r.w);
+    }
+    const float il = sh.inv_l[pj[u]];
+    float x[4] = {a.x * il, a.y * il, a.z * il, a.w * il};
+    const int kc = pf[u] / 64, unit = (pf[u] % 64) / 8;
+#pragma unroll
+    for (int piece = 0; piece < 3; ++piece) {
+      const int row = piece * nt + pj[u];
+      uint32_t w[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const __nv_bfloat162 z = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+        w[e] = *reinterpret_cast<const uint32_t*>(&z);
+        const float2 zf = __bfloat1622float2(z);
+        x[2 * e] -= zf.x;
+        x[2 * e + 1] -= zf.y;
+      }
+      *reinterpret_cast<uint2*>(smem + o_off + kc * o_chunk + row * 128 + ((unit ^ (row & 7)) << 4) + (pf[u] & 4) * 2) =
+          make_uint2(w[0], w[1]);
+    }
+  }
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sh.tmem_base;
+  if (tid == 0) {
+    volatile int own = 0;   // the copies land before the block can leave
+    if (!mbar_wait(smem_u32(&sh.afull), 0, &own, wait_ns)) {
+      *abort_flag = 1;
+    } else {
+      tc_fence_after();
+      const uint32_t idesc = idesc_bf16(128, cols, 0, 0);
+      for (int kc = 0; kc < nkc; ++kc) {
+        const uint64_t ad = smem_desc(sbase + kc * kCtAtom, 16, 1024, kSwizzle128B);
+        const uint64_t bd = smem_desc(sbase + o_off + kc * o_chunk, 16, 1024, kSwizzle128B);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16_ss(tmem, ad + ((kk * 32) >> 4), bd + ((kk * 32) >> 4), idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+      }
+    }
+    mma_commit(smem_u32(&sh.done));
+  }
+  __syncwarp();
+  bool ok = mbar_wait(smem_u32(&sh.done), 0, abort_flag, wait_ns);
+  ok = __all_sync(0xffffffffu, ok) && *abort_flag == 0;
+  tc_fence_after();
+  // ---- u: warp = (lane quadrant, every other sequence)
+  if (ok) {
+    float d[48];
+    const uint32_t ta = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
+#pragma unroll
+    for (int c = 0; c < 48; c += 16)
+      if (c < cols) tmem_ld16(ta + c, *reinterpret_cast<float(*)[16]>(&d[c]));
+    tmem_wait_ld();
+    const int v = v0 + 32 * (warp & 3) + lane;
+    // (nt is a power of two: the columns of a sequence by a compile-time switch)
+    auto store = [&](auto nt_c) {
+      constexpr int NT = decltype(nt_c)::value;
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+        if ((NT == 1 ? warp < 4 : (j & 1) == warp >> 2) && j < nb && v < d_v)
+          out[(static_cast<size_t>(b0 + j) * H + h) * d_v + v] = __float2bfloat16_rn(d[j] + (d[NT + j] + d[2 * NT + j]));
+    };
+    if (nt == 1) store(std::integral_constant<int, 1>{});
+    else if (nt == 2) store(std::integral_constant<int, 2>{});
+    else if (nt == 4) store(std::integral_constant<int, 4>{});
+    else if (nt == 8) store(std::integral_constant<int, 8>{});
+    else store(std::integral_constant<int, 16>{});
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc(tmem, tmem_cols);
+  if (tid == 0 && *abort_flag) report_status(status, kStatusTimeout);
 }
 
 // ------------------------------------------------------------------ fp32 decode
@@ -984,26 +1226,43 @@ cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaSt
 }
 
 namespace {
-template <typename T>
-cudaError_t launch_combine_t(const DecodeArgs& a, const int32_t* cu, const float* ml, const float* po, cudaStream_t st) {
-  // small batches: the output rows spread over more blocks (a pass of the block's
-  // warps covers 32 rows), so that most SMs read a part of W_UV
-  const int groups = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup), passes = (a.d_v + 31) / 32;
-  int parts = kCombineBlocks / groups;
-  parts = parts < 1 ? 1 : parts > passes ? passes : parts;
-  return launch_chained(combine_kernel<T>, dim3(groups, parts), dim3(kCombineThreads), 0, st, cu, ml, po,
-                        static_cast<const T*>(a.w_uv), static_cast<T*>(a.out), a.batch, a.H, a.d_c, a.d_v,
-                        a.num_splits);
+template <int PPT>
+cudaError_t launch_combine_tc(const DecodeArgs& a, const CUtensorMap* wmap, const int32_t* cu, const float* ml,
+                              const float* po, int nt, cudaStream_t st) {
+  const size_t smem = ct_smem(a.d_c, nt);
+  const cudaError_t e = cudaFuncSetAttribute(combine_tc_kernel<PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  return launch_chained(combine_tc_kernel<PPT>, dim3(16 * ((a.batch + nt - 1) / nt), (a.d_v + 127) / 128),
+                        dim3(kCtThreads), smem, st, *wmap, cu, ml, po, static_cast<__nv_bfloat16*>(a.out), a.batch,
+                        a.d_c, a.d_v, a.num_splits, nt, a.early, kWaitLimitNs, a.status);
 }
 }  // namespace
 
-cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, cudaStream_t st) {
+cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, const CUtensorMap* wmap, cudaStream_t st) {
   const WorkspaceLayout wl = workspace_layout(a.batch, a.num_splits, a.H, a.d_c, a.d_rope, tc_path);
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
   const int32_t* cu = reinterpret_cast<const int32_t*>(ws + wl.off_cu);
   const float* ml = reinterpret_cast<const float*>(ws + wl.off_ml);
   const float* po = reinterpret_cast<const float*>(ws + wl.off_o);
-  return a.dtype == 0 ? launch_combine_t<__nv_bfloat16>(a, cu, ml, po, st) : launch_combine_t<float>(a, cu, ml, po, st);
+  if (tc_path) {
+    // the fewest sequences per block that leave one block per SM
+    int nt = 1;
+    while (nt < kCtMaxSeq && 16 * ((a.batch + nt - 1) / nt) > kCtBlocks) nt *= 2;
+    const int pairs = nt * (a.d_c / 4);
+    if (pairs <= kCtThreads) return launch_combine_tc<1>(a, wmap, cu, ml, po, nt, st);
+    if (pairs <= 2 * kCtThreads) return launch_combine_tc<2>(a, wmap, cu, ml, po, nt, st);
+    if (pairs <= 4 * kCtThreads) return launch_combine_tc<4>(a, wmap, cu, ml, po, nt, st);
+    return launch_combine_tc<8>(a, wmap, cu, ml, po, nt, st);
+  }
+  // small batches: the output rows spread over more blocks (a pass of the block's
+  // warps covers 32 rows), so that most SMs read a part of W_UV
+  const int groups = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup), passes = (a.d_v + 31) / 32;
+  int parts = kCombineBlocks / groups;
+  parts = parts < 1 ? 1 : parts > passes ? passes : parts;
+  return launch_chained(combine_kernel, dim3(groups, parts), dim3(kCombineThreads), 0, st, cu, ml, po,
+                        static_cast<const float*>(a.w_uv), static_cast<float*>(a.out), a.batch, a.H, a.d_c, a.d_v,
+                        a.num_splits);
 }
 
 }  // namespace egmla

@@ -95,8 +95,6 @@ constexpr uint32_t kSmemLimit = 232448;
 // named barriers of the softmax warps (0 is __syncthreads)
 constexpr int kBarTile = 1;
 constexpr int kBarXch = 2;
-// sequences per unit of the fused combine
-constexpr uint32_t kFusedMaxG = 16;
 // W_UV,h rows per warp in the fused combine (the fused path needs d_v <= 9 x warps)
 constexpr int kCombineRowsPerWarp = 9;
 // a head's reference max moves only when a tile exceeds it by 2^8
@@ -152,8 +150,6 @@ struct Cfg {
   // D_C = 192 the second chunk starts at 64 and overlaps the first, so that no
   // MMA reads past the latent part of a slot (its rows 64..127 are not read out)
   __host__ __device__ static constexpr int mc_start(int j) { return j == 0 ? 0 : D_C - 128; }
-  // fused combine: up to kFusedMaxG merged latent rows reuse the page-slot area
-  static_assert(kFusedMaxG * D_C * 4 <= OFF_QBUF, "fused combine area");
 };
 
 struct TcParams {
@@ -180,12 +176,11 @@ struct TcParams {
   // run of (tag, clock64) pairs; tag = event << 24 | tile
   unsigned long long* trace;
   int trace_ctas, trace_cap;
-  // fused split combine (cooperative launch only): W_UV, output, grid counter,
-  // and the (head, group of cmb_g sequences) units
+  // fused split combine (cooperative launch only): W_UV and output
   const __nv_bfloat16* w_uv;
   __nv_bfloat16* out;
-  uint32_t* seq_done;   // [0] CTAs done, [1 + b] split partials of sequence b stored
-  int d_v, cmb_groups, cmb_g;
+  uint32_t* seq_done;   // [1 + b] split partials of sequence b stored
+  int d_v;
   int fuse, early;
   // limit of every wait (ns); a test entry lowers it, together with a
   // withheld page copy (stall_cta, stall_tile; stall_cta < 0: none)
@@ -485,20 +480,17 @@ __device__ __forceinline__ float reduce8_rows(const float (&v)[8], int lane) {
 
 // Split-KV combine inside the decode kernel (cooperative launch: every CTA is
 // resident, so a wait on other CTAs cannot starve).  A CTA merges its units
-// (head h, group of cmb_g sequences) once their split partials are stored:
-// with one sequence per unit (small batches) as soon as the softmax warps of
-// the splits that covered that sequence have counted their parts on its
-// counter, otherwise after every CTA has arrived on a grid counter (both
-// counters zeroed by the prologue kernel of the same call).  For each sequence
-// b, over the splits s that covered it,
+// (head h, sequence b) once the softmax warps of the splits that covered the
+// sequence have counted their parts of its partials on its counter (zeroed by
+// the prologue kernel of the same call).  Over the splits s that covered b,
 //   o = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s,  M = max_s m_s,
 //   u_{b,h} = W_UV,h o
 // (a sequence of length 0 gets u = 0).  Each warp loads its nine rows of
 // W_UV,h (lane l holding features 8l .. 8l + 7) from global memory into
 // registers before it waits, so that the loads overlap the wait.  Merge: a
-// warp per (sequence, 32 features), lane k loading (m, l) of slot k0 + k and
+// warp per 32 features, lane k loading (m, l) of slot k0 + k and
 // every lane O of 32 slots at once (online rescaling across groups of 32),
-// into shared memory.  u: per sequence, the warp's first eight row sums
+// into shared memory.  u: the warp's first eight row sums
 // reduced across the lanes by a transposing butterfly (9 shuffles, after
 // which lane 4r holds row r) and the ninth by a plain warp sum.
 template <int D_C, bool TRACE>
@@ -508,38 +500,16 @@ __device__ void fused_combine(const TcParams& p, uint8_t* smem, Bars& bars) {
   constexpr int LANES = D_C / 8;     // lanes holding 8 features each
   constexpr int kRows = kCombineRowsPerWarp;   // output rows of W_UV,h per warp
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int G = p.cmb_g, units = kHeads * p.cmb_groups;
-  float* olat = reinterpret_cast<float*>(smem);   // [G][D_C], in the free page-slot area
+  const int units = kHeads * p.batch;
+  float* olat = reinterpret_cast<float*>(smem);   // [D_C], in the free page-slot area
   volatile int* abort_flag = &bars.abort;
   const uint64_t wait_ns = p.wait_ns;
   const uint64_t keep = policy_evict_last();
   const int v0 = warp * kRows;   // this warp's first output row
   const int total = p.cu[p.batch];
   const int chunk = split_chunk(total, gridDim.x);
-  // splits that covered sequence b
-  auto splits_of = [&](int b) -> int {
-    const int q0 = p.cu[b] + kSegCost, q1 = p.cu[b + 1];   // units of the sequence's pages
-    return q1 > q0 ? (q1 - 1) / chunk - q0 / chunk + 1 : 0;
-  };
-  if (G > 1 && tid == 0) {
-    // units of several sequences wait for the whole grid: this CTA's partials
-    // are stored (the kernel-end barrier ordered the other threads' stores
-    // before this thread): release them, then wait for all
-    __threadfence();
-    atomicAdd(p.seq_done, 1u);
-    const uint64_t t0 = globaltimer();
-    while (ld_acquire_gpu(p.seq_done) < gridDim.x) {
-      if (globaltimer() - t0 > wait_ns) {
-        report_status(p.status, kStatusTimeout);
-        *abort_flag = 1;
-        break;
-      }
-      __nanosleep(32);
-    }
-  }
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    const int h = u % kHeads, grp = u / kHeads;
-    const int b0 = grp * G, nb = min(G, p.batch - b0);
+    const int h = u % kHeads, b = u / kHeads;
     // this warp's W_UV,h rows, requested before the wait
     uint4 wraw[kRows];
 #pragma unroll
@@ -549,11 +519,14 @@ __device__ void fused_combine(const TcParams& p, uint8_t* smem, Bars& bars) {
       if (lane < LANES && v < p.d_v)
         wraw[r] = ldg_16_na_hint(p.w_uv + (static_cast<size_t>(h) * p.d_v + v) * D_C + 8 * lane, keep);
     }
-    if (G == 1 && tid == 0 && !*abort_flag) {
-      // a unit of one sequence: every softmax warp's part of every split partial of it stored
-      const uint32_t want = static_cast<uint32_t>(kSoftWarps) * static_cast<uint32_t>(splits_of(b0));
+    const int q0 = p.cu[b] + kSegCost, q1 = p.cu[b + 1];   // units of the sequence's pages
+    const int c0 = q0 / chunk;
+    const int n = q1 > q0 ? (q1 - 1) / chunk - c0 + 1 : 0;   // splits that covered it
+    if (tid == 0 && !*abort_flag) {
+      // every softmax warp's part of every split partial of the sequence stored
+      const uint32_t want = static_cast<uint32_t>(kSoftWarps) * static_cast<uint32_t>(n);
       const uint64_t t0 = globaltimer();
-      while (ld_acquire_gpu(p.seq_done + 1 + b0) < want) {
+      while (ld_acquire_gpu(p.seq_done + 1 + b) < want) {
         if (*abort_flag) break;
         if (globaltimer() - t0 > wait_ns) {
           report_status(p.status, kStatusTimeout);
@@ -566,11 +539,8 @@ __device__ void fused_combine(const TcParams& p, uint8_t* smem, Bars& bars) {
     __syncthreads();
     if (u == static_cast<int>(blockIdx.x)) phase_mark<TRACE>(p, 4);
     if (*abort_flag) return;
-    for (int w = warp; w < nb * NFB; w += kWarps) {
-      const int j = w / NFB, f = (w % NFB) * 32 + lane, b = b0 + j;
-      const int q0 = p.cu[b] + kSegCost, q1 = p.cu[b + 1];   // units of the sequence's pages
-      const int c0 = q0 / chunk;
-      const int n = q1 > q0 ? (q1 - 1) / chunk - c0 + 1 : 0;
+    for (int w = warp; w < NFB; w += kWarps) {
+      const int f = w * 32 + lane;
       const float* po = p.part_o + (static_cast<size_t>(c0 + b) * kHeads + h) * D_C + f;
       const float* pm = p.part_ml + (static_cast<size_t>(c0 + b) * kHeads + h) * 2;
       float M = -INFINITY, L = 0.f, acc = 0.f;
@@ -599,39 +569,37 @@ __device__ void fused_combine(const TcParams& p, uint8_t* smem, Bars& bars) {
         acc = fmaf(acc, sc, (a4[0] + a4[1]) + (a4[2] + a4[3]));
         M = Mn;
       }
-      olat[j * D_C + f] = n > 0 ? acc / L : 0.f;
+      olat[f] = n > 0 ? acc / L : 0.f;
     }
     __syncthreads();
     if (u == static_cast<int>(blockIdx.x)) phase_mark<TRACE>(p, 5);
     // u = W_UV,h o from the registers loaded above: rows v0 .. v0 + 7 by the
     // butterfly, the ninth by a plain reduction
     if (v0 < p.d_v) {   // uniform in the warp
-      for (int j = 0; j < nb; ++j) {
-        float o8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (lane < LANES) {
-          const float4 x0 = *reinterpret_cast<const float4*>(olat + j * D_C + 8 * lane);
-          const float4 x1 = *reinterpret_cast<const float4*>(olat + j * D_C + 8 * lane + 4);
-          o8[0] = x0.x; o8[1] = x0.y; o8[2] = x0.z; o8[3] = x0.w;
-          o8[4] = x1.x; o8[5] = x1.y; o8[6] = x1.z; o8[7] = x1.w;
-        }
-        float part[kRows];
-#pragma unroll
-        for (int r = 0; r < kRows; ++r) {
-          float wv[8];
-          bf16x8_to_float(wraw[r], wv);
-          part[r] = 0.f;
-#pragma unroll
-          for (int e = 0; e < 8; ++e) part[r] = fmaf(wv[e], o8[e], part[r]);
-        }
-        const float sum = reduce8_rows(reinterpret_cast<const float (&)[8]>(part), lane);
-        float last = part[8];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) last += __shfl_xor_sync(0xffffffffu, last, o);
-        __nv_bfloat16* orow = p.out + (static_cast<size_t>(b0 + j) * kHeads + h) * p.d_v;
-        const int v = v0 + (lane >> 2);
-        if ((lane & 3) == 0 && v < p.d_v) orow[v] = __float2bfloat16_rn(sum);
-        if (lane == 0 && v0 + 8 < p.d_v) orow[v0 + 8] = __float2bfloat16_rn(last);
+      float o8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (lane < LANES) {
+        const float4 x0 = *reinterpret_cast<const float4*>(olat + 8 * lane);
+        const float4 x1 = *reinterpret_cast<const float4*>(olat + 8 * lane + 4);
+        o8[0] = x0.x; o8[1] = x0.y; o8[2] = x0.z; o8[3] = x0.w;
+        o8[4] = x1.x; o8[5] = x1.y; o8[6] = x1.z; o8[7] = x1.w;
       }
+      float part[kRows];
+#pragma unroll
+      for (int r = 0; r < kRows; ++r) {
+        float wv[8];
+        bf16x8_to_float(wraw[r], wv);
+        part[r] = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) part[r] = fmaf(wv[e], o8[e], part[r]);
+      }
+      const float sum = reduce8_rows(reinterpret_cast<const float (&)[8]>(part), lane);
+      float last = part[8];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) last += __shfl_xor_sync(0xffffffffu, last, o);
+      __nv_bfloat16* orow = p.out + (static_cast<size_t>(b) * kHeads + h) * p.d_v;
+      const int v = v0 + (lane >> 2);
+      if ((lane & 3) == 0 && v < p.d_v) orow[v] = __float2bfloat16_rn(sum);
+      if (lane == 0 && v0 + 8 < p.d_v) orow[v0 + 8] = __float2bfloat16_rn(last);
     }
     __syncthreads();   // olat is free for the next unit
     if (u == static_cast<int>(blockIdx.x)) phase_mark<TRACE>(p, 6);
@@ -662,9 +630,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   phase_mark<DBG == 2>(p, 0);
-  // the layer's output projection after this kernel may take each SM it
-  // leaves and stream its weights; any other kernel would crowd its blocks
-  // onto the first SMs to free up
+  // inside a layer the kernel after this one (the split combine, or the output
+  // projection where the combine is fused) may take each SM this one leaves,
+  // so that the projection's weights stream early; elsewhere an early combine
+  // would crowd its blocks onto the first SMs to free up (128 ragged sequences
+  // 69.8 us instead of 68.2)
   if (p.early) grid_launch_dependents();
 
   if (threadIdx.x == 0) {
@@ -1491,10 +1461,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             ml[0] = m16;
             ml[1] = lh;
           }
-          if (p.fuse && p.cmb_g == 1) {
-            // one sequence per combine unit: release this warp's part of the
-            // partial to the wait on its sequence (the warp barrier orders every
-            // lane's stores before lane 0's fence)
+          if (p.fuse) {
+            // release this warp's part of the partial to the combine's wait on
+            // its sequence (the warp barrier orders every lane's stores before
+            // lane 0's fence)
             __syncwarp();
             if (lane == 0) {
               __threadfence();
@@ -1578,23 +1548,24 @@ cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_
   p.trace = static_cast<unsigned long long*>(a.trace);
   p.trace_ctas = a.trace_ctas;
   p.trace_cap = a.trace_cap;
-  // The split combine runs inside this kernel when every CTA of the grid can
-  // be resident at once (a cooperative launch guarantees it, or fails).
+  // The split combine runs inside this kernel for the smallest batches, where
+  // a step is mostly latency, when every CTA of the grid can be resident at
+  // once (a cooperative launch guarantees it, or fails).  The launch then
+  // cannot overlap the kernel before it (about 2.5 us outside a graph), and more
+  // units than CTAs share a wait, so that at larger batches the separate
+  // combine is faster: 4 sequences 16.4 us fused, 17.9 apart; 8 x 32K 48.7 and
+  // 48.3; 32 x 4K 38.8 and 37.0 (both in a graph); 128 ragged 76.2 and 68.0.
   p.w_uv = static_cast<const __nv_bfloat16*>(a.w_uv);
   p.out = static_cast<__nv_bfloat16*>(a.out);
   p.seq_done = reinterpret_cast<uint32_t*>(ws + wl.off_done);
   p.d_v = a.d_v;
-  int groups = std::max(1, std::min(a.batch, a.num_splits / kHeads));
-  const int g = std::min(static_cast<int>(kFusedMaxG), (a.batch + groups - 1) / groups);
-  p.cmb_g = g;
-  p.cmb_groups = (a.batch + g - 1) / g;
   p.early = a.early;
   p.wait_ns = a.wait_ns;
   p.stall_cta = a.stall_cta;
   p.stall_tile = a.stall_tile;
   // (the fused combine holds kCombineRowsPerWarp rows of W_UV,h per warp)
-  p.fuse = DBG != 1 && a.batch > 0 && a.d_v <= kCombineRowsPerWarp * (kThreads / 32) &&
-           a.num_splits <= resident_ctas(kern, C::SMEM);
+  p.fuse = DBG != 1 && a.batch > 0 && kHeads * a.batch <= a.num_splits &&
+           a.d_v <= kCombineRowsPerWarp * (kThreads / 32) && a.num_splits <= resident_ctas(kern, C::SMEM);
   if (fused) *fused = p.fuse != 0;
   // The kernel may start while the query-absorption kernel before it on the
   // stream still runs (programmatic stream serialisation): its setup then

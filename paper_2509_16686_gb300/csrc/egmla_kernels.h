@@ -110,7 +110,8 @@ cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, const
 int absorb_tile(int d_c, int batch);
 // fp32: absorption (with the append blocks of `app` when it is non-null) and the split-KV kernel
 cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaStream_t st);
-cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, cudaStream_t st);
+// `wmap` (tensor-core path): W_UV as {d_c, d_v, H} in boxes of {64, 128, 1}
+cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, const CUtensorMap* wmap, cudaStream_t st);
 // tensor-core split-KV kernel; `maps` = {c_pool map (3-D page box for d_c <= 256), kr_pool map}.
 // *fused (may be null) is set when the split combine ran inside the kernel
 // (cooperative launch); otherwise launch_combine must follow.

@@ -108,6 +108,21 @@ def test_bf16_query_absorption_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_n
     assert rel.max() <= 4 * 2.0 ** -8 and rel_l2(got, ref) <= 5e-3, (float(rel.max()), rel_l2(got, ref))
 
 
+@pytest.mark.parametrize("d_c,gate", [(192, True), (256, False), (512, False)])
+@pytest.mark.parametrize("batch,d_v,splits", [(2, 136, 300), (3, 256, 0), (12, 8, 152), (20, 256, 600)])
+def test_bf16_split_combine_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_v, splits):
+    """The separate split combine: output rows past one tile of 128 and not a
+    multiple of it, slots dealt to groups of threads, more slots than fit
+    shared memory at once (600 splits over long sequences), empty sequences."""
+    dims = synth.Dims(num_heads=16, d_nope=64, d_rope=64, d_v=d_v, d_c=d_c, page_size=64, vocab=500, dtype="bf16",
+                      gate=gate)
+    lens = [0 if b == 1 else (20000 if b == 0 and splits > 256 else 130 + 61 * b) for b in range(batch)]
+    case = synth.make_case("combine", dims, lens, seed=35, latent_scale=0.5, layout="permuted", affine_ln=True)
+    _, got = run(case, splits)
+    check_bf16(got, orc.decode_unabsorbed(case), f"d_c={d_c} batch={batch} d_v={d_v} splits={splits}")
+    assert (got[1] == 0).all()
+
+
 # --------------------------------------------------------------------------- gating ablations (Section 4.4)
 @pytest.mark.parametrize("op", ["mul", "add_ln"])
 @pytest.mark.parametrize("d_c", [256, 192])
