@@ -80,46 +80,6 @@ EncodeFn get_encode() {
   return fn;
 }
 
-// 2D view [rows, cols] of a bf16 pool, boxes of 64 columns (128 bytes) x 64 rows,
-// 128-byte swizzle (the layout the MMA descriptors of the decode kernel expect)
-bool encode_pool_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols) {
-  EncodeFn enc = get_encode();
-  if (enc == nullptr) return false;
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {cols * 2};
-  const cuuint32_t box[2] = {64, 64};
-  const cuuint32_t estr[2] = {1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Latent pool as one 3-D box per page for the d_c <= 256 kernel: dims
-// {64 features, rows, d_c / 64 feature columns}, so that one copy writes the
-// page as its 128-byte-swizzled 64-feature columns one after another.
-bool encode_page_map_3d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols) {
-  EncodeFn enc = get_encode();
-  if (enc == nullptr) return false;
-  const cuuint64_t dims[3] = {64, rows, cols / 64};
-  const cuuint64_t strides[2] = {cols * 2, 128};
-  const cuuint32_t box[3] = {64, 64, static_cast<cuuint32_t>(cols / 64)};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// maps = {latent pool (3-D page box for d_c <= 256, 64x64 boxes otherwise), RoPE-key pool}
-bool encode_decode_maps(CUtensorMap (&maps)[2], const eg_mla_dims* d, const void* c_pool, const void* krope_pool,
-                        int32_t num_pages) {
-  std::memset(maps, 0, sizeof(maps));
-  const uint64_t rows = static_cast<uint64_t>(num_pages) * d->page_size;
-  const bool paged3d = d->d_c <= 256;
-  if (!(paged3d ? encode_page_map_3d(&maps[0], c_pool, rows, d->d_c) : encode_pool_map(&maps[0], c_pool, rows, d->d_c)))
-    return false;
-  return encode_pool_map(&maps[1], krope_pool, rows, d->d_rope);
-}
-
 // bf16 tensor {d0, d1, d2} with strides s1, s2 (elements) in boxes {64, b1, b2},
 // 128-byte swizzle, elements past an end read as zero
 bool encode_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1, uint64_t s2,
@@ -133,6 +93,19 @@ bool encode_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uin
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// maps = {latent pool, RoPE-key pool}: the latent as one 3-D box per tile, dims
+// {64 features, rows, d_c / 64 feature columns}, so that one copy writes the
+// tile as its 128-byte-swizzled 64-feature columns one after another; tiles of
+// 64 rows, 32 at d_c 512
+bool encode_decode_maps(CUtensorMap (&maps)[2], const eg_mla_dims* d, const void* c_pool, const void* krope_pool,
+                        int32_t num_pages) {
+  std::memset(maps, 0, sizeof(maps));
+  const uint64_t rows = static_cast<uint64_t>(num_pages) * d->page_size, dc = d->d_c, dr = d->d_rope;
+  const uint32_t tile = d->d_c <= 256 ? 64 : 32;
+  return encode_3d(&maps[0], c_pool, 64, rows, dc / 64, dc, 64, tile, static_cast<uint32_t>(dc / 64)) &&
+         encode_3d(&maps[1], krope_pool, dr, rows, 1, dr, rows * dr, tile, 1);
 }
 
 // maps of the tensor-core query absorption: {W_UK, q}

@@ -1,10 +1,10 @@
 // egmla_decode_tc.cu - split-KV EG-MLA decode on sm_103a tensor cores for the
-// latent widths 192 and 256 (gated or plain).
+// latent widths 192 and 256 (gated or plain) and 512 (plain).
 //
 // One CTA per split-KV work unit (see egmla_common.cuh for the schedule).  The
-// CTA streams its cache pages, one 64-token page per tile, through a ring of
-// shared-memory slots; the tiles are token rows of the tensor-core operations
-// (M = 64 tokens), the 16 heads their columns (N = 16).  Roles:
+// CTA streams its cache pages, one 64-token page per tile (half a page at width
+// 512), through a ring of shared-memory slots; the tiles are token rows of the
+// tensor-core operations (M = 64 tokens), the 16 heads their columns (N = 16).  Roles:
 //
 //   TMA (warp 4)      latent page [64 tok x d_c] (one 3-D box: 64-feature
 //                     columns x 64 rows) and RoPE-key page [64 x 64], both
@@ -26,14 +26,12 @@
 //   scores (warp 5)   S = Z (q^ gamma)^T and S_rope = K^R q^R^T (M = 64 tokens,
 //                     N = 16 heads, K = d_c and 64; fp32 in TMEM, four score
 //                     buffers) as soon as a gated page and a score buffer are
-//                     ready, and the query block of the next sequence segment;
-//                     with no query block to load the warp sleeps in hardware
-//                     on the gate's barrier.
+//                     ready, and the query block of the next sequence segment.
 //   output (warp 6)   O^T += Z^T P' (M = 128 latent features, N = 16 heads,
 //                     K = 64 tokens; O^T stays in TMEM over a sequence
 //                     segment).  An issuing thread stalls while the tensor
 //                     pipe's queue is full, so the two MMA streams have a
-//                     thread each.
+//                     thread each (which also does its own waits).
 //   softmax (warps 0-3, one per TMEM lane quadrant: tokens 16w .. 16w + 15)
 //                     thread t reads two tokens x four heads of S; the
 //                     LayerNorm is applied after the MMA, since
@@ -106,9 +104,15 @@ constexpr int kNP = 4;
 template <int D_C, bool GATE>
 struct Cfg {
   static constexpr int NCH = D_C / 64;                  // 64-feature swizzle-atom columns
-  static constexpr uint32_t PCHUNK = kPage * 128;       // one atom column of a page: 8 KB
+  // tokens per tile: a page, or half a page for the widest latent, whose pages
+  // are too large for a ring of three in shared memory: two slots of 72 KB took
+  // about 150 us for 128 ragged sequences, five of 36 KB about 105 (557 MB: 3.7
+  // and 5.3 TB/s; kernel alone, warm)
+  static constexpr int TOK = D_C > 256 ? kPage / 2 : kPage;
+  static constexpr int TPP = kPage / TOK;               // tiles per page
+  static constexpr uint32_t PCHUNK = TOK * 128;         // one atom column of a tile
   static constexpr uint32_t KR_OFF = NCH * PCHUNK;
-  static constexpr uint32_t SLOT = KR_OFF + PCHUNK;     // latent + RoPE key of one page
+  static constexpr uint32_t SLOT = KR_OFF + PCHUNK;     // latent + RoPE key of one tile
   static constexpr uint32_t STAT_BYTES = GATE ? 2 * kPage * 4 : 0;   // per slot: mu[64], r[64]
   static constexpr uint32_t QB_LAT = qprep_lat_bytes(D_C);
   static constexpr uint32_t QPREP = qprep_bytes_tc(D_C, kRope);
@@ -137,6 +141,7 @@ struct Cfg {
   static constexpr uint32_t SMEM = OFF_MISC + MISC + 1024;
   // TMEM columns: kNB score buffers of (latent 16 + RoPE 16) head columns,
   // then the latent output O^T (16 head columns per 128-feature M chunk)
+  static constexpr int NMC = (D_C + 127) / 128;
   static constexpr uint32_t S_COLS = 32;
   static constexpr uint32_t COL_S = 0, COL_O = kNB * S_COLS;
   static constexpr uint32_t TMEM_COLS = 256;
@@ -144,12 +149,16 @@ struct Cfg {
   static constexpr uint32_t ID_TX = GATE ? kPage * 4 : 0;   // the page's token ids
   static_assert(NS >= 3, "the ring needs three page slots");
   static_assert(SMEM <= kSmemLimit, "shared memory");
-  static_assert(D_C == 192 || D_C == 256, "latent widths of this kernel");
-  static_assert(COL_O + 32 <= TMEM_COLS, "tensor memory");
-  // first latent feature of output M chunk j (two chunks of 128 rows); for
+  static_assert(D_C == 192 || D_C == 256 || (D_C == 512 && !GATE), "latent widths of this kernel");
+  static_assert(COL_O + kHeads * NMC <= TMEM_COLS && NMC % 2 == 0, "tensor memory");
+  // the score MMAs read 64 rows of every atom column: at half pages the last
+  // 32 are the next column's (or what follows the slot), and their scores are
+  // not used
+  static_assert(OFF_QBUF + 64 * 128 <= SMEM, "score operand");
+  // first latent feature of output M chunk j (chunks of 128 rows); for
   // D_C = 192 the second chunk starts at 64 and overlaps the first, so that no
   // MMA reads past the latent part of a slot (its rows 64..127 are not read out)
-  __host__ __device__ static constexpr int mc_start(int j) { return j == 0 ? 0 : D_C - 128; }
+  __host__ __device__ static constexpr int mc_start(int j) { return j == NMC - 1 ? D_C - 128 : 128 * j; }
 };
 
 struct TcParams {
@@ -242,12 +251,15 @@ struct Tile {
   bool first, last;
 };
 
-// Walks this CTA's pages one at a time, segment by segment (identically in
-// every role, so no per-tile metadata needs to be exchanged).
+// Walks this CTA's tiles (TOK tokens: a page or half of one) one at a time,
+// segment by segment (identically in every role, so no per-tile metadata needs
+// to be exchanged).
+template <int TOK>
 struct Walker {
   const int32_t* cu;
   const int32_t* lens;
   int batch, g1, b, lp, lp_end, L;
+  int part = 0;   // tile of the page
   bool first, done;
 
   // the split's start record (written by the prologue kernel): one round of loads
@@ -277,10 +289,17 @@ struct Walker {
     if (done) return false;
     t.b = b;
     t.lp = lp;
-    t.tok0 = lp * kPage;
-    t.ntok = min(kPage, L - t.tok0);
+    t.tok0 = lp * kPage + part * TOK;
+    t.ntok = min(TOK, L - t.tok0);
     t.first = first;
     first = false;
+    if constexpr (TOK < kPage) {
+      if (++part < kPage / TOK && t.tok0 + TOK < L) {
+        t.last = false;
+        return true;
+      }
+      part = 0;
+    }
     lp += 1;
     t.last = lp >= lp_end;
     if (t.last) {
@@ -687,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // copies.  A slot is free once the output MMA of the tile that held it is
     // complete.
     const uint64_t pol_stream = policy_evict_first();
-    Walker w;
+    Walker<C::TOK> w;
     w.start(p);
     PageWindow pw;
     pw.init(p, lane);
@@ -716,9 +735,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_arrive_expect_tx(fb, ok ? C::PAGE_TX + C::ID_TX : 0u);
             if (ok) {
               const uint32_t dst = sbase + slot * C::SLOT;
-              const int y = pg * kPage;
+              const int y = pg * kPage + t.tok0 % kPage;
               tma_load_3d(dst, &cmap, 0, y, 0, fb, pol_stream);
-              tma_load_2d(dst + C::KR_OFF, &krmap, 0, y, fb, pol_stream);
+              tma_load_3d(dst + C::KR_OFF, &krmap, 0, y, 0, fb, pol_stream);
               // the page's token ids, into the half of the slot's statistics that
               // holds r once the gate has read them
               if (C::ID_TX)
@@ -749,121 +768,93 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------------- score MMAs, query blocks
-    // Converged warp; one elected lane issues.  The warp polls two queues and
-    // serves whichever is ready, so that neither waits for the other's
-    // condition:
-    //   query block of segment qn: its buffer's previous segment is done
-    //     (last score MMA complete, sums read by the softmax warps);
-    //   scores of tile js: its gated page (zready), a free score buffer (the
-    //     softmax warps read tile js - kNB's), and at a segment start the
-    //     segment's query block.
+    // One thread waits and issues.  Scores of tile js: at a segment start the
+    // segment's query block, a free score buffer (the softmax warps read tile
+    // js - kNB's), and the gated page.  The next segment's query block is
+    // requested once its buffer's previous segment is done with it (last score
+    // MMA complete, sums read by the softmax warps), tested after every tile.
+    // A warp that polled both queues, voted and elected for every tile took
+    // 135 us of the d_c 512 step where this takes 124 (its 36 MMAs per 32 tokens
+    // are short, so what lies between tiles counts), 48.4 instead of 47.9 of the
+    // 8 x 32K step, and 68.3 instead of 69.3 of 128 ragged sequences at d_c 192.
     // Loops are unrolled with compile-time accumulate flags.
-    if (!DUMP) {
+    if (!DUMP && elect_one()) {
       constexpr uint32_t IDESC_S = idesc_bf16(64, kHeads, 0, 0);
       // A operand: the page slot, 128-byte swizzled, K-major (tokens x
       // features); B: the query block in 8x8 core matrices, K cores 256 B
       // apart, head halves 128 B apart
       const uint64_t zdesc_k = smem_desc(sbase, 16, 1024, kSwizzle128B);
       const uint64_t qdesc0 = smem_desc(sbase + C::OFF_QBUF, kQGroupBytes, kQRowGroupBytes, kSwizzleNone);
-      Walker ws, wq;
+      Walker<C::TOK> ws, wq;
       ws.start(p);
       wq.start(p);
       Tile ts, tq;
-      bool s_more = ws.next(ts), q_more = wq.next(tq);
-      int js = 0, qn = 0, seg_s = -1;
-      int last_q[2] = {-1, -1};
+      bool q_more = wq.next(tq), q_walk = false;   // q_walk: tq's block is requested, the next segment not found yet
+      int qn = 0, seg = -1;   // query blocks requested, segment of the scores
       bool issued = false;
       Tracer tr;
       tr.init(p, 1, 0, 2);
-      if (lane != 0) tr.base = nullptr;
-      uint64_t idle_since = 0;
-      while (s_more) {
-        bool progress = false;
-        // ---- query block of the next segment
-        if (q_more && warp_test(smem_u32(&bars.qempty[qn % C::NQ]), ((qn / C::NQ) & 1) ^ 1)) {
-          const int qb = qn % C::NQ;
-          if (lane == 0) {
-            mbar_arrive_expect_tx(smem_u32(&bars.qfull[qb]), C::QPREP);
-            bulk_load(sbase + C::OFF_QBUF + qb * C::QBUF, p.qprep + static_cast<size_t>(tq.b) * C::QPREP, C::QPREP,
-                      smem_u32(&bars.qfull[qb]));
-          }
-          __syncwarp();
-          last_q[qb] = qn;
-          ++qn;
-          do {
-            q_more = wq.next(tq);
-          } while (q_more && !tq.first);
-          progress = true;
+      auto find_query = [&]() {
+        while (q_walk) {
+          q_more = wq.next(tq);
+          q_walk = q_more && !tq.first;
         }
-        // ---- scores of tile js
+      };
+      // the next segment's query block (its buffer is free)
+      auto load_query = [&]() {
+        const int qb = qn % C::NQ;
+        mbar_arrive_expect_tx(smem_u32(&bars.qfull[qb]), C::QPREP);
+        bulk_load(sbase + C::OFF_QBUF + qb * C::QBUF, p.qprep + static_cast<size_t>(tq.b) * C::QPREP, C::QPREP,
+                  smem_u32(&bars.qfull[qb]));
+        ++qn;
+        q_walk = true;
+      };
+      for (int js = 0; ws.next(ts); ++js) {
         const int slot = js % C::NS, sb = js % kNB;
-        const uint32_t zpar = (js / C::NS) & 1;
-        const int sg = seg_s + (ts.first ? 1 : 0);
-        bool ready = !ts.first || (qn > sg && warp_test(smem_u32(&bars.qfull[sg % C::NQ]), (sg / C::NQ) & 1));
-        ready = ready && warp_test(smem_u32(&bars.sfree[sb]), ((js / kNB) & 1) ^ 1);
-        if (ready && !(q_more && warp_test(smem_u32(&bars.qempty[qn % C::NQ]), ((qn / C::NQ) & 1) ^ 1))) {
-          // nothing else to serve: sleep in hardware until the gate warps
-          // release the slot (the gate waits on nothing this warp does)
-          ready = warp_wait(smem_u32(&bars.zready[slot]), zpar, abort_flag, wait_ns);
-          if (!ready) break;   // uniform: the wait ran out or another role aborted
-        } else {
-          ready = ready && warp_test(smem_u32(&bars.zready[slot]), zpar);
-        }
-        if (ready) {
-          seg_s = sg;
-          tr.mark(1, js);
-          if (lane == 0) mbar_arrive(smem_u32(&bars.sready[sb]));
-          tc_fence_after();
-          if (elect_one()) {
-            const uint64_t za = zdesc_k + ((slot * C::SLOT) >> 4);
-            const uint64_t qb = qdesc0 + (((seg_s % C::NQ) * C::QBUF) >> 4);
-            const uint32_t ds = tmem + C::COL_S + sb * C::S_COLS;
-#pragma unroll
-            for (int kk = 0; kk < D_C / 16; ++kk)
-              mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
-                          qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
-#pragma unroll
-            for (int kk = 0; kk < kRope / 16; ++kk)
-              mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
-                          qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
-            mma_commit(smem_u32(&bars.sready[sb]));
-            if (ts.last) mma_commit(smem_u32(&bars.qempty[seg_s % C::NQ]));
+        bool ok = true;
+        if (ts.first) {
+          ++seg;
+          if (qn <= seg) {
+            find_query();
+            ok = mbar_wait(smem_u32(&bars.qempty[seg % C::NQ]), ((seg / C::NQ) & 1) ^ 1, abort_flag, wait_ns);
+            if (ok) load_query();
           }
-          __syncwarp();
-          tr.mark(2, js);
-          issued = true;
-          ++js;
-          s_more = ws.next(ts);
-          progress = true;
         }
-        if (progress) {
-          idle_since = 0;
-        } else {
-          // nothing ready: bounded wait for the others (and their abort)
-          const uint64_t now = globaltimer();
-          if (idle_since == 0) idle_since = now;
-          bool stop = *abort_flag != 0;
-          if (!stop && now - idle_since > wait_ns) {
-            *abort_flag = 1;
-            stop = true;
-          }
-          if (__any_sync(0xffffffffu, stop)) break;
-          __nanosleep(32);   // leave the issue slots to the warps that do the work
-        }
+        if (ts.first)
+          ok = ok && mbar_wait(smem_u32(&bars.qfull[seg % C::NQ]), (seg / C::NQ) & 1, abort_flag, wait_ns);
+        ok = ok && mbar_wait(smem_u32(&bars.sfree[sb]), ((js / kNB) & 1) ^ 1, abort_flag, wait_ns);
+        ok = ok && mbar_wait(smem_u32(&bars.zready[slot]), (js / C::NS) & 1, abort_flag, wait_ns);
+        if (!ok) break;
+        tr.mark(1, js);
+        mbar_arrive(smem_u32(&bars.sready[sb]));
+        tc_fence_after();
+        const uint64_t za = zdesc_k + ((slot * C::SLOT) >> 4);
+        const uint64_t qb = qdesc0 + (((seg % C::NQ) * C::QBUF) >> 4);
+        const uint32_t ds = tmem + C::COL_S + sb * C::S_COLS;
+#pragma unroll
+        for (int kk = 0; kk < D_C / 16; ++kk)
+          mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
+                      qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+#pragma unroll
+        for (int kk = 0; kk < kRope / 16; ++kk)
+          mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
+                      qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+        mma_commit(smem_u32(&bars.sready[sb]));
+        if (ts.last) mma_commit(smem_u32(&bars.qempty[seg % C::NQ]));
+        tr.mark(2, js);
+        issued = true;
+        // (after the tile's MMAs: finding the next segment takes global loads)
+        find_query();
+        if (q_more && mbar_test_now(smem_u32(&bars.qempty[qn % C::NQ]), ((qn / C::NQ) & 1) ^ 1)) load_query();
       }
-      if (lane == 0) {
-        // drain: the query-block copies this warp issued must land, and every
-        // MMA must finish, before the CTA exits and TMEM is released (own flag:
-        // bounded but not cut short by an abort)
-        volatile int own = 0;
-        for (int b = 0; b < 2; ++b)
-          if (last_q[b] >= 0 && !mbar_wait(smem_u32(&bars.qfull[b]), (last_q[b] / C::NQ) & 1, &own, wait_ns)) *abort_flag = 1;
-      }
-      __syncwarp();
+      // drain: the query-block copies land and every MMA finishes before the
+      // CTA exits and TMEM is released (own flag: bounded but not cut short by
+      // an abort)
+      volatile int own = 0;
+      for (int n = qn > C::NQ ? qn - C::NQ : 0; n < qn; ++n)
+        if (!mbar_wait(smem_u32(&bars.qfull[n % C::NQ]), (n / C::NQ) & 1, &own, wait_ns)) *abort_flag = 1;
       if (issued) {
-        if (elect_one()) mma_commit(smem_u32(&bars.drain_s));
-        __syncwarp();
-        volatile int own = 0;
+        mma_commit(smem_u32(&bars.drain_s));
         if (!mbar_wait(smem_u32(&bars.drain_s), 0, &own, wait_ns)) *abort_flag = 1;
       }
     }
@@ -876,52 +867,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     // 64-feature atoms PCHUNK apart; tokens along K, 8-row groups 1 KB apart);
     // B: P' MN-major in 8x8 core matrices (token groups 256 B, head halves
     // 128 B).
-    if (!DUMP) {
+    if (!DUMP && elect_one()) {
       constexpr uint32_t IDESC_O = idesc_bf16(128, kHeads, 1, 1);
       const uint64_t zdesc_mn = smem_desc(sbase, C::PCHUNK, 1024, kSwizzle128B);
       const uint64_t pdesc0 = smem_desc(sbase + C::OFF_PBUF, 256, 128, kSwizzleNone);
-      Walker wo;
+      Walker<C::TOK> wo;
       wo.start(p);
       Tile to;
-      int jo = 0;
       bool issued = false;
       Tracer tr;
       tr.init(p, 1, 1, 2);   // second half of the MMA role's run
-      if (lane != 0) tr.base = nullptr;
-      while (wo.next(to)) {
-        if (!warp_wait(smem_u32(&bars.spdone[jo % kNP]), (jo / kNP) & 1, abort_flag, wait_ns)) break;
+      for (int jo = 0; wo.next(to); ++jo) {
+        if (!mbar_wait(smem_u32(&bars.spdone[jo % kNP]), (jo / kNP) & 1, abort_flag, wait_ns)) break;
         tr.mark(3, jo);
         tc_fence_after();
-        if (elect_one()) {
-          const int slot = jo % C::NS;
-          const uint64_t za = zdesc_mn + ((slot * C::SLOT) >> 4);
-          const uint64_t pb = pdesc0 + (((jo % kNP) * C::PBUF) >> 4);
-          if (to.first) {
+        const int slot = jo % C::NS;
+        const uint64_t za = zdesc_mn + ((slot * C::SLOT) >> 4);
+        const uint64_t pb = pdesc0 + (((jo % kNP) * C::PBUF) >> 4);
+        const uint32_t keep = to.first ? 0u : 1u;   // a segment's first MMAs overwrite O^T
 #pragma unroll
-            for (int ks = 0; ks < kPage / 16; ++ks)
+        for (int ks = 0; ks < C::TOK / 16; ++ks)
 #pragma unroll
-              for (int mc = 0; mc < 2; ++mc)
-                mma_bf16_ss(tmem + C::COL_O + kHeads * mc, za + (((C::mc_start(mc) / 64) * C::PCHUNK + ks * 2048) >> 4),
-                            pb + ((ks * 512) >> 4), IDESC_O, ks > 0);
-          } else {
-#pragma unroll
-            for (int ks = 0; ks < kPage / 16; ++ks)
-#pragma unroll
-              for (int mc = 0; mc < 2; ++mc)
-                mma_bf16_ss(tmem + C::COL_O + kHeads * mc, za + (((C::mc_start(mc) / 64) * C::PCHUNK + ks * 2048) >> 4),
-                            pb + ((ks * 512) >> 4), IDESC_O, 1);
-          }
-          mma_commit(smem_u32(&bars.empty[slot]));
-          mma_commit(smem_u32(&bars.pfree[jo % kNP]));
-        }
-        __syncwarp();
+          for (int mc = 0; mc < C::NMC; ++mc)
+            mma_bf16_ss(tmem + C::COL_O + kHeads * mc, za + (((C::mc_start(mc) / 64) * C::PCHUNK + ks * 2048) >> 4),
+                        pb + ((ks * 512) >> 4), IDESC_O, ks > 0 ? 1u : keep);
+        mma_commit(smem_u32(&bars.empty[slot]));
+        mma_commit(smem_u32(&bars.pfree[jo % kNP]));
         tr.mark(4, jo);
         issued = true;
-        ++jo;
       }
       if (issued) {
-        if (elect_one()) mma_commit(smem_u32(&bars.drain_o));
-        __syncwarp();
+        mma_commit(smem_u32(&bars.drain_o));
         volatile int own = 0;
         if (!mbar_wait(smem_u32(&bars.drain_o), 0, &own, wait_ns)) *abort_flag = 1;
       }
@@ -947,7 +923,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int row = gw * (32 / kGateLanesPerRow) + lane / kGateLanesPerRow;
     const uint64_t pol_keep = policy_evict_last();
     constexpr bool gate_ln = GATE_LN;
-    Walker w;
+    Walker<C::TOK> w;
     w.start(p);
     // id of this thread's row of tile jj, from the slot that holds its page (0
     // past the end of the page)
@@ -1043,7 +1019,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int fc = 0; fc < C::NCH; ++fc) load_next_column(fc);
         warp_arrive(smem_u32(&bars.empty[slot]));
       } else {
-        const bool full_page = t.ntok == kPage;   // uniform: no token masking needed
+        const bool full_page = t.ntok == C::TOK;   // uniform: no token masking needed
         if (GATE) {
           float* st = reinterpret_cast<float*>(smem + C::OFF_STAT + slot * C::STAT_BYTES);
           // all shared-memory reads of this thread's units first (the in-place
@@ -1162,7 +1138,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
         } else if (!full_page) {
-          if (row >= t.ntok) {
+          if (row >= t.ntok && row < C::TOK) {
 #pragma unroll
             for (int fc = 0; fc < C::NCH; ++fc)
 #pragma unroll
@@ -1226,7 +1202,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       wq[k] = 0.f;
       bsc[k] = 0.f;
     }
-    Walker w;
+    Walker<C::TOK> w;
     w.start(p);
     Tile t;
     int it = 0, seg = -1;
@@ -1343,12 +1319,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = warp_wait(smem_u32(&bars.pfree[pv]), ((it - 1) / kNP) & 1, abort_flag, wait_ns);
           if (ok) {
             tc_fence_after();
-            float o[32];
-            tmem_ld32(tq + C::COL_O, o);
-            tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) o[c] *= __shfl_sync(0xffffffffu, alpha, c & 15);
-            tmem_st32(tq + C::COL_O, o);
+            for (int m2 = 0; m2 < C::NMC / 2; ++m2) {   // two M chunks at a time
+              float o[32];
+              tmem_ld32(tq + C::COL_O + 32 * m2, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 32; ++c) o[c] *= __shfl_sync(0xffffffffu, alpha, c & 15);
+              tmem_st32(tq + C::COL_O + 32 * m2, o);
+            }
             tmem_wait_st();
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -1430,28 +1409,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         ok = warp_wait(smem_u32(&bars.pfree[pb]), (it / kNP) & 1, abort_flag, wait_ns);
         if (ok) {
           tc_fence_after();
-          float o[32];
-          tmem_ld32(tq + C::COL_O, o);
-          tmem_wait_ld();
           const int slot_out = blockIdx.x + t.b;
           float* po = p.part_o + static_cast<size_t>(slot_out) * kHeads * D_C;
 #pragma unroll
-          for (int mc = 0; mc < 2; ++mc) {
-            const int f = C::mc_start(mc) + 32 * warp + lane;
-            if (mc == 0 || C::mc_start(1) + 32 * warp >= 128) {   // uniform in the warp
-              float gm = 1.f, bt = 0.f;
-              if (GATE) {
-                gm = gb[f];
-                bt = gb[D_C + f];
-              }
+          for (int m2 = 0; m2 < C::NMC / 2; ++m2) {   // two M chunks at a time
+            float o[32];
+            tmem_ld32(tq + C::COL_O + 32 * m2, o);
+            tmem_wait_ld();
 #pragma unroll
-              for (int h = 0; h < kHeads; ++h) {
-                float v = o[mc * kHeads + h];
+            for (int mc = 2 * m2; mc < 2 * m2 + 2; ++mc) {
+              const int f = C::mc_start(mc) + 32 * warp + lane;
+              if (C::mc_start(mc) + 32 * warp >= 128 * mc) {   // uniform in the warp
+                float gm = 1.f, bt = 0.f;
                 if (GATE) {
-                  const float lhh = __shfl_sync(0xffffffffu, lh, h), bhh = __shfl_sync(0xffffffffu, bh, h);
-                  v = fmaf(gm, v - bhh, bt * lhh);
+                  gm = gb[f];
+                  bt = gb[D_C + f];
                 }
-                po[h * D_C + f] = v;
+#pragma unroll
+                for (int h = 0; h < kHeads; ++h) {
+                  float v = o[(mc & 1) * kHeads + h];
+                  if (GATE) {
+                    const float lhh = __shfl_sync(0xffffffffu, lh, h), bhh = __shfl_sync(0xffffffffu, bh, h);
+                    v = fmaf(gm, v - bhh, bt * lhh);
+                  }
+                  po[h * D_C + f] = v;
+                }
               }
             }
           }
@@ -1491,7 +1473,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   phase_mark<DBG == 2>(p, 2);
   if (warp == kMmaWarp) tmem_dealloc(tmem, C::TMEM_COLS);
   if (threadIdx.x == 0 && bars.abort) report_status(p.status, kStatusTimeout);
-  if (!DUMP && p.fuse) fused_combine<D_C, DBG == 2>(p, smem, bars);
+  if constexpr (!DUMP && D_C <= 256) {
+    if (p.fuse) fused_combine<D_C, DBG == 2>(p, smem, bars);
+  }
   phase_mark<DBG == 2>(p, 3);
 }
 
@@ -1564,7 +1548,7 @@ cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_
   p.stall_cta = a.stall_cta;
   p.stall_tile = a.stall_tile;
   // (the fused combine holds kCombineRowsPerWarp rows of W_UV,h per warp)
-  p.fuse = DBG != 1 && a.batch > 0 && kHeads * a.batch <= a.num_splits &&
+  p.fuse = DBG != 1 && D_C <= 256 && a.batch > 0 && kHeads * a.batch <= a.num_splits &&
            a.d_v <= kCombineRowsPerWarp * (kThreads / 32) && a.num_splits <= resident_ctas(kern, C::SMEM);
   if (fused) *fused = p.fuse != 0;
   // The kernel may start while the query-absorption kernel before it on the
@@ -1622,7 +1606,7 @@ cudaError_t launch_decode_tc(const DecodeArgs& a, const CUtensorMap* maps, bool 
     return cudaErrorInvalidValue;
   }
   if (!a.gate) {
-    if (a.d_c == 512) return launch_decode_wide(a, maps, st);
+    if (a.d_c == 512) return launch_one<512, 0, 0>(a, maps, st, fused);
     return launch_mode<0>(a, maps, st, fused);
   }
   if (a.gate_add) return launch_mode<3>(a, maps, st, fused);

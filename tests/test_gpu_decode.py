@@ -123,6 +123,18 @@ def test_bf16_split_combine_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_v, s
     assert (got[1] == 0).all()
 
 
+@pytest.mark.parametrize("splits", [1, 3, 0])
+def test_bf16_half_page_tiles_match_oracle(gpu_lib, splits):
+    """d_c 512 walks its pages in halves of 32 tokens: sequences that end in a
+    first half, at a half, in a second half and at a page, over one to all
+    splits."""
+    dims = synth.dims_bf16(d_c=512, vocab=300, gate=False)
+    case = synth.make_case("halves", dims, [1, 31, 32, 33, 0, 63, 64, 65, 96, 97, 128, 160, 200, 700], seed=36,
+                           latent_scale=0.5, layout="permuted", extra_pages=3)
+    _, got = run(case, splits)
+    check_bf16(got, orc.decode_unabsorbed(case), f"splits={splits}", scaled_abs=True)
+
+
 # --------------------------------------------------------------------------- gating ablations (Section 4.4)
 @pytest.mark.parametrize("op", ["mul", "add_ln"])
 @pytest.mark.parametrize("d_c", [256, 192])
