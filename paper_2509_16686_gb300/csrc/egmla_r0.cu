@@ -10,24 +10,29 @@
 //   q . k~ = r (q gamma) . z_k - r mu sum(q gamma) + q . beta,
 // so the up-projection computes every head's raw dot (q gamma) . z_k while
 // it has z_k in registers and keeps only the gated values.  Two kernels:
-//   r0_project_kernel  (tcgen05) one tile of two cache pages (128 tokens,
-//                      the MMA's M) of the walk over every sequence's pages:
-//                      for each head h, D = C W^UKV_h^T (N = 256 = d_n + d_v
-//                      features, K = d_c) in one of two TMEM accumulators, so
-//                      that the epilogue of head h overlaps the MMAs of head
-//                      h + 1.  Epilogue warps, one row each (their R0 gate
-//                      values G_R0[id] of head h + 1 requested a quarter at a
-//                      time while head h is processed): the key half gates
-//                      its 128 features, rounds z to bf16 and adds
-//                      (q gamma) . z to the row's head dots; the value half
-//                      gates and rounds its 128 features and stores them
-//                      head-major through a per-warp shared-memory tile (two
-//                      256-byte rows, 512 contiguous bytes, per store
-//                      instruction).  Both
-//                      add z and z^2 of the rounded values into the row's
-//                      statistics.  After the last head: (mu, 1/sqrt(var +
-//                      eps)) and every head's logit
+//   r0_project_kernel  (tcgen05, CTA pairs) one tile of two cache pages (128
+//                      tokens) per CTA of the walk over every sequence's
+//                      pages; the two CTAs of a cluster share the MMAs (M = 256
+//                      rows, both tiles): for each head h, D = C W^UKV_h^T (N =
+//                      256 = d_n + d_v features, K = d_c) with each CTA holding
+//                      half of W^UKV_h's rows, in one of two TMEM accumulators,
+//                      so that the epilogue of head h overlaps the MMAs of head
+//                      h + 1.  Epilogue: four groups of four warps, one row per
+//                      lane (its R0 gate values G_R0[id] of head h + 1 requested
+//                      a quarter at a time while head h is processed): the key
+//                      groups gate their 64 features each, round z to bf16 and
+//                      add (q gamma) . z to the row's head dots; the value
+//                      groups gate and round their 64 features and store them
+//                      head-major through a per-warp shared-memory tile (128
+//                      contiguous bytes per row).  All add z and z^2 of the
+//                      rounded values into the row's statistics.  After the last
+//                      head: (mu, 1/sqrt(var + eps)) and every head's logit
 //                        s = scale log2(e) (r ((q gamma) . z_k - mu sum(q gamma)) + q . beta + q^R . k^R).
+//                      Bound by the epilogue's latency (a warp's chain per head:
+//                      accumulator, gate values, conversions, statistics): eight
+//                      warps took 133 us for 8 x 4096 tokens whether each CTA
+//                      copied all of W^UKV or half of it, sixteen with packed
+//                      fp32 pairs about 110 (256 tiles are two waves on 152 SMs).
 //   r0_attend_kernel   one block per (sequence, head): an online softmax over
 //                      the logits and, with P' = p r,
 //                        o = gamma_v ((sum P' z_v - sum P' mu) / sum p) + beta_v,
@@ -60,24 +65,32 @@ constexpr int kR0Rows = 2 * kPage;              // tile rows: two pages (the MMA
 constexpr int kR0Chunk = 64;                    // K elements per operand chunk (128-byte swizzle atom)
 constexpr uint32_t kR0AChunkBytes = kR0Rows * kR0Chunk * 2;   // 16 KB
 constexpr uint32_t kR0APageBytes = kPage * kR0Chunk * 2;      // 8 KB: one page's rows of a chunk
-constexpr uint32_t kR0BChunkBytes = kR0Feat * kR0Chunk * 2;   // 32 KB
-constexpr int kR0BStages = 3;
-constexpr int kR0EpiWarps = 8;                  // warps 2-5 key half, 6-9 value half (one TMEM lane quadrant each)
-constexpr int kR0Threads = 32 * (2 + kR0EpiWarps);   // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+// the CTAs of a pair hold half of a head's 256 rows of W^UKV each (rank 0 its key
+// rows, rank 1 its value rows)
+constexpr uint32_t kR0BChunkBytes = kR0Half * kR0Chunk * 2;   // 16 KB
+constexpr int kR0BStages = 5;
+// epilogue: four groups of four warps (one TMEM lane quadrant each): the first
+// and last 64 key features, the first and last 64 value features of a head
+constexpr int kR0Groups = 4;
+constexpr int kR0GroupFeat = kR0Feat / kR0Groups;   // 64
+constexpr int kR0EpiWarps = 4 * kR0Groups;
+constexpr int kR0Threads = 32 * (2 + kR0EpiWarps);   // warp 0 TMA, warp 1 MMA, warps 2-17 epilogue
 constexpr uint32_t kR0TmemCols = 512;           // two 256-column accumulators
 constexpr int kR0S1Stride = kR0Heads + 1;       // row stride of the head dots (no bank conflicts)
 constexpr int kR0EpiBar = 1;                    // named barrier of the epilogue warps
 constexpr uint32_t kR0RowBytes = kR0Half * 2;   // one row's gated values of a head: 256 bytes
+constexpr uint32_t kR0GroupBytes = kR0GroupFeat * 2;   // .. and a value group's part of it
 
 // shared memory after the latent tile and the W^UKV stages
 struct R0Smem {
   float qg[2][kR0Heads][kR0Half];       // q_h (*) gamma_k,h of the tile's two sequences
   __nv_bfloat16 qr[2][kR0Heads][kR0Rope];   // q^R_h
   float2 wb[2][kR0Heads];               // (sum_f q gamma, q . beta)
-  float s1[kR0Rows][kR0S1Stride];       // (q gamma) . z_k per row and head
-  float2 half_sums[kR0Rows];            // the value half's (sum z, sum z^2) per row
-  uint8_t vstage[4][32 * kR0RowBytes];  // per value-half warp: its 32 rows, 16-byte chunks swizzled by row
+  float s1[2][kR0Rows][kR0S1Stride];    // (q gamma) . z_k per row and head, of each key group
+  float2 sums[kR0Groups][kR0Rows];      // each group's (sum z, sum z^2) per row
+  uint8_t vstage[8][32 * kR0GroupBytes];   // per value warp: its 32 rows, 16-byte chunks swizzled by row
   int tile_b[2], tile_lp[2], tile_page[2], tile_n[2];
+  int pair_live;
   uint64_t afull;
   uint64_t bfull[kR0BStages], bempty[kR0BStages];
   uint64_t dfull[2], dfree[2];
@@ -121,10 +134,16 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 
 __device__ __forceinline__ float bf(const __nv_bfloat16 x) { return __bfloat162float(x); }
 
+__device__ __forceinline__ float2 widen2(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
 // Pages 2t and 2t + 1 (t = blockIdx.x) of the walk over the sequences' pages
 // (sequence by sequence, each in logical order), found by warp 0: a prefix
 // sum of the page counts over the lanes, 32 sequences at a time.  A half with
-// no page (past the last) has n = 0 and repeats the other half's page.
+// no page (past the last) has n = 0 and repeats the other half's page (page 0
+// where neither has one: the other CTA of the pair may still have a tile).
+// pair_live: the walk reaches the pair's first page.
 __device__ void find_tile(const R0ProjParams& p, R0Smem& sm, int lane) {
   const int g0 = 2 * static_cast<int>(blockIdx.x);
   int fb[2] = {-1, -1}, flp[2] = {0, 0}, fl[2] = {0, 0};
@@ -157,6 +176,8 @@ __device__ void find_tile(const R0ProjParams& p, R0Smem& sm, int lane) {
     base += __shfl_sync(0xffffffffu, inc, 31);
   }
   if (lane == 0) {
+    // (base: the pages counted; the loop ends early only past this tile's pages)
+    sm.pair_live = base > 4 * static_cast<int>(blockIdx.x / 2) ? 1 : 0;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       int page = -1, n = 0;
@@ -179,10 +200,15 @@ __device__ void find_tile(const R0ProjParams& p, R0Smem& sm, int lane) {
     if (sm.tile_page[1] < 0) sm.tile_page[1] = sm.tile_page[0];
     if (sm.tile_b[0] < 0) sm.tile_b[0] = sm.tile_b[1];
     if (sm.tile_b[1] < 0) sm.tile_b[1] = sm.tile_b[0];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      sm.tile_page[k] = max(sm.tile_page[k], 0);
+      sm.tile_b[k] = max(sm.tile_b[k], 0);
+    }
   }
 }
 
-__global__ void __launch_bounds__(kR0Threads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kR0Threads, 1)
     r0_project_kernel(const __grid_constant__ CUtensorMap cmap, const __grid_constant__ CUtensorMap wmap,
                       const R0ProjParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -193,6 +219,7 @@ __global__ void __launch_bounds__(kR0Threads, 1)
   volatile int* abort_flag = &sm.abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+  const uint32_t rank = cluster_rank();
   if (tid == 0) {
     mbar_init(smem_u32(&sm.afull), 1);
     for (int s = 0; s < kR0BStages; ++s) {
@@ -201,7 +228,7 @@ __global__ void __launch_bounds__(kR0Threads, 1)
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(smem_u32(&sm.dfull[s]), 1);
-      mbar_init(smem_u32(&sm.dfree[s]), kR0EpiWarps);
+      mbar_init(smem_u32(&sm.dfree[s]), 2 * kR0EpiWarps);   // both CTAs' epilogue warps, on the leader's
     }
     mbar_init(smem_u32(&sm.drain), 1);
     sm.abort = 0;
@@ -212,97 +239,111 @@ __global__ void __launch_bounds__(kR0Threads, 1)
   grid_dependency_wait();
   if (warp == 0) find_tile(p, sm, lane);
   __syncthreads();
-  if (sm.tile_n[0] == 0 && sm.tile_n[1] == 0) return;   // past the last page (uniform)
+  if (!sm.pair_live) return;   // past the last page (uniform in both CTAs of the pair)
   if (warp == 1) {
-    tmem_alloc(smem_u32(&sm.tmem_base), kR0TmemCols);
-    tmem_relinquish();
+    tmem_alloc_pair(smem_u32(&sm.tmem_base), kR0TmemCols);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();   // both CTAs' barriers are ready before either signals them
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-  const int nsteps = kR0Heads * p.nkc;   // (head, K chunk) steps of the B stream
 
-  bool epi_key = false, epi_ok = false;
-  float epi_s1 = 0.f, epi_s2 = 0.f;
+  bool epi_ok = false;
   if (warp == 0) {
-    // ---- TMA: the tile's two pages (all K chunks), then W^UKV_h chunk by chunk
+    // ---- TMA: the tile's two pages (all K chunks), then this CTA's half of
+    // W^UKV_h chunk by chunk; both CTAs' copies complete on the leader's
+    // barriers, which its producer arms for both
     if (elect_one()) {
       const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
-      mbar_arrive_expect_tx(smem_u32(&sm.afull), static_cast<uint32_t>(p.nkc) * kR0AChunkBytes);
+      const uint32_t afull = map_to_rank(smem_u32(&sm.afull), 0);
+      if (rank == 0) mbar_arrive_expect_tx(smem_u32(&sm.afull), 2 * static_cast<uint32_t>(p.nkc) * kR0AChunkBytes);
       for (int kc = 0; kc < p.nkc; ++kc)
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-          tma_load_2d(sbase + kc * kR0AChunkBytes + k * kR0APageBytes, &cmap, kc * kR0Chunk, sm.tile_page[k] * kPage,
-                      smem_u32(&sm.afull), pol_stream);
-      int issued = 0;
-      for (int i = 0; i < nsteps; ++i) {
-        const int s = i % kR0BStages;
-        if (i >= kR0BStages &&
-            !mbar_wait(smem_u32(&sm.bempty[s]), ((i / kR0BStages) & 1) ^ 1, abort_flag, p.wait_ns))
-          break;
-        const int h = i / p.nkc, kc = i % p.nkc;
-        mbar_arrive_expect_tx(smem_u32(&sm.bfull[s]), kR0BChunkBytes);
-        tma_load_2d(sbase + b_off + s * kR0BChunkBytes, &wmap, kc * kR0Chunk, h * kR0Feat, smem_u32(&sm.bfull[s]),
-                    pol_keep);
-        issued = i + 1;
+          tma_load_2d_pair(sbase + kc * kR0AChunkBytes + k * kR0APageBytes, &cmap, kc * kR0Chunk,
+                           sm.tile_page[k] * kPage, afull, pol_stream);
+      int issued = 0, s = 0;
+      uint32_t ph = 0;   // phase of stage s
+      bool ok = true;
+      for (int h = 0; ok && h < kR0Heads; ++h) {
+        for (int kc = 0; kc < p.nkc; ++kc) {
+          if (issued >= kR0BStages) ok = mbar_wait(smem_u32(&sm.bempty[s]), ph ^ 1, abort_flag, p.wait_ns);
+          if (!ok) break;
+          if (rank == 0) mbar_arrive_expect_tx(smem_u32(&sm.bfull[s]), 2 * kR0BChunkBytes);
+          tma_load_2d_pair(sbase + b_off + s * kR0BChunkBytes, &wmap, kc * kR0Chunk,
+                           h * kR0Feat + static_cast<int>(rank) * kR0Half,
+                           map_to_rank(smem_u32(&sm.bfull[s]), 0), pol_keep);
+          ++issued;
+          if (++s == kR0BStages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
       }
-      // every copy issued lands before the CTA can leave (own flag: bounded, not cut short)
-      volatile int own = 0;
-      if (!mbar_wait(smem_u32(&sm.afull), 0, &own, p.wait_ns)) *abort_flag = 1;
-      for (int i = issued > kR0BStages ? issued - kR0BStages : 0; i < issued; ++i)
-        if (!mbar_wait(smem_u32(&sm.bfull[i % kR0BStages]), (i / kR0BStages) & 1, &own, p.wait_ns))
-          *abort_flag = 1;
+      // every copy issued lands before either CTA can leave (own flag: bounded,
+      // not cut short; the other CTA waits at the cluster barrier at the end)
+      if (rank == 0) {
+        volatile int own = 0;
+        if (!mbar_wait(smem_u32(&sm.afull), 0, &own, p.wait_ns)) *abort_flag = 1;
+        for (int i = issued > kR0BStages ? issued - kR0BStages : 0; i < issued; ++i)
+          if (!mbar_wait(smem_u32(&sm.bfull[i % kR0BStages]), (i / kR0BStages) & 1, &own, p.wait_ns))
+            *abort_flag = 1;
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ---- MMA: head h into accumulator h % 2 once the epilogue has read it out
-    constexpr uint32_t idesc = idesc_bf16(kR0Rows, kR0Feat, 0, 0);
-    bool ok = warp_all_wait(smem_u32(&sm.afull), 0, abort_flag, p.wait_ns);
-    bool issued = false;
-    for (int h = 0; ok && h < kR0Heads; ++h) {
-      const int db = h & 1;
-      if (h >= 2) ok = warp_all_wait(smem_u32(&sm.dfree[db]), ((h - 2) >> 1) & 1, abort_flag, p.wait_ns);
-      for (int kc = 0; ok && kc < p.nkc; ++kc) {
-        const int i = h * p.nkc + kc, s = i % kR0BStages;
-        ok = warp_all_wait(smem_u32(&sm.bfull[s]), (i / kR0BStages) & 1, abort_flag, p.wait_ns);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
+    // ---- MMA (one thread of the leader): head h into accumulator h % 2 once both
+    // CTAs' epilogues have read it out; M = 256 (both tiles' rows), N = 256
+    if (rank == 0 && elect_one()) {
+      constexpr uint32_t idesc = idesc_bf16(2 * kR0Rows, kR0Feat, 0, 0);
+      bool ok = mbar_wait(smem_u32(&sm.afull), 0, abort_flag, p.wait_ns), issued = false;
+      int s = 0;
+      uint32_t ph = 0;
+      for (int h = 0; ok && h < kR0Heads; ++h) {
+        const int db = h & 1;
+        if (h >= 2) ok = mbar_wait_cluster(smem_u32(&sm.dfree[db]), ((h - 2) >> 1) & 1, abort_flag, p.wait_ns);
+        for (int kc = 0; ok && kc < p.nkc; ++kc) {
+          ok = mbar_wait(smem_u32(&sm.bfull[s]), ph, abort_flag, p.wait_ns);
+          if (!ok) break;
+          tc_fence_after();
           const uint64_t ad = smem_desc(sbase + kc * kR0AChunkBytes, 16, 1024, kSwizzle128B);
           const uint64_t bd = smem_desc(sbase + b_off + s * kR0BChunkBytes, 16, 1024, kSwizzle128B);
 #pragma unroll
           for (int kk = 0; kk < kR0Chunk / 16; ++kk)
-            mma_bf16_ss(tmem + db * kR0Feat, ad + ((kk * 32) >> 4), bd + ((kk * 32) >> 4), idesc,
-                        (kc > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(smem_u32(&sm.bempty[s]));
-          if (kc == p.nkc - 1) mma_commit(smem_u32(&sm.dfull[db]));
+            mma_bf16_ss_pair(tmem + db * kR0Feat, ad + ((kk * 32) >> 4), bd + ((kk * 32) >> 4), idesc,
+                             (kc > 0 || kk > 0) ? 1u : 0u);
+          issued = true;
+          mma_commit_pair(smem_u32(&sm.bempty[s]));
+          if (++s == kR0BStages) {
+            s = 0;
+            ph ^= 1;
+          }
         }
-        __syncwarp();
-        issued = true;
+        if (ok) mma_commit_pair(smem_u32(&sm.dfull[db]));
       }
-    }
-    // every MMA issued completes before TMEM is released
-    if (issued) {
-      if (elect_one()) mma_commit(smem_u32(&sm.drain));
-      __syncwarp();
-      volatile int own = 0;
-      if (!mbar_wait(smem_u32(&sm.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
+      // every MMA issued completes before TMEM is released
+      if (issued) {
+        mma_commit_pair(smem_u32(&sm.drain));
+        volatile int own = 0;
+        if (!mbar_wait(smem_u32(&sm.drain), 0, &own, p.wait_ns)) *abort_flag = 1;
+      }
     }
     __syncwarp();
   } else {
     // ---- epilogue: tile row r is TMEM lane r (warp w reads lane quadrant
-    // w % 4); rows 0-63 are the first page, 64-127 the second.  Warps 2-5
-    // take the key features (columns 0-127) of every head, warps 6-9 the
-    // value features (columns 128-255).
-    const int quad = warp & 3, half = (warp - 2) / 4;
+    // w % 4); rows 0-63 are the first page, 64-127 the second.  Group g takes
+    // columns 64 g .. 64 g + 63 of every head: g < 2 key, g >= 2 value features.
+    const uint32_t dfree = map_to_rank(smem_u32(&sm.dfree[0]), 0);
+    const int quad = warp & 3, grp = (warp - 2) / 4;
+    const bool key = grp < 2;
     const int r = 32 * quad + lane, k = r >> 6, jrow = r & (kPage - 1);
     const int n = sm.tile_n[k], page = sm.tile_page[k];
     const bool valid = jrow < n;
     const size_t prow = static_cast<size_t>(page) * kPage + jrow;
     int id = p.id_pool[prow];
     if (static_cast<unsigned>(id) >= static_cast<unsigned>(p.vocab)) {
-      if (valid && half == 0) report_status(p.status, kStatusOutOfRange);   // the gate uses row 0
+      if (valid && grp == 0) report_status(p.status, kStatusOutOfRange);   // the gate uses row 0
       id = 0;
     }
     // the query terms of the tile's two sequences: q gamma (key features),
@@ -317,8 +358,8 @@ __global__ void __launch_bounds__(kR0Threads, 1)
       const int s = i / (kR0Heads * kR0Rope), h = (i / kR0Rope) % kR0Heads, d = i % kR0Rope;
       sm.qr[s][h][d] = p.q[(static_cast<size_t>(sm.tile_b[s]) * kR0Heads + h) * (kR0Half + kR0Rope) + kR0Half + d];
     }
-    for (int pr = 0; pr < 4; ++pr) {
-      const int pidx = 4 * (warp - 2) + pr, s = pidx / kR0Heads, h = pidx % kR0Heads;
+    for (int pidx = warp - 2; pidx < 2 * kR0Heads; pidx += kR0EpiWarps) {
+      const int s = pidx / kR0Heads, h = pidx % kR0Heads;
       const __nv_bfloat16* qh = p.q + (static_cast<size_t>(sm.tile_b[s]) * kR0Heads + h) * (kR0Half + kR0Rope);
       float w = 0.f, bq = 0.f;
 #pragma unroll
@@ -337,145 +378,130 @@ __global__ void __launch_bounds__(kR0Threads, 1)
     }
     epi_sync();
 
-    const __nv_bfloat16* grow = p.gate + static_cast<size_t>(id) * kR0Width + half * kR0Half;
+    const __nv_bfloat16* grow = p.gate + static_cast<size_t>(id) * kR0Width + grp * kR0GroupFeat;
     const uint64_t pol_gate = policy_evict_last();
-    uint8_t* vst = sm.vstage[quad];
-    const bool store_v = half == 1 && n > 0;   // uniform in the warp
-    float s1 = 0.f, s2 = 0.f;
+    uint8_t* vst = sm.vstage[(warp - 2) & 7];
+    const bool store_v = !key && n > 0;   // uniform in the warp
+    float2 s1 = make_float2(0.f, 0.f), s2 = make_float2(0.f, 0.f);
     bool ok = true;
-    // this half of the row's gate values of a head (128 bf16): each quarter
-    // of them is requested for head h + 1 as soon as head h has used it, so
-    // that the loads run while the rest of head h is processed
-    uint4 g[kR0Half / 8];
+    // this group's part of the row's gate values of a head (64 bf16): each
+    // quarter of them is requested for head h + 1 as soon as head h has used
+    // it, so that the loads run while the rest of head h is processed
+    uint4 g[kR0GroupFeat / 8];
     auto load_g = [&](int hh, int i) { ldg_32_na_hint(grow + hh * kR0Feat + 16 * i, pol_gate, g[2 * i], g[2 * i + 1]); };
 #pragma unroll
-    for (int i = 0; i < kR0Half / 16; ++i) load_g(0, i);
+    for (int i = 0; i < kR0GroupFeat / 16; ++i) load_g(0, i);
     for (int h = 0; h < kR0Heads; ++h) {
       const int db = h & 1;
-      if (h + 2 < kR0Heads) {   // two heads ahead into L2
-        prefetch_l2(grow + (h + 2) * kR0Feat);
-        prefetch_l2(grow + (h + 2) * kR0Feat + 64);
-      }
+      if (h + 2 < kR0Heads) prefetch_l2(grow + (h + 2) * kR0Feat);   // two heads ahead into L2
       ok = ok && warp_all_wait(smem_u32(&sm.dfull[db]), (h >> 1) & 1, abort_flag, p.wait_ns);
       if (!ok) break;
       tc_fence_after();
-      const float* qgh = &sm.qg[k][h][0];
-      float dot = 0.f;
+      const float* qgh = &sm.qg[k][h][(grp & 1) * kR0GroupFeat];
+      float2 dot2 = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int c0 = 0; c0 < kR0Half; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + (static_cast<uint32_t>(32 * quad) << 16) + db * kR0Feat + half * kR0Half + c0, v);
+      for (int c0 = 0; c0 < kR0GroupFeat; c0 += 32) {
+        float v[32];
+        const uint32_t ta = tmem + (static_cast<uint32_t>(32 * quad) << 16) + db * kR0Feat + grp * kR0GroupFeat + c0;
+        tmem_ld16(ta, *reinterpret_cast<float(*)[16]>(&v[0]));
+        tmem_ld16(ta + 16, *reinterpret_cast<float(*)[16]>(&v[16]));
         tmem_wait_ld();
-        const __nv_bfloat162* ge0 = reinterpret_cast<const __nv_bfloat162*>(&g[c0 / 8]);
-        const __nv_bfloat162* ge1 = reinterpret_cast<const __nv_bfloat162*>(&g[c0 / 8 + 1]);
-        uint32_t packed[8];
-        float zf[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float2 gf = __bfloat1622float2(i < 4 ? ge0[i] : ge1[i - 4]);
-          const __nv_bfloat162 zb = __floats2bfloat162_rn(v[2 * i] * gf.x, v[2 * i + 1] * gf.y);
-          const float2 zr = __bfloat1622float2(zb);   // statistics and dots of the rounded values
-          s1 += zr.x + zr.y;
-          s2 = fmaf(zr.x, zr.x, fmaf(zr.y, zr.y, s2));
-          zf[2 * i] = zr.x;
-          zf[2 * i + 1] = zr.y;
-          packed[i] = *reinterpret_cast<const uint32_t*>(&zb);
-        }
-        if (half == 0) {
+        for (int u = 0; u < 4; ++u) {   // 8 columns: one 16-byte unit
+          const uint32_t* gw = reinterpret_cast<const uint32_t*>(&g[c0 / 8 + u]);
+          uint32_t packed[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const float4 qv = *reinterpret_cast<const float4*>(qgh + c0 + 4 * i);
-            dot = fmaf(qv.x, zf[4 * i], dot);
-            dot = fmaf(qv.y, zf[4 * i + 1], dot);
-            dot = fmaf(qv.z, zf[4 * i + 2], dot);
-            dot = fmaf(qv.w, zf[4 * i + 3], dot);
+            const float2 z = __fmul2_rn(make_float2(v[8 * u + 2 * i], v[8 * u + 2 * i + 1]), widen2(gw[i]));
+            const __nv_bfloat162 zb = __floats2bfloat162_rn(z.x, z.y);
+            packed[i] = *reinterpret_cast<const uint32_t*>(&zb);
+            const float2 zr = widen2(packed[i]);   // statistics and dots of the rounded values
+            s1 = __fadd2_rn(s1, zr);
+            s2 = __ffma2_rn(zr, zr, s2);
+            if (key) {
+              const float2 qv = *reinterpret_cast<const float2*>(qgh + c0 + 8 * u + 2 * i);
+              dot2 = __ffma2_rn(qv, zr, dot2);
+            }
           }
-        } else {
-          // chunks c0/8 and c0/8 + 1 of this row, at (chunk ^ (row % 16)) in its 256-byte row
-          const int ch = c0 / 8;
-          *reinterpret_cast<uint4*>(vst + lane * kR0RowBytes + ((ch ^ (lane & 15)) << 4)) =
-              make_uint4(packed[0], packed[1], packed[2], packed[3]);
-          *reinterpret_cast<uint4*>(vst + lane * kR0RowBytes + (((ch + 1) ^ (lane & 15)) << 4)) =
-              make_uint4(packed[4], packed[5], packed[6], packed[7]);
-        }
-        if (c0 % 32 == 16 && h + 1 < kR0Heads) {   // columns c0 - 16 .. c0 + 15 done
-          load_g(h + 1, c0 / 16 - 1);
-          load_g(h + 1, c0 / 16);
+          if (!key)   // this unit of the row, at (unit ^ (row % 8)) in its 128-byte row
+            *reinterpret_cast<uint4*>(vst + lane * kR0GroupBytes + (((c0 / 8 + u) ^ (lane & 7)) << 4)) =
+                make_uint4(packed[0], packed[1], packed[2], packed[3]);
+          if ((u & 1) && h + 1 < kR0Heads) load_g(h + 1, c0 / 16 + u / 2);   // these 16 columns done
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&sm.dfree[db]));
-      if (half == 0) {
-        sm.s1[r][h] = dot;
+      if (lane == 0) mbar_arrive_cluster(dfree + db * 8);
+      if (key) {
+        sm.s1[grp][r][h] = dot2.x + dot2.y;
       } else if (store_v) {
-        // the warp's 32 rows of head h are 8 KB in one piece (head-major):
-        // two whole rows per store instruction
+        // the warp's 32 rows of head h (head-major), its 128 bytes of each:
+        // four rows per store instruction
         uint8_t* dst = reinterpret_cast<uint8_t*>(
-            p.zv + (static_cast<size_t>(h) * p.pool_rows + static_cast<size_t>(page) * kPage + 32 * (quad & 1)) *
-                       kR0Half);
+                           p.zv + (static_cast<size_t>(h) * p.pool_rows + static_cast<size_t>(page) * kPage +
+                                   32 * (quad & 1)) * kR0Half) + (grp & 1) * kR0GroupBytes;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int rr = 2 * i + (lane >> 4), c = lane & 15;
+        for (int i = 0; i < 8; ++i) {
+          const int rr = 4 * i + (lane >> 3), c = lane & 7;
           *reinterpret_cast<uint4*>(dst + rr * kR0RowBytes + c * 16) =
-              *reinterpret_cast<const uint4*>(vst + rr * kR0RowBytes + ((c ^ (rr & 15)) << 4));
+              *reinterpret_cast<const uint4*>(vst + rr * kR0GroupBytes + ((c ^ (rr & 7)) << 4));
         }
         __syncwarp();   // the tile is read before the next head rewrites it
       }
     }
-    if (half == 1) sm.half_sums[r] = make_float2(s1, s2);
-    epi_key = half == 0 && n > 0;
+    sm.sums[grp][r] = make_float2(s1.x + s1.y, s2.x + s2.y);
     epi_ok = ok;
-    epi_s1 = s1;
-    epi_s2 = s2;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (epi_key && epi_ok && !sm.abort) {
-    // the row's statistics over all 4096 features, then every head's logit
-    const int r = 32 * (warp & 3) + lane, k = r >> 6, jrow = r & (kPage - 1);
+  if (epi_ok && !sm.abort) {
+    // the row's statistics over all 4096 features, then its logits: four heads
+    // per group
+    const int grp = (warp - 2) / 4, r = 32 * (warp & 3) + lane, k = r >> 6, jrow = r & (kPage - 1);
     const size_t prow = static_cast<size_t>(sm.tile_page[k]) * kPage + jrow;
-    const float2 o = sm.half_sums[r];
-    const float mu = (epi_s1 + o.x) / kR0Width;
-    const float var = fmaxf((epi_s2 + o.y) / kR0Width - mu * mu, 0.f);
+    float t1 = 0.f, t2 = 0.f;
+#pragma unroll
+    for (int g = 0; g < kR0Groups; ++g) {
+      t1 += sm.sums[g][r].x;
+      t2 += sm.sums[g][r].y;
+    }
+    const float mu = t1 / kR0Width;
+    const float var = fmaxf(t2 / kR0Width - mu * mu, 0.f);
     const float rinv = rsqrtf(var + p.eps);
-    p.stats[prow] = make_float2(mu, rinv);
+    if (grp == 0 && sm.tile_n[k] > 0) p.stats[prow] = make_float2(mu, rinv);
     if (jrow < sm.tile_n[k]) {
-      float kr[kR0Rope];
       const uint4* kr4 = reinterpret_cast<const uint4*>(p.kr_pool + prow * kR0Rope);
+      uint4 kr[kR0Rope / 8];
 #pragma unroll
-      for (int i = 0; i < kR0Rope / 8; ++i) {
-        const uint4 u = kr4[i];
-        const __nv_bfloat162* e = reinterpret_cast<const __nv_bfloat162*>(&u);
+      for (int i = 0; i < kR0Rope / 8; ++i) kr[i] = kr4[i];
+      float lg[kR0Heads / kR0Groups];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 f = __bfloat1622float2(e[j]);
-          kr[8 * i + 2 * j] = f.x;
-          kr[8 * i + 2 * j + 1] = f.y;
-        }
-      }
-      float lg[kR0Heads];
-#pragma unroll
-      for (int h = 0; h < kR0Heads; ++h) {
+      for (int e = 0; e < kR0Heads / kR0Groups; ++e) {
+        const int h = 4 * grp + e;
         const __nv_bfloat162* qr2 = reinterpret_cast<const __nv_bfloat162*>(&sm.qr[k][h][0]);
         float sr = 0.f;
 #pragma unroll
         for (int d = 0; d < kR0Rope / 2; ++d) {
           const float2 qf = __bfloat1622float2(qr2[d]);
-          sr = fmaf(qf.x, kr[2 * d], fmaf(qf.y, kr[2 * d + 1], sr));
+          const float2 kf = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(kr)[d]);
+          sr = fmaf(qf.x, kf.x, fmaf(qf.y, kf.y, sr));
         }
         const float2 wb = sm.wb[k][h];
-        lg[h] = p.scale_log2 * (rinv * (sm.s1[r][h] - mu * wb.x) + wb.y + sr);
+        lg[e] = p.scale_log2 * (rinv * (sm.s1[0][r][h] + sm.s1[1][r][h] - mu * wb.x) + wb.y + sr);
       }
       const size_t pos = static_cast<size_t>(sm.tile_b[k]) * p.max_pages * kPage +
                          static_cast<size_t>(sm.tile_lp[k]) * kPage + jrow;
-      float4* dst = reinterpret_cast<float4*>(p.logit + pos * kR0Heads);
-#pragma unroll
-      for (int i = 0; i < kR0Heads / 4; ++i) dst[i] = make_float4(lg[4 * i], lg[4 * i + 1], lg[4 * i + 2], lg[4 * i + 3]);
+      reinterpret_cast<float4*>(p.logit + pos * kR0Heads)[grp] = make_float4(lg[0], lg[1], lg[2], lg[3]);
     }
   }
-  if (warp == 1) tmem_dealloc(tmem, kR0TmemCols);
+  // neither CTA leaves (or frees its tensor memory) while the other's copies,
+  // MMAs or arrivals may still reach it
+  __syncwarp();
+  tc_fence_before();
+  cluster_sync();
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc_pair(tmem, kR0TmemCols);
   if (tid == 0 && sm.abort) report_status(p.status, kStatusTimeout);
 }
 
@@ -648,7 +674,7 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   float* logit = reinterpret_cast<float*>(ws + off);
   CUtensorMap cmap, wmap;
   if (!r0_encode(&cmap, a.c_pool, rows, static_cast<uint64_t>(a.d_c), kPage)) return cudaErrorInvalidValue;
-  if (!r0_encode(&wmap, a.w_ukv, kR0Width, static_cast<uint64_t>(a.d_c), kR0Feat)) return cudaErrorInvalidValue;
+  if (!r0_encode(&wmap, a.w_ukv, kR0Width, static_cast<uint64_t>(a.d_c), kR0Half)) return cudaErrorInvalidValue;
   const int nkc = a.d_c / kR0Chunk;
   const int smem = static_cast<int>(nkc * kR0AChunkBytes + kR0BStages * kR0BChunkBytes + sizeof(R0Smem) + 1024);
   cudaError_t e = cudaFuncSetAttribute(r0_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -676,7 +702,8 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   pp.wait_ns = kWaitLimitNs;
   pp.status = a.status;
   // one CTA per two pages of the walk: the block table bounds the pages in use
-  const int tiles = static_cast<int>((static_cast<int64_t>(a.batch) * a.max_pages + 1) / 2);
+  // (an even number: the CTAs work in pairs)
+  const int tiles = static_cast<int>((static_cast<int64_t>(a.batch) * a.max_pages + 3) / 4 * 2);
   e = launch_chained(r0_project_kernel, dim3(tiles), dim3(kR0Threads), smem, st, cmap, wmap, pp);
   if (e != cudaSuccess) return e;
   R0AttnParams ap;
