@@ -107,92 +107,16 @@ struct PfGateParams {
 };
 
 constexpr int kGateWarps = 8;
-
-// c~ of one row from its loaded c and g units, stored, and the row's cache write
-__device__ __forceinline__ void gate_row(const PfGateParams& p, int t, int b, int pos, int lane, int nu,
-                                         const uint4 (&craw)[2], const uint4 (&graw)[2], bool& bad) {
-  float z[2][8];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int u = lane + 32 * i;
-    const __nv_bfloat162* c2 = reinterpret_cast<const __nv_bfloat162*>(&craw[i]);
-    const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&graw[i]);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 cf = __bfloat1622float2(c2[e]);
-      float2 v = cf;
-      if (p.gate) {
-        const float2 gf = __bfloat1622float2(g2[e]);
-        v = p.gate_add ? make_float2(cf.x + gf.x, cf.y + gf.y) : make_float2(cf.x * gf.x, cf.y * gf.y);
-      }
-      z[i][2 * e] = u < nu ? v.x : 0.f;
-      z[i][2 * e + 1] = u < nu ? v.y : 0.f;
-    }
-  }
-  if (p.gate && p.gate_ln) {
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s += z[i][e];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float mu = s / p.d_c;
-    float q = 0.f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (lane + 32 * i < nu)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) q = fmaf(z[i][e] - mu, z[i][e] - mu, q);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    const float r = rsqrtf(q / p.d_c + p.eps);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int u = lane + 32 * i;
-      if (u >= nu) continue;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float gm = p.gamma ? __ldg(p.gamma + 8 * u + e) : 1.f;
-        const float bt = p.beta ? __ldg(p.beta + 8 * u + e) : 0.f;
-        z[i][e] = fmaf((z[i][e] - mu) * r, gm, bt);
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int u = lane + 32 * i;
-    if (u >= nu) continue;
-    uint4 o;
-    o.x = pack_bf16x2(z[i][0], z[i][1]);
-    o.y = pack_bf16x2(z[i][2], z[i][3]);
-    o.z = pack_bf16x2(z[i][4], z[i][5]);
-    o.w = pack_bf16x2(z[i][6], z[i][7]);
-    reinterpret_cast<uint4*>(p.ctil + static_cast<size_t>(t) * p.d_c)[u] = o;
-  }
-  if (p.c_pool) {
-    const int lp = pos / kPage;
-    const int page = lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
-    if (page < 0 || page >= p.num_pages) {
-      bad = true;
-    } else {
-      const size_t slot = static_cast<size_t>(page) * kPage + pos % kPage;
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int u = lane + 32 * i;
-        if (u < nu) reinterpret_cast<uint4*>(p.c_pool + slot * p.d_c)[u] = craw[i];
-      }
-      if (lane < p.d_r / 8)
-        reinterpret_cast<uint4*>(p.kr_pool + slot * p.d_r)[lane] =
-            __ldg(reinterpret_cast<const uint4*>(p.kr + static_cast<size_t>(t) * p.d_r) + lane);
-      if (lane == 0 && p.id_pool && p.ids) p.id_pool[slot] = __ldg(p.ids + t);
-    }
-  }
-}
+constexpr int kGateRows = 1;   // token rows of a warp, their loads in flight together (2: 28 us, 4: 39, 1: 25 at 8 x 4096)
 
 constexpr int kSortMaxBatch = 2048;   // larger batches keep the given order
 
-// One warp per token row.
+// A warp takes kGateRows consecutive token rows; NU 16-byte units of a row per
+// lane (d_c <= 256 NU).  Everything a row needs is requested before anything is
+// used: its latent, id, RoPE key and page, then its gate row.  Bound by that
+// chain's latency at few tokens and by DRAM at many (75 MB at 8 x 4096 with the
+// gate: 29 us with every row looped over as if 512 wide, 25 now).
+template <int NU>
 __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfGateParams p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_launch_dependents();
@@ -215,28 +139,120 @@ __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfG
       p.order[rank] = b;
     }
   }
-  const int t = blockIdx.x * kGateWarps + warp;
-  if (t >= p.total) return;
-  const int nu = p.d_c / 8;   // 16-byte units of a row (at most 64: two per lane)
-  const int b = prompt_of_row(p.cu, p.batch, t);
-  const int pos = t - __ldg(p.cu + b);
+  const int t0 = (blockIdx.x * kGateWarps + warp) * kGateRows;
+  if (t0 >= p.total) return;
+  const int nu = p.d_c / 8;   // 16-byte units of a row
+  uint4 craw[kGateRows][NU], graw[kGateRows][NU], kraw[kGateRows];
+  int id[kGateRows], page[kGateRows], slot[kGateRows];
   bool bad = false;
-  int id = p.ids ? __ldg(p.ids + t) : 0;
-  if (p.gate && static_cast<unsigned>(id) >= static_cast<unsigned>(p.vocab)) {
-    bad = true;
-    id = 0;
-  }
-  uint4 craw[2], graw[2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int u = lane + 32 * i;
-    craw[i] = make_uint4(0u, 0u, 0u, 0u);
-    graw[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (u < nu) craw[i] = __ldg(reinterpret_cast<const uint4*>(p.c + static_cast<size_t>(t) * p.d_c) + u);
-    if (p.gate && u < nu)
-      graw[i] = __ldg(reinterpret_cast<const uint4*>(p.gate_table + static_cast<size_t>(id) * p.d_c) + u);
+  for (int k = 0; k < kGateRows; ++k) {
+    const int t = min(t0 + k, p.total - 1);
+    id[k] = p.ids ? __ldg(p.ids + t) : 0;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int u = lane + 32 * i;
+      craw[k][i] = make_uint4(0u, 0u, 0u, 0u);
+      if (u < nu) craw[k][i] = __ldg(reinterpret_cast<const uint4*>(p.c + static_cast<size_t>(t) * p.d_c) + u);
+    }
+    if (p.c_pool && lane < p.d_r / 8)
+      kraw[k] = __ldg(reinterpret_cast<const uint4*>(p.kr + static_cast<size_t>(t) * p.d_r) + lane);
   }
-  gate_row(p, t, b, pos, lane, nu, craw, graw, bad);
+#pragma unroll
+  for (int k = 0; k < kGateRows; ++k) {
+    const int t = min(t0 + k, p.total - 1);
+    const bool live = t0 + k < p.total;
+    if (p.gate && static_cast<unsigned>(id[k]) >= static_cast<unsigned>(p.vocab)) {
+      bad = bad || live;
+      id[k] = 0;
+    }
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int u = lane + 32 * i;
+      graw[k][i] = make_uint4(0u, 0u, 0u, 0u);
+      if (p.gate && u < nu)
+        graw[k][i] = __ldg(reinterpret_cast<const uint4*>(p.gate_table + static_cast<size_t>(id[k]) * p.d_c) + u);
+    }
+    page[k] = -1;
+    if (p.c_pool) {
+      const int b = prompt_of_row(p.cu, p.batch, t);
+      const int pos = t - __ldg(p.cu + b), lp = pos / kPage;
+      slot[k] = pos % kPage;
+      page[k] = lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kGateRows; ++k) {
+    const int t = t0 + k;
+    if (t >= p.total) break;
+    // c~ of the row
+    float z[NU][8];
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const __nv_bfloat162* c2 = reinterpret_cast<const __nv_bfloat162*>(&craw[k][i]);
+      const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&graw[k][i]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 cf = __bfloat1622float2(c2[e]);
+        float2 v = cf;
+        if (p.gate) {
+          const float2 gf = __bfloat1622float2(g2[e]);
+          v = p.gate_add ? make_float2(cf.x + gf.x, cf.y + gf.y) : make_float2(cf.x * gf.x, cf.y * gf.y);
+        }
+        z[i][2 * e] = v.x;   // (units past the row: 0)
+        z[i][2 * e + 1] = v.y;
+      }
+    }
+    if (p.gate && p.gate_ln) {
+      float sum = 0.f;
+#pragma unroll
+      for (int i = 0; i < NU; ++i)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum += z[i][e];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      const float mu = sum / p.d_c;
+      float q = 0.f;
+#pragma unroll
+      for (int i = 0; i < NU; ++i)
+        if (lane + 32 * i < nu)
+#pragma unroll
+          for (int e = 0; e < 8; ++e) q = fmaf(z[i][e] - mu, z[i][e] - mu, q);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      const float r = rsqrtf(q / p.d_c + p.eps);
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const int u = lane + 32 * i;
+        if (u >= nu) continue;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float gm = p.gamma ? __ldg(p.gamma + 8 * u + e) : 1.f;
+          const float bt = p.beta ? __ldg(p.beta + 8 * u + e) : 0.f;
+          z[i][e] = fmaf((z[i][e] - mu) * r, gm, bt);
+        }
+      }
+    }
+    const bool write = page[k] >= 0 && page[k] < p.num_pages;
+    if (p.c_pool && !write) bad = true;
+    const size_t row = write ? static_cast<size_t>(page[k]) * kPage + slot[k] : 0;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) {
+      const int u = lane + 32 * i;
+      if (u >= nu) continue;
+      uint4 o;
+      o.x = pack_bf16x2(z[i][0], z[i][1]);
+      o.y = pack_bf16x2(z[i][2], z[i][3]);
+      o.z = pack_bf16x2(z[i][4], z[i][5]);
+      o.w = pack_bf16x2(z[i][6], z[i][7]);
+      reinterpret_cast<uint4*>(p.ctil + static_cast<size_t>(t) * p.d_c)[u] = o;
+      if (p.c_pool && write) reinterpret_cast<uint4*>(p.c_pool + row * p.d_c)[u] = craw[k][i];
+    }
+    if (p.c_pool && write) {
+      if (lane < p.d_r / 8) reinterpret_cast<uint4*>(p.kr_pool + row * p.d_r)[lane] = kraw[k];
+      if (lane == 0 && p.id_pool && p.ids) p.id_pool[row] = __ldg(p.ids + t);
+    }
+  }
   if (bad && lane == 0) report_status(p.status, kStatusOutOfRange);
 }
 
@@ -1118,8 +1134,10 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   gp.gate_ln = a.gate_ln;
   gp.eps = a.eps;
   gp.status = a.status;
-  cudaError_t e =
-      launch_chained(prefill_gate_kernel, dim3((a.total + kGateWarps - 1) / kGateWarps), dim3(32 * kGateWarps), 0, st, gp);
+  const dim3 gate_grid((a.total + kGateWarps * kGateRows - 1) / (kGateWarps * kGateRows));
+  cudaError_t e = a.d_c <= 256
+                      ? launch_chained(prefill_gate_kernel<1>, gate_grid, dim3(32 * kGateWarps), 0, st, gp)
+                      : launch_chained(prefill_gate_kernel<2>, gate_grid, dim3(32 * kGateWarps), 0, st, gp);
   if (e != cudaSuccess) return e;
 
   // 2. keys and values of every head: the units shared equally by one CTA per SM
