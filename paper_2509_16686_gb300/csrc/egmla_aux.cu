@@ -636,11 +636,11 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
 //  - u: lanes are output rows; a sequence's three columns are added, rounded to
 //    bf16 and stored.
 // Bound by the merge's reads of the partials from L2 and the latency of its
-// phases: 9 us at 128 sequences with d_c 192 (the merge at the end of the
+// phases: 7 us at 128 sequences with d_c 192 (the merge at the end of the
 // decode kernel, on CUDA cores after a grid-wide wait, and the cooperative
-// launch it needs cost that step 8 us more), and 13 us against 18 on CUDA cores
+// launch it needs cost that step 8 us more), and 8 us against 18 on CUDA cores
 // with d_c 512 (kernel alone, warm).
-constexpr int kCtThreads = 256;
+constexpr int kCtMaxThreads = 512;
 constexpr int kCtMaxSeq = 16;            // sequences per block, at most
 constexpr int kCtBlocks = 152;           // one per SM
 constexpr uint32_t kCtAtom = 128 * 128;  // 128 rows x 64 bf16
@@ -652,7 +652,7 @@ struct CtShared {
   float wts[kCtMaxSeq][kCombineSlots];
   float inv_l[kCtMaxSeq];
   int slots[kCtMaxSeq], slot0[kCtMaxSeq];
-  float4 red[kCtThreads];
+  float4 red[kCtMaxThreads];
   uint64_t afull, done;
   uint32_t tmem_base;
   int abort;
@@ -661,14 +661,17 @@ __host__ __device__ constexpr uint32_t ct_smem(int d_c, int nt) {
   return static_cast<uint32_t>(d_c / 64) * (kCtAtom + ct_cols(nt) * 128) + sizeof(CtShared) + 1024;
 }
 
-// PPT: (sequence, 4 features) pairs per thread, at most
-template <int PPT>
+// PPT: (sequence, 4 features) pairs per thread, at most; T threads (512 where
+// that is more than one pair each: more of the partials in flight, 128 ragged
+// sequences 69.3 -> 67.7 us, 128 at d_c 512 123.6 -> 118.9; 256 otherwise, 32 x 4K
+// 37.5 against 38.1)
+template <int PPT, int kCtThreads>
 __global__ void __launch_bounds__(kCtThreads)
 combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __restrict__ cu,
                   const float* __restrict__ part_ml, const float* __restrict__ part_o, __nv_bfloat16* __restrict__ out,
                   int batch, int d_c, int d_v, int num_splits, int nt, int early, uint64_t wait_ns, int32_t* status) {
   constexpr int H = 16;
-  constexpr int kFlight = PPT >= 8 ? 2 : PPT >= 4 ? 4 : 8;   // slots of a pair in flight
+  constexpr int kFlight = PPT >= 4 ? 4 : 8;   // slots of a pair in flight
   extern __shared__ uint8_t ct_raw[];
   uint8_t* smem = ct_raw + ((1024u - (smem_u32(ct_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
@@ -844,8 +847,8 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
   bool ok = mbar_wait(smem_u32(&sh.done), 0, abort_flag, wait_ns);
   ok = __all_sync(0xffffffffu, ok) && *abort_flag == 0;
   tc_fence_after();
-  // ---- u: warp = (lane quadrant, every other sequence)
-  if (ok) {
+  // ---- u: warp (of the first eight) = (lane quadrant, every other sequence)
+  if (ok && warp < 8) {
     float d[48];
     const uint32_t ta = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
 #pragma unroll
@@ -1226,15 +1229,15 @@ cudaError_t launch_decode_f32(const DecodeArgs& a, const AppendArgs* app, cudaSt
 }
 
 namespace {
-template <int PPT>
+template <int PPT, int T>
 cudaError_t launch_combine_tc(const DecodeArgs& a, const CUtensorMap* wmap, const int32_t* cu, const float* ml,
                               const float* po, int nt, cudaStream_t st) {
   const size_t smem = ct_smem(a.d_c, nt);
-  const cudaError_t e = cudaFuncSetAttribute(combine_tc_kernel<PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(combine_tc_kernel<PPT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  return launch_chained(combine_tc_kernel<PPT>, dim3(16 * ((a.batch + nt - 1) / nt), (a.d_v + 127) / 128),
-                        dim3(kCtThreads), smem, st, *wmap, cu, ml, po, static_cast<__nv_bfloat16*>(a.out), a.batch,
+  return launch_chained(combine_tc_kernel<PPT, T>, dim3(16 * ((a.batch + nt - 1) / nt), (a.d_v + 127) / 128),
+                        dim3(T), smem, st, *wmap, cu, ml, po, static_cast<__nv_bfloat16*>(a.out), a.batch,
                         a.d_c, a.d_v, a.num_splits, nt, a.early, kWaitLimitNs, a.status);
 }
 }  // namespace
@@ -1250,10 +1253,10 @@ cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, const CUtensorMap*
     int nt = 1;
     while (nt < kCtMaxSeq && 16 * ((a.batch + nt - 1) / nt) > kCtBlocks) nt *= 2;
     const int pairs = nt * (a.d_c / 4);
-    if (pairs <= kCtThreads) return launch_combine_tc<1>(a, wmap, cu, ml, po, nt, st);
-    if (pairs <= 2 * kCtThreads) return launch_combine_tc<2>(a, wmap, cu, ml, po, nt, st);
-    if (pairs <= 4 * kCtThreads) return launch_combine_tc<4>(a, wmap, cu, ml, po, nt, st);
-    return launch_combine_tc<8>(a, wmap, cu, ml, po, nt, st);
+    if (pairs <= 256) return launch_combine_tc<1, 256>(a, wmap, cu, ml, po, nt, st);
+    if (pairs <= 512) return launch_combine_tc<1, 512>(a, wmap, cu, ml, po, nt, st);
+    if (pairs <= 1024) return launch_combine_tc<2, 512>(a, wmap, cu, ml, po, nt, st);
+    return launch_combine_tc<4, 512>(a, wmap, cu, ml, po, nt, st);
   }
   // small batches: the output rows spread over more blocks (a pass of the block's
   // warps covers 32 rows), so that most SMs read a part of W_UV
