@@ -580,11 +580,13 @@ constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffK = kOffQ + 2 * kAttnQBytes;
 constexpr uint32_t kOffV = kOffK + kAttnKSlots * kPfAtom;
 constexpr uint32_t kOffBars = kOffV + kAttnVStages * kAttnVBytes;
-// warp 0: work items, query and key copies; warp 1: MMAs; warps 2-9: softmax
-// and epilogue (2-5 tile A, 6-9 tile B, warp w reading TMEM lane quadrant
-// w % 4); warp 10: value copies
+// warp 0: work items, query and key copies; warp 1: MMAs; warps 2-17: softmax
+// and epilogue (2-9 tile A, 10-17 tile B; warp w reads TMEM lane quadrant w % 4,
+// the first four of a tile's eight warps its first 16 lanes, the others its last
+// 16); warp 18: value copies
 constexpr int kAttnSoftWarp0 = 2;
-constexpr int kAttnVWarp = 10;
+constexpr int kAttnSoftWarps = 16;
+constexpr int kAttnVWarp = kAttnSoftWarp0 + kAttnSoftWarps;
 constexpr int kAttnThreads = 32 * (kAttnVWarp + 1);
 // TMEM columns: S_X (P_X over its first 64 columns) and O_X
 __host__ __device__ constexpr uint32_t col_s(int x) { return x * kAttnKeys; }
@@ -608,7 +610,7 @@ struct AttnBars {
   int abort;
 };
 constexpr uint32_t kAttnSmem = kOffBars + sizeof(AttnBars) + 1024;
-constexpr int kAttnItemReaders = 2 + 8;   // MMA warp, value loader, eight softmax warps
+constexpr int kAttnItemReaders = 2 + kAttnSoftWarps;   // MMA warp, value loader, softmax warps
 
 struct AttnParams {
   const int32_t* cu;
@@ -648,9 +650,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(smem_u32(&bars.sfull[x]), 1);
-      for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&bars.pfull[x][h]), 4);
+      for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&bars.pfull[x][h]), 8);
       mbar_init(smem_u32(&bars.odone[x]), 1);
-      mbar_init(smem_u32(&bars.ofree[x]), 4);
+      mbar_init(smem_u32(&bars.ofree[x]), 8);
       mbar_init(smem_u32(&bars.ifull[x]), 1);
       mbar_init(smem_u32(&bars.iempty[x]), kAttnItemReaders);
     }
@@ -895,11 +897,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---- softmax and epilogue of query tile x: query row r = TMEM lane r
-    const int x = (warp - kAttnSoftWarp0) >> 2;
-    const int quad = warp & 3;
-    const int r = 32 * quad + lane;
-    const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * quad) << 16);
+    // ---- softmax and epilogue of query tile x: query row = TMEM lane.  The score
+    // MMAs of one tile cover only so many cycles of the other tile's softmax, so
+    // its latency counts.  A warp has 16 rows, four lanes per row (16x256b loads:
+    // lane t has rows t/4 and t/4 + 8, columns 2 (t%4) and + 1 of every 8-column
+    // group), so a thread's chains are 2 x 32 scores long and a row's maximum
+    // takes two shuffles; the scores are read twice (once for the maximum), which
+    // keeps a thread within its registers.  Whole calls against a thread per row
+    // (8 warps): 604 -> 581 us at 8 x 4096, 201 -> 187 for 16 ragged prompts, 26.8
+    // -> 24.8 for one of 777 tokens.
+    const int x = (warp - kAttnSoftWarp0) >> 3, sub = ((warp - kAttnSoftWarp0) >> 2) & 1;
+    const int lane0 = 32 * (warp & 3) + 16 * sub;   // the warp's first row
+    const int r0 = lane0 + (lane >> 2), c2 = 2 * (lane & 3);
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(lane0) << 16);
     const float sl2 = p.scale_log2;
     int tx = 0, kx = 0;   // tiles and items of X before this item
     bool ok = true;
@@ -910,103 +920,125 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       tiles_of(it, ntile);
       const int nx = ntile[x];
       if (nx == 0) continue;
-      const int qrow = it.qb * 2 * kPfRows + x * kPfRows + r;   // this row's position in the prompt
-      float m_ref = 0.f, l = 0.f;
+      const int qrow = it.qb * 2 * kPfRows + x * kPfRows + r0;   // the thread's rows in the prompt: qrow, qrow + 8
+      float m_ref[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};
       for (int j = 0; ok && j < nx; ++j) {
         // S_X(j) complete (and with it every earlier MMA: O_X is current)
         ok = pf_warp_wait(smem_u32(&bars.sfull[x]), (tx + j) & 1, abort_flag, p.wait_ns);
         if (!ok) break;
         tc_fence_after();
-        float sv[kAttnKeys];
-#pragma unroll
-        for (int c = 0; c < kAttnKeys; c += 16)
-          tmem_ld16(lane_base + col_s(x) + c, *reinterpret_cast<float(*)[16]>(&sv[c]));
-        tmem_wait_ld();
         const int k0 = j * kAttnKeys;
-        if (k0 + kAttnKeys - 1 > qrow) {
-          // keys after the query (the tile on the diagonal)
+        const bool diag = k0 + kAttnKeys - 1 > qrow;   // the tile on the diagonal: keys after the query
+        // 64 columns of the tile, keys after the query at -inf
+        auto load_s = [&](int g, float (&v)[32]) {
+          tmem_ld_16x256b_x8(lane_base + col_s(x) + 64 * g, v);
+          tmem_wait_ld();
+          if (diag) {
+            const int lim = qrow - k0 - 64 * g - c2;   // last column of the first row
 #pragma unroll
-          for (int c = 0; c < kAttnKeys; ++c)
-            if (k0 + c > qrow) sv[c] = -INFINITY;
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (8 * k + (e & 1) > lim + 8 * (e >> 1)) v[4 * k + e] = -INFINITY;
+          }
+        };
+        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          float v[32];
+          load_s(g, v);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) m4[e] = fmaxf(m4[e], v[4 * k + e]);
         }
-        // row maximum and sum as interleaved chains (short dependencies)
-        float m8[8];
+        float alpha[2] = {1.f, 1.f};
 #pragma unroll
-        for (int e = 0; e < 8; ++e) m8[e] = sv[e];
-#pragma unroll
-        for (int c = 8; c < kAttnKeys; c += 16)
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            m8[e] = c + 8 < kAttnKeys ? fmaxf(fmaxf(m8[e], sv[c + e]), sv[(c + 8 + e) % kAttnKeys])
-                                      : fmaxf(m8[e], sv[c + e]);
-        float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), m8[2]), fmaxf(fmaxf(m8[3], m8[4]), m8[5]));
-        mx = fmaxf(fmaxf(mx, m8[6]), m8[7]) * sl2;
-        float alpha = 1.f;
-        if (j == 0) {
-          m_ref = mx;
-        } else if (mx > m_ref + kRescaleLog2) {
-          alpha = pf_ex2(m_ref - mx);
-          m_ref = mx;
+        for (int e = 0; e < 2; ++e) {
+          float mx = fmaxf(m4[2 * e], m4[2 * e + 1]);
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) * sl2;
+          if (j == 0) {
+            m_ref[e] = mx;
+          } else if (mx > m_ref[e] + kRescaleLog2) {
+            alpha[e] = pf_ex2(m_ref[e] - mx);
+            m_ref[e] = mx;
+          }
         }
-        if (__any_sync(0xffffffffu, alpha != 1.f)) {
+        if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f)) {
 #pragma unroll
-          for (int c = 0; c < kPfDv; c += 16) {
-            float o[16];
-            tmem_ld16(lane_base + col_o(x) + c, o);
+          for (int g = 0; g < 2; ++g) {
+            float o[32];
+            tmem_ld_16x256b_x8(lane_base + col_o(x) + 64 * g, o);
             tmem_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 16; ++e) o[e] *= alpha;
-            tmem_st16(lane_base + col_o(x) + c, o);
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o[4 * k + e] *= alpha[e >> 1];
+            tmem_st_16x256b_x8(lane_base + col_o(x) + 64 * g, o);
           }
         }
         // P_X over the first 64 columns of S_X, each half of 64 keys handed to
-        // the PV MMAs as soon as it is written
-        const float2 sl2v = make_float2(sl2, sl2), mrv = make_float2(-m_ref, -m_ref);
-        float2 r4[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        // the PV MMAs as soon as it is written (a half's P goes over columns
+        // that the warp has read)
+        const float2 sl2v = make_float2(sl2, sl2);
+        float2 rs[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float pk[kAttnKeys / 4];   // bf16 pairs, kept as 32-bit words for the TMEM store
+        for (int g = 0; g < 2; ++g) {
+          float v[32];
+          load_s(g, v);
+          uint32_t pk[16];
 #pragma unroll
-          for (int i = 0; i < kAttnKeys / 4; ++i) {
-            const int c = h * (kAttnKeys / 2) + 2 * i;
-            const float2 e = __ffma2_rn(make_float2(sv[c], sv[c + 1]), sl2v, mrv);
-            const float2 pr = make_float2(pf_ex2(e.x), pf_ex2(e.y));
-            r4[i & 3] = __fadd2_rn(r4[i & 3], pr);
-            pk[i] = __uint_as_float(pack_bf16x2(pr.x, pr.y));
-          }
+          for (int k = 0; k < 8; ++k)
 #pragma unroll
-          for (int c = 0; c < kAttnKeys / 4; c += 16)
-            tmem_st16(lane_base + col_s(x) + h * (kAttnKeys / 4) + c, *reinterpret_cast<const float(*)[16]>(&pk[c]));
+            for (int e = 0; e < 2; ++e) {
+              const float2 t = __ffma2_rn(make_float2(v[4 * k + 2 * e], v[4 * k + 2 * e + 1]), sl2v,
+                                          make_float2(-m_ref[e], -m_ref[e]));
+              const float2 pr = make_float2(pf_ex2(t.x), pf_ex2(t.y));
+              rs[e] = __fadd2_rn(rs[e], pr);
+              pk[2 * k + e] = pack_bf16x2(pr.x, pr.y);
+            }
+          tmem_st_16x128b_x8(lane_base + col_s(x) + 32 * g, pk);
           tmem_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&bars.pfull[x][h]));
+          if (lane == 0) mbar_arrive(smem_u32(&bars.pfull[x][g]));
         }
-        const float2 rs2 = __fadd2_rn(__fadd2_rn(r4[0], r4[1]), __fadd2_rn(r4[2], r4[3]));
-        l = fmaf(l, alpha, rs2.x + rs2.y);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) l[e] = fmaf(l[e], alpha[e], rs[e].x + rs[e].y);
       }
       // ---- epilogue: O_X / l of the live rows, then O_X is free for the next item
       if (ok) ok = pf_warp_wait(smem_u32(&bars.odone[x]), kx & 1, abort_flag, p.wait_ns);
       if (!ok) break;
       tc_fence_after();
-      const float inv = 1.f / l;
-      const bool live = qrow < it.L;
-      __nv_bfloat16* orow = p.out + (static_cast<size_t>(it.start + (live ? qrow : 0)) * p.H + it.h) * kPfDv;
-      float o[kPfDv];
+      float inv[2];
 #pragma unroll
-      for (int c = 0; c < kPfDv; c += 16) tmem_ld16(lane_base + col_o(x) + c, *reinterpret_cast<float(*)[16]>(&o[c]));
-      tmem_wait_ld();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars.ofree[x]));
-      if (live) {
-        uint4* d = reinterpret_cast<uint4*>(orow);
+      for (int e = 0; e < 2; ++e) {
+        float t = l[e];
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        inv[e] = 1.f / t;
+      }
 #pragma unroll
-        for (int q = 0; q < kPfDv / 8; ++q)
-          d[q] = make_uint4(pack_bf16x2(o[8 * q] * inv, o[8 * q + 1] * inv),
-                            pack_bf16x2(o[8 * q + 2] * inv, o[8 * q + 3] * inv),
-                            pack_bf16x2(o[8 * q + 4] * inv, o[8 * q + 5] * inv),
-                            pack_bf16x2(o[8 * q + 6] * inv, o[8 * q + 7] * inv));
+      for (int g = 0; g < 2; ++g) {
+        float o[32];
+        tmem_ld_16x256b_x8(lane_base + col_o(x) + 64 * g, o);
+        tmem_wait_ld();
+        if (g == 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&bars.ofree[x]));
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          if (qrow + 8 * e >= it.L) continue;
+          uint32_t* d = reinterpret_cast<uint32_t*>(
+              p.out + (static_cast<size_t>(it.start + qrow + 8 * e) * p.H + it.h) * kPfDv + 64 * g + c2);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            d[4 * k] = pack_bf16x2(o[4 * k + 2 * e] * inv[e], o[4 * k + 2 * e + 1] * inv[e]);
+        }
+        __syncwarp();
       }
       tx += nx;
       ++kx;

@@ -444,6 +444,19 @@ __device__ __forceinline__ void tmem_st_16x256b_x8(uint32_t taddr, const float (
       : "memory");
 }
 
+// 16 lanes x 32 columns of 32-bit, spread over the whole warp: thread t writes
+// lanes t/4 and t/4 + 8 at column 4k + t%4 of every 4-column group k, as
+// v[2k] = (t/4, 4k + t%4), v[2k + 1] = (t/4 + 8, 4k + t%4).  Two packed values
+// per column: what tmem_ld_16x256b_x8 gives a thread of 64 columns, in 32.
+__device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+      : "memory");
+}
+
 // one lane of a converged warp returns true
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred = 0;
