@@ -444,136 +444,183 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
   }
 }
 
-// ------------------------------------------------------------------ combine, fp32
-// Block per (head h, group of kCombineGroup sequences; blockIdx.y: a part of the
-// d_v output rows, each part repeating the merge), 256 threads: the
-// sequences of a group share one pass over W_UV,h.  The splits that covered
-// sequence b are the CTAs c0..c1 of the page schedule; their partials sit in
-// slots c + b.  M = max_s m_s; o = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M)
-// l_s (m in log2 units); then u = W_UV,h o.  A sequence of length 0 gets
-// u = 0.
-//  - weights: warp j takes sequence b0 + j, its lanes the slots: M, then
-//    2^(m_s - M) into shared memory, kCombineSlots at a time, and the
-//    denominator;
-//  - merge: thread t takes (sequence, 4 features) pairs t, t + 256, ..: up to
-//    four pairs and four slots of each in flight, so that the time is a few
-//    round trips whatever the number of slots (a warp per sequence, one slot
-//    after another, took 60 us of an fp32 step of 8 sequences of 100 to 3000
-//    tokens, up to 47 slots each; 15 us now: ncu, cold caches);
-//  - u: warp w takes groups of four W_UV,h rows; a lane loads its 16-byte
-//    pieces of the four rows once and multiplies them into all the group's
-//    merged vectors (shared memory), then the 32 sums (sequence, row) are
-//    reduced across the lanes by a transposing butterfly (31 shuffles), after
-//    which lane t holds sequence t / 4, row t % 4.
-constexpr int kCombineThreads = 256;
-constexpr int kCombineGroup = 8;        // sequences per block (one warp each for the weights)
-constexpr int kCombineMaxDc = 512;
-constexpr int kCombineBlocks = 304;     // two blocks per SM
-constexpr int kCombineSlots = 128;      // slots whose weights are in shared memory at a time
-constexpr int kCombinePairs = kCombineGroup * kCombineMaxDc / 4 / kCombineThreads;   // pairs per thread, at most
+// ------------------------------------------------------------------ merge of the split partials
+// For head h and the sequences b0 .. b0 + nt - 1 of a block of T threads: the
+// splits that covered sequence b are the CTAs c0..c1 of the page schedule, their
+// partials sit in slots c + b, and with M = max_s m_s (log2 units)
+//   o = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s,
+// 0 for a sequence of length 0.
+//  - weights: a warp takes a sequence, its lanes the slots: M, then 2^(m_s - M)
+//    into shared memory, kCombineSlots at a time, and the denominator;
+//  - sums: thread t takes (sequence, 4 features) pairs t, t + T, .. (PPT of them
+//    at most), with several slots of each in flight; where the block has fewer
+//    pairs than threads, the slots are dealt to groups of threads whose sums are
+//    added in group order.  The time is then a few round trips to L2 whatever
+//    the number of slots.
+// emit(j, f, o) is called for features f .. f + 3 of sequence b0 + j, by one
+// thread; the caller's next __syncthreads makes what it stored visible.
+constexpr int kCombineSlots = 128;
+constexpr int kMergeMaxSeq = 16;         // sequences per block, at most
+constexpr int kMergeBlocks = 152;        // blocks wanted at most: one per SM
 
-__global__ void __launch_bounds__(kCombineThreads)
-combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml, const float* __restrict__ part_o,
-               const float* __restrict__ w_uv, float* __restrict__ out, int batch, int H, int d_c, int d_v,
-               int num_splits) {
-  __shared__ __align__(16) float olat[kCombineGroup][kCombineMaxDc];
-  __shared__ float wts[kCombineGroup][kCombineSlots];
-  __shared__ float inv_l[kCombineGroup];
-  __shared__ int slots_s[kCombineGroup], slot0_s[kCombineGroup];
-  const int h = blockIdx.x % H, b0 = (blockIdx.x / H) * kCombineGroup;
-  const int nb = min(kCombineGroup, batch - b0);
+template <int T>
+struct MergeShared {
+  float wts[kMergeMaxSeq][kCombineSlots];
+  float inv_l[kMergeMaxSeq];
+  int slots[kMergeMaxSeq], slot0[kMergeMaxSeq];
+  float4 red[T];
+};
+
+// the fewest sequences per block (a power of two up to `most`) that leave at most
+// one block per SM
+int merge_group(int H, int batch, int most) {
+  int nt = 1;
+  while (nt < most && H * ((batch + nt - 1) / nt) > kMergeBlocks) nt *= 2;
+  return nt;
+}
+
+template <int PPT, int T, int TS, typename Emit>
+__device__ void merge_partials(MergeShared<TS>& sh, const int32_t* cu, const float* part_ml, const float* part_o,
+                               int batch, int H, int h, int b0, int nt, int d_c, int num_splits, Emit emit) {
+  static_assert(T <= TS, "threads");
+  constexpr int kFlight = PPT >= 4 ? 4 : 8;   // slots of a pair in flight
+  constexpr int kWarps = T / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kWarps = kCombineThreads / 32;
-  grid_dependency_wait();
-  const int total = cu[batch];
-  const int chunk = split_chunk(total, num_splits);
+  const int nb = min(nt, batch - b0), ncol = d_c / 4, pairs = nt * ncol;
+  const int chunk = split_chunk(cu[batch], num_splits);
   const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
-  // the slots of sequence b0 + warp and their maximum
-  int n = 0, c0 = 0;
-  float M = -INFINITY, lsum = 0.f;
-  const float* pml = part_ml;
-  if (warp < nb) {
-    const int b = b0 + warp;
-    const int p0 = cu[b] + kSegCost, p1 = cu[b + 1];   // units of the sequence's pages
-    c0 = p0 / chunk;
-    n = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
-    pml += (static_cast<size_t>(c0 + b) * H + h) * 2;
-    for (int k = lane; k < n; k += 32) M = fmaxf(M, pml[k * mlstride]);
+  // the slots of this warp's sequences (warp, warp + kWarps) and their maxima
+  int n[2] = {0, 0};
+  float M[2] = {-INFINITY, -INFINITY}, lsum[2] = {0.f, 0.f};
+  const float* pml[2] = {part_ml, part_ml};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  for (int e = 0; e < 2; ++e) {
+    const int j = warp + kWarps * e;
+    if (j >= nb) continue;
+    const int b = b0 + j, p0 = cu[b] + kSegCost, p1 = cu[b + 1], c0 = p0 / chunk;   // units of the sequence's pages
+    n[e] = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
+    pml[e] += (static_cast<size_t>(c0 + b) * H + h) * 2;
+    if (lane == 0) {
+      sh.slots[j] = n[e];
+      sh.slot0[j] = c0 + b;
+    }
+    for (int k = lane; k < n[e]; k += 32) M[e] = fmaxf(M[e], pml[e][k * mlstride]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M[e] = fmaxf(M[e], __shfl_xor_sync(0xffffffffu, M[e], o));
   }
-  if (warp < kCombineGroup && lane == 0) {
-    slots_s[warp] = n;
-    slot0_s[warp] = c0 + b0 + warp;
-  }
-  // this thread's (sequence, 4 features) pairs
-  const int ncol = d_c / 4;
-  int pj[kCombinePairs];
-  const float* po[kCombinePairs];
-  float4 acc4[kCombinePairs];
-  int nmax = 0;   // slots of the group's longest sequence
+  // this thread's pairs, and its group where the slots are dealt out
+  const int groups = pairs < T ? T / pairs : 1;
+  const int grp = groups > 1 ? tid / pairs : 0;
+  int pj[PPT], pf[PPT];
+  const float* po[PPT];
+  float4 acc[PPT];
   __syncthreads();
+  int nmax = 0;
+  for (int j = 0; j < nb; ++j) nmax = max(nmax, sh.slots[j]);
 #pragma unroll
-  for (int j = 0; j < kCombineGroup; ++j) nmax = max(nmax, slots_s[j]);
-#pragma unroll
-  for (int u = 0; u < kCombinePairs; ++u) {
-    const int i = tid + u * kCombineThreads, j = i / ncol, f = 4 * (i - j * ncol);
-    pj[u] = j < nb ? j : -1;
-    acc4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    po[u] = part_o + (static_cast<size_t>(j < nb ? slot0_s[j] : 0) * H + h) * d_c + f;
+  for (int u = 0; u < PPT; ++u) {
+    const int i = groups > 1 ? tid - grp * pairs : tid + u * T;
+    const int j = i / ncol;
+    const bool live = grp < groups && j < nb && (groups == 1 || u == 0);
+    pj[u] = live ? j : -1;
+    pf[u] = 4 * (i - j * ncol);
+    acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    po[u] = part_o + (static_cast<size_t>(live ? sh.slot0[j] : 0) * H + h) * d_c + pf[u];
   }
   for (int k0 = 0; k0 < nmax; k0 += kCombineSlots) {
-    if (warp < nb) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = warp + kWarps * e;
+      if (j >= nb) continue;
       for (int k = lane; k < kCombineSlots; k += 32) {
         float wk = 0.f;
-        if (k0 + k < n) {
-          const float2 ml = *reinterpret_cast<const float2*>(pml + (k0 + k) * mlstride);
-          wk = exp2f(ml.x - M);
-          lsum = fmaf(wk, ml.y, lsum);
+        if (k0 + k < n[e]) {
+          const float2 ml = *reinterpret_cast<const float2*>(pml[e] + (k0 + k) * mlstride);
+          wk = exp2f(ml.x - M[e]);
+          lsum[e] = fmaf(wk, ml.y, lsum[e]);
         }
-        wts[warp][k] = wk;
+        sh.wts[j][k] = wk;
       }
     }
     __syncthreads();
     const int kn = min(kCombineSlots, nmax - k0);
-    for (int k = 0; k < kn; k += 4) {
-      float4 v[kCombinePairs][4];
+    for (int k = grp; k < kn; k += groups * kFlight) {
+      float4 v[PPT][kFlight];
 #pragma unroll
-      for (int u = 0; u < kCombinePairs; ++u)
+      for (int u = 0; u < PPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < kFlight; ++e) {
+          const int kk = k + e * groups;
           v[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (pj[u] >= 0 && k0 + k + e < slots_s[pj[u]])
-            v[u][e] = *reinterpret_cast<const float4*>(po[u] + (k0 + k + e) * sstride);
+          if (pj[u] >= 0 && kk < kn && k0 + kk < sh.slots[pj[u]])
+            v[u][e] = *reinterpret_cast<const float4*>(po[u] + (k0 + kk) * sstride);
         }
 #pragma unroll
-      for (int u = 0; u < kCombinePairs; ++u)
+      for (int u = 0; u < PPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float w = pj[u] >= 0 ? wts[pj[u]][k + e] : 0.f;   // 0 past the sequence's slots
-          acc4[u].x = fmaf(w, v[u][e].x, acc4[u].x);
-          acc4[u].y = fmaf(w, v[u][e].y, acc4[u].y);
-          acc4[u].z = fmaf(w, v[u][e].z, acc4[u].z);
-          acc4[u].w = fmaf(w, v[u][e].w, acc4[u].w);
+        for (int e = 0; e < kFlight; ++e) {
+          const int kk = k + e * groups;
+          const float w = pj[u] >= 0 && kk < kn ? sh.wts[pj[u]][kk] : 0.f;   // 0 past the sequence's slots
+          acc[u].x = fmaf(w, v[u][e].x, acc[u].x);
+          acc[u].y = fmaf(w, v[u][e].y, acc[u].y);
+          acc[u].z = fmaf(w, v[u][e].z, acc[u].z);
+          acc[u].w = fmaf(w, v[u][e].w, acc[u].w);
         }
     }
     __syncthreads();   // the weights are read: the next slots' may overwrite them
   }
-  if (warp < nb) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) inv_l[warp] = n > 0 ? 1.f / lsum : 0.f;
+  for (int e = 0; e < 2; ++e) {
+    const int j = warp + kWarps * e;
+    if (j >= nb) continue;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lsum[e] += __shfl_xor_sync(0xffffffffu, lsum[e], o);
+    if (lane == 0) sh.inv_l[j] = n[e] > 0 ? 1.f / lsum[e] : 0.f;
   }
+  if (groups > 1) sh.red[tid] = acc[0];
   __syncthreads();
 #pragma unroll
-  for (int u = 0; u < kCombinePairs; ++u) {
-    const int i = tid + u * kCombineThreads;
-    if (pj[u] >= 0) {
-      const float il = inv_l[pj[u]];
-      *reinterpret_cast<float4*>(&olat[pj[u]][4 * (i - pj[u] * ncol)]) =
-          make_float4(acc4[u].x * il, acc4[u].y * il, acc4[u].z * il, acc4[u].w * il);
+  for (int u = 0; u < PPT; ++u) {
+    if (pj[u] < 0 || grp > 0) continue;
+    float4 a = acc[u];
+    for (int g = 1; g < groups; ++g) {
+      const float4 r = sh.red[tid + g * pairs];
+      a = make_float4(a.x + r.x, a.y + r.y, a.z + r.z, a.w + r.w);
     }
+    const float il = sh.inv_l[pj[u]];
+    emit(pj[u], pf[u], make_float4(a.x * il, a.y * il, a.z * il, a.w * il));
   }
+}
+
+// ------------------------------------------------------------------ combine, fp32
+// Block per (head h, `nt` sequences; blockIdx.y: a part of the d_v output rows,
+// each part repeating the merge), 256 threads: the merge, then u = W_UV,h o: warp
+// w takes groups of four W_UV,h rows; a lane loads its 16-byte pieces of the four
+// rows once and multiplies them into all the group's merged vectors (shared
+// memory), then the 32 sums (sequence, row) are reduced across the lanes by a
+// transposing butterfly (31 shuffles), after which lane t holds sequence t / 4,
+// row t % 4.  8 sequences of 100 to 3000 tokens (up to 47 slots each) took 60 us
+// with a warp per sequence, one slot after another; 10 us now (ncu, cold
+// caches).
+constexpr int kCombineThreads = 256;
+constexpr int kCombineGroup = 8;        // sequences per block, at most
+constexpr int kCombineMaxDc = 512;
+constexpr int kCombineBlocks = 304;     // two blocks per SM
+
+template <int PPT>
+__global__ void __launch_bounds__(kCombineThreads)
+combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml, const float* __restrict__ part_o,
+               const float* __restrict__ w_uv, float* __restrict__ out, int batch, int H, int d_c, int d_v,
+               int num_splits, int nt) {
+  __shared__ __align__(16) float olat[kCombineGroup][kCombineMaxDc];
+  __shared__ __align__(16) MergeShared<kCombineThreads> sh;
+  const int h = blockIdx.x % H, b0 = (blockIdx.x / H) * nt;
+  const int nb = min(nt, batch - b0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kCombineThreads / 32;
+  grid_dependency_wait();
+  merge_partials<PPT, kCombineThreads>(sh, cu, part_ml, part_o, batch, H, h, b0, nt, d_c, num_splits,
+                                       [&](int j, int f, const float4& o) { *reinterpret_cast<float4*>(&olat[j][f]) = o; });
   __syncthreads();
   // u[j][v] = sum_f W_UV[h][v][f] olat[j][f]
   constexpr int VEC = 4;
@@ -641,18 +688,13 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
 // launch it needs cost that step 8 us more), and 8 us against 18 on CUDA cores
 // with d_c 512 (kernel alone, warm).
 constexpr int kCtMaxThreads = 512;
-constexpr int kCtMaxSeq = 16;            // sequences per block, at most
-constexpr int kCtBlocks = 152;           // one per SM
 constexpr uint32_t kCtAtom = 128 * 128;  // 128 rows x 64 bf16
 
 // the N operand's rows: three per sequence, a multiple of the MMA's 16
 __host__ __device__ constexpr int ct_cols(int nt) { return (3 * nt + 15) / 16 * 16; }
 
 struct CtShared {
-  float wts[kCtMaxSeq][kCombineSlots];
-  float inv_l[kCtMaxSeq];
-  int slots[kCtMaxSeq], slot0[kCtMaxSeq];
-  float4 red[kCtMaxThreads];
+  MergeShared<kCtMaxThreads> merge;
   uint64_t afull, done;
   uint32_t tmem_base;
   int abort;
@@ -671,18 +713,16 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
                   const float* __restrict__ part_ml, const float* __restrict__ part_o, __nv_bfloat16* __restrict__ out,
                   int batch, int d_c, int d_v, int num_splits, int nt, int early, uint64_t wait_ns, int32_t* status) {
   constexpr int H = 16;
-  constexpr int kFlight = PPT >= 4 ? 4 : 8;   // slots of a pair in flight
   extern __shared__ uint8_t ct_raw[];
   uint8_t* smem = ct_raw + ((1024u - (smem_u32(ct_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
-  const int nkc = d_c / 64, cols = ct_cols(nt), ncol = d_c / 4, pairs = nt * ncol;
+  const int nkc = d_c / 64, cols = ct_cols(nt);
   const uint32_t o_off = static_cast<uint32_t>(nkc) * kCtAtom, o_chunk = static_cast<uint32_t>(cols) * 128;
   CtShared& sh = *reinterpret_cast<CtShared*>(smem + o_off + nkc * o_chunk);
   volatile int* abort_flag = &sh.abort;
   const int h = blockIdx.x % H, b0 = (blockIdx.x / H) * nt, v0 = blockIdx.y * 128;
   const int nb = min(nt, batch - b0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kWarps = kCtThreads / 32;
   if (tid == 0) {
     mbar_init(smem_u32(&sh.afull), 1);
     mbar_init(smem_u32(&sh.done), 1);
@@ -700,114 +740,15 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
     tmem_relinquish();
   }
   grid_dependency_wait();
-  const int chunk = split_chunk(cu[batch], num_splits);
-  const size_t mlstride = static_cast<size_t>(H) * 2, sstride = static_cast<size_t>(H) * d_c;
-  // the slots of this warp's sequences (warp, warp + 8) and their maxima
-  int n[2] = {0, 0};
-  float M[2] = {-INFINITY, -INFINITY}, lsum[2] = {0.f, 0.f};
-  const float* pml[2] = {part_ml, part_ml};
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int j = warp + kWarps * e;
-    if (j >= nb) continue;
-    const int b = b0 + j, p0 = cu[b] + kSegCost, p1 = cu[b + 1], c0 = p0 / chunk;   // units of the sequence's pages
-    n[e] = p1 > p0 ? (p1 - 1) / chunk - c0 + 1 : 0;
-    pml[e] += (static_cast<size_t>(c0 + b) * H + h) * 2;
-    if (lane == 0) {
-      sh.slots[j] = n[e];
-      sh.slot0[j] = c0 + b;
-    }
-    for (int k = lane; k < n[e]; k += 32) M[e] = fmaxf(M[e], pml[e][k * mlstride]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M[e] = fmaxf(M[e], __shfl_xor_sync(0xffffffffu, M[e], o));
-  }
-  // this thread's pairs, and its group where the slots are dealt out
-  const int groups = pairs < kCtThreads ? kCtThreads / pairs : 1;
-  const int grp = groups > 1 ? tid / pairs : 0;
-  int pj[PPT], pf[PPT];
-  const float* po[PPT];
-  float4 acc[PPT];
-  __syncthreads();
-  int nmax = 0;
-  for (int j = 0; j < nb; ++j) nmax = max(nmax, sh.slots[j]);
-#pragma unroll
-  for (int u = 0; u < PPT; ++u) {
-    const int i = groups > 1 ? tid - grp * pairs : tid + u * kCtThreads;
-    const int j = i / ncol;
-    const bool live = grp < groups && j < nb && (groups == 1 || u == 0);
-    pj[u] = live ? j : -1;
-    pf[u] = 4 * (i - j * ncol);
-    acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-    po[u] = part_o + (static_cast<size_t>(live ? sh.slot0[j] : 0) * H + h) * d_c + pf[u];
-  }
-  for (int k0 = 0; k0 < nmax; k0 += kCombineSlots) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int j = warp + kWarps * e;
-      if (j >= nb) continue;
-      for (int k = lane; k < kCombineSlots; k += 32) {
-        float wk = 0.f;
-        if (k0 + k < n[e]) {
-          const float2 ml = *reinterpret_cast<const float2*>(pml[e] + (k0 + k) * mlstride);
-          wk = exp2f(ml.x - M[e]);
-          lsum[e] = fmaf(wk, ml.y, lsum[e]);
-        }
-        sh.wts[j][k] = wk;
-      }
-    }
-    __syncthreads();
-    const int kn = min(kCombineSlots, nmax - k0);
-    for (int k = grp; k < kn; k += groups * kFlight) {
-      float4 v[PPT][kFlight];
-#pragma unroll
-      for (int u = 0; u < PPT; ++u)
-#pragma unroll
-        for (int e = 0; e < kFlight; ++e) {
-          const int kk = k + e * groups;
-          v[u][e] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (pj[u] >= 0 && kk < kn && k0 + kk < sh.slots[pj[u]])
-            v[u][e] = *reinterpret_cast<const float4*>(po[u] + (k0 + kk) * sstride);
-        }
-#pragma unroll
-      for (int u = 0; u < PPT; ++u)
-#pragma unroll
-        for (int e = 0; e < kFlight; ++e) {
-          const int kk = k + e * groups;
-          const float w = pj[u] >= 0 && kk < kn ? sh.wts[pj[u]][kk] : 0.f;   // 0 past the sequence's slots
-          acc[u].x = fmaf(w, v[u][e].x, acc[u].x);
-          acc[u].y = fmaf(w, v[u][e].y, acc[u].y);
-          acc[u].z = fmaf(w, v[u][e].z, acc[u].z);
-          acc[u].w = fmaf(w, v[u][e].w, acc[u].w);
-        }
-    }
-    __syncthreads();   // the weights are read: the next slots' may overwrite them
-  }
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const int j = warp + kWarps * e;
-    if (j >= nb) continue;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lsum[e] += __shfl_xor_sync(0xffffffffu, lsum[e], o);
-    if (lane == 0) sh.inv_l[j] = n[e] > 0 ? 1.f / lsum[e] : 0.f;
-  }
-  if (groups > 1) sh.red[tid] = acc[0];
-  __syncthreads();
   // the merged vectors as three bf16 pieces, rows j, nt + j and 2 nt + j of the N
   // operand (K-major, 128-byte swizzle)
-#pragma unroll
-  for (int u = 0; u < PPT; ++u) {
-    if (pj[u] < 0 || grp > 0) continue;
-    float4 a = acc[u];
-    for (int g = 1; g < groups; ++g) {
-      const float4 r = sh.red[tid + g * pairs];
-      a = make_float4(a.x + r.x, a.y + r.y, a.z + r.z, a.w + r.w);
-    }
-    const float il = sh.inv_l[pj[u]];
-    float x[4] = {a.x * il, a.y * il, a.z * il, a.w * il};
-    const int kc = pf[u] / 64, unit = (pf[u] % 64) / 8;
+  merge_partials<PPT, kCtThreads>(sh.merge, cu, part_ml, part_o, batch, H, h, b0, nt, d_c, num_splits,
+                                  [&](int j, int f, const float4& o) {
+    float x[4] = {o.x, o.y, o.z, o.w};
+    const int kc = f / 64, unit = (f % 64) / 8;
 #pragma unroll
     for (int piece = 0; piece < 3; ++piece) {
-      const int row = piece * nt + pj[u];
+      const int row = piece * nt + j;
       uint32_t w[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -817,10 +758,10 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
         x[2 * e] -= zf.x;
         x[2 * e + 1] -= zf.y;
       }
-      *reinterpret_cast<uint2*>(smem + o_off + kc * o_chunk + row * 128 + ((unit ^ (row & 7)) << 4) + (pf[u] & 4) * 2) =
+      *reinterpret_cast<uint2*>(smem + o_off + kc * o_chunk + row * 128 + ((unit ^ (row & 7)) << 4) + (f & 4) * 2) =
           make_uint2(w[0], w[1]);
     }
-  }
+  });
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -1249,9 +1190,7 @@ cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, const CUtensorMap*
   const float* ml = reinterpret_cast<const float*>(ws + wl.off_ml);
   const float* po = reinterpret_cast<const float*>(ws + wl.off_o);
   if (tc_path) {
-    // the fewest sequences per block that leave one block per SM
-    int nt = 1;
-    while (nt < kCtMaxSeq && 16 * ((a.batch + nt - 1) / nt) > kCtBlocks) nt *= 2;
+    const int nt = merge_group(16, a.batch, kMergeMaxSeq);
     const int pairs = nt * (a.d_c / 4);
     if (pairs <= 256) return launch_combine_tc<1, 256>(a, wmap, cu, ml, po, nt, st);
     if (pairs <= 512) return launch_combine_tc<1, 512>(a, wmap, cu, ml, po, nt, st);
@@ -1260,12 +1199,18 @@ cudaError_t launch_combine(const DecodeArgs& a, bool tc_path, const CUtensorMap*
   }
   // small batches: the output rows spread over more blocks (a pass of the block's
   // warps covers 32 rows), so that most SMs read a part of W_UV
-  const int groups = a.H * ((a.batch + kCombineGroup - 1) / kCombineGroup), passes = (a.d_v + 31) / 32;
+  const int nt = merge_group(a.H, a.batch, kCombineGroup), pairs = nt * (a.d_c / 4);
+  const int groups = a.H * ((a.batch + nt - 1) / nt), passes = (a.d_v + 31) / 32;
   int parts = kCombineBlocks / groups;
   parts = parts < 1 ? 1 : parts > passes ? passes : parts;
-  return launch_chained(combine_kernel, dim3(groups, parts), dim3(kCombineThreads), 0, st, cu, ml, po,
-                        static_cast<const float*>(a.w_uv), static_cast<float*>(a.out), a.batch, a.H, a.d_c, a.d_v,
-                        a.num_splits);
+  auto launch = [&](auto kernel) {
+    return launch_chained(kernel, dim3(groups, parts), dim3(kCombineThreads), 0, st, cu, ml, po,
+                          static_cast<const float*>(a.w_uv), static_cast<float*>(a.out), a.batch, a.H, a.d_c, a.d_v,
+                          a.num_splits, nt);
+  };
+  if (pairs <= kCombineThreads) return launch(combine_kernel<1>);
+  if (pairs <= 2 * kCombineThreads) return launch(combine_kernel<2>);
+  return launch(combine_kernel<4>);
 }
 
 }  // namespace egmla
