@@ -199,7 +199,8 @@ int eg_mla_layer_decode(const eg_mla_dims* dims, const eg_mla_layer_dims* layer,
                               st) != cudaSuccess)
     return EG_MLA_ERR_CUDA;
   if (egmla::launch_chained(
-      layer_qkv_kernel, dim3(batch, kQkvParts + (do_kv ? 1 : 0)), dim3(kQkvThreads), 0, st, static_cast<const float*>(qkv32), positions,
+      layer_qkv_kernel, dim3(batch, kQkvParts + (do_kv ? 1 : 0)), dim3(kQkvThreads), 0, st,
+      static_cast<const float*>(qkv32), positions,
       static_cast<const __nv_bfloat16*>(wt->kv_norm_w), H, dims->d_nope, dims->d_rope, dims->d_c, freqs, eps,
       qb, cb, krb) != cudaSuccess)
     return EG_MLA_ERR_CUDA;

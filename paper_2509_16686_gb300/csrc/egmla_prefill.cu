@@ -15,10 +15,11 @@
 //                        attention's launch order) and zeroes the attention's
 //                        work counter.
 //   prefill_kv_kernel    (tcgen05) [k^C_h ; v^C_h] = [W_UK,h ; W_UV,h] c~ for
-//                        128 tokens per CTA (RT = 1; RT = 2 row tiles share each
-//                        weight chunk in the gate-table mode) and every head h
-//                        (Eqs. 2 and 6): per output block of 128 columns (the
-//                        key or the value rows of a head) M = 128 tokens per
+//                        every token and head h (Eqs. 2 and 6), in units of a
+//                        tile of 128 tokens (RT = 1; RT = 2 row tiles share each
+//                        weight chunk in the gate-table mode) and an output block
+//                        of 128 columns (the key or the value rows of a head),
+//                        shared equally by one CTA per SM: M = 128 tokens per
 //                        row tile, N = 128, K = d_c; two TMEM accumulators so
 //                        the epilogue of one block overlaps the MMAs of the
 //                        next; the output leaves through TMA tensor stores.
