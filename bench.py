@@ -178,12 +178,19 @@ def max_over_ranks(ms, dist, device):
     return float(t.item())
 
 
-def algorithmic_bytes(case, cache_bytes):
+def combine_fused(d, batch, splits, sms):
+    """Whether the decode kernel merges the splits and applies W_UV itself (bf16,
+    d_c 192/256, a grid of at most one CTA per SM with a CTA for every sequence
+    and head) or leaves that to the combine kernel after it."""
+    return d.dtype == "bf16" and d.d_c in (192, 256) and splits <= sms and 16 * batch <= splits
+
+
+def algorithmic_bytes(case, cache_bytes, fused):
     """Bytes one decode launch must move at least: the latent-cache stream
     (c^KV, k^R and the token id of every cached token), each distinct gate row
     G[id] once (the ids of the cached tokens after the step's append), and
-    W_UV of every head.  Queries, outputs, split partials and LayerNorm
-    parameters (under 1 % here) are left out."""
+    W_UV of every head where the kernel applies it (`fused`).  Queries, outputs,
+    split partials and LayerNorm parameters (under 1 % here) are left out."""
     d = case.dims
     elem = 2 if d.dtype == "bf16" else 4
     gate_rows = 0
@@ -198,7 +205,7 @@ def algorithmic_bytes(case, cache_bytes):
             ids.append(case.id_pool[pages].reshape(-1)[:L - 1])
             ids.append(case.ids_new[b:b + 1])
         gate_rows = int(np.unique(np.concatenate(ids)).size) * d.d_c * elem if ids else 0
-    w_uv = d.num_heads * d.d_v * d.d_c * elem
+    w_uv = d.num_heads * d.d_v * d.d_c * elem if fused else 0
     return {"cache": int(cache_bytes), "gate_rows_unique": gate_rows, "w_uv": w_uv,
             "total": int(cache_bytes) + gate_rows + w_uv}
 
@@ -483,7 +490,9 @@ def run_gpu_full_layers(args, workload, torch, dist, ws, rank):
     stream = torch.cuda.Stream()
     tokens_cached = int(case.seq_lens.astype(np.int64).sum())
     cache_bytes = tokens_cached * ((d.d_c + d.d_rope) * 2 + 4)
-    algo = algorithmic_bytes(case, cache_bytes)
+    splits = _lib.eg_mla_default_num_splits()   # one per SM
+    fused = combine_fused(d, B, splits, splits)
+    algo = algorithmic_bytes(case, cache_bytes, fused)
     splits = base.dc.num_splits or _lib.eg_mla_default_num_splits()
 
     def run_step():
@@ -598,8 +607,10 @@ def run_gpu_full_layers(args, workload, torch, dist, ws, rank):
                 "d2h_bytes_per_step": d2h},
         # this library's kernels per layer: the query/latent projection,
         # kv_norm + RoPE, query absorption (with the append in its grid in the
-        # first layer of a group), decode, the output projection
-        "gpu_launches": steps_arg * n_layers * 5,
+        # first layer of a group), decode, its split combine (a kernel of its
+        # own for more sequences than a sixteenth of the splits), the output
+        # projection
+        "gpu_launches": steps_arg * n_layers * (5 if fused else 6),
         "clocks": clk.summary(),
     }
 
@@ -698,7 +709,8 @@ def mla_baseline(case, torch, stream, peak, steps=600):
     k_ms = ms_sum / max(1, n_l)
     tokens = int(case.seq_lens.astype(np.int64).sum())
     kvb = (d.d_c + d.d_rope) * (2 if d.dtype == "bf16" else 4)
-    algo = algorithmic_bytes(mcase, tokens * kvb)
+    splits = _lib.eg_mla_default_num_splits()   # one per SM
+    algo = algorithmic_bytes(mcase, tokens * kvb, combine_fused(mcase.dims, mcase.batch, splits, splits))
     achieved = algo["total"] / (k_ms * 1e-3) / 1e9
     del units, graph
     torch.cuda.empty_cache()
@@ -987,15 +999,14 @@ def run_gpu(args, workload, torch, dist, ws, rank):
     elem = 2 if d.dtype == "bf16" else 4
     id_bytes = 4 if d.gate else 0
     cache_bytes = tokens_cached * ((d.d_c + d.d_rope) * elem + id_bytes)     # per unit (layer)
-    # algorithmic bytes of one decode launch: the cache stream, each distinct
-    # gate row once, and W_UV of every head
-    algo = algorithmic_bytes(case, cache_bytes)
     splits = units[0].num_splits or _lib.eg_mla_default_num_splits()
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    # bf16: query absorption (with the append in its grid) + decode, + the
-    # combine kernel unless the decode kernel runs fused (d_c 192/256, a grid
-    # of at most one CTA per SM); fp32: append + decode + combine
-    fused = d.dtype == "bf16" and d.d_c in (192, 256) and splits <= sms
+    # query absorption (with the append in its grid) + decode, + the combine
+    # kernel unless the decode kernel runs fused
+    fused = combine_fused(d, B, splits, sms)
+    # algorithmic bytes of one decode launch: the cache stream, each distinct
+    # gate row once, and W_UV of every head where the kernel applies it
+    algo = algorithmic_bytes(case, cache_bytes, fused)
     launches_per_step = n_layers * ((2 if fused else 3) if d.dtype == "bf16" else 3)
     if workload.endswith("_embed"):
         launches_per_step += n_layers
