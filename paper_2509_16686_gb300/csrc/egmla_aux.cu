@@ -677,8 +677,9 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
 //    then thread t takes (sequence, 4 features) pairs; where the block has fewer
 //    pairs than threads, the slots are dealt to groups of threads whose sums
 //    are added in group order;
-//  - the merged fp32 vector is split into three bf16 pieces (o = o1 + o2 + o3 to
-//    2^-24 |o|), which become three columns of the N operand, so that
+//  - the merged fp32 vector is split into three bf16 pieces, its significand's
+//    three bytes (o = o1 + o2 + o3 exactly; an infinite or NaN o is its first
+//    piece), which become three columns of the N operand, so that
 //    u = W_UV,h o1 + W_UV,h o2 + W_UV,h o3 keeps the fp32 value of o (the weights
 //    are bf16 as stored), accumulated in fp32;
 //  - u: lanes are output rows; a sequence's three columns are added, rounded to
@@ -753,11 +754,13 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
       uint32_t w[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const __nv_bfloat162 z = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
-        w[e] = *reinterpret_cast<const uint32_t*>(&z);
-        const float2 zf = __bfloat1622float2(z);
-        x[2 * e] -= zf.x;
-        x[2 * e + 1] -= zf.y;
+        const uint32_t lo = __float_as_uint(x[2 * e]), hi = __float_as_uint(x[2 * e + 1]);
+        w[e] = __byte_perm(lo, hi, 0x7632);   // the upper halves
+#pragma unroll
+        for (int k = 2 * e; k < 2 * e + 2; ++k) {
+          const float rest = x[k] - __uint_as_float(__float_as_uint(x[k]) & 0xffff0000u);
+          x[k] = fabsf(x[k]) < INFINITY ? rest : 0.f;
+        }
       }
       *reinterpret_cast<uint2*>(smem + o_off + kc * o_chunk + row * 128 + ((unit ^ (row & 7)) << 4) + (f & 4) * 2) =
           make_uint2(w[0], w[1]);

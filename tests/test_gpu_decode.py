@@ -123,6 +123,26 @@ def test_bf16_split_combine_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_v, s
     assert (got[1] == 0).all()
 
 
+@pytest.mark.parametrize("d_c", [192, 256, 512])
+def test_bf16_split_combine_keeps_infinities(gpu_lib, d_c):
+    """A latent feature whose weighted sum overflows fp32 (q = 0: every weight 1)
+    gives outputs of W_UV's sign times infinity in its own sequence, and leaves
+    the other sequences of the block as they are."""
+    dims = synth.dims_bf16(d_c=d_c, vocab=300, gate=False)
+    case = synth.make_case("overflow", dims, [140 + b for b in range(20)], seed=37, latent_scale=0.5,
+                           layout="permuted")
+    case.q[:] = 0
+    f, big = 70, orc.to_bf16_bits(np.array([3e38]))[0]
+    case.c_pool[case.block_table[0], :, f] = big
+    case.c_new[0, f] = big
+    case.w_uv[0, :, f] |= 0x3C00   # no zeros
+    _, got = run(case, 0)
+    w = orc.widen(case.w_uv, "bf16")[0, :, f]
+    np.testing.assert_array_equal(got[0, 0], np.sign(w) * np.inf)
+    ref = orc.decode_unabsorbed(case)
+    check_bf16(got[1:], ref[1:], f"d_c={d_c}")
+
+
 @pytest.mark.parametrize("splits", [1, 3, 0])
 def test_bf16_half_page_tiles_match_oracle(gpu_lib, splits):
     """d_c 512 walks its pages in halves of 32 tokens: sequences that end in a
