@@ -649,12 +649,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   phase_mark<DBG == 2>(p, 0);
-  // inside a layer the kernel after this one (the split combine, or the output
-  // projection where the combine is fused) may take each SM this one leaves,
-  // so that the projection's weights stream early; elsewhere an early combine
-  // would crowd its blocks onto the first SMs to free up (128 ragged sequences
-  // 69.8 us instead of 68.2)
-  if (p.early) grid_launch_dependents();
+  // a fused launch inside a layer lets the output projection take each SM this
+  // kernel leaves, so that its weights stream early
+  if (p.early && p.fuse) grid_launch_dependents();
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NS; ++s) {
@@ -759,6 +756,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       ++it;
     }
     if (lane == 0) {
+      // The split combine may take its place once every CTA's last page is
+      // requested, a few microseconds before this kernel ends (at the start it
+      // would crowd its blocks onto the first SMs to free up: 128 ragged
+      // sequences 69.8 us against 68.2).  128 at d_c 512 119.7 -> 118.5 us, 32 x
+      // 4K 37.7 -> 37.2, 64 x 8K layer 102.4 -> 101.5 (against a trigger at the
+      // start), at d_c 192 91.3 -> 90.8; outside layers d_c 192 lost (67.7 ->
+      // 67.9, 32 x 4K 33.7 -> 33.9).
+      if (!p.fuse && (D_C > 192 || p.early)) grid_launch_dependents();
       // drain: every copy this thread issued must land before the CTA exits,
       // also after an abort (own flag: the wait is bounded but not cut short)
       volatile int own = 0;
