@@ -57,6 +57,11 @@ __device__ void append_row(const AppendArgs& a, int b, int thr, int nthr) {
 __global__ void append_latent_kernel(const AppendArgs a) { append_row(a, blockIdx.x, threadIdx.x, blockDim.x); }
 
 // ------------------------------------------------------------------ helpers
+// brings the 128-byte line of p into L2
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(p)));
+}
+
 // v[i] (i < 32) summed over the warp; lane t returns the sum of v[t]
 __device__ __forceinline__ float reduce32_transpose(float (&v)[32], int lane) {
 #pragma unroll
@@ -375,7 +380,7 @@ prologue_tc_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_consta
 // parts of a sum are added in shared memory.  Bound by the latency of one
 // round of loads: 17.5 us for 8 sequences when a thread walked all of d_nope
 // for one sequence, 9 us now (ncu, cold caches).
-constexpr int kPfBatch = 8, kPfFeat = 64, kPfParts = 16;
+constexpr int kPfBatch = 8, kPfFeat = 64, kPfParts = 16, kPfRows = 8;
 
 __global__ void __launch_bounds__(256)
 prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk, const int32_t* __restrict__ seq_lens,
@@ -399,27 +404,40 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
   const int h = item % H, fc = (item / H) % nfc, b0 = (item / (H * nfc)) * kPfBatch;
   const int nb = min(kPfBatch, batch - b0), tid = threadIdx.x;
   const int qrow = d_nope + d_rope;
+  const int f4 = 4 * (tid % (kPfFeat / 4)), part = tid / (kPfFeat / 4), f = fc * kPfFeat + f4;
+  const float* w = w_uk + static_cast<size_t>(h) * d_nope * d_c + f;
+  // the first kPfRows rows of this thread, in flight while q is staged
+  float4 wv[kPfRows];
+  auto load_rows = [&](int n0) {
+#pragma unroll
+    for (int k = 0; k < kPfRows; ++k) {
+      const int n = n0 + kPfParts * k;
+      wv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (f < d_c && n < d_nope) wv[k] = __ldg(reinterpret_cast<const float4*>(w + static_cast<size_t>(n) * d_c));
+    }
+  };
+  load_rows(part);
   for (int i = tid; i < kPfBatch * d_nope; i += 256) {
     const int j = i / d_nope, n = i % d_nope;
     qn[j][n] = j < nb ? q[(static_cast<size_t>(b0 + j) * H + h) * qrow + n] : 0.f;
   }
   __syncthreads();
-  const int f4 = 4 * (tid % (kPfFeat / 4)), part = tid / (kPfFeat / 4), f = fc * kPfFeat + f4;
   float4 acc[kPfBatch];
 #pragma unroll
   for (int j = 0; j < kPfBatch; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (f < d_c) {
-    const float* w = w_uk + static_cast<size_t>(h) * d_nope * d_c + f;
-#pragma unroll 8
-    for (int n = part; n < d_nope; n += kPfParts) {
-      const float4 wv = __ldg(reinterpret_cast<const float4*>(w + static_cast<size_t>(n) * d_c));
+  for (int n0 = part; n0 < d_nope; n0 += kPfParts * kPfRows) {
+    if (n0 != part) load_rows(n0);
+#pragma unroll
+    for (int k = 0; k < kPfRows; ++k) {
+      const int n = n0 + kPfParts * k;
+      if (n >= d_nope) break;
 #pragma unroll
       for (int j = 0; j < kPfBatch; ++j) {
         const float x = qn[j][n];
-        acc[j].x = fmaf(wv.x, x, acc[j].x);
-        acc[j].y = fmaf(wv.y, x, acc[j].y);
-        acc[j].z = fmaf(wv.z, x, acc[j].z);
-        acc[j].w = fmaf(wv.w, x, acc[j].w);
+        acc[j].x = fmaf(wv[k].x, x, acc[j].x);
+        acc[j].y = fmaf(wv[k].y, x, acc[j].y);
+        acc[j].z = fmaf(wv[k].z, x, acc[j].z);
+        acc[j].w = fmaf(wv[k].w, x, acc[j].w);
       }
     }
   }
@@ -619,6 +637,11 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
   const int nb = min(nt, batch - b0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kCombineThreads / 32;
+  const float* wh = w_uv + static_cast<size_t>(h) * d_v * d_c;
+  // this block's rows of W_UV,h (groups of 4 kWarps, one in gridDim.y) on their way to L2 meanwhile
+  for (int v = 4 * kWarps * blockIdx.y; v < d_v; v += 4 * kWarps * gridDim.y)
+    for (int i = 32 * tid; i < min(4 * kWarps, d_v - v) * d_c; i += 32 * kCombineThreads)
+      prefetch_l2(wh + static_cast<size_t>(v) * d_c + i);
   grid_dependency_wait();
   merge_partials<PPT, kCombineThreads>(sh, cu, part_ml, part_o, batch, H, h, b0, nt, d_c, num_splits,
                                        [&](int j, int f, const float4& o) { *reinterpret_cast<float4*>(&olat[j][f]) = o; });
@@ -626,7 +649,6 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
   // u[j][v] = sum_f W_UV[h][v][f] olat[j][f]
   constexpr int VEC = 4;
   const int npieces = d_c / VEC;   // d_c is a multiple of 4
-  const float* wh = w_uv + static_cast<size_t>(h) * d_v * d_c;
   for (int v0 = 4 * (warp + kWarps * blockIdx.y); v0 < d_v; v0 += 4 * kWarps * gridDim.y) {
     float acc[32];
 #pragma unroll
@@ -832,12 +854,17 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
 //           2 tokens;
 //   softmax warp = head: the parts added, the tile's maximum, P and the
 //           running max and denominator;
-//   output  thread = (4 features, 4 heads), accumulated in registers.
+//   output  thread = (4 features, 4 heads, every n-th token), accumulated in
+//           registers, the token groups added at the segment's end.
 // All sums are fp32 on CUDA cores.  A tile's four phases cost five block
 // barriers for 64 tokens; processing one token at a time cost 36 barriers per
 // token, 651 us for 8 sequences of 100 to 3000 tokens (d_c 256, 16 heads)
 // against 20 us now (ncu, cold caches).  At that size a split holds one
-// page, so the time is the latency of one tile's phases.
+// page, so the time is the latency of one tile's phases: the sequence found by
+// one round of loads, the page requested before the query block, the tokens of
+// the output dealt to groups of threads where d_c leaves threads without work,
+// W_UK requested before q is staged and W_UV brought to L2 before the combine
+// waits took the step from 28.4 to 26.4 us.
 constexpr int kF32Threads = 512, kF32Warps = kF32Threads / 32;
 constexpr int kF32Parts = 8;      // parts of a dot product
 constexpr int kF32Heads = 16;     // heads, at most
@@ -881,21 +908,40 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
   const int g0 = blockIdx.x * chunk;
   const int g1 = min(g0 + chunk, total);
   if (g0 >= g1) return;
-  int b = find_sequence(cu, batch, g0);
+  // the sequence of unit g0: the last that starts at or before it, by one round of loads
+  int b = batch <= kF32Threads ? __syncthreads_count(tid < batch && cu[min(tid, batch)] <= g0) - 1
+                               : find_sequence(cu, batch, g0);
   int g = g0;
-  // output: features 4 ocol .., heads 4 ohg ..
-  const int ocol = tid % ncol, ohg = tid / ncol;
-  const bool oact = ohg < kF32Heads / 4 && 4 * ohg < H;
+  // output: features 4 ocol .., heads 4 ohg .., every og-th token of ogroups
+  const int ocols = ncol * (kF32Heads / 4), ogroups = min(kF32Threads / ocols, 8);
+  const int ocol = tid % ncol, ohg = tid % ocols / ncol, og = tid / ocols;
+  const bool oact = og < ogroups && 4 * ohg < H;
   while (g < g1) {
     const int pend = min(g1, cu[b + 1]);
     const int L = seq_lens[b];
     const int s0 = cu[b] + kSegCost;   // unit of the sequence's first page
     const int lp0 = max(g - s0, 0), lp1 = pend - s0;
     if (min(lp1 * kPage, L) <= lp0 * kPage) break;   // the range ends inside the sequence's start cost
-    const float* qsrc = reinterpret_cast<const float*>(qprep + static_cast<size_t>(b) * qstride);
-    for (int i = tid; i < kF32Heads * d; i += kF32Threads) {
-      const int h = i / d, f = i - h * d;
-      qs[i] = h >= H ? 0.f : f < d_c ? qsrc[h * d_c + f] : qsrc[H * d_c + h * d_rope + f - d_c];
+    int page = block_table[static_cast<size_t>(b) * max_pages + lp0];   // (requested before the query block)
+    {
+      // warp = head
+      const float* qsrc = reinterpret_cast<const float*>(qprep + static_cast<size_t>(b) * qstride);
+      float4 qv[NV], qr = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int u = lane + 32 * i;
+        qv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (warp < H && u < ncol) qv[i] = reinterpret_cast<const float4*>(qsrc + static_cast<size_t>(warp) * d_c)[u];
+      }
+      if (warp < H && lane < d_rope / 4)
+        qr = reinterpret_cast<const float4*>(qsrc + static_cast<size_t>(H) * d_c + warp * d_rope)[lane];
+      float* qd = qs + warp * d;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int u = lane + 32 * i;
+        if (u < ncol) *reinterpret_cast<float4*>(qd + 4 * u) = qv[i];
+      }
+      if (lane < d_rope / 4) *reinterpret_cast<float4*>(qd + d_c + 4 * lane) = qr;
     }
     float4 acc[4];
 #pragma unroll
@@ -903,7 +949,7 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
     float mrun = -INFINITY, lrun = 0.f;   // head `warp`, the same in every lane
     for (int lp = lp0; lp < lp1; ++lp) {
       const int ntok = min(kPage, L - lp * kPage);
-      const int page = block_table[static_cast<size_t>(b) * max_pages + lp];
+      if (lp > lp0) page = block_table[static_cast<size_t>(b) * max_pages + lp];
       const bool page_ok = page >= 0 && page < num_pages;
       if (!page_ok && tid == 0) report_status(status, kStatusOutOfRange);
       const size_t row0 = static_cast<size_t>(page_ok ? page : 0) * kPage;
@@ -1064,7 +1110,7 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
         const float* zc = ct + 4 * ocol;
         const float* pc = pw + 4 * ohg;
 #pragma unroll 4
-        for (int t = 0; t < ntok; ++t) {
+        for (int t = og; t < ntok; t += ogroups) {
           const float4 x = *reinterpret_cast<const float4*>(zc + t * row_f);
           const float4 p4 = *reinterpret_cast<const float4*>(pc + t * kF32Heads);
           const float pk[4] = {p4.x, p4.y, p4.z, p4.w};
@@ -1080,7 +1126,21 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
       __syncthreads();   // the tile is read: the next one may overwrite it
     }
     const size_t slot = blockIdx.x + b;
-    if (oact) {
+    if (ogroups > 1) {   // the token groups' sums, added in order (the scores' space is free)
+      float4* red = reinterpret_cast<float4*>(sp);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) red[k * kF32Threads + tid] = acc[k];
+      __syncthreads();
+      if (og == 0) {
+        for (int i = 1; i < ogroups; ++i)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 r = red[k * kF32Threads + tid + i * ocols];
+            acc[k] = make_float4(acc[k].x + r.x, acc[k].y + r.y, acc[k].z + r.z, acc[k].w + r.w);
+          }
+      }
+    }
+    if (oact && og == 0) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if (4 * ohg + k < H)
