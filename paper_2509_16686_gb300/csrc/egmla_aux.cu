@@ -349,7 +349,7 @@ prologue_tc_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_consta
       tmem_ld16(tmem + (static_cast<uint32_t>(32 * quad) << 16) + c0, v);
       tmem_wait_ld();
       float part[32];
-      uint8_t* qb = qprep + static_cast<size_t>(b0 + c0) * qstride + qop_offset(h, f);
+      uint8_t* qb = qprep + static_cast<size_t>(b0 + c0) * qstride + qlat_offset(h, f, d_c);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const __nv_bfloat16 bq = __float2bfloat16_rn(v[j] * gm);

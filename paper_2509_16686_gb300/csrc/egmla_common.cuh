@@ -36,6 +36,13 @@ constexpr int kQRowGroupBytes = 128;
 __host__ __device__ constexpr size_t qop_offset(int h, int k) {
   return static_cast<size_t>(k / 8) * kQGroupBytes + (h / 8) * kQRowGroupBytes + (h % 8) * 16 + (k % 8) * 2;
 }
+// Latent widths walked in half pages: the K cores of two 64-feature columns
+// alternate, so that the score MMA takes both as one operand of 32 rows (the row
+// groups of the even column, then of the odd one, 128 B apart; K cores 512 B apart).
+__host__ __device__ constexpr size_t qlat_offset(int h, int f, int d_c) {
+  const int core = f / 8;
+  return qop_offset(h, d_c <= 256 ? f : 8 * (core / 16 * 16 + core % 8 * 2 + core / 8 % 2) + f % 8);
+}
 __host__ __device__ constexpr size_t qprep_lat_bytes(int d_c) { return static_cast<size_t>(d_c / 8) * kQGroupBytes; }
 __host__ __device__ constexpr size_t qprep_rope_bytes(int d_rope) {
   return static_cast<size_t>(d_rope / 8) * kQGroupBytes;

@@ -106,8 +106,8 @@ struct Cfg {
   static constexpr int NCH = D_C / 64;                  // 64-feature swizzle-atom columns
   // tokens per tile: a page, or half a page for the widest latent, whose pages
   // are too large for a ring of three in shared memory: two slots of 72 KB took
-  // about 150 us for 128 ragged sequences, five of 36 KB about 105 (557 MB: 3.7
-  // and 5.3 TB/s; kernel alone, warm)
+  // about 150 us for 128 ragged sequences, five of 36 KB about 92 (562 MB: 3.7
+  // and 6.1 TB/s; kernel alone, warm)
   static constexpr int TOK = D_C > 256 ? kPage / 2 : kPage;
   static constexpr int TPP = kPage / TOK;               // tiles per page
   static constexpr uint32_t PCHUNK = TOK * 128;         // one atom column of a tile
@@ -121,8 +121,9 @@ struct Cfg {
   static constexpr uint32_t PBUF = kPage * kHeads * 2;
   // LayerNorm gamma and beta of the segment read-out
   static constexpr uint32_t GB_BYTES = GATE ? 2 * D_C * 4 : 0;
-  // softmax exchange: tile maxima [4 warps][16], segment sums [4 warps][16][2]
-  static constexpr uint32_t XCH = 1024;
+  // softmax exchange: tile maxima [4 warps][16], segment sums [4 warps][16][2],
+  // with half pages the odd latent columns' scores [32 tokens][16]
+  static constexpr uint32_t XCH = 1024 + (TOK < kPage ? TOK * kHeads * 4 : 0);
   static constexpr uint32_t MISC = 1024;
   static constexpr uint32_t FIXED = kNP * PBUF + GB_BYTES + XCH + MISC + 1024;
   // slots with two query buffers (the next segment's loaded while this one is
@@ -151,9 +152,8 @@ struct Cfg {
   static_assert(SMEM <= kSmemLimit, "shared memory");
   static_assert(D_C == 192 || D_C == 256 || (D_C == 512 && !GATE), "latent widths of this kernel");
   static_assert(COL_O + kHeads * NMC <= TMEM_COLS && NMC % 2 == 0, "tensor memory");
-  // the score MMAs read 64 rows of every atom column: at half pages the last
-  // 32 are the next column's (or what follows the slot), and their scores are
-  // not used
+  // the score MMAs read 64 rows: at half pages two atom columns' 32, for the
+  // RoPE key its 32 and what follows the slot, whose scores are not used
   static_assert(OFF_QBUF + 64 * 128 <= SMEM, "score operand");
   // first latent feature of output M chunk j (chunks of 128 rows); for
   // D_C = 192 the second chunk starts at 64 and overlaps the first, so that no
@@ -779,8 +779,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // requested once its buffer's previous segment is done with it (last score
     // MMA complete, sums read by the softmax warps), tested after every tile.
     // A warp that polled both queues, voted and elected for every tile took
-    // 135 us of the d_c 512 step where this takes 124 (its 36 MMAs per 32 tokens
-    // are short, so what lies between tiles counts), 48.4 instead of 47.9 of the
+    // 135 us of the d_c 512 step where this took 124 (then 36 MMAs per 32 tokens,
+    // short, so that what lies between tiles counts), 48.4 instead of 47.9 of the
     // 8 x 32K step, and 68.3 instead of 69.3 of 128 ragged sequences at d_c 192.
     // Loops are unrolled with compile-time accumulate flags.
     if (!DUMP && elect_one()) {
@@ -790,6 +790,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       // apart, head halves 128 B apart
       const uint64_t zdesc_k = smem_desc(sbase, 16, 1024, kSwizzle128B);
       const uint64_t qdesc0 = smem_desc(sbase + C::OFF_QBUF, kQGroupBytes, kQRowGroupBytes, kSwizzleNone);
+      // half pages: two latent columns per MMA.  The 64 rows of the A operand at an
+      // even column are its 32 tokens and the next column's 32, B's N = 32 the two
+      // columns' query values; the scores are D's two diagonal blocks (the others
+      // are not used), added by the softmax warps.  The MMAs are bound by the
+      // operand bytes they read from shared memory, 59 KB per half page against 92
+      // with a column at a time and half the rows unused: 128 ragged sequences at
+      // d_c 512 118.4 -> 106.2 us.
+      constexpr uint32_t IDESC_S2 = idesc_bf16(64, 2 * kHeads, 0, 0);
+      const uint64_t qdesc2 = smem_desc(sbase + C::OFF_QBUF, 2 * kQGroupBytes, kQRowGroupBytes, kSwizzleNone);
       Walker<C::TOK> ws, wq;
       ws.start(p);
       wq.start(p);
@@ -836,14 +845,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t za = zdesc_k + ((slot * C::SLOT) >> 4);
         const uint64_t qb = qdesc0 + (((seg % C::NQ) * C::QBUF) >> 4);
         const uint32_t ds = tmem + C::COL_S + sb * C::S_COLS;
+        if constexpr (C::TOK < kPage) {
+          const uint64_t qb2 = qdesc2 + (((seg % C::NQ) * C::QBUF) >> 4);
 #pragma unroll
-        for (int kk = 0; kk < D_C / 16; ++kk)
-          mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
-                      qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+          for (int kk = 0; kk < D_C / 32; ++kk)
+            mma_bf16_ss(ds, za + (((kk >> 2) * 2 * C::PCHUNK + (kk & 3) * 32) >> 4),
+                        qb2 + ((kk * 4 * kQGroupBytes) >> 4), IDESC_S2, kk > 0);
 #pragma unroll
-        for (int kk = 0; kk < kRope / 16; ++kk)
-          mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
-                      qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+          for (int kk = 0; kk < kRope / 16; ++kk)
+            mma_bf16_ss(ds, za + ((C::KR_OFF + kk * 32) >> 4),
+                        qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, 1);
+        } else {
+#pragma unroll
+          for (int kk = 0; kk < D_C / 16; ++kk)
+            mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
+                        qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+#pragma unroll
+          for (int kk = 0; kk < kRope / 16; ++kk)
+            mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
+                        qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+        }
         mma_commit(smem_u32(&bars.sready[sb]));
         if (ts.last) mma_commit(smem_u32(&bars.qempty[seg % C::NQ]));
         tr.mark(2, js);
@@ -1187,6 +1208,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float scale = p.scale_log2;
     float* xmax = reinterpret_cast<float*>(smem + C::OFF_XCH);        // [4 warps][16 heads]
     float* xsum = xmax + kSoftWarps * kHeads;                         // [4 warps][16 heads][2]
+    float* xodd = xmax + 256;                                         // half pages: [32 tokens][16 heads]
     auto head_of = [&](int k) { return (k & 1) + 2 * q + 8 * (k >> 1); };
     // gamma and beta of the segment read-out in shared memory (written once by
     // the four warps; the first tile's barrier orders the writes before any read)
@@ -1258,9 +1280,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       float s[2][4];
       float mu[2] = {0.f, 0.f}, rr[2] = {1.f, 1.f};
       bool exceed = false;
+      float v[16];
       if (ok) {
         tc_fence_after();
-        float v[16];
         tmem_ld_16x256b_x4(tq + C::COL_S + sb * C::S_COLS, v);
         if (GATE) {
           const float* st = reinterpret_cast<const float*>(smem + C::OFF_STAT + slot * C::STAT_BYTES);
@@ -1273,6 +1295,20 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         warp_arrive(smem_u32(&bars.sfree[sb]));   // score buffer read: tile it + kNB may overwrite it
         tr.mark(7, it);
+        if constexpr (C::TOK < kPage) {
+          // rows 32 .. 63 are the odd columns' part of tokens 0 .. 31: to their owners
+          if (warp >= 2) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+              for (int hp = 0; hp < 2; ++hp)
+                *reinterpret_cast<float2*>(xodd + ((e ? r1 : r0) - C::TOK) * kHeads + head_of(2 * hp)) =
+                    make_float2(v[8 + hp * 4 + 2 * e], v[8 + hp * 4 + 2 * e + 1]);
+          }
+        }
+      }
+      if constexpr (C::TOK < kPage) soft_sync(kBarXch);   // (every warp, also after an error)
+      if (ok) {
         const bool full_page = t.ntok == kPage;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -1280,7 +1316,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float lat = v[(k >> 1) * 4 + 2 * e + (k & 1)];
-            const float rope = v[8 + (k >> 1) * 4 + 2 * e + (k & 1)];
+            const float rope = C::TOK == kPage ? v[8 + (k >> 1) * 4 + 2 * e + (k & 1)]
+                               : warp < 2      ? xodd[(e ? r1 : r0) * kHeads + head_of(k)]
+                                               : 0.f;
             float x;
             if (GATE) {
               x = fmaf(rr[e] * scale, fmaf(-mu[e], wq[k], lat), fmaf(rope, scale, bsc[k]));
