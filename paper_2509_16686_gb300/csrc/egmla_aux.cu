@@ -379,7 +379,7 @@ prologue_tc_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_consta
 // for all the group's sequences with no load depending on another; the 16
 // parts of a sum are added in shared memory.  Bound by the latency of one
 // round of loads: 17.5 us for 8 sequences when a thread walked all of d_nope
-// for one sequence, 9 us now (ncu, cold caches).
+// for one sequence, 6 us now (ncu, cold caches).
 constexpr int kPfBatch = 8, kPfFeat = 64, kPfParts = 16, kPfRows = 8;
 
 __global__ void __launch_bounds__(256)
@@ -859,7 +859,7 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
 // All sums are fp32 on CUDA cores.  A tile's four phases cost five block
 // barriers for 64 tokens; processing one token at a time cost 36 barriers per
 // token, 651 us for 8 sequences of 100 to 3000 tokens (d_c 256, 16 heads)
-// against 20 us now (ncu, cold caches).  At that size a split holds one
+// against 17 us now (ncu, cold caches).  At that size a split holds one
 // page, so the time is the latency of one tile's phases: the sequence found by
 // one round of loads, the page requested before the query block, the tokens of
 // the output dealt to groups of threads where d_c leaves threads without work,
