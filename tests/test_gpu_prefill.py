@@ -216,3 +216,25 @@ def test_prefill_offsets_past_the_tokens_are_reported(gpu_lib):
     got = device.output_f64(dp.out)
     ref = orc.prefill(pc)
     check_close(got[:150], ref[:150], positions_of(pc)[:150])
+
+
+@pytest.mark.parametrize("d_c", [192, 512])
+def test_prefill_layernorm_parameters_at_any_alignment(gpu_lib, d_c):
+    """gamma and beta are read 16 bytes at a time where their addresses allow it:
+    the same values at addresses that do not give the same bytes."""
+    pc = synth.make_prefill_case("align", synth.dims_bf16(d_c=d_c, vocab=3000), [70, 129], seed=69)
+    dp = device.upload_prefill(pc)
+    g = torch.Generator().manual_seed(70)
+    gamma, beta = (1 + torch.randn(d_c, generator=g) / 10).cuda(), (torch.randn(d_c, generator=g) / 10).cuda()
+    outs = []
+    for shift in (0, 1, 2):
+        for name, v in (("ln_gamma", gamma), ("ln_beta", beta)):
+            room = torch.empty(d_c + shift, device="cuda")
+            room[shift:] = v
+            setattr(dp, name, room[shift:])
+            assert getattr(dp, name).data_ptr() % 16 == 4 * shift
+        dp.run()
+        torch.cuda.synchronize()
+        assert dp.read_status() == 0
+        outs.append(dp.out.clone())
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
