@@ -168,6 +168,28 @@ def test_bf16_ablation_gates_match_oracle(gpu_lib, op, d_c):
         check_bf16(got, ref, f"{op} d_c={d_c} splits={splits}", scaled_abs=True)
 
 
+@pytest.mark.parametrize("d_c", [64, 256])
+def test_fp32_layernorm_parameters_at_any_alignment(gpu_lib, d_c):
+    """gamma and beta are read 16 bytes at a time where their addresses allow it:
+    the same values at addresses that do not give the same bits."""
+    dims = synth.Dims(num_heads=4, d_nope=32, d_rope=16, d_v=32, d_c=d_c, page_size=64, vocab=500, dtype="fp32",
+                      gate=True)
+    case = synth.make_case("f32-align", dims, [1, 70, 130], seed=38, affine_ln=True, layout="permuted")
+    dc = device.upload(case)
+    gamma, beta = dc.ln_gamma.clone(), dc.ln_beta.clone()
+    outs = []
+    for shift in (0, 1, 2):
+        for name, v in (("ln_gamma", gamma), ("ln_beta", beta)):
+            room = torch.empty(d_c + shift, device="cuda")
+            room[shift:] = v
+            setattr(dc, name, room[shift:])
+        dc.step()
+        torch.cuda.synchronize()
+        assert dc.read_status() == 0
+        outs.append(dc.out.clone())
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
 @pytest.mark.parametrize("heads,d_nope,d_rope,d_v,d_c,gate", [
     (16, 256, 64, 256, 512, True),    # the largest shape: four units per lane, all shared memory
     (3, 7, 12, 9, 100, True),         # d_c + d_rope an even number of units (padded rows), odd sizes
