@@ -238,6 +238,8 @@ __host__ __device__ constexpr uint32_t pm_smem(int nk, int nt) {
          sizeof(PmBars);
 }
 
+static_assert(pm_smem(kPmMaxNope / 64, kPmMaxSeq) <= kSmemMost, "shared memory");
+
 __global__ void __launch_bounds__(kPmThreads)
 prologue_tc_kernel(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap qmap,
                     const __nv_bfloat16* __restrict__ q, const float* __restrict__ gamma,
@@ -727,6 +729,8 @@ __host__ __device__ constexpr uint32_t ct_smem(int d_c, int nt) {
   return static_cast<uint32_t>(d_c / 64) * (kCtAtom + ct_cols(nt) * 128) + sizeof(CtShared) + 1024;
 }
 
+static_assert(ct_smem(kCombineMaxDc, kMergeMaxSeq) <= kSmemMost, "shared memory");
+
 // PPT: (sequence, 4 features) pairs per thread, at most; T threads (512 where
 // that is more than one pair each: more of the partials in flight, 128 ragged
 // sequences 69.3 -> 67.7 us, 128 at d_c 512 123.6 -> 118.9; 256 otherwise, 32 x 4K
@@ -876,6 +880,7 @@ __device__ __forceinline__ float4 load_features4(const float* p, int f, float no
 constexpr int kF32Threads = 512, kF32Warps = kF32Threads / 32;
 constexpr int kF32Parts = 8;      // parts of a dot product
 constexpr int kF32Heads = 16;     // heads, at most
+constexpr int kF32MaxRope = 64;   // d_rope, at most
 
 // row stride of the tile in floats: a multiple of 4 and an odd number of 16-byte
 // units, so that the lanes' rows start in different bank groups
@@ -885,6 +890,8 @@ __host__ __device__ constexpr size_t f32_smem_floats(int d_c, int d_rope) {
   return static_cast<size_t>(kF32Heads) * d + static_cast<size_t>(kPage) * f32_row(d) +
          kF32Parts * kF32Heads * kPage + kPage * kF32Heads + kF32Heads;
 }
+
+static_assert(f32_smem_floats(512, kF32MaxRope) * sizeof(float) <= kSmemMost, "shared memory");
 
 // NV: 16-byte units of a latent row per lane (d_c <= 128 NV)
 template <int NV>
@@ -1194,8 +1201,7 @@ cudaError_t launch_prologue_tc(const DecodeArgs& a, const AppendArgs* app, const
   const int tiles = a.q != nullptr ? 16 * mt * ((a.batch + nt - 1) / nt) : 0;
   const int blocks = tiles + 1 + (ap.batch + kPmThreads / 32 - 1) / (kPmThreads / 32);
   const size_t smem = pm_smem(nk, nt);
-  const cudaError_t e =
-      cudaFuncSetAttribute(prologue_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(prologue_tc_kernel, pm_smem(kPmMaxNope / 64, kPmMaxSeq));
   if (e != cudaSuccess) return e;
   return launch_chained(
       prologue_tc_kernel, dim3(blocks), dim3(kPmThreads), smem, st, maps[0], maps[1],
@@ -1210,8 +1216,7 @@ template <int NV>
 cudaError_t launch_decode_f32_t(const DecodeArgs& a, const WorkspaceLayout& wl, cudaStream_t st) {
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
   const size_t smem = f32_smem_floats(a.d_c, a.d_rope) * sizeof(float);
-  const cudaError_t e =
-      cudaFuncSetAttribute(decode_f32_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(decode_f32_kernel<NV>, f32_smem_floats(128 * NV, kF32MaxRope) * sizeof(float));
   if (e != cudaSuccess) return e;
   return launch_chained(
       decode_f32_kernel<NV>, dim3(a.num_splits), dim3(kF32Threads), smem, st,
@@ -1247,8 +1252,7 @@ template <int PPT, int T>
 cudaError_t launch_combine_tc(const DecodeArgs& a, const CUtensorMap* wmap, const int32_t* cu, const float* ml,
                               const float* po, int nt, cudaStream_t st) {
   const size_t smem = ct_smem(a.d_c, nt);
-  const cudaError_t e = cudaFuncSetAttribute(combine_tc_kernel<PPT, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+  const cudaError_t e = allow_smem(combine_tc_kernel<PPT, T>, ct_smem(kCombineMaxDc, kMergeMaxSeq));
   if (e != cudaSuccess) return e;
   return launch_chained(combine_tc_kernel<PPT, T>, dim3(16 * ((a.batch + nt - 1) / nt), (a.d_v + 127) / 128),
                         dim3(T), smem, st, *wmap, cu, ml, po, static_cast<__nv_bfloat16*>(a.out), a.batch,

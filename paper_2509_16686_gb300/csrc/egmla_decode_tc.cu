@@ -1552,7 +1552,7 @@ template <int D_C, int GM, int DBG>
 cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_t st, bool* fused) {
   using C = Cfg<D_C, GM != 0>;
   auto kern = decode_tc_kernel<D_C, GM, DBG>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  cudaError_t e = allow_smem(kern, C::SMEM);
   if (e != cudaSuccess) return e;
   const WorkspaceLayout wl = workspace_layout(a.batch, a.num_splits, kHeads, D_C, kRope, true);
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);

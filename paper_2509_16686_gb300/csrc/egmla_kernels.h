@@ -39,6 +39,17 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Lets `kernel` be launched with up to `most` bytes of dynamic shared memory.  The
+// limit belongs to the function, not to the calling thread, so every call of a
+// kernel sets the same one, the most that any supported shape needs: a call that
+// set its own smaller need would take the launch of another thread's larger call
+// from under it.
+constexpr size_t kSmemMost = 227 * 1024;   // of a block, on this GPU
+template <typename K>
+cudaError_t allow_smem(K* kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
+
 struct AppendArgs {
   void* c_pool;
   void* kr_pool;

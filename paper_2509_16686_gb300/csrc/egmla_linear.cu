@@ -392,8 +392,7 @@ bool linear_tc_supported(int n_out, int k, int batch) {
 cudaError_t linear_tc_plan(int n_out, int k, int batch, int* cluster, int* stages, int* max_clusters) {
   *cluster = *stages = *max_clusters = 0;
   if (n_out <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kLinSmemLimit));
+  cudaError_t e = allow_smem(linear_tc_kernel, kLinSmemLimit);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
@@ -427,15 +426,10 @@ cudaError_t linear_tc_plan(int n_out, int k, int batch, int* cluster, int* stage
 cudaError_t launch_linear_tc(const void* w, int n_out, int k, const void* x, int batch, void* out, int ldo,
                              bool out_f32, int32_t* status, cudaStream_t st) {
   if (batch == 0) return cudaSuccess;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(linear_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kLinSmemLimit));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  cudaError_t e = allow_smem(linear_tc_kernel, kLinSmemLimit);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;

@@ -331,7 +331,7 @@ struct KvParams {
 // weight stages that fit next to RT x nkc latent atoms and the output staging
 template <int RT>
 __host__ __device__ constexpr int kv_stages(int nkc) {
-  const long long room = 227LL * 1024 - 2048 - static_cast<long long>(RT * nkc) * kPfAtom - kKvOutBytes;
+  const long long room = static_cast<long long>(kSmemMost) - 2048 - static_cast<long long>(RT * nkc) * kPfAtom - kKvOutBytes;
   const long long st = room / kKvBBytes;
   return st > kKvMaxStages ? kKvMaxStages : static_cast<int>(st);
 }
@@ -1213,7 +1213,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   {
     kp.stages = kv_stages<1>(nkc);
     const int kv_smem = static_cast<int>(kv_smem_bytes<1>(nkc));
-    e = cudaFuncSetAttribute(prefill_kv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kv_smem);
+    e = allow_smem(prefill_kv_kernel<1>, kSmemMost);
     if (e != cudaSuccess) return e;
     kp.units = static_cast<long long>((a.total + kPfRows - 1) / kPfRows) * kp.nblocks;
     const int grid = static_cast<int>(kp.units < sms ? kp.units : sms);
@@ -1226,8 +1226,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   if (!pf_encode(&qmap, a.q, a.total, static_cast<uint64_t>(a.H) * kPfDqk, static_cast<uint64_t>(a.H) * kPfDqk))
     return cudaErrorInvalidValue;
   if (!pf_encode(&krmap, a.kr, a.total, kPfDr, kPfDr)) return cudaErrorInvalidValue;
-  e = cudaFuncSetAttribute(prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kAttnSmem));
+  e = allow_smem(prefill_attn_kernel, kAttnSmem);
   if (e != cudaSuccess) return e;
   AttnParams ap;
   ap.cu = a.cu_seqlens;
@@ -1271,7 +1270,7 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
   if (nkc <= 4) {
     kp.stages = kv_stages<2>(nkc);
     const int smem = static_cast<int>(kv_smem_bytes<2>(nkc));
-    e = cudaFuncSetAttribute(prefill_kv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = allow_smem(prefill_kv_kernel<2>, kSmemMost);
     if (e != cudaSuccess) return e;
     const int tiles = (vocab + 2 * kPfRows - 1) / (2 * kPfRows);
     kp.units = static_cast<long long>(tiles) * kp.nblocks;   // whole tiles: a table row's few blocks share its copy
@@ -1279,7 +1278,7 @@ cudaError_t launch_gate_table(const void* emb, const void* w_ue, int vocab, int 
   } else {
     kp.stages = kv_stages<1>(nkc);
     const int smem = static_cast<int>(kv_smem_bytes<1>(nkc));
-    e = cudaFuncSetAttribute(prefill_kv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = allow_smem(prefill_kv_kernel<1>, kSmemMost);
     if (e != cudaSuccess) return e;
     const int tiles = (vocab + kPfRows - 1) / kPfRows;
     kp.units = static_cast<long long>(tiles) * kp.nblocks;

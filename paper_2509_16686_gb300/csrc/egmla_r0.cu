@@ -99,6 +99,12 @@ struct R0Smem {
   int abort;
 };
 
+constexpr int kR0MaxChunks = 4;   // d_c 256
+__host__ __device__ constexpr size_t r0_smem(int nkc) {
+  return nkc * kR0AChunkBytes + kR0BStages * kR0BChunkBytes + sizeof(R0Smem) + 1024;
+}
+static_assert(r0_smem(kR0MaxChunks) <= kSmemMost, "shared memory");
+
 struct R0ProjParams {
   const __nv_bfloat16* q;        // [B, 16, d_n + d_r]
   const __nv_bfloat16* kr_pool;  // [pool rows, d_r]
@@ -676,8 +682,8 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   if (!r0_encode(&cmap, a.c_pool, rows, static_cast<uint64_t>(a.d_c), kPage)) return cudaErrorInvalidValue;
   if (!r0_encode(&wmap, a.w_ukv, kR0Width, static_cast<uint64_t>(a.d_c), kR0Half)) return cudaErrorInvalidValue;
   const int nkc = a.d_c / kR0Chunk;
-  const int smem = static_cast<int>(nkc * kR0AChunkBytes + kR0BStages * kR0BChunkBytes + sizeof(R0Smem) + 1024);
-  cudaError_t e = cudaFuncSetAttribute(r0_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const size_t smem = r0_smem(nkc);
+  cudaError_t e = allow_smem(r0_project_kernel, r0_smem(kR0MaxChunks));
   if (e != cudaSuccess) return e;
   R0ProjParams pp;
   pp.q = static_cast<const __nv_bfloat16*>(a.q);
