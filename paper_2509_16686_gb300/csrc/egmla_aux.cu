@@ -831,9 +831,13 @@ combine_tc_kernel(const __grid_constant__ CUtensorMap wmap, const int32_t* __res
     auto store = [&](auto nt_c) {
       constexpr int NT = decltype(nt_c)::value;
 #pragma unroll
-      for (int j = 0; j < NT; ++j)
+      for (int j = 0; j < NT; ++j) {
+        // (an infinite first column, of an infinite o or weight, is the sum: the
+        // other pieces may be zero, and their product with such a weight no number)
+        const float u = fabsf(d[j]) < INFINITY ? d[j] + (d[NT + j] + d[2 * NT + j]) : d[j];
         if ((NT == 1 ? warp < 4 : (j & 1) == warp >> 2) && j < nb && v < d_v)
-          out[(static_cast<size_t>(b0 + j) * H + h) * d_v + v] = __float2bfloat16_rn(d[j] + (d[NT + j] + d[2 * NT + j]));
+          out[(static_cast<size_t>(b0 + j) * H + h) * d_v + v] = __float2bfloat16_rn(u);
+      }
     };
     if (nt == 1) store(std::integral_constant<int, 1>{});
     else if (nt == 2) store(std::integral_constant<int, 2>{});

@@ -143,6 +143,27 @@ def test_bf16_split_combine_keeps_infinities(gpu_lib, d_c):
     check_bf16(got[1:], ref[1:], f"d_c={d_c}")
 
 
+@pytest.mark.parametrize("d_c", [192, 256, 512])
+def test_bf16_split_combine_of_an_infinite_weight(gpu_lib, d_c):
+    """An infinite element of W_UV makes its output row infinite in every sequence,
+    also where the merged latent needs one or two bf16 pieces only (latents of one
+    and q = 0: a merged value of one, or the fp32 number next to it), and leaves
+    the other rows as they are."""
+    dims = synth.dims_bf16(d_c=d_c, vocab=300, gate=False)
+    case = synth.make_case("inf-weight", dims, [1 << (b % 9) for b in range(20)], seed=39, latent_scale=0.5,
+                           layout="permuted")
+    case.q[:] = 0
+    f, row, one = 70, 3, orc.to_bf16_bits(np.array([1.0]))[0]
+    case.c_pool[..., f] = one
+    case.c_new[:, f] = one
+    ref = orc.decode_unabsorbed(case)
+    case.w_uv[0, row, f] = orc.to_bf16_bits(np.array([-np.inf]))[0]
+    _, got = run(case, 0)
+    assert (got[:, 0, row] == -np.inf).all()
+    got[:, 0, row] = ref[:, 0, row]
+    check_bf16(got, ref, f"d_c={d_c}", scaled_abs=True)
+
+
 @pytest.mark.parametrize("splits", [1, 3, 0])
 def test_bf16_half_page_tiles_match_oracle(gpu_lib, splits):
     """d_c 512 walks its pages in halves of 32 tokens: sequences that end in a
