@@ -192,10 +192,12 @@ __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfG
     }
     page[k] = -1;
     if (p.c_pool) {
-      const int b = prompt_of_row(p.cu, p.batch, t);
-      const int pos = t - __ldg(p.cu + b), lp = pos / kPage;
+      // a row before the first prompt's start or past its prompt's end has no slot
+      // (inconsistent offsets: nothing is written, and it is reported below)
+      const int b = prompt_of_row(p.cu, p.batch, t), start = __ldg(p.cu + b);
+      const int pos = start >= 0 && start <= t && t < __ldg(p.cu + b + 1) ? t - start : -1, lp = pos / kPage;
       slot[k] = pos % kPage;
-      page[k] = lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
+      page[k] = pos >= 0 && lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
     }
   }
 #pragma unroll

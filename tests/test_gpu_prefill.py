@@ -218,6 +218,30 @@ def test_prefill_offsets_past_the_tokens_are_reported(gpu_lib):
     check_close(got[:150], ref[:150], positions_of(pc)[:150])
 
 
+@pytest.mark.parametrize("cu", [(70, 150, 240), (1, 150, 240), (0, 150, 200), (70, 150, 160)])
+def test_prefill_rows_outside_every_prompt_are_not_cached(gpu_lib, cu):
+    """Offsets that start past row 0 or end before the last row: the rows in no
+    prompt are reported and written to no slot (a row before the first prompt
+    would sit before the first page), the others go to their prompts' slots."""
+    pc = synth.make_prefill_case("outside", synth.dims_bf16(d_c=256, vocab=3000), [150, 90], seed=71, extra_pages=4)
+    dp = device.upload_prefill(pc)
+    dp.cu_seqlens.copy_(torch.tensor(cu, dtype=torch.int32))
+    dp.out.fill_(float("nan"))
+    dp.run()
+    torch.cuda.synchronize()
+    assert dp.read_status() == _lib.EG_MLA_ERR_OUT_OF_RANGE
+    c_pool, kr_pool, id_pool = pc.c_pool.copy(), pc.kr_pool.copy(), pc.id_pool.copy()
+    for b in range(2):
+        for pos in range(cu[b + 1] - cu[b]):
+            at = pc.block_table[b, pos // 64], pos % 64
+            c_pool[at], kr_pool[at], id_pool[at] = (x[cu[b] + pos] for x in (pc.c, pc.kr, pc.ids))
+    np.testing.assert_array_equal(device.bf16_tensor_to_bits(dp.c_pool), c_pool)
+    np.testing.assert_array_equal(device.bf16_tensor_to_bits(dp.kr_pool), kr_pool)
+    np.testing.assert_array_equal(dp.id_pool.cpu().numpy(), id_pool)
+    rows = slice(cu[1], cu[2])   # the second prompt starts where it should
+    check_close(device.output_f64(dp.out)[rows], orc.prefill(pc)[rows], positions_of(pc)[rows])
+
+
 @pytest.mark.parametrize("d_c", [192, 512])
 def test_prefill_layernorm_parameters_at_any_alignment(gpu_lib, d_c):
     """gamma and beta are read 16 bytes at a time where their addresses allow it:
