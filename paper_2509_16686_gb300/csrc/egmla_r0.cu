@@ -214,6 +214,9 @@ __device__ void find_tile(const R0ProjParams& p, R0Smem& sm, int lane) {
   }
 }
 
+// WIDE: the gate's rows are 32-byte aligned and read in 32-byte pieces, otherwise
+// in 16-byte ones (all that the contract asks for)
+template <bool WIDE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kR0Threads, 1)
     r0_project_kernel(const __grid_constant__ CUtensorMap cmap, const __grid_constant__ CUtensorMap wmap,
                       const R0ProjParams p) {
@@ -394,7 +397,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kR0Threads, 1)
     // quarter of them is requested for head h + 1 as soon as head h has used
     // it, so that the loads run while the rest of head h is processed
     uint4 g[kR0GroupFeat / 8];
-    auto load_g = [&](int hh, int i) { ldg_32_na_hint(grow + hh * kR0Feat + 16 * i, pol_gate, g[2 * i], g[2 * i + 1]); };
+    auto load_g = [&](int hh, int i) {
+      const __nv_bfloat16* src = grow + hh * kR0Feat + 16 * i;
+      if constexpr (WIDE) {
+        ldg_32_na_hint(src, pol_gate, g[2 * i], g[2 * i + 1]);
+      } else {
+        g[2 * i] = ldg_16_na_hint(src, pol_gate);
+        g[2 * i + 1] = ldg_16_na_hint(src + 8, pol_gate);
+      }
+    };
 #pragma unroll
     for (int i = 0; i < kR0GroupFeat / 16; ++i) load_g(0, i);
     for (int h = 0; h < kR0Heads; ++h) {
@@ -683,7 +694,8 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   if (!r0_encode(&wmap, a.w_ukv, kR0Width, static_cast<uint64_t>(a.d_c), kR0Half)) return cudaErrorInvalidValue;
   const int nkc = a.d_c / kR0Chunk;
   const size_t smem = r0_smem(nkc);
-  cudaError_t e = allow_smem(r0_project_kernel, r0_smem(kR0MaxChunks));
+  const auto project = (reinterpret_cast<uintptr_t>(a.gate_r0) & 31) == 0 ? r0_project_kernel<true> : r0_project_kernel<false>;
+  cudaError_t e = allow_smem(project, r0_smem(kR0MaxChunks));
   if (e != cudaSuccess) return e;
   R0ProjParams pp;
   pp.q = static_cast<const __nv_bfloat16*>(a.q);
@@ -710,7 +722,7 @@ cudaError_t launch_decode_r0(const R0Args& a, cudaStream_t st) {
   // one CTA per two pages of the walk: the block table bounds the pages in use
   // (an even number: the CTAs work in pairs)
   const int tiles = static_cast<int>((static_cast<int64_t>(a.batch) * a.max_pages + 3) / 4 * 2);
-  e = launch_chained(r0_project_kernel, dim3(tiles), dim3(kR0Threads), smem, st, cmap, wmap, pp);
+  e = launch_chained(project, dim3(tiles), dim3(kR0Threads), smem, st, cmap, wmap, pp);
   if (e != cudaSuccess) return e;
   R0AttnParams ap;
   ap.block_table = a.block_table;

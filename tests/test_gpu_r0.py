@@ -22,11 +22,14 @@ def rel_l2(got, ref):
     return float(np.linalg.norm(got - ref) / max(np.linalg.norm(ref), 1e-30))
 
 
-def run_r0(case, r0):
+def run_r0(case, r0, gate_shift=0):
+    """gate_shift: elements between an aligned address and the gate's first"""
     dc = device.upload(case)
     dc.append()
     w_ukv = device.to_device_array(r0.w_ukv, "bf16", "cuda")
     gate = device.to_device_array(r0.gate_r0, "bf16", "cuda")
+    room = torch.empty(gate.numel() + gate_shift, dtype=gate.dtype, device="cuda")
+    gate = room[gate_shift:].view(gate.shape).copy_(gate)
     gamma = torch.from_numpy(r0.gamma).cuda()
     beta = torch.from_numpy(r0.beta).cuda()
     ws = torch.empty(_lib.eg_mla_decode_r0_workspace_size(dc.dims, case.batch, dc.block_table.shape[1],
@@ -51,6 +54,21 @@ def test_r0_decode_matches_oracle(gpu_lib, d_c, lens, affine):
     diff = np.abs(got - ref)
     rel = rel_l2(got, ref)
     assert (diff <= 1e-2 * np.maximum(1.0, np.abs(ref))).all() and rel <= 5e-3, (diff.max(), rel)
+
+
+@pytest.mark.parametrize("d_c", [192, 256])
+def test_r0_gate_at_a_16_byte_address(gpu_lib, d_c):
+    """The gate's rows are read 32 bytes at a time where the address allows it:
+    the same output bit for bit at an address that is 16-byte aligned only."""
+    case = synth.make_case("r0-align", synth.dims_bf16(d_c=d_c, vocab=3000), [70, 200, 1], seed=62, latent_scale=0.5,
+                           layout="permuted", affine_ln=True)
+    r0 = synth.make_r0_inputs(case, seed=63)
+    outs = []
+    for shift in (0, 8):
+        dc, got = run_r0(case, r0, gate_shift=shift)
+        assert dc.read_status() == 0
+        outs.append(got)
+    np.testing.assert_array_equal(outs[0], outs[1])
 
 
 def test_r0_out_of_range_id_is_reported(gpu_lib):
