@@ -935,13 +935,15 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
   const int ocols = ncol * (kF32Heads / 4), ogroups = min(kF32Threads / ocols, 8);
   const int ocol = tid % ncol, ohg = tid % ocols / ncol, og = tid / ocols;
   const bool oact = og < ogroups && 4 * ohg < H;
+  // a page past the block table's row is out of range like any other bad id
+  auto page_of = [&](int lp) { return lp < max_pages ? block_table[static_cast<size_t>(b) * max_pages + lp] : -1; };
   while (g < g1) {
     const int pend = min(g1, cu[b + 1]);
     const int L = seq_lens[b];
     const int s0 = cu[b] + kSegCost;   // unit of the sequence's first page
     const int lp0 = max(g - s0, 0), lp1 = pend - s0;
     if (min(lp1 * kPage, L) <= lp0 * kPage) break;   // the range ends inside the sequence's start cost
-    int page = block_table[static_cast<size_t>(b) * max_pages + lp0];   // (requested before the query block)
+    int page = page_of(lp0);   // (requested before the query block)
     {
       // warp = head
       const float* qsrc = reinterpret_cast<const float*>(qprep + static_cast<size_t>(b) * qstride);
@@ -968,7 +970,7 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
     float mrun = -INFINITY, lrun = 0.f;   // head `warp`, the same in every lane
     for (int lp = lp0; lp < lp1; ++lp) {
       const int ntok = min(kPage, L - lp * kPage);
-      if (lp > lp0) page = block_table[static_cast<size_t>(b) * max_pages + lp];
+      if (lp > lp0) page = page_of(lp);
       const bool page_ok = page >= 0 && page < num_pages;
       if (!page_ok && tid == 0) report_status(status, kStatusOutOfRange);
       const size_t row0 = static_cast<size_t>(page_ok ? page : 0) * kPage;

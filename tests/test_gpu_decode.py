@@ -443,6 +443,24 @@ def test_out_of_range_page_is_reported(gpu_lib):
     assert dc.read_status() == _lib.EG_MLA_ERR_OUT_OF_RANGE
 
 
+def test_fp32_sequence_past_its_block_table_is_reported(gpu_lib):
+    """A device-side length of more pages than the block table has: nothing is
+    read behind the table's last row (the pages past it count as out of range),
+    and the other sequence is right."""
+    case = synth.make_case("f32-past", synth.dims_tiny(), [150, 70], seed=40, layout="permuted")
+    dc = device.upload(case)
+    dc.append()
+    ref = orc.decode_unabsorbed(case)
+    dc.seq_lens[1] = 64 * dc.block_table.shape[1] + 100
+    for splits in (0, 1):
+        dc.num_splits = splits
+        dc.status.zero_()
+        dc.decode()
+        torch.cuda.synchronize()
+        assert dc.read_status() == _lib.EG_MLA_ERR_OUT_OF_RANGE
+        assert rel_l2(device.output_f64(dc.out)[0], ref[0]) <= F32_REL_L2
+
+
 # --------------------------------------------------------------------------- full-size workloads (sampled)
 def sampled_check(case, batches, num_splits=0):
     _, got = run(case, num_splits)
