@@ -60,6 +60,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 
@@ -1532,20 +1533,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   phase_mark<DBG == 2>(p, 3);
 }
 
-// CTAs of `kern` that the current device holds at once (1 per SM here), cached per kernel
-template <typename K>
-int resident_ctas(K kern, uint32_t smem) {
-  static int cached[64] = {0};
+// CTAs of Kern (with its one shared-memory size) that the current device holds at
+// once (1 per SM here), looked up once per kernel and device
+template <auto Kern>
+int resident_ctas(uint32_t smem) {
+  static std::atomic<int> cached[64];   // 0: not looked up yet
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (cached[dev] == 0) {
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
     int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kern, kThreads, smem) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return 0;
-    cached[dev] = std::max(0, per_sm) * sms;
+    n = std::max(0, per_sm) * sms;
+    cached[dev].store(n, std::memory_order_relaxed);
   }
-  return cached[dev];
+  return n;
 }
 
 template <int D_C, int GM, int DBG>
@@ -1602,7 +1606,8 @@ cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_
   p.stall_tile = a.stall_tile;
   // (the fused combine holds kCombineRowsPerWarp rows of W_UV,h per warp)
   p.fuse = DBG != 1 && D_C <= 256 && a.batch > 0 && kHeads * a.batch <= a.num_splits &&
-           a.d_v <= kCombineRowsPerWarp * (kThreads / 32) && a.num_splits <= resident_ctas(kern, C::SMEM);
+           a.d_v <= kCombineRowsPerWarp * (kThreads / 32) &&
+           a.num_splits <= resident_ctas<decode_tc_kernel<D_C, GM, DBG>>(C::SMEM);
   if (fused) *fused = p.fuse != 0;
   // The kernel may start while the query-absorption kernel before it on the
   // stream still runs (programmatic stream serialisation): its setup then
