@@ -372,10 +372,7 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
     if (!encode_decode_maps(maps, dims, c_pool, krope_pool, num_pages)) return EG_MLA_ERR_CUDA;
     apply_trace(a);
     apply_fault(a);
-    CUtensorMap amaps[2], wmap;
-    std::memset(&wmap, 0, sizeof(wmap));
-    const uint64_t dc = a.d_c, dv = a.d_v;
-    if (!encode_3d(&wmap, w_uv, dc, dv, a.H, dc, dv * dc, 128, 1)) return EG_MLA_ERR_CUDA;
+    CUtensorMap amaps[2];
     if (!encode_absorb_maps(amaps, a, egmla::absorb_tile(a.d_c, a.batch))) return EG_MLA_ERR_CUDA;
     cudaError_t e = egmla::launch_prologue_tc(a, app, amaps, st);
     bool fused = false;
@@ -384,7 +381,13 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
       e = egmla::launch_decode_tc(a, maps, false, st, &fused);
       prof_mark(st, false);
     }
-    if (e == cudaSuccess && !fused) e = egmla::launch_combine(a, true, &wmap, st);
+    if (e == cudaSuccess && !fused) {
+      CUtensorMap wmap;
+      std::memset(&wmap, 0, sizeof(wmap));
+      const uint64_t dc = a.d_c, dv = a.d_v;
+      if (!encode_3d(&wmap, w_uv, dc, dv, a.H, dc, dv * dc, 128, 1)) return EG_MLA_ERR_CUDA;
+      e = egmla::launch_combine(a, true, &wmap, st);
+    }
     return to_status(e);
   }
   cudaError_t e = egmla::launch_decode_f32(a, app, st);
