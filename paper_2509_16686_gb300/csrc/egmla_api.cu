@@ -61,38 +61,11 @@ int resolve_splits(int32_t num_splits, int32_t* out) {
   return EG_MLA_OK;
 }
 
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn get_encode() {
-  static EncodeFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeFn>(p);
-  });
-  return fn;
-}
-
 // bf16 tensor {d0, d1, d2} with strides s1, s2 (elements) in boxes {64, b1, b2},
 // 128-byte swizzle, elements past an end read as zero
 bool encode_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1, uint64_t s2,
                uint32_t b1, uint32_t b2) {
-  EncodeFn enc = get_encode();
-  if (enc == nullptr) return false;
-  const cuuint64_t dims[3] = {d0, d1, d2};
-  const cuuint64_t strides[2] = {s1 * 2, s2 * 2};
-  const cuuint32_t box[3] = {64, b1, b2};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return egmla::encode_map(map, base, {d0, d1, d2}, {s1, s2}, {64, b1, b2});
 }
 
 // maps = {latent pool, RoPE-key pool}: the latent as one 3-D box per tile, dims

@@ -6,6 +6,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 
 #include "../../include/egmla.h"
 
@@ -37,6 +38,57 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+inline EncodeFn encode_fn() {
+  static EncodeFn fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+            cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<EncodeFn>(p);
+  });
+  return fn;
+}
+
+// Map of a bf16 tensor of R dimensions (innermost first) with the strides of the
+// outer ones in elements; 128-byte swizzle, elements past an end read as zero and
+// are not written.
+template <size_t R>
+bool encode_map(CUtensorMap* map, const void* base, const uint64_t (&dims)[R], const uint64_t (&strides)[R - 1],
+                const uint32_t (&box)[R]) {
+  const EncodeFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  cuuint64_t d[R], s[R - 1];
+  cuuint32_t b[R], step[R];
+  for (size_t i = 0; i < R; ++i) {
+    d[i] = dims[i];
+    b[i] = box[i];
+    step[i] = 1;
+    if (i + 1 < R) s[i] = strides[i] * 2;
+  }
+  auto encode = [&] {
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, R, const_cast<void*>(base), d, s, b, step,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  if (r == CUDA_ERROR_INVALID_CONTEXT) {
+    // a host thread that has made no call on the device yet has no current context,
+    // which the encoder needs: cudaSetDevice makes the device's own current
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return false;
+    r = encode();
+  }
+  return r == CUDA_SUCCESS;
 }
 
 // Lets `kernel` be launched with up to `most` bytes of dynamic shared memory.  The

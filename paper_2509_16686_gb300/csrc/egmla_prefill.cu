@@ -41,7 +41,6 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
-#include <mutex>
 
 #include "egmla_common.cuh"
 #include "egmla_kernels.h"
@@ -1070,54 +1069,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 }
 
 // ---------------------------------------------------------------- host
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn pf_encode_fn() {
-  static EncodeFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeFn>(ptr);
-  });
-  return fn;
-}
-
 // bf16 planes of [rows, 64] with row stride `ld` and plane stride `plane`
 // elements; boxes of 64 columns x box_rows rows of one plane, 128-byte swizzle,
 // rows past the end read as zero and are not written
 bool pf_encode_planes(CUtensorMap* map, const void* base, uint64_t rows, uint64_t ld, uint64_t planes, uint64_t plane,
                       uint32_t box_rows) {
-  EncodeFn enc = pf_encode_fn();
-  if (enc == nullptr) return false;
   std::memset(map, 0, sizeof(*map));
-  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(kPfChunk), rows, planes};
-  const cuuint64_t strides[2] = {ld * 2, plane * 2};
-  const cuuint32_t box[3] = {static_cast<cuuint32_t>(kPfChunk), box_rows, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(map, base, {kPfChunk, rows, planes}, {ld, plane}, {kPfChunk, box_rows, 1});
 }
 
 // row-major bf16 [rows, cols] with row stride `ld` elements; boxes of 64
 // columns x 128 rows, 128-byte swizzle, rows past the end read as zero
 bool pf_encode(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld) {
-  EncodeFn enc = pf_encode_fn();
-  if (enc == nullptr) return false;
   std::memset(map, 0, sizeof(*map));
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {ld * 2};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(kPfChunk), static_cast<cuuint32_t>(kPfRows)};
-  const cuuint32_t estr[2] = {1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(map, base, {cols, rows}, {ld}, {kPfChunk, kPfRows});
 }
 
 struct PfWorkspace {

@@ -1,6 +1,7 @@
-"""Two host threads issuing calls of different shapes at once, each on its own
-stream with its own buffers (the binding releases the interpreter lock inside a
-call): every call is accepted and every output is bit for bit that of the call
+"""Calls from several host threads: two threads issuing calls of different shapes
+at once, each on its own stream with its own buffers (the binding releases the
+interpreter lock inside a call), and a thread whose first use of the GPU is the
+call.  Every call is accepted and every output is bit for bit that of the call
 alone."""
 import threading
 
@@ -102,3 +103,27 @@ def test_calls_of_two_threads_leave_each_other_alone(gpu_lib, name):
     for (_, out, status), want in zip(work, alone):
         assert int(status.item()) == 0
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("name", sorted(PAIRS))
+def test_call_from_a_thread_that_has_used_no_gpu_yet(gpu_lib, name):
+    bind, out, status = PAIRS[name]()[0]
+    call = bind(torch.cuda.current_stream())
+    call()
+    want = out.clone()
+    out.fill_(0)
+    torch.cuda.synchronize()
+    errors = []
+
+    def run():
+        try:
+            call()
+        except Exception as e:   # noqa: BLE001 - shown below
+            errors.append(e)
+
+    t = threading.Thread(target=run)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    assert int(status.item()) == 0 and torch.equal(out, want)
