@@ -31,7 +31,8 @@
 //                     K = 64 tokens; O^T stays in TMEM over a sequence
 //                     segment).  An issuing thread stalls while the tensor
 //                     pipe's queue is full, so the two MMA streams have a
-//                     thread each (which also does its own waits).
+//                     warp each (of which one thread does the waits; see
+//                     WARP_ISSUE).
 //   softmax (warps 0-3, one per TMEM lane quadrant: tokens 16w .. 16w + 15)
 //                     thread t reads two tokens x four heads of S; the
 //                     LayerNorm is applied after the MMA, since
@@ -639,6 +640,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr bool GATE_ADD = GM == 3;             // ablation: c + g
   constexpr bool GATE_LN = GM == 1 || GM == 3;   // LayerNorm after the gate
   using C = Cfg<D_C, GATE>;
+  // The MMA issuers: one thread of the warp, or (d_c 192 gated with a product) the
+  // whole warp waiting together and electing a thread for each tile's MMAs.  Steps
+  // replayed 24 to a graph, one thread / whole warp: d_c 192 with c (*) g 65.7 / 65.1
+  // us for 16 x 32K, 114.1 / 112.9 for 31 x 32K, 65.9 / 65.2 for 128 ragged
+  // sequences; with LN(c + g) 119.3 / 119.7 for 31 x 32K, and 79.9 / 84.2 at d_c 256
+  // (ragged); ungated 52.8 / 55.0 and, at d_c 256, 59.0 / 61.3 (ragged; there the warps
+  // also polled their queues); 124 / 135 at d_c 512, when its tiles had 36 short MMAs.
+  constexpr bool WARP_ISSUE = D_C == 192 && GATE && !GATE_ADD;
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte aligned base (128-byte swizzle atoms); derived by an offset from the
   // __shared__ array so that every access through it stays a shared-memory access
@@ -698,6 +707,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   // split schedule, zeroed counters) and the cache it may have appended to.
   grid_dependency_wait();
 
+  // an issuer's wait, the choice of the thread that issues, and the warp's joining after it
+  auto issuer_wait = [&](uint64_t& bar, uint32_t parity) {
+    return WARP_ISSUE ? warp_wait(smem_u32(&bar), parity, abort_flag, wait_ns)
+                      : mbar_wait(smem_u32(&bar), parity, abort_flag, wait_ns);
+  };
+  auto issuer_one = [] { return !WARP_ISSUE || elect_one(); };
+  auto issuer_join = [] {
+    if (WARP_ISSUE) __syncwarp();
+  };
+
   if (warp == kTmaWarp) {
     // ---------------------------------------------------------------- TMA producer
     // The whole warp walks the tiles; lane 0 waits for the slot and issues the
@@ -735,7 +754,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const uint32_t dst = sbase + slot * C::SLOT;
               const int y = pg * kPage + t.tok0 % kPage;
               tma_load_3d(dst, &cmap, 0, y, 0, fb, pol_stream);
-              tma_load_3d(dst + C::KR_OFF, &krmap, 0, y, 0, fb, pol_stream);
+              tma_load_2d(dst + C::KR_OFF, &krmap, 0, y, fb, pol_stream);
               // the page's token ids, into the half of the slot's statistics that
               // holds r once the gate has read them
               if (C::ID_TX)
@@ -774,17 +793,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------------- score MMAs, query blocks
-    // One thread waits and issues.  Scores of tile js: at a segment start the
-    // segment's query block, a free score buffer (the softmax warps read tile
-    // js - kNB's), and the gated page.  The next segment's query block is
-    // requested once its buffer's previous segment is done with it (last score
-    // MMA complete, sums read by the softmax warps), tested after every tile.
-    // A warp that polled both queues, voted and elected for every tile took
-    // 135 us of the d_c 512 step where this took 124 (then 36 MMAs per 32 tokens,
-    // short, so that what lies between tiles counts), 48.4 instead of 47.9 of the
-    // 8 x 32K step, and 68.3 instead of 69.3 of 128 ragged sequences at d_c 192.
-    // Loops are unrolled with compile-time accumulate flags.
-    if (!DUMP && elect_one()) {
+    // Scores of tile js: at a segment start the segment's query block, a free score
+    // buffer (the softmax warps read tile js - kNB's), and the gated page.  The
+    // next segment's query block is requested once its buffer's previous segment
+    // is done with it (last score MMA complete, sums read by the softmax warps),
+    // tested after every tile.  Loops are unrolled with compile-time accumulate
+    // flags.
+    if (!DUMP && (WARP_ISSUE || elect_one())) {
       constexpr uint32_t IDESC_S = idesc_bf16(64, kHeads, 0, 0);
       // A operand: the page slot, 128-byte swizzled, K-major (tokens x
       // features); B: the query block in 8x8 core matrices, K cores 256 B
@@ -809,6 +824,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool issued = false;
       Tracer tr;
       tr.init(p, 1, 0, 2);
+      if (WARP_ISSUE && lane != 0) tr.base = nullptr;
       auto find_query = [&]() {
         while (q_walk) {
           q_more = wq.next(tq);
@@ -818,11 +834,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the next segment's query block (its buffer is free)
       auto load_query = [&]() {
         const int qb = qn % C::NQ;
-        mbar_arrive_expect_tx(smem_u32(&bars.qfull[qb]), C::QPREP);
-        bulk_load(sbase + C::OFF_QBUF + qb * C::QBUF, p.qprep + static_cast<size_t>(tq.b) * C::QPREP, C::QPREP,
-                  smem_u32(&bars.qfull[qb]));
+        if (issuer_one()) {
+          mbar_arrive_expect_tx(smem_u32(&bars.qfull[qb]), C::QPREP);
+          bulk_load(sbase + C::OFF_QBUF + qb * C::QBUF, p.qprep + static_cast<size_t>(tq.b) * C::QPREP, C::QPREP,
+                    smem_u32(&bars.qfull[qb]));
+        }
+        issuer_join();
         ++qn;
         q_walk = true;
+      };
+      auto query_free = [&]() {   // the next query block's buffer, tested without waiting
+        const uint32_t bar = smem_u32(&bars.qempty[qn % C::NQ]), parity = ((qn / C::NQ) & 1) ^ 1;
+        return WARP_ISSUE ? warp_test(bar, parity) : mbar_test_now(bar, parity);
       };
       for (int js = 0; ws.next(ts); ++js) {
         const int slot = js % C::NS, sb = js % kNB;
@@ -831,48 +854,50 @@ __global__ void __launch_bounds__(kThreads, 1)
           ++seg;
           if (qn <= seg) {
             find_query();
-            ok = mbar_wait(smem_u32(&bars.qempty[seg % C::NQ]), ((seg / C::NQ) & 1) ^ 1, abort_flag, wait_ns);
+            ok = issuer_wait(bars.qempty[seg % C::NQ], ((seg / C::NQ) & 1) ^ 1);
             if (ok) load_query();
           }
         }
-        if (ts.first)
-          ok = ok && mbar_wait(smem_u32(&bars.qfull[seg % C::NQ]), (seg / C::NQ) & 1, abort_flag, wait_ns);
-        ok = ok && mbar_wait(smem_u32(&bars.sfree[sb]), ((js / kNB) & 1) ^ 1, abort_flag, wait_ns);
-        ok = ok && mbar_wait(smem_u32(&bars.zready[slot]), (js / C::NS) & 1, abort_flag, wait_ns);
+        if (ts.first) ok = ok && issuer_wait(bars.qfull[seg % C::NQ], (seg / C::NQ) & 1);
+        ok = ok && issuer_wait(bars.sfree[sb], ((js / kNB) & 1) ^ 1);
+        ok = ok && issuer_wait(bars.zready[slot], (js / C::NS) & 1);
         if (!ok) break;
         tr.mark(1, js);
-        mbar_arrive(smem_u32(&bars.sready[sb]));
         tc_fence_after();
-        const uint64_t za = zdesc_k + ((slot * C::SLOT) >> 4);
-        const uint64_t qb = qdesc0 + (((seg % C::NQ) * C::QBUF) >> 4);
-        const uint32_t ds = tmem + C::COL_S + sb * C::S_COLS;
-        if constexpr (C::TOK < kPage) {
-          const uint64_t qb2 = qdesc2 + (((seg % C::NQ) * C::QBUF) >> 4);
+        if (issuer_one()) {
+          mbar_arrive(smem_u32(&bars.sready[sb]));
+          const uint64_t za = zdesc_k + ((slot * C::SLOT) >> 4);
+          const uint64_t qb = qdesc0 + (((seg % C::NQ) * C::QBUF) >> 4);
+          const uint32_t ds = tmem + C::COL_S + sb * C::S_COLS;
+          if constexpr (C::TOK < kPage) {
+            const uint64_t qb2 = qdesc2 + (((seg % C::NQ) * C::QBUF) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < D_C / 32; ++kk)
-            mma_bf16_ss(ds, za + (((kk >> 2) * 2 * C::PCHUNK + (kk & 3) * 32) >> 4),
-                        qb2 + ((kk * 4 * kQGroupBytes) >> 4), IDESC_S2, kk > 0);
+            for (int kk = 0; kk < D_C / 32; ++kk)
+              mma_bf16_ss(ds, za + (((kk >> 2) * 2 * C::PCHUNK + (kk & 3) * 32) >> 4),
+                          qb2 + ((kk * 4 * kQGroupBytes) >> 4), IDESC_S2, kk > 0);
 #pragma unroll
-          for (int kk = 0; kk < kRope / 16; ++kk)
-            mma_bf16_ss(ds, za + ((C::KR_OFF + kk * 32) >> 4),
-                        qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, 1);
-        } else {
+            for (int kk = 0; kk < kRope / 16; ++kk)
+              mma_bf16_ss(ds, za + ((C::KR_OFF + kk * 32) >> 4),
+                          qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, 1);
+          } else {
 #pragma unroll
-          for (int kk = 0; kk < D_C / 16; ++kk)
-            mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
-                        qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+            for (int kk = 0; kk < D_C / 16; ++kk)
+              mma_bf16_ss(ds, za + (((kk >> 2) * C::PCHUNK + (kk & 3) * 32) >> 4),
+                          qb + ((kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
 #pragma unroll
-          for (int kk = 0; kk < kRope / 16; ++kk)
-            mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
-                        qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+            for (int kk = 0; kk < kRope / 16; ++kk)
+              mma_bf16_ss(ds + kHeads, za + ((C::KR_OFF + kk * 32) >> 4),
+                          qb + ((C::QB_LAT + kk * 2 * kQGroupBytes) >> 4), IDESC_S, kk > 0);
+          }
+          mma_commit(smem_u32(&bars.sready[sb]));
+          if (ts.last) mma_commit(smem_u32(&bars.qempty[seg % C::NQ]));
         }
-        mma_commit(smem_u32(&bars.sready[sb]));
-        if (ts.last) mma_commit(smem_u32(&bars.qempty[seg % C::NQ]));
+        issuer_join();
         tr.mark(2, js);
         issued = true;
         // (after the tile's MMAs: finding the next segment takes global loads)
         find_query();
-        if (q_more && mbar_test_now(smem_u32(&bars.qempty[qn % C::NQ]), ((qn / C::NQ) & 1) ^ 1)) load_query();
+        if (q_more && query_free()) load_query();
       }
       // drain: the query-block copies land and every MMA finishes before the
       // CTA exits and TMEM is released (own flag: bounded but not cut short by
@@ -881,7 +906,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int n = qn > C::NQ ? qn - C::NQ : 0; n < qn; ++n)
         if (!mbar_wait(smem_u32(&bars.qfull[n % C::NQ]), (n / C::NQ) & 1, &own, wait_ns)) *abort_flag = 1;
       if (issued) {
-        mma_commit(smem_u32(&bars.drain_s));
+        if (issuer_one()) mma_commit(smem_u32(&bars.drain_s));
+        issuer_join();
         if (!mbar_wait(smem_u32(&bars.drain_s), 0, &own, wait_ns)) *abort_flag = 1;
       }
     }
@@ -894,7 +920,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // 64-feature atoms PCHUNK apart; tokens along K, 8-row groups 1 KB apart);
     // B: P' MN-major in 8x8 core matrices (token groups 256 B, head halves
     // 128 B).
-    if (!DUMP && elect_one()) {
+    if (!DUMP && (WARP_ISSUE || elect_one())) {
       constexpr uint32_t IDESC_O = idesc_bf16(128, kHeads, 1, 1);
       const uint64_t zdesc_mn = smem_desc(sbase, C::PCHUNK, 1024, kSwizzle128B);
       const uint64_t pdesc0 = smem_desc(sbase + C::OFF_PBUF, 256, 128, kSwizzleNone);
@@ -904,27 +930,32 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool issued = false;
       Tracer tr;
       tr.init(p, 1, 1, 2);   // second half of the MMA role's run
+      if (WARP_ISSUE && lane != 0) tr.base = nullptr;
       for (int jo = 0; wo.next(to); ++jo) {
-        if (!mbar_wait(smem_u32(&bars.spdone[jo % kNP]), (jo / kNP) & 1, abort_flag, wait_ns)) break;
+        if (!issuer_wait(bars.spdone[jo % kNP], (jo / kNP) & 1)) break;
         tr.mark(3, jo);
         tc_fence_after();
-        const int slot = jo % C::NS;
-        const uint64_t za = zdesc_mn + ((slot * C::SLOT) >> 4);
-        const uint64_t pb = pdesc0 + (((jo % kNP) * C::PBUF) >> 4);
-        const uint32_t keep = to.first ? 0u : 1u;   // a segment's first MMAs overwrite O^T
+        if (issuer_one()) {
+          const int slot = jo % C::NS;
+          const uint64_t za = zdesc_mn + ((slot * C::SLOT) >> 4);
+          const uint64_t pb = pdesc0 + (((jo % kNP) * C::PBUF) >> 4);
+          const uint32_t keep = to.first ? 0u : 1u;   // a segment's first MMAs overwrite O^T
 #pragma unroll
-        for (int ks = 0; ks < C::TOK / 16; ++ks)
+          for (int ks = 0; ks < C::TOK / 16; ++ks)
 #pragma unroll
-          for (int mc = 0; mc < C::NMC; ++mc)
-            mma_bf16_ss(tmem + C::COL_O + kHeads * mc, za + (((C::mc_start(mc) / 64) * C::PCHUNK + ks * 2048) >> 4),
-                        pb + ((ks * 512) >> 4), IDESC_O, ks > 0 ? 1u : keep);
-        mma_commit(smem_u32(&bars.empty[slot]));
-        mma_commit(smem_u32(&bars.pfree[jo % kNP]));
+            for (int mc = 0; mc < C::NMC; ++mc)
+              mma_bf16_ss(tmem + C::COL_O + kHeads * mc, za + (((C::mc_start(mc) / 64) * C::PCHUNK + ks * 2048) >> 4),
+                          pb + ((ks * 512) >> 4), IDESC_O, ks > 0 ? 1u : keep);
+          mma_commit(smem_u32(&bars.empty[slot]));
+          mma_commit(smem_u32(&bars.pfree[jo % kNP]));
+        }
+        issuer_join();
         tr.mark(4, jo);
         issued = true;
       }
       if (issued) {
-        mma_commit(smem_u32(&bars.drain_o));
+        if (issuer_one()) mma_commit(smem_u32(&bars.drain_o));
+        issuer_join();
         volatile int own = 0;
         if (!mbar_wait(smem_u32(&bars.drain_o), 0, &own, wait_ns)) *abort_flag = 1;
       }
