@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -357,6 +358,20 @@ bool plan_smem(int nb, int bp, SmemPlan& sp) {
   return sp.smem <= static_cast<int>(kLinSmemLimit);
 }
 
+// once per device: a layer launches this kernel twice, and 0.4 us of host time each
+// show in a layer of few tokens
+cudaError_t allow_linear_smem() {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < 64;
+  if (known && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+  e = allow_smem(linear_tc_kernel, kLinSmemLimit);
+  if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_relaxed);
+  return e;
+}
+
 }  // namespace
 
 bool linear_tc_supported(int n_out, int k, int batch) {
@@ -366,7 +381,7 @@ bool linear_tc_supported(int n_out, int k, int batch) {
 cudaError_t linear_tc_plan(int n_out, int k, int batch, int* cluster, int* stages, int* max_clusters) {
   *cluster = *stages = *max_clusters = 0;
   if (n_out <= 0 || k <= 0 || batch <= 0) return cudaErrorInvalidValue;
-  cudaError_t e = allow_smem(linear_tc_kernel, kLinSmemLimit);
+  cudaError_t e = allow_linear_smem();
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
@@ -400,7 +415,7 @@ cudaError_t linear_tc_plan(int n_out, int k, int batch, int* cluster, int* stage
 cudaError_t launch_linear_tc(const void* w, int n_out, int k, const void* x, int batch, void* out, int ldo,
                              bool out_f32, int32_t* status, cudaStream_t st) {
   if (batch == 0) return cudaSuccess;
-  cudaError_t e = allow_smem(linear_tc_kernel, kLinSmemLimit);
+  cudaError_t e = allow_linear_smem();
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
