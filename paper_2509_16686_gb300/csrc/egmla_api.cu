@@ -71,14 +71,14 @@ bool encode_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uin
 // maps = {latent pool, RoPE-key pool}: the latent as one 3-D box per tile, dims
 // {64 features, rows, d_c / 64 feature columns}, so that one copy writes the
 // tile as its 128-byte-swizzled 64-feature columns one after another; tiles of
-// 64 rows, 32 at d_c 512; the RoPE keys in 2-D boxes of as many rows
+// 64 rows, 32 at d_c 512
 bool encode_decode_maps(CUtensorMap (&maps)[2], const eg_mla_dims* d, const void* c_pool, const void* krope_pool,
                         int32_t num_pages) {
   std::memset(maps, 0, sizeof(maps));
   const uint64_t rows = static_cast<uint64_t>(num_pages) * d->page_size, dc = d->d_c, dr = d->d_rope;
   const uint32_t tile = d->d_c <= 256 ? 64 : 32;
   return encode_3d(&maps[0], c_pool, 64, rows, dc / 64, dc, 64, tile, static_cast<uint32_t>(dc / 64)) &&
-         egmla::encode_map(&maps[1], krope_pool, {dr, rows}, {dr}, {64, tile});
+         encode_3d(&maps[1], krope_pool, dr, rows, 1, dr, rows * dr, tile, 1);
 }
 
 // maps of the tensor-core query absorption: {W_UK, q}

@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const uint32_t dst = sbase + slot * C::SLOT;
               const int y = pg * kPage + t.tok0 % kPage;
               tma_load_3d(dst, &cmap, 0, y, 0, fb, pol_stream);
-              tma_load_2d(dst + C::KR_OFF, &krmap, 0, y, fb, pol_stream);
+              tma_load_3d(dst + C::KR_OFF, &krmap, 0, y, 0, fb, pol_stream);
               // the page's token ids, into the half of the slot's statistics that
               // holds r once the gate has read them
               if (C::ID_TX)
