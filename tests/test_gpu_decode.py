@@ -90,8 +90,7 @@ def test_bf16_small_matches_oracle(gpu_lib, d_c, lens):
 @pytest.mark.parametrize("batch,d_nope", [(15, 128), (16, 40), (17, 128), (33, 256), (70, 72), (140, 128), (300, 64)])
 def test_bf16_query_absorption_tiles_match_oracle(gpu_lib, d_c, gate, batch, d_nope):
     """The query absorption at the edges of its tiles: sequences per block (16 to
-    128, part-filled last blocks, both sides of the batch from which it runs on
-    the tensor cores), d_nope below, on and off a multiple of 64, the
+    128, part-filled last blocks), d_nope below, on and off a multiple of 64, the
     overlapping feature tile of d_c 192; short contexts."""
     dims = synth.Dims(num_heads=16, d_nope=d_nope, d_rope=64, d_v=64, d_c=d_c, page_size=64, vocab=500, dtype="bf16",
                       gate=gate)
@@ -266,9 +265,9 @@ def test_bf16_empty_sequences(gpu_lib):
 def test_split_count_invariance(gpu_lib):
     case = small_bf16((1000, 37, 513))
     outs = []
-    # up to 152 splits the combine runs inside the decode kernel (cooperative
-    # launch); 400 exceeds the resident CTAs of the GPU, so it takes the
-    # separate combine kernel
+    # at 64 and 152 splits (16 per sequence or more, all CTAs resident at once)
+    # the combine runs inside the decode kernel (cooperative launch); below, and at
+    # 400, it is a kernel of its own
     for splits in (1, 2, 7, 64, 152, 400):
         _, got = run(case, splits)
         outs.append(got)
@@ -346,7 +345,8 @@ def test_step_equals_append_then_decode(gpu_lib, kind, splits):
     """eg_mla_step (the append inside the query-absorption grid on the bf16
     path, the split-KV kernel launched to overlap its setup with it) leaves the
     cache and the output bit-identical to eg_mla_append_latent followed by
-    eg_mla_decode; 400 splits take the unfused path (separate combine)."""
+    eg_mla_decode; 0 splits (one per SM) take the fused combine, the others the
+    separate one."""
     if kind == "fp32":
         case = synth.case_tiny()
     else:
@@ -430,6 +430,27 @@ def test_withheld_page_times_out_and_gpu_stays_usable(gpu_lib):
     check_bf16(got, orc.decode_unabsorbed(case), "after a timed-out step", scaled_abs=True)
     _, got = run(case, 0)
     check_bf16(got, orc.decode_unabsorbed(case), "after a timed-out step, default splits", scaled_abs=True)
+
+
+@pytest.mark.parametrize("d_c,gate,splits,cta,tile", [
+    (256, True, 64, 1, 0),     # the merge inside the kernel: other CTAs wait for this one's partial
+    (192, True, 4, 0, 2),      # the issuers as whole warps
+    (512, False, 4, 0, 3),     # half a page per tile
+])
+def test_withheld_page_times_out_in_every_form(gpu_lib, d_c, gate, splits, cta, tile):
+    """The test above in the kernel's other forms.  Every wait of the launch gives
+    up after 1 ms, every CTA returns, the next step is right."""
+    case = small_bf16((700, 65, 300), d_c=d_c, gate=gate)
+    dc = device.upload(case, num_splits=splits)
+    _lib.eg_mla_debug_set_fault(cta, tile, 1_000_000)
+    try:
+        dc.step()
+        torch.cuda.synchronize()
+    finally:
+        _lib.eg_mla_debug_set_fault(-1)
+    assert dc.read_status() == _lib.EG_MLA_ERR_TIMEOUT
+    _, got = run(case, splits)
+    check_bf16(got, orc.decode_unabsorbed(case), "after a timed-out step", scaled_abs=True)
 
 
 def test_out_of_range_page_is_reported(gpu_lib):
@@ -516,7 +537,7 @@ def growing_rope_case(d_c, gate, lens=(3000, 700, 1280), seed=23):
     return case
 
 
-@pytest.mark.parametrize("d_c,gate", [(256, True), (192, True), (256, False)])
+@pytest.mark.parametrize("d_c,gate", [(256, True), (192, True), (256, False), (512, False)])
 def test_rising_scores_move_the_reference_max(gpu_lib, d_c, gate):
     case = growing_rope_case(d_c, gate)
     ref = orc.decode_unabsorbed(case)
