@@ -107,9 +107,6 @@ struct PfGateParams {
 };
 
 constexpr int kGateWarps = 8;
-// token rows of a warp, their loads in flight together (2: 25.3 us for a call
-// over 777 tokens against 24.3, 187.7 against 185.8 for 16 ragged prompts)
-constexpr int kGateRows = 1;
 
 constexpr int kSortMaxBatch = 2048;   // larger batches keep the given order
 
@@ -125,12 +122,13 @@ __device__ __forceinline__ void load_features(const float* p, int f, float none,
   }
 }
 
-// A warp takes kGateRows consecutive token rows; NU 16-byte units of a row per
-// lane (d_c <= 256 NU).  Everything a row needs is requested before anything is
-// used: its latent, id, RoPE key and page, then its gate row.  Bound by that
-// chain's latency at few tokens and by DRAM at many (75 MB at 8 x 4096 with the
-// gate: 29 us with every row looped over as if 512 wide, 20 now).  gamma and
-// beta a float at a time cost more L1 accesses than the row's own data: the
+// A warp takes a token row; NU 16-byte units of it per lane (d_c <= 256 NU).
+// Everything the row needs is requested before anything is used: its latent, id,
+// RoPE key and page, then its gate row.  Bound by that chain's latency at few tokens
+// and by DRAM at many (75 MB at 8 x 4096 with the gate: 29 us with every row looped
+// over as if 512 wide, 20 now; two rows per warp in flight together: 25.3 us for a
+// call over 777 tokens against 24.3, 187.7 against 185.8 for 16 ragged prompts).
+// gamma and beta a float at a time cost more L1 accesses than the row's own data: the
 // call over 777 tokens 24.65 -> 24.3 us, 16 ragged prompts 187.5 -> 185.8.
 template <int NU>
 __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfGateParams p) {
@@ -155,120 +153,105 @@ __global__ void __launch_bounds__(32 * kGateWarps) prefill_gate_kernel(const PfG
       p.order[rank] = b;
     }
   }
-  const int t0 = (blockIdx.x * kGateWarps + warp) * kGateRows;
-  if (t0 >= p.total) return;
+  const int t = blockIdx.x * kGateWarps + warp;
+  if (t >= p.total) return;
   const int nu = p.d_c / 8;   // 16-byte units of a row
-  uint4 craw[kGateRows][NU], graw[kGateRows][NU], kraw[kGateRows];
-  int id[kGateRows], page[kGateRows], slot[kGateRows];
   bool bad = false;
+  uint4 craw[NU], graw[NU], kraw;
+  int id = p.ids ? __ldg(p.ids + t) : 0;
 #pragma unroll
-  for (int k = 0; k < kGateRows; ++k) {
-    const int t = min(t0 + k, p.total - 1);
-    id[k] = p.ids ? __ldg(p.ids + t) : 0;
-#pragma unroll
-    for (int i = 0; i < NU; ++i) {
-      const int u = lane + 32 * i;
-      craw[k][i] = make_uint4(0u, 0u, 0u, 0u);
-      if (u < nu) craw[k][i] = __ldg(reinterpret_cast<const uint4*>(p.c + static_cast<size_t>(t) * p.d_c) + u);
-    }
-    if (p.c_pool && lane < p.d_r / 8)
-      kraw[k] = __ldg(reinterpret_cast<const uint4*>(p.kr + static_cast<size_t>(t) * p.d_r) + lane);
+  for (int i = 0; i < NU; ++i) {
+    const int u = lane + 32 * i;
+    craw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (u < nu) craw[i] = __ldg(reinterpret_cast<const uint4*>(p.c + static_cast<size_t>(t) * p.d_c) + u);
+  }
+  if (p.c_pool && lane < p.d_r / 8)
+    kraw = __ldg(reinterpret_cast<const uint4*>(p.kr + static_cast<size_t>(t) * p.d_r) + lane);
+  if (p.gate && static_cast<unsigned>(id) >= static_cast<unsigned>(p.vocab)) {
+    bad = true;
+    id = 0;
   }
 #pragma unroll
-  for (int k = 0; k < kGateRows; ++k) {
-    const int t = min(t0 + k, p.total - 1);
-    const bool live = t0 + k < p.total;
-    if (p.gate && static_cast<unsigned>(id[k]) >= static_cast<unsigned>(p.vocab)) {
-      bad = bad || live;
-      id[k] = 0;
-    }
+  for (int i = 0; i < NU; ++i) {
+    const int u = lane + 32 * i;
+    graw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (p.gate && u < nu)
+      graw[i] = __ldg(reinterpret_cast<const uint4*>(p.gate_table + static_cast<size_t>(id) * p.d_c) + u);
+  }
+  int page = -1, slot = 0;
+  if (p.c_pool) {
+    // a row before the first prompt's start or past its prompt's end has no slot
+    // (inconsistent offsets: nothing is written, and it is reported below)
+    const int b = prompt_of_row(p.cu, p.batch, t), start = __ldg(p.cu + b), end = __ldg(p.cu + b + 1);
+    const int pos = start >= 0 && start <= t && t < end ? t - start : -1, lp = pos / kPage;
+    slot = pos % kPage;
+    page = pos >= 0 && lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
+  }
+  // c~ of the row
+  float z[NU][8];
 #pragma unroll
-    for (int i = 0; i < NU; ++i) {
-      const int u = lane + 32 * i;
-      graw[k][i] = make_uint4(0u, 0u, 0u, 0u);
-      if (p.gate && u < nu)
-        graw[k][i] = __ldg(reinterpret_cast<const uint4*>(p.gate_table + static_cast<size_t>(id[k]) * p.d_c) + u);
-    }
-    page[k] = -1;
-    if (p.c_pool) {
-      // a row before the first prompt's start or past its prompt's end has no slot
-      // (inconsistent offsets: nothing is written, and it is reported below)
-      const int b = prompt_of_row(p.cu, p.batch, t), start = __ldg(p.cu + b);
-      const int pos = start >= 0 && start <= t && t < __ldg(p.cu + b + 1) ? t - start : -1, lp = pos / kPage;
-      slot[k] = pos % kPage;
-      page[k] = pos >= 0 && lp < p.max_pages ? __ldg(p.block_table + static_cast<size_t>(b) * p.max_pages + lp) : -1;
+  for (int i = 0; i < NU; ++i) {
+    const __nv_bfloat162* c2 = reinterpret_cast<const __nv_bfloat162*>(&craw[i]);
+    const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&graw[i]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 cf = __bfloat1622float2(c2[e]);
+      float2 v = cf;
+      if (p.gate) {
+        const float2 gf = __bfloat1622float2(g2[e]);
+        v = p.gate_add ? make_float2(cf.x + gf.x, cf.y + gf.y) : make_float2(cf.x * gf.x, cf.y * gf.y);
+      }
+      z[i][2 * e] = v.x;   // (units past the row: 0)
+      z[i][2 * e + 1] = v.y;
     }
   }
+  if (p.gate && p.gate_ln) {
+    float sum = 0.f;
 #pragma unroll
-  for (int k = 0; k < kGateRows; ++k) {
-    const int t = t0 + k;
-    if (t >= p.total) break;
-    // c~ of the row
-    float z[NU][8];
+    for (int i = 0; i < NU; ++i)
 #pragma unroll
-    for (int i = 0; i < NU; ++i) {
-      const __nv_bfloat162* c2 = reinterpret_cast<const __nv_bfloat162*>(&craw[k][i]);
-      const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&graw[k][i]);
+      for (int e = 0; e < 8; ++e) sum += z[i][e];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 cf = __bfloat1622float2(c2[e]);
-        float2 v = cf;
-        if (p.gate) {
-          const float2 gf = __bfloat1622float2(g2[e]);
-          v = p.gate_add ? make_float2(cf.x + gf.x, cf.y + gf.y) : make_float2(cf.x * gf.x, cf.y * gf.y);
-        }
-        z[i][2 * e] = v.x;   // (units past the row: 0)
-        z[i][2 * e + 1] = v.y;
-      }
-    }
-    if (p.gate && p.gate_ln) {
-      float sum = 0.f;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const float mu = sum / p.d_c;
+    float q = 0.f;
 #pragma unroll
-      for (int i = 0; i < NU; ++i)
+    for (int i = 0; i < NU; ++i)
+      if (lane + 32 * i < nu)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) sum += z[i][e];
+        for (int e = 0; e < 8; ++e) q = fmaf(z[i][e] - mu, z[i][e] - mu, q);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      const float mu = sum / p.d_c;
-      float q = 0.f;
-#pragma unroll
-      for (int i = 0; i < NU; ++i)
-        if (lane + 32 * i < nu)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) q = fmaf(z[i][e] - mu, z[i][e] - mu, q);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      const float r = rsqrtf(q / p.d_c + p.eps);
-#pragma unroll
-      for (int i = 0; i < NU; ++i) {
-        const int u = lane + 32 * i;
-        if (u >= nu) continue;
-        float gm[8], bt[8];
-        load_features(p.gamma, 8 * u, 1.f, gm);
-        load_features(p.beta, 8 * u, 0.f, bt);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) z[i][e] = fmaf((z[i][e] - mu) * r, gm[e], bt[e]);
-      }
-    }
-    const bool write = page[k] >= 0 && page[k] < p.num_pages;
-    if (p.c_pool && !write) bad = true;
-    const size_t row = write ? static_cast<size_t>(page[k]) * kPage + slot[k] : 0;
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    const float r = rsqrtf(q / p.d_c + p.eps);
 #pragma unroll
     for (int i = 0; i < NU; ++i) {
       const int u = lane + 32 * i;
       if (u >= nu) continue;
-      uint4 o;
-      o.x = pack_bf16x2(z[i][0], z[i][1]);
-      o.y = pack_bf16x2(z[i][2], z[i][3]);
-      o.z = pack_bf16x2(z[i][4], z[i][5]);
-      o.w = pack_bf16x2(z[i][6], z[i][7]);
-      reinterpret_cast<uint4*>(p.ctil + static_cast<size_t>(t) * p.d_c)[u] = o;
-      if (p.c_pool && write) reinterpret_cast<uint4*>(p.c_pool + row * p.d_c)[u] = craw[k][i];
+      float gm[8], bt[8];
+      load_features(p.gamma, 8 * u, 1.f, gm);
+      load_features(p.beta, 8 * u, 0.f, bt);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) z[i][e] = fmaf((z[i][e] - mu) * r, gm[e], bt[e]);
     }
-    if (p.c_pool && write) {
-      if (lane < p.d_r / 8) reinterpret_cast<uint4*>(p.kr_pool + row * p.d_r)[lane] = kraw[k];
-      if (lane == 0 && p.id_pool && p.ids) p.id_pool[row] = __ldg(p.ids + t);
-    }
+  }
+  const bool write = page >= 0 && page < p.num_pages;
+  if (p.c_pool && !write) bad = true;
+  const size_t row = write ? static_cast<size_t>(page) * kPage + slot : 0;
+#pragma unroll
+  for (int i = 0; i < NU; ++i) {
+    const int u = lane + 32 * i;
+    if (u >= nu) continue;
+    uint4 o;
+    o.x = pack_bf16x2(z[i][0], z[i][1]);
+    o.y = pack_bf16x2(z[i][2], z[i][3]);
+    o.z = pack_bf16x2(z[i][4], z[i][5]);
+    o.w = pack_bf16x2(z[i][6], z[i][7]);
+    reinterpret_cast<uint4*>(p.ctil + static_cast<size_t>(t) * p.d_c)[u] = o;
+    if (write) reinterpret_cast<uint4*>(p.c_pool + row * p.d_c)[u] = craw[i];
+  }
+  if (write) {
+    if (lane < p.d_r / 8) reinterpret_cast<uint4*>(p.kr_pool + row * p.d_r)[lane] = kraw;
+    if (lane == 0 && p.id_pool && p.ids) p.id_pool[row] = __ldg(p.ids + t);
   }
   if (bad && lane == 0) report_status(p.status, kStatusOutOfRange);
 }
@@ -1149,7 +1132,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st, void (*mark)(c
   gp.gate_ln = a.gate_ln;
   gp.eps = a.eps;
   gp.status = a.status;
-  const dim3 gate_grid((a.total + kGateWarps * kGateRows - 1) / (kGateWarps * kGateRows));
+  const dim3 gate_grid((a.total + kGateWarps - 1) / kGateWarps);
   cudaError_t e = a.d_c <= 256
                       ? launch_chained(prefill_gate_kernel<1>, gate_grid, dim3(32 * kGateWarps), 0, st, gp)
                       : launch_chained(prefill_gate_kernel<2>, gate_grid, dim3(32 * kGateWarps), 0, st, gp);
