@@ -180,9 +180,11 @@ def max_over_ranks(ms, dist, device):
 
 def combine_fused(d, batch, splits, sms):
     """Whether the decode kernel merges the splits and applies W_UV itself (bf16,
-    d_c 192/256, a grid of at most one CTA per SM with a CTA for every sequence
-    and head) or leaves that to the combine kernel after it."""
-    return d.dtype == "bf16" and d.d_c in (192, 256) and splits <= sms and 16 * batch <= splits
+    d_c 192/256, at most nine rows of W_UV,h for each of its 15 warps, a grid
+    resident at once, that is of at most one CTA per SM, with a CTA for every
+    sequence and head) or leaves that to the combine kernel after it."""
+    return (d.dtype == "bf16" and d.d_c in (192, 256) and d.d_v <= 9 * 15 and splits <= sms
+            and 16 * batch <= splits)
 
 
 def algorithmic_bytes(case, cache_bytes, fused):

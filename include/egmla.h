@@ -291,14 +291,15 @@ typedef struct {
                          cache with its own W_UK, W_UV, gate table and LayerNorm */
 } eg_mla_layer_dims;
 
-/* Device pointers of one layer's weights, each 16-byte aligned, in the
- * PyTorch Linear layout [out, in] of the model dtype (bf16) unless stated. */
+/* Device pointers of one layer's weights, each 16-byte aligned (gate_table 32, as
+ * for eg_mla_decode), in the PyTorch Linear layout [out, in] of the model dtype
+ * (bf16) unless stated. */
 typedef struct {
   const void* w_qkv_a;      /* [H (d_nope + d_rope) + d_c + d_rope, E]: the rows of
                                W^Q, then those of W^{DKV,KR} (one projection GEMM) */
   const void* kv_norm_w;    /* [d_c] */
   const void* w_o;          /* [E, H d_v] */
-  const void* gate_table;   /* [vocab, d_c]  as for eg_mla_decode */
+  const void* gate_table;   /* [vocab, d_c] as for eg_mla_decode; 32-byte aligned */
   const float* ln_gamma;    /* [d_c] fp32 or NULL, as for eg_mla_decode */
   const float* ln_beta;     /* [d_c] fp32 or NULL */
   const void* w_uk;         /* [H, d_nope, d_c] */
@@ -335,13 +336,15 @@ size_t eg_mla_layer_attn_offset(const eg_mla_dims* dims, const eg_mla_layer_dims
  *   y          [batch, E] bf16 output, caller-owned
  *   workspace  >= eg_mla_layer_workspace_size(...) bytes, 256-byte aligned
  *
- The projections run in this library's weight-streaming tcgen05 GEMM
+ * The projections run in this library's weight-streaming tcgen05 GEMM
  * (fp32 accumulation, the reduction dimension split over the CTAs of a
  * thread-block cluster and summed in rank order, so results do not depend on
- * timing).  The call allocates nothing.  The first call with a given shape
- * runs a host-side occupancy query for the GEMM's cluster size (cached
- * afterwards); make it before any stream capture.  Host-side argument errors
- * return a negative status and launch nothing; device errors go to
+ * timing).  The first one starts reading w_qkv_a while the kernel before the
+ * call on the stream may still run: that kernel must not be the one that writes
+ * w_qkv_a.  The call allocates nothing.  The first call with a given shape runs
+ * a host-side occupancy query for the GEMM's cluster size (cached afterwards);
+ * make it before any stream capture.  Host-side argument errors return a
+ * negative status and launch nothing; device errors go to
  * *dev_status as for eg_mla_decode.
  */
 int eg_mla_layer_decode(const eg_mla_dims* dims, const eg_mla_layer_dims* layer,
@@ -564,16 +567,16 @@ int eg_mla_debug_set_trace(void* dev_buf, int64_t bytes, int32_t ctas);
 
 /*
  * eg_mla_debug_set_fault - test entry for the failure path of the split-KV
- * decode kernel (d_c 192 and 256, bf16).  With cta >= 0, later eg_mla_decode
- * calls withhold one page copy: CTA `cta` skips the copy of its tile `tile`
- * (0-based in its walk) and its arrival, and every pipeline wait of those
- * launches gives up after wait_limit_ns (1 us .. 2 s) instead of the default
+ * decode kernel (bf16).  With cta >= 0, later eg_mla_decode calls withhold one
+ * page copy: CTA `cta` skips the copy of its tile `tile` (0-based in its walk; a
+ * page, half a page at d_c 512) and its arrival, and every pipeline wait of
+ * those launches gives up after wait_limit_ns (1 us .. 2 s) instead of the default
  * 2 s.  The wait on the withheld page then runs out: the kernel records
  * EG_MLA_ERR_TIMEOUT in *dev_status, every role leaves its loop, the copies
  * and MMAs already issued are waited for, TMEM is freed and the kernel
- * returns; the rest of the grid reports the same status when its split merge
- * waits for the missing partial.  No fault, trap or hang is involved, and the
- * device stays usable.  cta < 0 restores normal operation.  Returns
+ * returns; where the split merge runs in the same kernel, the rest of the grid
+ * reports the same status when it waits for the missing partial.  No fault,
+ * trap or hang is involved, and the device stays usable.  cta < 0 restores normal operation.  Returns
  * EG_MLA_ERR_INVALID_ARG for a negative tile or a limit out of range.
  */
 int eg_mla_debug_set_fault(int32_t cta, int32_t tile, int64_t wait_limit_ns);

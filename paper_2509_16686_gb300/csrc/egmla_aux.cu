@@ -190,7 +190,7 @@ __device__ void schedule_block(const int32_t* seq_lens, int batch, int page_size
                                int num_splits, const int32_t* block_table, int max_pages, SplitStart* starts,
                                int32_t* smem, int words, int32_t* wsum) {
   if (seq_done != nullptr)
-    for (int i = threadIdx.x; i <= batch; i += blockDim.x) seq_done[i] = 0u;
+    for (int i = threadIdx.x; i < batch; i += blockDim.x) seq_done[i] = 0u;
   if (batch + 1 <= words) {
     page_prefix_sums_block(seq_lens, batch, page_size, cu, smem, wsum);
     __syncthreads();   // the prefix sums are visible to the whole block
@@ -223,7 +223,6 @@ constexpr int kPmThreads = 256;
 constexpr int kPmTile = 128;                    // features per block (the MMA's M)
 constexpr uint32_t kPmAtomRow = 128;            // bytes of a swizzled 64-element row
 constexpr int kPmMaxSeq = 128;                  // sequences per block, at most (the MMA's N)
-constexpr int kPmBlocks = 152;                  // one per SM
 constexpr int kPmMaxNope = 256;
 
 struct PmBars {
@@ -482,7 +481,6 @@ prologue_f32_kernel(const float* __restrict__ q, const float* __restrict__ w_uk,
 // thread; the caller's next __syncthreads makes what it stored visible.
 constexpr int kCombineSlots = 128;
 constexpr int kMergeMaxSeq = 16;         // sequences per block, at most
-constexpr int kMergeBlocks = 152;        // blocks wanted at most: one per SM
 
 template <int T>
 struct MergeShared {
@@ -496,7 +494,7 @@ struct MergeShared {
 // one block per SM
 int merge_group(int H, int batch, int most) {
   int nt = 1;
-  while (nt < most && H * ((batch + nt - 1) / nt) > kMergeBlocks) nt *= 2;
+  while (nt < most && H * ((batch + nt - 1) / nt) > kSms) nt *= 2;
   return nt;
 }
 
@@ -626,7 +624,7 @@ __device__ void merge_partials(MergeShared<TS>& sh, const int32_t* cu, const flo
 constexpr int kCombineThreads = 256;
 constexpr int kCombineGroup = 8;        // sequences per block, at most
 constexpr int kCombineMaxDc = 512;
-constexpr int kCombineBlocks = 304;     // two blocks per SM
+constexpr int kCombineBlocks = 2 * kSms;
 
 template <int PPT>
 __global__ void __launch_bounds__(kCombineThreads)
@@ -696,7 +694,8 @@ combine_kernel(const int32_t* __restrict__ cu, const float* __restrict__ part_ml
 // kernel does not fuse them.  A block takes (head h, `nt` sequences, 128 output
 // rows):
 //  - W_UV,h's rows (the MMA's M = 128 operand, K = d_c) are copied by TMA before
-//    the block waits for the decode kernel, which does not write them;
+//    the block waits for the decode kernel (which lets it start only when all that
+//    comes before that kernel is complete);
 //  - merge as in combine_kernel: weights per (sequence, slot) in shared memory,
 //    then thread t takes (sequence, 4 features) pairs; where the block has fewer
 //    pairs than threads, the slots are dealt to groups of threads whose sums
@@ -920,6 +919,9 @@ decode_f32_kernel(const float* __restrict__ c_pool, const float* __restrict__ kr
   float* al = pw + kPage * kF32Heads;                // [16]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the combine may start (with this trigger / without: 64 short sequences 38.4 / 38.9
+  // us, but 8 of 100 to 3000 tokens 25.2 / 24.2 and one of 3000 22.6 / 21.8); before
+  // its wait it only brings W_UV to L2
   grid_launch_dependents();
   grid_dependency_wait();
   const int total = cu[batch];
@@ -1190,7 +1192,7 @@ cudaError_t launch_append(const AppendArgs& a, cudaStream_t st) {
 int absorb_tile(int d_c, int batch) {
   const int mt = (d_c + kPmTile - 1) / kPmTile;
   int nt = 16;
-  while (nt < kPmMaxSeq && 16 * mt * ((batch + nt - 1) / nt) > kPmBlocks) nt *= 2;
+  while (nt < kPmMaxSeq && 16 * mt * ((batch + nt - 1) / nt) > kSms) nt *= 2;
   return nt;
 }
 

@@ -87,8 +87,8 @@ __host__ __device__ inline WorkspaceLayout workspace_layout(int batch, int num_s
   size_t off = 0;
   w.off_cu = off;
   off = align_up(off + static_cast<size_t>(batch + 1) * 4, 256);
-  // the fused combine's counters (zeroed by the prologue each call): [0] the
-  // CTAs done, [1 + b] the split partials of sequence b stored
+  // the fused combine's counters (zeroed by the prologue each call): the split
+  // partials of each sequence stored (the area is as large as the prefix sums')
   w.off_done = off;
   off = align_up(off + static_cast<size_t>(batch + 1) * 4, 256);
   w.off_start = off;

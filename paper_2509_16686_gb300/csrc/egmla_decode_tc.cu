@@ -111,7 +111,6 @@ struct Cfg {
   // about 150 us for 128 ragged sequences, five of 36 KB about 92 (562 MB: 3.7
   // and 6.1 TB/s; kernel alone, warm)
   static constexpr int TOK = D_C > 256 ? kPage / 2 : kPage;
-  static constexpr int TPP = kPage / TOK;               // tiles per page
   static constexpr uint32_t PCHUNK = TOK * 128;         // one atom column of a tile
   static constexpr uint32_t KR_OFF = NCH * PCHUNK;
   static constexpr uint32_t SLOT = KR_OFF + PCHUNK;     // latent + RoPE key of one tile
@@ -190,7 +189,7 @@ struct TcParams {
   // fused split combine (cooperative launch only): W_UV and output
   const __nv_bfloat16* w_uv;
   __nv_bfloat16* out;
-  uint32_t* seq_done;   // [1 + b] split partials of sequence b stored
+  uint32_t* seq_done;   // [b]: the split partials of sequence b stored
   int d_v;
   int fuse, early;
   // limit of every wait (ns); a test entry lowers it, together with a
@@ -547,7 +546,7 @@ __device__ void fused_combine(const TcParams& p, uint8_t* smem, Bars& bars) {
       // every softmax warp's part of every split partial of the sequence stored
       const uint32_t want = static_cast<uint32_t>(kSoftWarps) * static_cast<uint32_t>(n);
       const uint64_t t0 = globaltimer();
-      while (ld_acquire_gpu(p.seq_done + 1 + b) < want) {
+      while (ld_acquire_gpu(p.seq_done + b) < want) {
         if (*abort_flag) break;
         if (globaltimer() - t0 > wait_ns) {
           report_status(p.status, kStatusTimeout);
@@ -777,7 +776,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (lane == 0) {
       // The split combine may take its place once every CTA's last page is
-      // requested, a few microseconds before this kernel ends (at the start it
+      // requested, a few microseconds before this kernel ends.  Never before this
+      // kernel's wait: the combine copies W_UV before its own, and only this wait
+      // stands for the kernel before the call, which may write W_UV.  (At the start it
       // would crowd its blocks onto the first SMs to free up: 128 ragged
       // sequences 69.8 us against 68.2).  128 at d_c 512 119.7 -> 118.5 us, 32 x
       // 4K 37.7 -> 37.2, 64 x 8K layer 102.4 -> 101.5 (against a trigger at the
@@ -1535,7 +1536,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             if (lane == 0) {
               __threadfence();
-              atomicAdd(p.seq_done + 1 + t.b, 1u);
+              atomicAdd(p.seq_done + t.b, 1u);
             }
           }
         }
@@ -1620,13 +1621,16 @@ cudaError_t launch_one(const DecodeArgs& a, const CUtensorMap* maps, cudaStream_
   p.trace = static_cast<unsigned long long*>(a.trace);
   p.trace_ctas = a.trace_ctas;
   p.trace_cap = a.trace_cap;
-  // The split combine runs inside this kernel for the smallest batches, where
-  // a step is mostly latency, when every CTA of the grid can be resident at
-  // once (a cooperative launch guarantees it, or fails).  The launch then
-  // cannot overlap the kernel before it (about 2.5 us outside a graph), and more
-  // units than CTAs share a wait, so that at larger batches the separate
-  // combine is faster: 4 sequences 16.4 us fused, 17.9 apart; 8 x 32K 48.7 and
-  // 48.3; 32 x 4K 38.8 and 37.0 (both in a graph); 128 ragged 76.2 and 68.0.
+  // The split combine runs inside this kernel for the smallest batches, where a
+  // step is mostly latency, when every CTA of the grid can be resident at once (a
+  // cooperative launch guarantees it, or fails): a CTA for every sequence and head.
+  // Beyond that, units share a wait, and the separate combine is faster.  us per
+  // step, fused / apart: replayed 24 to a graph at d_c 256, 4 x 100 12.0 / 13.4, 9 x
+  // 100 12.4 / 14.1, 8 x 32K 43.8 / 45.6, 9 x 32K 48.2 / 49.7, 10 x 100 14.7 / 13.9,
+  // 10 x 32K 53.0 / 53.7, 12 x 8K 27.9 / 26.9, 32 x 8K 52.8 / 46.8; at d_c 192, 9 x 1K
+  // 13.2 / 15.0, 10 x 1K 15.5 / 14.9, 10 x 32K 45.8 / 46.6, 12 x 32K 54.0 / 53.6.
+  // Issued eagerly, where a cooperative launch cannot overlap the kernel before it,
+  // the two are closer: 8 x 32K 46.9 / 46.5, 4 x 100 14.4 / 14.5, 4 x 8K 20.6 / 19.8.
   p.w_uv = static_cast<const __nv_bfloat16*>(a.w_uv);
   p.out = static_cast<__nv_bfloat16*>(a.out);
   p.seq_done = reinterpret_cast<uint32_t*>(ws + wl.off_done);

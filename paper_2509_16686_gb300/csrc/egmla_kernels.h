@@ -14,17 +14,25 @@ namespace egmla {
 
 // Launch with programmatic stream serialisation: the grid is set up while the
 // kernel before it on the stream drains, instead of after it has completed and
-// flushed.  Every kernel launched this way executes grid_dependency_wait
-// before its first access to global memory, in every block, so it (and what
-// waits for it) runs after everything before it on the stream.  A kernel that
-// is followed by another of the same call lets it start early
-// (grid_launch_dependents) only where that one's blocks take a whole SM each:
+// flushed.  What holds the order:
+//  - every block of a kernel launched this way executes grid_dependency_wait,
+//    and before it touches nothing that a kernel before it writes, and writes
+//    nothing, so that a completed kernel stands for everything before it;
+//  - before the wait a kernel may read inputs that no kernel of the call writes:
+//    the split combine copies W_UV, the fp32 one brings it to L2, the projection
+//    GEMM copies its weights.  The caller's kernel before the call may write
+//    W_UV: the combine must not start before that one is complete, so the bf16
+//    split-KV kernel triggers a separate combine only after its own wait.  (An
+//    L2 prefetch reads nothing that could be old.  The first projection's weights
+//    must not be written by the kernel directly before the layer call.)
+// A kernel lets its successor start early (grid_launch_dependents) where that was
+// measured to pay: mostly where the successor's blocks take a whole SM each, since
 // smaller blocks, started early, crowd onto the first SMs to free up (the R0
 // attention took 42 us instead of 33, the layer's query absorption 13 instead
-// of 8).  Measured, whole calls against plain launches: one 777-token prefill
-// 34.8 -> 26.8 us, the fp32 step 38.9 -> 32.6, 8 x 32K decode step 51.2 -> 48.9,
-// 128 ragged sequences 84.2 -> 81.7, the d_c 512 step 188 -> 186, a layer of
-// 64 x 8K 119.6 -> 115.1, R0 at 8 x 4K 169.6 -> 164.0.
+// of 8); the figures stand at the triggers.  Whole calls against plain launches:
+// one 777-token prefill 34.8 -> 26.8 us, the fp32 step 38.9 -> 32.6, 8 x 32K decode
+// step 51.2 -> 48.9, 128 ragged sequences 84.2 -> 81.7, the d_c 512 step 188 -> 186,
+// a layer of 64 x 8K 119.6 -> 115.1, R0 at 8 x 4K 169.6 -> 164.0.
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -39,6 +47,10 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+
+// SMs of a GB300: what the tile sizes of the small kernels aim at (their results do
+// not depend on it; grids that must cover the device ask it)
+constexpr int kSms = 152;
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
