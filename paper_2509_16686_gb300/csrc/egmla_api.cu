@@ -317,13 +317,15 @@ int fill_append_args(egmla::AppendArgs& a, const eg_mla_dims* dims, void* c_pool
 }
 
 // eg_mla_decode, preceded by the append of `app` when it is non-null (in the
-// query-absorption kernel's grid).  Every argument is checked before anything is launched.
+// query-absorption kernel's grid).  Every argument is checked before anything is
+// launched (`launch` false: checked only).
 int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, const void* krope_pool,
                 const int32_t* id_pool, const int32_t* block_table, int32_t max_pages_per_seq,
                 const int32_t* seq_lens, int32_t max_seq_len, int32_t batch, int32_t num_pages,
                 const void* gate_table, const float* ln_gamma, const float* ln_beta, const void* w_uk,
                 const void* w_uv, void* out, int32_t num_splits, void* workspace, size_t workspace_bytes,
-                int32_t* dev_status, const egmla::AppendArgs* app, cudaStream_t st, bool early = false) {
+                int32_t* dev_status, const egmla::AppendArgs* app, cudaStream_t st, bool early = false,
+                bool launch = true) {
   DecodeArgs a;
   int rc = fill_decode_args(a, dims, c_pool, krope_pool, id_pool, block_table, max_pages_per_seq, seq_lens,
                             max_seq_len, batch, num_pages, gate_table, num_splits, workspace, workspace_bytes,
@@ -333,6 +335,7 @@ int decode_impl(const eg_mla_dims* dims, const void* q, const void* c_pool, cons
   if (q == nullptr || w_uk == nullptr || w_uv == nullptr || out == nullptr) return EG_MLA_ERR_INVALID_ARG;
   // q, W_UK and W_UV rows are read in 16-byte pieces
   if (!aligned(w_uv, 16) || !aligned(w_uk, 16) || !aligned(q, 16)) return EG_MLA_ERR_INVALID_ARG;
+  if (!launch) return EG_MLA_OK;
   a.q = q;
   a.ln_gamma = ln_gamma;
   a.ln_beta = ln_beta;
@@ -375,7 +378,8 @@ int egmla_layer_step(const eg_mla_dims* dims, bool append, void* c_pool, void* k
                      const void* q, const int32_t* block_table, int32_t max_pages_per_seq, const int32_t* seq_lens,
                      int32_t max_seq_len, int32_t batch, int32_t num_pages, const void* gate_table,
                      const float* ln_gamma, const float* ln_beta, const void* w_uk, const void* w_uv, void* out,
-                     int32_t num_splits, void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
+                     int32_t num_splits, void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream,
+                     bool launch) {
   egmla::AppendArgs app;
   if (append) {
     const int rc = fill_append_args(app, dims, c_pool, krope_pool, id_pool, c_new, krope_new, ids_new, block_table,
@@ -384,7 +388,7 @@ int egmla_layer_step(const eg_mla_dims* dims, bool append, void* c_pool, void* k
   }
   return decode_impl(dims, q, c_pool, krope_pool, id_pool, block_table, max_pages_per_seq, seq_lens, max_seq_len,
                      batch, num_pages, gate_table, ln_gamma, ln_beta, w_uk, w_uv, out, num_splits, workspace,
-                     workspace_bytes, dev_status, append ? &app : nullptr, static_cast<cudaStream_t>(stream), true);
+                     workspace_bytes, dev_status, append ? &app : nullptr, static_cast<cudaStream_t>(stream), true, launch);
 }
 
 namespace {

@@ -267,10 +267,11 @@ cudaError_t linear_tc_plan(int n_out, int k, int batch, int* cluster, int* stage
 
 // The step inside eg_mla_layer_decode (egmla_api.cu): eg_mla_step (`append`)
 // or eg_mla_decode, whose split-KV kernel lets the output projection after it
-// start early.
+// start early.  `launch` false: its arguments are checked and nothing is launched.
 int egmla_layer_step(const eg_mla_dims* dims, bool append, void* c_pool, void* krope_pool, int32_t* id_pool,
                      const void* c_new, const void* krope_new, const int32_t* ids_new, const int32_t* positions,
                      const void* q, const int32_t* block_table, int32_t max_pages_per_seq, const int32_t* seq_lens,
                      int32_t max_seq_len, int32_t batch, int32_t num_pages, const void* gate_table,
                      const float* ln_gamma, const float* ln_beta, const void* w_uk, const void* w_uv, void* out,
-                     int32_t num_splits, void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream);
+                     int32_t num_splits, void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream,
+                     bool launch);

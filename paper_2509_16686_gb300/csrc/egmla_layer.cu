@@ -192,9 +192,19 @@ int eg_mla_layer_decode(const eg_mla_dims* dims, const eg_mla_layer_dims* layer,
   auto* krb = reinterpret_cast<__nv_bfloat16*>(base + ws.off_kr);
   void* ub = base + ws.off_u;
 
+  // the append (first layer of a group) and the decode as one step, whose
+  // arguments are checked before the projections are launched
+  const bool do_kv = layer->share_kv == 0;
+  auto step = [&](bool launch) {
+    return egmla_layer_step(dims, do_kv, c_pool, krope_pool, id_pool, cb, krb, ids_new, positions, qb, block_table,
+                            max_pages_per_seq, seq_lens, max_seq_len, batch, num_pages, wt->gate_table, wt->ln_gamma,
+                            wt->ln_beta, wt->w_uk, wt->w_uv, ub, num_splits, base + ws.off_dec, ws.dec_bytes,
+                            dev_status, stream, launch);
+  };
+  int rc = step(false);
+  if (rc != EG_MLA_OK) return rc;
   // the query and latent projections, fp32 out (a later layer of a layer
   // group projects only its query)
-  const bool do_kv = layer->share_kv == 0;
   if (egmla::launch_linear_tc(wt->w_qkv_a, do_kv ? nq + nkv : nq, E, x, batch, qkv32, nq + nkv, true, dev_status,
                               st) != cudaSuccess)
     return EG_MLA_ERR_CUDA;
@@ -204,11 +214,7 @@ int eg_mla_layer_decode(const eg_mla_dims* dims, const eg_mla_layer_dims* layer,
       static_cast<const __nv_bfloat16*>(wt->kv_norm_w), H, dims->d_nope, dims->d_rope, dims->d_c, freqs, eps,
       qb, cb, krb) != cudaSuccess)
     return EG_MLA_ERR_CUDA;
-  // the append (first layer of a group) and the decode as one step
-  const int rc = egmla_layer_step(dims, do_kv, c_pool, krope_pool, id_pool, cb, krb, ids_new, positions, qb,
-                                  block_table, max_pages_per_seq, seq_lens, max_seq_len, batch, num_pages,
-                                  wt->gate_table, wt->ln_gamma, wt->ln_beta, wt->w_uk, wt->w_uv, ub, num_splits,
-                                  base + ws.off_dec, ws.dec_bytes, dev_status, stream);
+  rc = step(true);
   if (rc != EG_MLA_OK) return rc;
   // Eq. 14: the output projection of the heads' concatenated outputs
   if (egmla::launch_linear_tc(wt->w_o, E, nu, ub, batch, y, E, false, dev_status, st) != cudaSuccess)

@@ -142,6 +142,11 @@ def test_layer_decode_rejects_before_launch(lib):
     assert call(x=fake + 8) == _lib.EG_MLA_ERR_INVALID_ARG              # 16-byte alignment
     assert call(ws_bytes=1 << 20) == _lib.EG_MLA_ERR_WORKSPACE         # far below the layer's workspace
     assert call(batch=0) == _lib.EG_MLA_OK                              # nothing to do, nothing launched
+    # the step's own arguments, before the projections are launched
+    for name, value in (("gate_table", 0), ("gate_table", fake + 16), ("w_uk", fake + 8), ("w_uv", 0)):
+        bad = _lib.EgMlaLayerWeights(*([fake] * 8))
+        setattr(bad, name, value)
+        assert call(weights=bad, ws_bytes=1 << 24) == _lib.EG_MLA_ERR_INVALID_ARG, name
 
 
 def test_fault_entry_validates_its_arguments(lib):
